@@ -68,9 +68,12 @@ typedef enum {
     MHS_EDEVICE = 7    /* a kernel reported an internal error status */
 } mhs_status;
 
-/* How the pair counts I^E_ij / I^V_ij are contracted. */
+/* How the pairs of a pass are decided. */
 typedef enum {
-    MHS_CONTRACT_AUTO = 0,     /* library choice by size */
+    MHS_CONTRACT_AUTO = 0,     /* library choice: sparse hypergraphs by candidate lists (the pairs
+                                  that can fire, found from the incidence lists; no contraction),
+                                  others, and those whose tile shape or sparsity the options
+                                  name, as MHS_CONTRACT_FP8 */
     MHS_CONTRACT_FP8 = 1,      /* tcgen05 tensor cores, E4M3 0/1, FP32 accumulate */
     MHS_CONTRACT_POPCOUNT = 2  /* bit-packed AND + popcount on the integer units */
 } mhs_contraction;
@@ -332,13 +335,16 @@ mhs_status mhs_export(const mhs_instance *inst, int32_t index, int32_t *edge_ptr
  * Per-round device time split of the last mhs_kernelize / mhs_reduce_round
  * call, in milliseconds (CUDA events on the instance's stream):
  * ms[0] DP contraction, ms[1] MD contraction, ms[2] encode + compaction,
- * ms[3] total.  Timing is recorded only if enabled with mhs_set_timing.
+ * ms[3] total (candidate lists: the DP and MD tests, the rest, the launch;
+ * a batch's split by the sums over its instances).  Timing is recorded only
+ * if enabled with mhs_set_timing.
  */
 mhs_status mhs_set_timing(mhs_instance *inst, int32_t enable);
 /*
  * Tensor-core work done since load (tcgen05 contraction): MMA work in units
  * of 128 x 128 x 32 MACs issued, and tiles contracted.  With block-sparse
- * skipping this is below the dense formulation's count.
+ * skipping this is below the dense formulation's count; candidate lists
+ * contract nothing and count 0.
  */
 mhs_status mhs_work_stats(const mhs_instance *inst, int64_t *mma_kblocks, int64_t *mma_tiles);
 

@@ -111,6 +111,39 @@ cudaError_t launch_server_cond(cudaGraphConditionalHandle h, const BatchCounters
 cudaError_t launch_alive_masks_batch(const InstState *st, int count, uint8_t *alive_v,
                                      uint8_t *alive_e, cudaStream_t s);
 
+// ---- candidate lists instead of a contraction (sparse.cu) ----
+// What a load reads back: the list entries the first round's walks may visit
+// (summed over a batch) and the OR of the status words.
+struct SpTotals {
+    unsigned long long cost;
+    int32_t status;
+    int32_t pad;
+};
+// Time spent in the DP and MD tests and in all, summed over the instances (ns).
+struct SpTimes {
+    unsigned long long dp, md, all;
+};
+// CTAs per instance (all of the launch resident together), or 0: one CTA per
+// instance of a batch, from a queue.  nnz, items (n + m): of the largest one.
+int sparse_team(int count, int64_t nnz, int64_t items, int sms);
+// Structural checks (status bits), rows, vertex lists and the cost of every
+// instance.  The caller has zeroed every sp_ctl, sp_vrec, sp_vagg and stamp
+// array, *queue (used for team = 0) and *out.
+cudaError_t launch_sparse_build(InstState *st, int count, int team, int32_t max_rounds,
+                                int32_t *queue, SpTotals *out, int sms, cudaStream_t s);
+// At most `limit` rounds (0: to the fixpoint); adds to *ctr and *times
+// (which the caller has zeroed, like *queue).
+cudaError_t launch_sparse_rounds(InstState *st, int count, int team, int32_t limit,
+                                 BatchCounters *ctr, int32_t *queue, SpTimes *times, int sms,
+                                 cudaStream_t s);
+// One part of a sharded round of a single instance.
+enum SpPass : int {
+    kSpBegin0, kSpContract0, kSpExport0, kSpImport0,
+    kSpBegin1, kSpContract1, kSpExport1, kSpImport1, kSpEnd1
+};
+cudaError_t launch_sparse_pass(InstState *st, int team, int op, int shard, int nshards,
+                               BatchCounters *ctr, void *buf, cudaStream_t s);
+
 // tcgen05 contraction (contract_tc.cu)
 cudaError_t launch_tc_contract(InstState *st, Plan *plan, BatchCounters *ctr, int phase, int sms,
                                int tile_n, int32_t *kerr, cudaStream_t s);

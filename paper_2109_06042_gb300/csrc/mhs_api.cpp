@@ -219,6 +219,17 @@ struct Arena {
     }
 };
 
+// Sparse path: words zeroed before every launch of the rounds.
+struct SpWords {
+    BatchCounters ctr;
+    SpTimes times;
+    int32_t queue;     // next instance of a batch
+    int32_t pad;
+    SpTotals totals;   // written by the build
+    int32_t build_queue;
+    int32_t pad2;
+};
+
 struct HostInst {  // per-instance host bookkeeping
     int32_t n0, m0;
     int64_t nnz0;
@@ -275,6 +286,10 @@ struct mhs_instance {
     cudaEvent_t ev[6] = {};
     float last_ms[4] = {0, 0, 0, 0};
     int32_t rounds_done = 0;
+    // sparse path (contraction == kSparse): CTAs per instance (0: a queue)
+    // and its words in the arena
+    int sp_team = 0;
+    SpWords *sp = nullptr;
     // sharded passes (mhs_pass_*): 0 between rounds, 1 DP pass open,
     // 2 DP pass ended, 3 MD pass open
     int32_t pass_state = 0;
@@ -424,17 +439,65 @@ struct Layout {  // byte offsets inside the arena for one instance
     int64_t v_o2c, v_c2o, e_o2c, e_c2o, e_f, e_s, v_deg, v_maxf, v_cnt, e_del, v_del, forced;
     int64_t e_dirty_rb, v_dirty, v_dirty_rb, e_prev, e_rec, scan;
     int64_t A, At, Ab, Atb;
+    int64_t gone, row, pos, tmp, vedge, erec, vrec, vagg, vaux, estamp, vstamp, tstamp, task, heavy;
+    int64_t pairs, pair_tab;
+    int32_t task_cap, pair_cap;
 };
+
+// Vertices of more than 256 hyperedges (sparse.cu's limit for a group of lanes).
+inline int64_t heavy_cap(int64_t nnz) { return nnz / 257 + 1; }
+
+// Slots of the pair table: a power of two, about one per 4 hyperedges (power
+// law 20,000 x 40,000: 2,020 pairs).
+inline int64_t pair_slots(int64_t m) {
+    int64_t s = 16;
+    while (s < m / 4 && s < (1 << 20)) s <<= 1;
+    return s;
+}
+
+// Can MHS_CONTRACT_AUTO take the sparse path?  Options that name the operands
+// of the contraction ask for the contraction.
+bool auto_sparse(const mhs_options *opt) {
+    return !opt || (opt->contraction == MHS_CONTRACT_AUTO && opt->sparsity == MHS_SPARSITY_AUTO &&
+                    !opt->tile_m && !opt->tile_n && !opt->group_rows && !opt->half_stages);
+}
+
+// Does the sparse path pay?  cost: list entries its first round may visit;
+// pairs: m^2 + n^2 summed over the instances, what the contraction's
+// epilogue tests.  Measured (load and kernelization, sparse / FP8, us):
+//   n 200, m 20,000, |e| 16..32: cost 118 M, pairs 0.4 G    1240 /  768
+//   n 64, m 20,000, |e| 3..6:    cost  62 M, pairs 0.4 G     298 /  497
+//   n 16,000, m 24,000, |e| 32..64: cost 3.5 M, pairs 0.8 G  258 / 5248
+// and by the mean size, where the searches in rows and the work per
+// incidence grow:
+//   n 2,000, m 4,000, |e| 256..512: mean 384                1567 / 1302
+//   n 2,000, m 4,000, |e| 128..256: mean 192                 726 /  804
+constexpr double kSparseBase = 64e6, kSparsePerPair = 1.0 / 20;
+constexpr double kSparseMeanSize = 256;
+bool sparse_pays(double cost, double pairs) { return cost <= kSparseBase + kSparsePerPair * pairs; }
+// A lower estimate of the cost before anything is loaded: every hyperedge
+// walks one list of mean length.
+bool sparse_may_pay(int32_t count, const int32_t *n, const int32_t *m, const int64_t *nnz) {
+    double cost = 0, pairs = 0, edges = 0, inc = 0;
+    for (int32_t b = 0; b < count; ++b) {
+        if (n[b] > 0) cost += (double)m[b] * (double)nnz[b] / n[b];
+        pairs += (double)m[b] * m[b] + (double)n[b] * n[b];
+        edges += m[b];
+        inc += (double)nnz[b];
+    }
+    return inc <= kSparseMeanSize * edges && sparse_pays(cost / 4, pairs);
+}
 
 mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64_t *nnz,
                   const int64_t *k, const mhs_options *opt_in, void *cuda_stream,
-                  mhs_instance **out, std::vector<Layout> &lay, int64_t &glob_off) {
+                  mhs_instance **out, std::vector<Layout> &lay, int64_t &glob_off,
+                  bool sparse = false) {
     mhs_options opt;
     mhs_status st = check_options(opt_in, &opt);
     if (st) return st;
     auto *h = new mhs_instance();
     h->opt = opt;
-    h->contraction = opt.contraction == kPopcount ? kPopcount : kFp8;
+    h->contraction = sparse ? kSparse : opt.contraction == kPopcount ? kPopcount : kFp8;
     h->count = count;
     if (cudaGetDevice(&h->device) != cudaSuccess) {
         destroy(h);
@@ -469,7 +532,7 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
     h->sum_m = sum_m;
     int64_t c_m1 = 0, c_z = 0, c_m = 0;
     int64_t tiles_dp = 0, tiles_md = 0;
-    if (dense) {  // the tile shape: options, else the autotuner's table for this size class
+    if (dense || sparse) {  // the tile shape: options, else the autotuner's table for this size class
         int64_t rows = 0;
         for (int b = 0; b < count; ++b) rows += std::max<int64_t>(n[b], m[b]);
         h->tiles = choose_tiles(count, rows / std::max(count, 1), opt);
@@ -493,17 +556,31 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
         c_z += z;
         c_m += m0;
         L.v_o2c = ar.take(4 * n0);
-        L.v_c2o = ar.take(4 * n0);
         L.e_o2c = ar.take(4 * m0);
+        L.v_cnt = ar.take(4 * (n0 + 1));
+        L.forced = opt.full_edges ? ar.take(n0) : -1;
+        if (sparse) {
+            L.row = ar.take(4 * z);
+            L.pos = ar.take(4 * z);
+            L.tmp = ar.take(4 * z);
+            L.vedge = ar.take(8 * z);
+            L.erec = ar.take(16 * m0);
+            L.vaux = ar.take(16 * n0);
+            L.task_cap = (int32_t)std::min<int64_t>(count == 1 ? 16384 + 4 * m0 : 64 + m0 / 8, 1 << 20);
+            L.task = ar.take(16 * (int64_t)L.task_cap);
+            L.pair_cap = (int32_t)std::min<int64_t>(count == 1 ? 65536 + 64 * m0 : 256 + 2 * m0, 1 << 22);
+            L.pairs = ar.take(8 * (int64_t)L.pair_cap);
+            L.heavy = ar.take(4 * heavy_cap(z));
+            continue;
+        }
+        L.v_c2o = ar.take(4 * n0);
         L.e_c2o = ar.take(4 * m0);
         L.e_f = ar.take(4 * m0);
         L.e_s = ar.take(4 * m0);
         L.v_deg = ar.take(4 * (n0 + 1));
         L.v_maxf = ar.take(4 * n0);
-        L.v_cnt = ar.take(4 * (n0 + 1));
         L.e_del = ar.take(m0);
         L.v_del = ar.take(n0);
-        L.forced = opt.full_edges ? ar.take(n0) : -1;
         L.v_dirty = ar.take(n0);
         L.e_prev = ar.take(4 * m0);
         L.e_rec = dense ? ar.take(16 * m0) : -1;
@@ -526,7 +603,7 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
     // all zero at load: the scatter/clear passes leave them all-zero between
     // phases
     Arena ad;
-    for (int b = 0; b < count; ++b) {
+    for (int b = 0; b < count && !sparse; ++b) {
         Layout &L = lay[b];
         const int64_t n0 = n[b], m0 = m[b];
         const int64_t arows = round_up(std::max<int64_t>(m0, 1), kRowAlign);
@@ -552,17 +629,29 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
     const int64_t off_tmaps = ar.take(dense ? (int64_t)tmap_bytes() * 2 * count : 0);
     const int64_t list_cap = dense ? std::max<int64_t>(std::max(tiles_dp, tiles_md), 1) : 0;
     const int64_t off_list = ar.take(8 * list_cap);
+    const int64_t off_sp = ar.take(sparse ? (int64_t)sizeof(SpWords) : 0);
+    const int64_t off_ctl = ar.take(sparse ? (int64_t)sizeof(SpCtl) * count : 0);
+    for (int b = 0; b < count && sparse; ++b) {  // what starts at zero, with the words above
+        lay[b].vrec = ar.take(16 * (int64_t)n[b]);
+        lay[b].vagg = ar.take(16 * (int64_t)n[b]);
+        lay[b].pair_tab = ar.take((int64_t)sizeof(SpPair) * pair_slots(m[b]));
+        lay[b].gone = ar.take(4 * (((int64_t)m[b] + 31) / 32));
+        lay[b].estamp = ar.take(4 * (int64_t)m[b]);
+        lay[b].vstamp = ar.take(4 * (int64_t)n[b]);
+        lay[b].tstamp = ar.take(4 * (int64_t)n[b]);
+    }
+    const int64_t ctl_end = ar.bytes;
     glob_off = off_tmaps;
 
     cudaMemPool_t pool;
     cudaError_t ce = pool_for(h->device, &pool);
-    h->dense = zero_take(h->device, h->dense_bytes);
+    h->dense = sparse ? nullptr : zero_take(h->device, h->dense_bytes);
     h->dense_zeroed = h->dense != nullptr;
     for (int attempt = 0; attempt < 2 && ce == cudaSuccess; ++attempt) {
         if (!h->arena)
             ce = cudaMallocFromPoolAsync(reinterpret_cast<void **>(&h->arena), (size_t)ar.bytes,
                                          pool, h->stream);
-        if (ce == cudaSuccess && !h->dense)
+        if (ce == cudaSuccess && !h->dense && !sparse)
             ce = cudaMallocFromPoolAsync(reinterpret_cast<void **>(&h->dense),
                                          (size_t)h->dense_bytes, pool, h->stream);
         if (ce != cudaErrorMemoryAllocation || attempt == 1) break;
@@ -589,6 +678,7 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
     }
     h->hctr = reinterpret_cast<BatchCounters *>(h->pin);
     h->hkerr = reinterpret_cast<int32_t *>(h->pin + 64);
+    *h->hkerr = 0;
     h->hstate.resize(count);
     if (count > 1) {  // without it the copies stage through pageable memory
         h->stage_tmaps = round_up((int64_t)sizeof(InstState) * count, 128);
@@ -614,6 +704,36 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
         s.edge_rule = opt.edge_rule;
         s.full_edges = opt.full_edges;
         s.forced = L.forced >= 0 ? base + L.forced : nullptr;
+        s.eptr = reinterpret_cast<int32_t *>(base + L.eptr);
+        s.evtx = reinterpret_cast<int32_t *>(base + L.evtx);
+        s.f = reinterpret_cast<int32_t *>(base + L.f);
+        s.v_o2c = reinterpret_cast<int32_t *>(base + L.v_o2c);
+        s.e_o2c = reinterpret_cast<int32_t *>(base + L.e_o2c);
+        s.v_cnt = reinterpret_cast<int32_t *>(base + L.v_cnt);
+        if (sparse) {
+            s.sp_row = reinterpret_cast<uint32_t *>(base + L.row);
+            s.sp_pos = reinterpret_cast<int32_t *>(base + L.pos);
+            s.sp_tmp = reinterpret_cast<uint32_t *>(base + L.tmp);
+            s.sp_vedge = reinterpret_cast<unsigned long long *>(base + L.vedge);
+            s.sp_erec = reinterpret_cast<int4 *>(base + L.erec);
+            s.sp_vrec = reinterpret_cast<int4 *>(base + L.vrec);
+            s.sp_vagg = reinterpret_cast<SpAgg *>(base + L.vagg);
+            s.sp_vaux = reinterpret_cast<int4 *>(base + L.vaux);
+            s.sp_gone = reinterpret_cast<uint32_t *>(base + L.gone);
+            s.sp_estamp = reinterpret_cast<int32_t *>(base + L.estamp);
+            s.sp_vstamp = reinterpret_cast<int32_t *>(base + L.vstamp);
+            s.sp_tstamp = reinterpret_cast<int32_t *>(base + L.tstamp);
+            s.sp_task = reinterpret_cast<int4 *>(base + L.task);
+            s.sp_task_cap = L.task_cap;
+            s.sp_pair_tab = reinterpret_cast<SpPair *>(base + L.pair_tab);
+            s.sp_pair_mask = (uint32_t)pair_slots(s.m0) - 1;
+            s.sp_pairs = reinterpret_cast<int2 *>(base + L.pairs);
+            s.sp_pair_cap = L.pair_cap;
+            s.sp_heavy = reinterpret_cast<int32_t *>(base + L.heavy);
+            s.sp_ctl = reinterpret_cast<SpCtl *>(base + off_ctl) + b;
+            h->hstate[b] = s;
+            continue;
+        }
         s.v_dirty = base + L.v_dirty;
         s.e_prev = reinterpret_cast<int32_t *>(base + L.e_prev);
         s.scan_status =
@@ -625,18 +745,12 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
         s.e_rec = L.e_rec >= 0 ? reinterpret_cast<int4 *>(base + L.e_rec) : nullptr;
         s.e_dirty_rb = base + L.e_dirty_rb;
         s.v_dirty_rb = base + L.v_dirty_rb;
-        s.eptr = reinterpret_cast<int32_t *>(base + L.eptr);
-        s.evtx = reinterpret_cast<int32_t *>(base + L.evtx);
-        s.f = reinterpret_cast<int32_t *>(base + L.f);
-        s.v_o2c = reinterpret_cast<int32_t *>(base + L.v_o2c);
         s.v_c2o = reinterpret_cast<int32_t *>(base + L.v_c2o);
-        s.e_o2c = reinterpret_cast<int32_t *>(base + L.e_o2c);
         s.e_c2o = reinterpret_cast<int32_t *>(base + L.e_c2o);
         s.e_f = reinterpret_cast<int32_t *>(base + L.e_f);
         s.e_s = reinterpret_cast<int32_t *>(base + L.e_s);
         s.v_deg = reinterpret_cast<int32_t *>(base + L.v_deg);
         s.v_maxf = reinterpret_cast<int32_t *>(base + L.v_maxf);
-        s.v_cnt = reinterpret_cast<int32_t *>(base + L.v_cnt);
         s.e_del = base + L.e_del;
         s.v_del = base + L.v_del;
         const int64_t arows = round_up(std::max<int64_t>(m[b], 1), kRowAlign);
@@ -662,6 +776,23 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
             s.Atb_pitch = (int32_t)kpad_words(m[b]);
         }
         h->hstate[b] = s;
+    }
+    if (sparse) {  // control words: zero; no plan
+        h->sp = reinterpret_cast<SpWords *>(base + off_sp);
+        h->dctr = &h->sp->ctr;
+        int64_t big_nnz = 0, big_items = 0;
+        for (int b = 0; b < count; ++b) {
+            big_nnz = std::max(big_nnz, nnz[b]);
+            big_items = std::max(big_items, (int64_t)n[b] + m[b]);
+        }
+        h->sp_team = sparse_team(count, big_nnz, big_items, h->sms);
+        ce = cudaMemsetAsync(base + off_sp, 0, (size_t)(ctl_end - off_sp), h->stream);
+        if (ce != cudaSuccess) {
+            destroy(h);
+            return fail(MHS_ECUDA, "setup failed: %s", cudaGetErrorString(ce));
+        }
+        *out = h;
+        return MHS_OK;
     }
     // device plan header
     Plan p;
@@ -769,6 +900,24 @@ mhs_status finish_load(mhs_instance *h, int64_t tmap_off) {
     return MHS_OK;
 }
 
+// Sparse path, once the inputs are on their way: the states, the build
+// kernel, and what it found.  Synchronises.  *pays: the instance stays on
+// this path.
+mhs_status build_sparse(mhs_instance *h, SpTotals *found, bool *pays) {
+    CUDA_TRY(launch_sparse_build(h->dstate, h->count, h->sp_team, h->opt.max_rounds,
+                                 &h->sp->build_queue, &h->sp->totals, h->sms, h->stream));
+    SpTotals *host = reinterpret_cast<SpTotals *>(h->pin + 128);
+    CUDA_TRY(cudaMemcpyAsync(host, &h->sp->totals, sizeof(SpTotals), cudaMemcpyDeviceToHost,
+                             h->stream));
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    *found = *host;
+    double pairs = 0;
+    for (const HostInst &i : h->hinst)
+        pairs += (double)i.m0 * i.m0 + (double)i.n0 * i.n0;
+    *pays = sparse_pays((double)host->cost, pairs);
+    return MHS_OK;
+}
+
 const char *status_text(int32_t st) {
     if (st & kErrBadVertex) return "vertex id out of range";
     if (st & kErrBadPtr) return "bad edge_ptr";
@@ -776,6 +925,34 @@ const char *status_text(int32_t st) {
     if (st & kErrCapacity) return "index beyond capacity";
     if (st & kErrTimeout) return "bounded wait timed out";
     return "unknown";
+}
+
+// The end of a load on the sparse path (inputs and states are on their
+// way): build and checks.  *again: the
+// instance is better contracted (the caller loads it again on that path).
+// On an error or *again the caller destroys the handle.
+mhs_status finish_sparse(mhs_instance *h, bool *again) {
+    SpTotals found;
+    bool pays = true;
+    mhs_status st = build_sparse(h, &found, &pays);
+    if (st) return st;
+    if (found.status) {
+        if (h->count == 1)
+            return fail(MHS_EINVAL, "malformed device instance (status 0x%x: %s)", found.status,
+                        status_text(found.status));
+        // read the states to name the first
+        std::vector<InstState> chk(h->count);
+        CUDA_TRY(cudaMemcpyAsync(chk.data(), h->dstate, sizeof(InstState) * h->count,
+                                 cudaMemcpyDeviceToHost, h->stream));
+        CUDA_TRY(cudaStreamSynchronize(h->stream));
+        for (int b = 0; b < h->count; ++b)
+            if (chk[b].status)
+                return fail(MHS_EINVAL, "instance %d malformed (status 0x%x: %s)", b,
+                            chk[b].status, status_text(chk[b].status));
+        return fail(MHS_ECUDA, "batch device load: status read back inconsistent");
+    }
+    *again = !pays;
+    return MHS_OK;
 }
 
 mhs_status check_device_status(mhs_instance *h) {
@@ -888,9 +1065,50 @@ mhs_status build_loop_graph(mhs_instance *h) {
     return MHS_OK;
 }
 
+void stats_from(const BatchCounters &c, mhs_round_stats *stats) {
+    stats->n_alive = c.n_alive;
+    stats->m_alive = c.m_alive;
+    stats->rounds = c.max_rounds_seen;
+    stats->changed = c.changed_any;
+    stats->dp_deleted = c.dp_deleted;
+    stats->md_deleted = c.md_deleted;
+    stats->active = c.active;
+}
+
+// Rounds of the sparse path: one launch.
+mhs_status run_sparse(mhs_instance *h, int32_t limit, mhs_round_stats *stats) {
+    if (h->timing)
+        for (auto &e : h->ev)
+            if (!e) CUDA_TRY(cudaEventCreate(&e));
+    CUDA_TRY(cudaMemsetAsync(h->sp, 0, offsetof(SpWords, totals), h->stream));
+    if (h->timing) CUDA_TRY(cudaEventRecord(h->ev[4], h->stream));
+    CUDA_TRY(launch_sparse_rounds(h->dstate, h->count, h->sp_team, limit, &h->sp->ctr,
+                                  &h->sp->queue, &h->sp->times, h->sms, h->stream));
+    if (h->timing) CUDA_TRY(cudaEventRecord(h->ev[5], h->stream));
+    CUDA_TRY(cudaMemcpyAsync(h->hctr, &h->sp->ctr, sizeof(BatchCounters), cudaMemcpyDeviceToHost,
+                             h->stream));
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    if (h->timing) {  // the launch's time, split by where its lead threads spent theirs
+        SpTimes t;
+        CUDA_TRY(cudaMemcpy(&t, &h->sp->times, sizeof(t), cudaMemcpyDeviceToHost));
+        float ms = 0;
+        cudaEventElapsedTime(&ms, h->ev[4], h->ev[5]);
+        const double all = std::max<double>((double)t.all, 1.0);
+        h->last_ms[0] = (float)(ms * (double)t.dp / all);
+        h->last_ms[1] = (float)(ms * (double)t.md / all);
+        h->last_ms[2] = ms - h->last_ms[0] - h->last_ms[1];
+        h->last_ms[3] = ms;
+    }
+    mhs_status st = check_device_status(h);
+    if (st) return st;
+    if (stats) stats_from(*h->hctr, stats);
+    return MHS_OK;
+}
+
 mhs_status run_rounds(mhs_instance *h, int32_t limit, mhs_round_stats *stats) {
     if (h->pass_state != 0)
         return fail(MHS_EINVAL, "a sharded round is in progress (finish it with mhs_pass_end)");
+    if (h->contraction == kSparse) return run_sparse(h, limit, stats);
     if (limit <= 0 && h->opt.use_graphs && !h->timing) {
         if (!h->loop_graph) {
             mhs_status st = build_loop_graph(h);
@@ -902,15 +1120,7 @@ mhs_status run_rounds(mhs_instance *h, int32_t limit, mhs_round_stats *stats) {
             return fail(MHS_EDEVICE, "device round loop reached its cap of %d rounds", h->round_cap);
         mhs_status st = check_device_status(h);
         if (st) return st;
-        if (stats) {
-            stats->n_alive = h->hctr->n_alive;
-            stats->m_alive = h->hctr->m_alive;
-            stats->rounds = h->hctr->max_rounds_seen;
-            stats->changed = h->hctr->changed_any;
-            stats->dp_deleted = h->hctr->dp_deleted;
-            stats->md_deleted = h->hctr->md_deleted;
-            stats->active = h->hctr->active;
-        }
+        if (stats) stats_from(*h->hctr, stats);
         return MHS_OK;
     }
     if (h->timing) {
@@ -948,17 +1158,8 @@ mhs_status run_rounds(mhs_instance *h, int32_t limit, mhs_round_stats *stats) {
         if (h->hctr->active == 0) break;
     }
     if (stats) {
-        if (any) {
-            stats->n_alive = h->hctr->n_alive;
-            stats->m_alive = h->hctr->m_alive;
-            stats->rounds = h->hctr->max_rounds_seen;
-            stats->changed = h->hctr->changed_any;
-            stats->dp_deleted = h->hctr->dp_deleted;
-            stats->md_deleted = h->hctr->md_deleted;
-            stats->active = h->hctr->active;
-        } else {
-            std::memset(stats, 0, sizeof(*stats));
-        }
+        if (any) stats_from(*h->hctr, stats);
+        else std::memset(stats, 0, sizeof(*stats));
     }
     return MHS_OK;
 }
@@ -997,59 +1198,80 @@ mhs_status mhs_load(int32_t n, int32_t m, const int32_t *edge_ptr, const int32_t
         }
     if (m > 0 && edge_ptr[m] > 0 && !edge_vtx) return fail(MHS_EINVAL, "edge_vtx is NULL");
     int64_t nnz = edge_ptr[m];
-    std::vector<Layout> lay;
-    int64_t tmoff = 0;
-    mhs_instance *h = nullptr;
-    mhs_status st = create(1, &n, &m, &nnz, &k, opt, cuda_stream, &h, lay, tmoff);
-    if (st) return st;
     // The host checks the incidences, several threads each taking a range
     // of hyperedges and, once it has checked it, copying the range into
     // page-locked staging (a buffer of its own, nothing else writes it while
     // the copies run); the copies to the device follow.  Without staging the
     // inputs are copied from the caller's arrays while the host checks them.
     // No kernel reads them before the checks have passed.
-    const InstState &s = h->hstate[0];
     const size_t b_ptr = 4 * ((size_t)m + 1), b_vtx = 4 * (size_t)nnz, b_f = 4 * (size_t)m;
-    h->in_stage = static_cast<uint8_t *>(pinned_take(b_ptr + b_vtx + b_f, &h->in_stage_cls));
-    const void *src_ptr = edge_ptr, *src_vtx = edge_vtx, *src_f = demand;
-    if (uint8_t *in = h->in_stage) {
-        st = validate_host_parallel(n, m, edge_ptr, edge_vtx, demand, nnz, "instance", in);
+    uint8_t *stage = nullptr;  // kept over a second try on the other path
+    size_t stage_cls = 0;
+    bool checked = false;
+    bool sparse = auto_sparse(opt) && sparse_may_pay(1, &n, &m, &nnz);
+    for (;;) {
+        std::vector<Layout> lay;
+        int64_t tmoff = 0;
+        mhs_instance *h = nullptr;
+        mhs_status st = create(1, &n, &m, &nnz, &k, opt, cuda_stream, &h, lay, tmoff, sparse);
+        if (st) {
+            pinned_give(stage, stage_cls);
+            return st;
+        }
+        if (!checked) stage = static_cast<uint8_t *>(pinned_take(b_ptr + b_vtx + b_f, &stage_cls));
+        h->in_stage = stage;
+        h->in_stage_cls = stage_cls;
+        const InstState &s = h->hstate[0];
+        const void *src_ptr = edge_ptr, *src_vtx = edge_vtx, *src_f = demand;
+        if (stage) {
+            if (!checked)
+                st = validate_host_parallel(n, m, edge_ptr, edge_vtx, demand, nnz, "instance", stage);
+            if (st) {
+                destroy(h);
+                return st;
+            }
+            checked = true;
+            src_ptr = stage;
+            src_vtx = stage + b_ptr;
+            src_f = stage + b_ptr + b_vtx;
+        }
+        cudaError_t e = cudaMemcpyAsync(const_cast<int32_t *>(s.eptr), src_ptr, b_ptr,
+                                        cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess && b_vtx)
+            e = cudaMemcpyAsync(const_cast<int32_t *>(s.evtx), src_vtx, b_vtx,
+                                cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess && b_f)
+            e = cudaMemcpyAsync(const_cast<int32_t *>(s.f), src_f, b_f, cudaMemcpyHostToDevice,
+                                h->stream);
+        if (e != cudaSuccess) {
+            destroy(h);
+            return fail(MHS_ECUDA, "input copy failed: %s", cudaGetErrorString(e));
+        }
+        if (!checked) {
+            st = validate_host_parallel(n, m, edge_ptr, edge_vtx, demand, nnz, "instance");
+            if (st) {
+                destroy(h);  // (waits for the copies)
+                return st;
+            }
+            checked = true;
+        }
+        bool again = false;
+        if (sparse && upload_states(h) != cudaSuccess) st = fail(MHS_ECUDA, "state copy failed");
+        else st = sparse ? finish_sparse(h, &again) : finish_load(h, tmoff);
+        if (st == MHS_OK && !sparse && cudaStreamSynchronize(h->stream) != cudaSuccess)
+            st = fail(MHS_ECUDA, "load failed: %s", cudaGetErrorString(cudaGetLastError()));
         if (st) {
             destroy(h);
             return st;
         }
-        src_ptr = in;
-        src_vtx = in + b_ptr;
-        src_f = in + b_ptr + b_vtx;
-    }
-    cudaError_t e = cudaMemcpyAsync(const_cast<int32_t *>(s.eptr), src_ptr, b_ptr,
-                                    cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess && b_vtx)
-        e = cudaMemcpyAsync(const_cast<int32_t *>(s.evtx), src_vtx, b_vtx, cudaMemcpyHostToDevice,
-                            h->stream);
-    if (e == cudaSuccess && b_f)
-        e = cudaMemcpyAsync(const_cast<int32_t *>(s.f), src_f, b_f, cudaMemcpyHostToDevice,
-                            h->stream);
-    if (e != cudaSuccess) {
-        destroy(h);
-        return fail(MHS_ECUDA, "input copy failed: %s", cudaGetErrorString(e));
-    }
-    if (!h->in_stage) {
-        st = validate_host_parallel(n, m, edge_ptr, edge_vtx, demand, nnz, "instance");
-        if (st) {
-            destroy(h);  // (waits for the copies)
-            return st;
+        if (!again) {
+            *out = h;
+            return MHS_OK;
         }
-    }
-    st = finish_load(h, tmoff);
-    if (st == MHS_OK && cudaStreamSynchronize(h->stream) != cudaSuccess)
-        st = fail(MHS_ECUDA, "load failed: %s", cudaGetErrorString(cudaGetLastError()));
-    if (st) {
+        h->in_stage = nullptr;  // the second try copies from it
         destroy(h);
-        return st;
+        sparse = false;
     }
-    *out = h;
-    return MHS_OK;
 }
 
 mhs_status mhs_load_device(int32_t n, int32_t m, const int32_t *edge_ptr, const int32_t *edge_vtx,
@@ -1067,44 +1289,58 @@ mhs_status mhs_load_device(int32_t n, int32_t m, const int32_t *edge_ptr, const 
     if (nnz32 < 0) return fail(MHS_EINVAL, "edge_ptr[m] < 0");
     if (nnz32 > 0 && !edge_vtx) return fail(MHS_EINVAL, "edge_vtx is NULL");
     int64_t nnz = nnz32;
-    std::vector<Layout> lay;
-    int64_t tmoff = 0;
-    mhs_instance *h = nullptr;
-    mhs_status st = create(1, &n, &m, &nnz, &k, opt, cuda_stream, &h, lay, tmoff);
-    if (st) return st;
-    InstState &s = h->hstate[0];
-    cudaError_t e = cudaMemcpyAsync(const_cast<int32_t *>(s.eptr), edge_ptr, 4 * ((size_t)m + 1),
-                                    cudaMemcpyDeviceToDevice, h->stream);
-    if (e == cudaSuccess && nnz > 0)
-        e = cudaMemcpyAsync(const_cast<int32_t *>(s.evtx), edge_vtx, 4 * (size_t)nnz,
-                            cudaMemcpyDeviceToDevice, h->stream);
-    if (e == cudaSuccess && m > 0)
-        e = cudaMemcpyAsync(const_cast<int32_t *>(s.f), demand, 4 * (size_t)m,
-                            cudaMemcpyDeviceToDevice, h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(h->dstate, h->hstate.data(), sizeof(InstState), cudaMemcpyHostToDevice,
-                            h->stream);
-    if (e == cudaSuccess) e = launch_validate(h->dstate, 1, h->stream);
-    int32_t status = 0;
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&status, &h->dstate->status, 4, cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) {
-        destroy(h);
-        return fail(MHS_ECUDA, "device load failed: %s", cudaGetErrorString(e));
+    for (bool sparse = auto_sparse(opt) && sparse_may_pay(1, &n, &m, &nnz);; sparse = false) {
+        std::vector<Layout> lay;
+        int64_t tmoff = 0;
+        mhs_instance *h = nullptr;
+        mhs_status st = create(1, &n, &m, &nnz, &k, opt, cuda_stream, &h, lay, tmoff, sparse);
+        if (st) return st;
+        InstState &s = h->hstate[0];
+        cudaError_t e = cudaMemcpyAsync(const_cast<int32_t *>(s.eptr), edge_ptr,
+                                        4 * ((size_t)m + 1), cudaMemcpyDeviceToDevice, h->stream);
+        if (e == cudaSuccess && nnz > 0)
+            e = cudaMemcpyAsync(const_cast<int32_t *>(s.evtx), edge_vtx, 4 * (size_t)nnz,
+                                cudaMemcpyDeviceToDevice, h->stream);
+        if (e == cudaSuccess && m > 0)
+            e = cudaMemcpyAsync(const_cast<int32_t *>(s.f), demand, 4 * (size_t)m,
+                                cudaMemcpyDeviceToDevice, h->stream);
+        bool again = false;
+        if (e == cudaSuccess && sparse) e = upload_states(h);
+        if (e == cudaSuccess && sparse) {
+            st = finish_sparse(h, &again);
+            if (st || again) {
+                destroy(h);
+                if (st) return st;
+                continue;
+            }
+            *out = h;
+            return MHS_OK;
+        }
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(h->dstate, h->hstate.data(), sizeof(InstState),
+                                cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess) e = launch_validate(h->dstate, 1, h->stream);
+        int32_t status = 0;
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(&status, &h->dstate->status, 4, cudaMemcpyDeviceToHost, h->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        if (e != cudaSuccess) {
+            destroy(h);
+            return fail(MHS_ECUDA, "device load failed: %s", cudaGetErrorString(e));
+        }
+        if (status) {
+            destroy(h);
+            return fail(MHS_EINVAL, "malformed device instance (status 0x%x: %s)", status,
+                        status_text(status));
+        }
+        st = finish_load(h, tmoff);  // device inputs: nothing to wait for before returning
+        if (st) {
+            destroy(h);
+            return st;
+        }
+        *out = h;
+        return MHS_OK;
     }
-    if (status) {
-        destroy(h);
-        return fail(MHS_EINVAL, "malformed device instance (status 0x%x: %s)", status,
-                    status_text(status));
-    }
-    st = finish_load(h, tmoff);  // device inputs: nothing to wait for before returning
-    if (st) {
-        destroy(h);
-        return st;
-    }
-    *out = h;
-    return MHS_OK;
 }
 
 mhs_status mhs_load_batch(int32_t count, const int32_t *n, const int32_t *m,
@@ -1206,81 +1442,83 @@ mhs_status mhs_load_batch(int32_t count, const int32_t *n, const int32_t *m,
                                       demand + eoff[bad], mark, 0, what);
         return st ? st : fail(MHS_EINVAL, "%s: malformed", what);
     };
-    std::vector<Layout> lay;
-    int64_t tmoff = 0;
-    mhs_instance *h = nullptr;
-    mhs_status st = create(count, n, m, nnz.data(), k, opt, cuda_stream, &h, lay, tmoff);
-    if (st) {  // a malformed input is reported first, as a check before the allocation would
-        const std::string msg = g_err;
-        const mhs_status vst = finish_checks();
-        pinned_give(stage, stage_cls);
-        if (vst) return vst;
-        return fail(st, "%s", msg.c_str());
-    }
-    if (stage) {  // checked and staged: three copies; the buffer lives as long as the handle
-        h->in_stage = stage;
-        h->in_stage_cls = stage_cls;
-        st = finish_checks();
-        if (st) {
-            destroy(h);
-            return st;
+    std::vector<int32_t> local_ptr;  // (without staging) local int32 offsets
+    bool sparse = auto_sparse(opt) && sparse_may_pay(count, n, m, nnz.data());
+    for (bool first = true;; first = false, sparse = false) {
+        std::vector<Layout> lay;
+        int64_t tmoff = 0;
+        mhs_instance *h = nullptr;
+        mhs_status st =
+            create(count, n, m, nnz.data(), k, opt, cuda_stream, &h, lay, tmoff, sparse);
+        if (st) {  // a malformed input is reported first, as a check before the allocation would
+            const std::string msg = g_err;
+            const mhs_status vst = first ? finish_checks() : MHS_OK;
+            pinned_give(stage, stage_cls);
+            if (vst) return vst;
+            return fail(st, "%s", msg.c_str());
         }
-        cudaError_t e = cudaMemcpyAsync(h->arena + h->in_eptr, s_ptr, 4 * (size_t)sum_m1,
-                                        cudaMemcpyHostToDevice, h->stream);
-        if (e == cudaSuccess && sum_z > 0)
-            e = cudaMemcpyAsync(h->arena + h->in_evtx, s_vtx, 4 * (size_t)sum_z,
+        cudaError_t e = cudaSuccess;
+        if (stage) {  // checked and staged: three copies; the buffer lives as long as the handle
+            h->in_stage = stage;
+            h->in_stage_cls = stage_cls;
+            if (first) st = finish_checks();
+            if (st) {
+                destroy(h);
+                return st;
+            }
+            e = cudaMemcpyAsync(h->arena + h->in_eptr, s_ptr, 4 * (size_t)sum_m1,
                                 cudaMemcpyHostToDevice, h->stream);
-        if (e == cudaSuccess && sum_m > 0)
-            e = cudaMemcpyAsync(h->arena + h->in_f, s_f, 4 * (size_t)sum_m,
+            if (e == cudaSuccess && sum_z > 0)
+                e = cudaMemcpyAsync(h->arena + h->in_evtx, s_vtx, 4 * (size_t)sum_z,
+                                    cudaMemcpyHostToDevice, h->stream);
+            if (e == cudaSuccess && sum_m > 0)
+                e = cudaMemcpyAsync(h->arena + h->in_f, s_f, 4 * (size_t)sum_m,
+                                    cudaMemcpyHostToDevice, h->stream);
+        } else {  // one copy per input array, from the caller's
+            if (first) {
+                local_ptr.resize((size_t)h->sum_m1);
+                size_t w = 0;
+                for (int b = 0; b < count; ++b) {
+                    const int64_t e0 = eoff[b];
+                    for (int32_t i = 0; i <= m[b]; ++i)
+                        local_ptr[w++] = (int32_t)(edge_ptr[e0 + i] - edge_ptr[e0]);
+                }
+            }
+            e = cudaMemcpyAsync(h->arena + h->in_eptr, local_ptr.data(), 4 * local_ptr.size(),
                                 cudaMemcpyHostToDevice, h->stream);
-        if (e == cudaSuccess) st = finish_load(h, tmoff);
-        else st = fail(MHS_ECUDA, "input copy failed: %s", cudaGetErrorString(e));
-        if (st == MHS_OK && cudaStreamSynchronize(h->stream) != cudaSuccess)
+            if (e == cudaSuccess && h->sum_nnz > 0)
+                e = cudaMemcpyAsync(h->arena + h->in_evtx, edge_vtx, 4 * (size_t)h->sum_nnz,
+                                    cudaMemcpyHostToDevice, h->stream);
+            if (e == cudaSuccess && h->sum_m > 0)
+                e = cudaMemcpyAsync(h->arena + h->in_f, demand, 4 * (size_t)h->sum_m,
+                                    cudaMemcpyHostToDevice, h->stream);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);  // local_ptr is pageable
+            if (first) st = finish_checks();
+            if (st) {
+                destroy(h);
+                return st;
+            }
+        }
+        if (e != cudaSuccess) {
+            destroy(h);
+            return fail(MHS_ECUDA, "input copy failed: %s", cudaGetErrorString(e));
+        }
+        bool again = false;
+        if (sparse && upload_states(h) != cudaSuccess) st = fail(MHS_ECUDA, "state copy failed");
+        else st = sparse ? finish_sparse(h, &again) : finish_load(h, tmoff);
+        if (st == MHS_OK && !sparse && cudaStreamSynchronize(h->stream) != cudaSuccess)
             st = fail(MHS_ECUDA, "load failed");
         if (st) {
             destroy(h);
             return st;
         }
-        *out = h;
-        return MHS_OK;
-    }
-    // one copy per input array: local int32 offsets, vertex ids, demands
-    std::vector<int32_t> local_ptr((size_t)h->sum_m1);
-    {
-        size_t w = 0;
-        for (int b = 0; b < count; ++b) {
-            const int64_t e0 = eoff[b];
-            for (int32_t i = 0; i <= m[b]; ++i)
-                local_ptr[w++] = (int32_t)(edge_ptr[e0 + i] - edge_ptr[e0]);
+        if (!again) {
+            *out = h;
+            return MHS_OK;
         }
-    }
-    cudaError_t e = cudaMemcpyAsync(h->arena + h->in_eptr, local_ptr.data(), 4 * local_ptr.size(),
-                                    cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess && h->sum_nnz > 0)
-        e = cudaMemcpyAsync(h->arena + h->in_evtx, edge_vtx, 4 * (size_t)h->sum_nnz,
-                            cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess && h->sum_m > 0)
-        e = cudaMemcpyAsync(h->arena + h->in_f, demand, 4 * (size_t)h->sum_m,
-                            cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);  // local_ptr is pageable
-    st = finish_checks();
-    if (st) {
+        h->in_stage = nullptr;  // the second try copies from it
         destroy(h);
-        return st;
     }
-    if (e != cudaSuccess) {
-        destroy(h);
-        return fail(MHS_ECUDA, "input copy failed: %s", cudaGetErrorString(e));
-    }
-    st = finish_load(h, tmoff);
-    if (st == MHS_OK && cudaStreamSynchronize(h->stream) != cudaSuccess)
-        st = fail(MHS_ECUDA, "load failed");
-    if (st) {
-        destroy(h);
-        return st;
-    }
-    *out = h;
-    return MHS_OK;
 }
 
 mhs_status mhs_load_batch_device(int32_t count, const int32_t *n, const int32_t *m,
@@ -1340,63 +1578,78 @@ mhs_status mhs_load_batch_device(int32_t count, const int32_t *n, const int32_t 
         cudaFreeAsync(tmp, cs);
         return fail(MHS_EINVAL, "edge_vtx is NULL");
     }
-    std::vector<Layout> lay;
-    int64_t tmoff = 0;
-    mhs_instance *h = nullptr;
-    mhs_status st = create(count, n, m, nnz.data(), k, opt, cuda_stream, &h, lay, tmoff);
-    if (st) {
-        cudaFreeAsync(tmp, cs);
-        return st;
-    }
-    // device-to-device: vertex ids and demands in one copy each, local offsets by a kernel
-    e = cudaSuccess;
-    if (h->sum_nnz > 0)
-        e = cudaMemcpyAsync(h->arena + h->in_evtx, edge_vtx, 4 * (size_t)h->sum_nnz,
-                            cudaMemcpyDeviceToDevice, h->stream);
-    if (e == cudaSuccess && h->sum_m > 0)
-        e = cudaMemcpyAsync(h->arena + h->in_f, demand, 4 * (size_t)h->sum_m,
-                            cudaMemcpyDeviceToDevice, h->stream);
-    if (e == cudaSuccess) e = upload_states(h);
-    if (e == cudaSuccess) e = launch_localize_ptr(h->dstate, count, edge_ptr, tmp, h->stream);
-    if (e == cudaSuccess) e = launch_validate(h->dstate, count, h->stream);
-    int32_t *any_status = reinterpret_cast<int32_t *>(tmp + 2 * ((int64_t)count + 1));
-    int32_t hany = 0;
-    if (e == cudaSuccess) e = cudaMemsetAsync(any_status, 0, sizeof(int32_t), h->stream);
-    if (e == cudaSuccess) e = launch_status_or(h->dstate, count, any_status, h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&hany, any_status, sizeof(int32_t), cudaMemcpyDeviceToHost,
-                            h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    cudaFreeAsync(tmp, h->stream);
-    if (e != cudaSuccess) {
-        destroy(h);
-        return fail(MHS_ECUDA, "batch device load: %s", cudaGetErrorString(e));
-    }
-    if (hany) {  // some instance is malformed: read the states to name the first
-        std::vector<InstState> chk(count);
-        e = cudaMemcpyAsync(chk.data(), h->dstate, sizeof(InstState) * count,
-                            cudaMemcpyDeviceToHost, h->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-        for (int b = 0; e == cudaSuccess && b < count; ++b)
-            if (chk[b].status) {
-                const int32_t sv = chk[b].status;
+    for (bool sparse = auto_sparse(opt) && sparse_may_pay(count, n, m, nnz.data());; sparse = false) {
+        std::vector<Layout> lay;
+        int64_t tmoff = 0;
+        mhs_instance *h = nullptr;
+        mhs_status st =
+            create(count, n, m, nnz.data(), k, opt, cuda_stream, &h, lay, tmoff, sparse);
+        if (st) {
+            cudaFreeAsync(tmp, cs);
+            return st;
+        }
+        // device-to-device: vertex ids and demands in one copy each, local offsets by a kernel
+        e = cudaSuccess;
+        if (h->sum_nnz > 0)
+            e = cudaMemcpyAsync(h->arena + h->in_evtx, edge_vtx, 4 * (size_t)h->sum_nnz,
+                                cudaMemcpyDeviceToDevice, h->stream);
+        if (e == cudaSuccess && h->sum_m > 0)
+            e = cudaMemcpyAsync(h->arena + h->in_f, demand, 4 * (size_t)h->sum_m,
+                                cudaMemcpyDeviceToDevice, h->stream);
+        if (e == cudaSuccess) e = upload_states(h);
+        if (e == cudaSuccess) e = launch_localize_ptr(h->dstate, count, edge_ptr, tmp, h->stream);
+        if (e == cudaSuccess && sparse) {
+            bool again = false;
+            st = finish_sparse(h, &again);
+            if (st || !again) cudaFreeAsync(tmp, h->stream);
+            if (st || again) {
                 destroy(h);
-                return fail(MHS_EINVAL, "instance %d malformed (status 0x%x: %s)", b, sv,
-                            status_text(sv));
+                if (st) return st;
+                continue;
             }
-        destroy(h);
-        return fail(MHS_ECUDA, "batch device load: %s",
-                    e != cudaSuccess ? cudaGetErrorString(e) : "status read back inconsistent");
+            *out = h;
+            return MHS_OK;
+        }
+        if (e == cudaSuccess) e = launch_validate(h->dstate, count, h->stream);
+        int32_t *any_status = reinterpret_cast<int32_t *>(tmp + 2 * ((int64_t)count + 1));
+        int32_t hany = 0;
+        if (e == cudaSuccess) e = cudaMemsetAsync(any_status, 0, sizeof(int32_t), h->stream);
+        if (e == cudaSuccess) e = launch_status_or(h->dstate, count, any_status, h->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(&hany, any_status, sizeof(int32_t), cudaMemcpyDeviceToHost,
+                                h->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        cudaFreeAsync(tmp, h->stream);
+        if (e != cudaSuccess) {
+            destroy(h);
+            return fail(MHS_ECUDA, "batch device load: %s", cudaGetErrorString(e));
+        }
+        if (hany) {  // some instance is malformed: read the states to name the first
+            std::vector<InstState> chk(count);
+            e = cudaMemcpyAsync(chk.data(), h->dstate, sizeof(InstState) * count,
+                                cudaMemcpyDeviceToHost, h->stream);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+            for (int b = 0; e == cudaSuccess && b < count; ++b)
+                if (chk[b].status) {
+                    const int32_t sv = chk[b].status;
+                    destroy(h);
+                    return fail(MHS_EINVAL, "instance %d malformed (status 0x%x: %s)", b, sv,
+                                status_text(sv));
+                }
+            destroy(h);
+            return fail(MHS_ECUDA, "batch device load: %s",
+                        e != cudaSuccess ? cudaGetErrorString(e) : "status read back inconsistent");
+        }
+        st = finish_load(h, tmoff);
+        if (st == MHS_OK && cudaStreamSynchronize(h->stream) != cudaSuccess)
+            st = fail(MHS_ECUDA, "load failed");
+        if (st) {
+            destroy(h);
+            return st;
+        }
+        *out = h;
+        return MHS_OK;
     }
-    st = finish_load(h, tmoff);
-    if (st == MHS_OK && cudaStreamSynchronize(h->stream) != cudaSuccess)
-        st = fail(MHS_ECUDA, "load failed");
-    if (st) {
-        destroy(h);
-        return st;
-    }
-    *out = h;
-    return MHS_OK;
 }
 
 int32_t mhs_count(const mhs_instance *inst) { return inst ? inst->count : 0; }
@@ -1432,13 +1685,43 @@ mhs_status pass_check(const mhs_instance *h, int32_t phase, bool open) {
 }
 }  // namespace
 
+namespace {
+cudaError_t pass_exchange(const mhs_instance *h, int phase, int import, void *buf) {
+    if (h->contraction != kSparse)
+        return launch_pass_exchange(h->dstate, phase, import, buf, h->sms, h->stream);
+    const int op = import ? (phase == 0 ? kSpImport0 : kSpImport1)
+                          : (phase == 0 ? kSpExport0 : kSpExport1);
+    return launch_sparse_pass(h->dstate, h->sp_team, op, 0, 1, nullptr, buf, h->stream);
+}
+
+// The end of a pass: the decision, and for MD the round's books and FE.
+cudaError_t pass_finish(mhs_instance *h, int phase) {
+    if (h->contraction == kSparse) {
+        if (phase == 0) return cudaSuccess;  // DP's deletions are booked with MD's
+        cudaError_t e = cudaMemsetAsync(&h->sp->ctr, 0, sizeof(BatchCounters), h->stream);
+        if (e != cudaSuccess) return e;
+        return launch_sparse_pass(h->dstate, h->sp_team, kSpEnd1, 0, 1, &h->sp->ctr, nullptr,
+                                  h->stream);
+    }
+    cudaError_t e = launch_phase_epilogue(h->dstate, h->dplan, h->dctr, 1, phase, h->contraction,
+                                          h->sms, h->stream, nullptr, h->compact_blocks);
+    if (e == cudaSuccess && phase == 1 && h->opt.full_edges)
+        e = launch_full_edges(h->dstate, 1, h->dctr, nullptr, h->sms, h->stream);
+    return e;
+}
+}  // namespace
+
 mhs_status mhs_pass_begin(mhs_instance *inst, int32_t phase) {
     mhs_status st = pass_check(inst, phase, false);
     if (st) return st;
     if (inst->opt.full_edges && inst->opt.max_rounds)
         return fail(MHS_EINVAL, "full_edges needs max_rounds = 0");
-    CUDA_TRY(launch_phase_prologue(inst->dstate, inst->dplan, inst->dctr, phase, inst->contraction,
-                                   inst->sms, inst->stream));
+    if (inst->contraction == kSparse)
+        CUDA_TRY(launch_sparse_pass(inst->dstate, inst->sp_team, phase == 0 ? kSpBegin0 : kSpBegin1,
+                                    0, 1, nullptr, nullptr, inst->stream));
+    else
+        CUDA_TRY(launch_phase_prologue(inst->dstate, inst->dplan, inst->dctr, phase,
+                                       inst->contraction, inst->sms, inst->stream));
     inst->pass_state = phase == 0 ? 1 : 3;
     return MHS_OK;
 }
@@ -1448,6 +1731,12 @@ mhs_status mhs_pass_contract(mhs_instance *inst, int32_t phase, int32_t shard, i
     if (st) return st;
     if (nshards < 1 || nshards > 4096 || shard < 0 || shard >= nshards)
         return fail(MHS_EINVAL, "need 1 <= nshards <= 4096 and 0 <= shard < nshards");
+    if (inst->contraction == kSparse) {
+        CUDA_TRY(launch_sparse_pass(inst->dstate, inst->sp_team,
+                                    phase == 0 ? kSpContract0 : kSpContract1, shard, nshards,
+                                    nullptr, nullptr, inst->stream));
+        return MHS_OK;
+    }
     CUDA_TRY(launch_phase_contract(inst->dstate, inst->dplan, inst->dctr, phase,
                                    inst->contraction, inst->sms, inst->dkerr, inst->stream,
                                    inst->tiles.tile_n, shard, nshards));
@@ -1462,7 +1751,7 @@ mhs_status mhs_pass_partial(const mhs_instance *inst, int32_t phase, void *dev_o
     const int64_t elems = phase == 0 ? s.m0 : s.n0;
     if (elems_out) *elems_out = elems;
     if (dev_out && elems > 0) {
-        CUDA_TRY(launch_pass_exchange(inst->dstate, phase, 0, dev_out, inst->sms, inst->stream));
+        CUDA_TRY(pass_exchange(inst, phase, 0, dev_out));
         CUDA_TRY(cudaStreamSynchronize(inst->stream));
     }
     return MHS_OK;
@@ -1475,8 +1764,7 @@ mhs_status mhs_pass_merge(mhs_instance *inst, int32_t phase, const void *dev_in)
     const InstState &s = inst->hstate[0];
     const int64_t elems = phase == 0 ? s.m0 : s.n0;
     if (elems > 0) {
-        CUDA_TRY(launch_pass_exchange(inst->dstate, phase, 1, const_cast<void *>(dev_in),
-                                      inst->sms, inst->stream));
+        CUDA_TRY(pass_exchange(inst, phase, 1, const_cast<void *>(dev_in)));
         CUDA_TRY(cudaStreamSynchronize(inst->stream));
     }
     return MHS_OK;
@@ -1485,11 +1773,7 @@ mhs_status mhs_pass_merge(mhs_instance *inst, int32_t phase, const void *dev_in)
 mhs_status mhs_pass_end(mhs_instance *inst, int32_t phase, mhs_round_stats *stats) {
     mhs_status st = pass_check(inst, phase, true);
     if (st) return st;
-    cudaError_t e = launch_phase_epilogue(inst->dstate, inst->dplan, inst->dctr, 1, phase,
-                                          inst->contraction, inst->sms, inst->stream, nullptr,
-                                          inst->compact_blocks);
-    if (e == cudaSuccess && phase == 1 && inst->opt.full_edges)
-        e = launch_full_edges(inst->dstate, 1, inst->dctr, nullptr, inst->sms, inst->stream);
+    const cudaError_t e = pass_finish(inst, phase);
     if (e != cudaSuccess) {
         inst->faulted = true;
         return fail(MHS_ECUDA, "pass end: %s", cudaGetErrorString(e));
@@ -1501,20 +1785,13 @@ mhs_status mhs_pass_end(mhs_instance *inst, int32_t phase, mhs_round_stats *stat
     }
     CUDA_TRY(cudaMemcpyAsync(inst->hctr, inst->dctr, sizeof(BatchCounters), cudaMemcpyDeviceToHost,
                              inst->stream));
-    CUDA_TRY(cudaMemcpyAsync(inst->hkerr, inst->dkerr, sizeof(int32_t), cudaMemcpyDeviceToHost,
-                             inst->stream));
+    if (inst->contraction != kSparse)
+        CUDA_TRY(cudaMemcpyAsync(inst->hkerr, inst->dkerr, sizeof(int32_t),
+                                 cudaMemcpyDeviceToHost, inst->stream));
     CUDA_TRY(cudaStreamSynchronize(inst->stream));
     st = check_device_status(inst);
     if (st) return st;
-    if (stats) {
-        stats->n_alive = inst->hctr->n_alive;
-        stats->m_alive = inst->hctr->m_alive;
-        stats->rounds = inst->hctr->max_rounds_seen;
-        stats->changed = inst->hctr->changed_any;
-        stats->dp_deleted = inst->hctr->dp_deleted;
-        stats->md_deleted = inst->hctr->md_deleted;
-        stats->active = inst->hctr->active;
-    }
+    if (stats) stats_from(*inst->hctr, stats);
     return MHS_OK;
 }
 
@@ -1535,6 +1812,30 @@ mhs_status mhs_result_at(const mhs_instance *inst, int32_t index, int32_t *vtx_o
     if ((vtx_out && vtx_cap < s.n) || ((edge_out || demand_out) && edge_cap < s.m))
         return fail(MHS_EINVAL, "output capacity too small (need %d vertices, %d edges)", s.n,
                     s.m);
+    if (inst->contraction == kSparse) {  // kept by input id: no positions
+        const auto alive = [&](const int32_t *o2c, int32_t size, std::vector<int32_t> *map) {
+            map->resize(size);
+            return size ? cudaMemcpyAsync(map->data(), o2c, 4 * (size_t)size,
+                                          cudaMemcpyDeviceToHost, cs)
+                        : cudaSuccess;
+        };
+        std::vector<int32_t> vmap, emap, fall;
+        if (vtx_out) CUDA_TRY(alive(s.v_o2c, s.n0, &vmap));
+        if (edge_out || demand_out) CUDA_TRY(alive(s.e_o2c, s.m0, &emap));
+        if (demand_out) CUDA_TRY(alive(s.f, s.m0, &fall));
+        CUDA_TRY(cudaStreamSynchronize(cs));
+        int32_t w = 0;
+        for (int32_t v = 0; v < (int32_t)vmap.size(); ++v)
+            if (vmap[v] >= 0 && w < s.n) vtx_out[w++] = v;
+        w = 0;
+        for (int32_t e = 0; e < (int32_t)emap.size(); ++e) {
+            if (emap[e] < 0 || w >= s.m) continue;
+            if (edge_out) edge_out[w] = e;
+            if (demand_out) demand_out[w] = fall[e];
+            ++w;
+        }
+        return MHS_OK;
+    }
     if (vtx_out && s.n > 0)
         CUDA_TRY(cudaMemcpyAsync(vtx_out, s.v_c2o, 4 * (size_t)s.n, cudaMemcpyDeviceToHost, cs));
     std::vector<int32_t> eids;
@@ -1643,9 +1944,21 @@ mhs_status mhs_export(const mhs_instance *inst, int32_t index, int32_t *edge_ptr
         CUDA_TRY(cudaMemcpyAsync(f.data(), s.f, 4 * (size_t)s.m0, cudaMemcpyDeviceToHost, cs));
     if (s.n0 > 0)
         CUDA_TRY(cudaMemcpyAsync(vmap.data(), s.v_o2c, 4 * (size_t)s.n0, cudaMemcpyDeviceToHost, cs));
-    if (s.m > 0)
+    std::vector<int32_t> emap;
+    if (inst->contraction == kSparse) {
+        emap.resize(std::max(s.m0, 1));
+        if (s.m0 > 0)
+            CUDA_TRY(cudaMemcpyAsync(emap.data(), s.e_o2c, 4 * (size_t)s.m0,
+                                     cudaMemcpyDeviceToHost, cs));
+    } else if (s.m > 0) {
         CUDA_TRY(cudaMemcpyAsync(ec2o.data(), s.e_c2o, 4 * (size_t)s.m, cudaMemcpyDeviceToHost, cs));
+    }
     CUDA_TRY(cudaStreamSynchronize(cs));
+    if (!emap.empty()) {
+        int32_t w = 0;
+        for (int32_t e = 0; e < s.m0 && w < s.m; ++e)
+            if (emap[e] >= 0) ec2o[w++] = e;
+    }
     // renumber in input order: vertex v -> number of surviving vertices before it
     std::sort(ec2o.begin(), ec2o.begin() + s.m);
     {

@@ -29,7 +29,8 @@ constexpr int kOccK = 64;        // K columns per occupancy bit (half a stage)
 constexpr int kRowAlign = 256;   // row capacity rounded to this
 constexpr int kTraceRounds = 32; // rounds whose sizes an instance records
 
-enum Contraction : int32_t { kAuto = 0, kFp8 = 1, kPopcount = 2 };
+// (kSparse: no contraction; what MHS_CONTRACT_AUTO takes for sparse hypergraphs)
+enum Contraction : int32_t { kAuto = 0, kFp8 = 1, kPopcount = 2, kSparse = 3 };
 
 // Status bits written by kernels (OR-ed into InstState::status).
 enum : int32_t {
@@ -39,6 +40,40 @@ enum : int32_t {
     kErrCapacity = 8,      // an index exceeded an allocated capacity
     kErrBadDemand = 16,    // a demand f(e) < 1 in the input
     kErrRoundCap = 32,     // the device-side round loop hit its hard cap
+};
+
+// Sparse path (sparse.cu): per vertex, the bounds that delete hyperedges
+// holding it, and whether whole CTAs handle it.
+struct alignas(16) SpAgg {
+    int32_t m1;                 // largest f_i - |e_i| + 1 over its hyperedges of |e_i| >= 2
+    int32_t heavy;              // bit 0: whole CTAs handle it; above: its pairs' largest bound
+    unsigned long long s1;      // hyperedges of this vertex alone: largest f << 32 | ~index
+};
+// Bounds of a pair of vertices (a hash table, linear probing).
+struct alignas(32) SpPair {
+    unsigned long long key;     // 0: free
+    unsigned long long s2;      // hyperedges of this pair alone: largest f << 32 | ~index
+    int32_t m2;                 // largest f_i - |e_i| + 2 over its hyperedges of |e_i| >= 3
+    int32_t pad[3];
+};
+// Counters of one round; rounds alternate between two.
+struct SpRound {
+    int32_t dp, md;             // deletions
+    int32_t ntask;              // tasks reserved
+    int32_t npair[2];           // pairs listed: by the walks, by the tasks
+    int32_t scan_all;           // an instance-wide bound rose
+};
+// Sparse path: control words of one instance.
+struct SpCtl {
+    uint32_t bar;               // team barrier: arrivals over all launches
+    uint32_t cursor;            // places handed out in the vertex lists
+    int32_t n_heavy;            // entries of sp_heavy
+    int32_t full;               // the next round takes every hyperedge and vertex
+    int32_t loose;              // largest f_i - |e_i| over nonempty hyperedges (> 0), else 0
+    int32_t pairs_full;         // the pair table ran out of places: its bounds are incomplete
+    SpRound fe;                 // deletions of an FE pass
+    unsigned long long empty;   // empty hyperedges: largest f << 32 | ~index
+    SpRound c[2];
 };
 
 struct InstState {
@@ -130,6 +165,26 @@ struct InstState {
     int32_t has_loose;     // zero counts matter in this hyperedge pass: DP, some
                            // hyperedge has f > |e|; SE, some hyperedge is empty
     int32_t no_skip;       // 1: contract every tile and K block (dense formulation)
+    // sparse path (sparse.cu), by input id; rows and lists share eptr's offsets
+    uint32_t *sp_row;      // [nnz0] rows in key order, alive vertices first
+    int32_t *sp_pos;       // [nnz0] (build) an incidence's place in its vertex's list
+    uint32_t *sp_tmp;      // [nnz0] (build) keys of long rows
+    unsigned long long *sp_vedge;  // [nnz0] the vertices' lists of hyperedges
+    int4 *sp_erec;         // [m0] {signature (2 words), f or "gone", |e|}
+    int4 *sp_vrec;         // [n0] {signature (2 words), degree, place of the list}
+    SpAgg *sp_vagg;        // [n0]
+    int4 *sp_vaux;         // [n0] {smallest hyperedge, largest demand, its row's place and length}
+    uint32_t *sp_gone;     // [m0 / 32] bit: the hyperedge is deleted
+    int32_t *sp_estamp;    // [m0] round for which the hyperedge is a DP candidate
+    int32_t *sp_vstamp;    // [n0] round for which the vertex is an MD candidate
+    int32_t *sp_tstamp;    // [n0] round in which the vertex's bounds rose
+    int2 *sp_pairs;        // [sp_pair_cap] {i, j} the walks have found
+    SpPair *sp_pair_tab;   // [sp_pair_mask + 1]
+    uint32_t sp_pair_mask;
+    int4 *sp_task;         // [sp_task_cap] {i, vertex, p, part}
+    int32_t *sp_heavy;     // vertices of high degree
+    SpCtl *sp_ctl;
+    int32_t sp_task_cap, sp_pair_cap;
     // offsets of this instance's ids in the concatenated ids of its batch
     int64_t v_base, e_base;
     // per round r < kTraceRounds: hyperedges and vertices entering DP, hyperedges after DP

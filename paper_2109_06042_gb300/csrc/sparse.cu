@@ -1,0 +1,1939 @@
+// sparse.cu -- Algorithm 3 by candidate lists instead of pair tiles.
+//
+// The contractions decide every pair (i, j) of a row block; of those pairs
+// almost none can fire.  For sparse hypergraphs the pairs that can are found
+// directly from the vertex -> hyperedge lists, and the result is the same
+// set of deletions, pass by pass:
+//
+//  DP (Algorithm 1).  e_i supersedes e_j iff |e_i \ e_j| <= t, t = f_i - f_j,
+//  i.e. iff they share at least need = |e_i| - t vertices.
+//   * need >= 2: e_j holds one of any t + 1 vertices of e_i, so it is in the
+//     list of one of its rarest ones.  The p-th rarest (p from 0) has to be
+//     walked only for f_j <= f_i - p: an e_j that holds none of the p rarer
+//     ones has missed p already.  The most popular vertex of e_i is never
+//     walked (p <= |e_i| - 2).
+//   * need = 1: every e_j holding a vertex v of e_i with f_j = f_i - |e_i| + 1
+//     goes.  Per vertex the largest such bound is kept (m1), and every e_j
+//     tests its own vertices.  Hyperedges of one vertex keep per vertex the
+//     largest demand and, among equals, the lowest index (s1).
+//   * need = 2 with both vertices heavy (192 hyperedges or more): the same
+//     bound per pair of vertices, in a hash table.  What is left to walk in a
+//     heavy vertex's list is need >= 3: 5.7 of 30 million entries on the
+//     power-law instance.
+//   * need <= 0 (only f_i > |e_i|, or an empty e_i): every e_j with
+//     f_j <= f_i - |e_i| goes; one maximum over the instance (loose, empty).
+//  A pair is mutual iff both sets and demands are equal; the lower input
+//  index stays.  "Supersedes or wins the tie" is transitive and acyclic, so a
+//  hyperedge that is deleted need not be tested as a superseder: whatever it
+//  supersedes, a surviving one does too.  Deleted hyperedges are therefore
+//  skipped as soon as they are flagged, in any order, with the same result.
+//  Rule SE is the case t = 0 whatever the demands, with f_i >= f_j.
+//
+//  MD (Algorithm 2).  A dominator of v_j is in every hyperedge of v_j, so only
+//  the members of its smallest one are tested; fewer members than the
+//  largest demand decide at once.
+//
+// Pairs are filtered by 64-bit signatures (a set bit of e_i missing in e_j
+// is a vertex missed; a set bit of v_j missing in v_i rules v_i out), then
+// decided exactly by searching the sorted rows.  After the first round only
+// hyperedges that lost a vertex are superseders and only vertices that lost
+// a hyperedge are tested (the incremental argument of the contractions).
+//
+// What bounds it: latency.  A pass reads a few megabytes from L2 in chains of
+// two or three dependent loads, so the whole fixpoint runs in ONE kernel: a
+// team of CTAs per instance with a barrier between the phases (a cooperative
+// launch), or one CTA per instance of a batch.  Eight lanes share a
+// hyperedge or vertex, a warp's four groups in step; lists longer than
+// kHeavyList become tasks of kTaskLen entries for whole warps, vertices with
+// more than kHeavyDeg hyperedges are handled by whole CTAs.
+// Measured on one GB300, the rounds alone (load, kernelization and result
+// through the C ABI beside the FP8 contraction's):
+//   power law 20,000 x 40,000: 280 us (474 / 1,690)
+//   interval 50,000 x 100,000: 358 us (628 / 11,357)
+//   uniform 16,000 x 32,000, |e| 2..16: 68 us (197 / 6,145)
+#include <algorithm>
+
+#include <cuda_runtime.h>
+
+#include "bounded_wait.cuh"
+#include "kernels.h"
+#include "mhs_internal.h"
+
+namespace mhs {
+
+namespace {
+
+typedef unsigned long long u64;
+
+constexpr int kG = 8;                  // lanes per hyperedge / vertex
+// Loads in flight per lane, in the phases, a task and the build.  Small: the
+// phases are short and each round runs through all of them, so what they
+// cost most is their code (at 4 throughout, and with the helpers inlined, the
+// kernel was 236 KB and every phase waited 5 to 10 us for instructions).
+constexpr int kU = 2;
+constexpr int kTaskU = 4;
+constexpr int kRowU = 4;
+constexpr int kHeavyList = 192;        // longer lists are walked by whole warps (see kHeavyKey)
+constexpr int kTaskLen = 1024;         // entries per such task
+constexpr int kHeavyDeg = 256;         // vertices of a higher degree: whole CTAs
+constexpr int32_t kNoTask = -1, kBoundTask = -2;  // Task.x: unused; a vertex's bounds
+constexpr int32_t kGone = 0x7fffffff;  // demand of a deleted hyperedge: no test passes it
+constexpr int kSpThreads = 1024;       // threads of a CTA of a team
+constexpr int kSpBatchThreads = 512;   // threads of a CTA of a batch
+constexpr int kSpBatchBlocks = 2;      // such CTAs per SM
+constexpr int64_t kSpTeamNnz = 512;    // incidences per CTA of a team
+constexpr int64_t kSpTeamItems = 256;  // hyperedges and vertices per CTA of a team
+constexpr uint64_t kTeamWaitNs = 4000000000ull;  // 4 s bound on a team barrier
+
+__device__ __forceinline__ u64 sig_bit(int32_t id) {
+    return 1ull << (((uint32_t)id * 2654435761u) >> 26);
+}
+__device__ __forceinline__ u64 rec_sig(int4 r) {
+    return (u64)(uint32_t)r.x | ((u64)(uint32_t)r.y << 32);
+}
+// Rows hold keys: the vertex's degree at load, in 8 bits (exact below 16,
+// then 8 steps per octave), above its id.  A row in key order is sorted by one
+// order common to all rows, its rarest vertices first.
+constexpr uint32_t kIdMask = 0xffffffu;
+__device__ __forceinline__ uint32_t row_key(int32_t id, int32_t deg) {
+    const uint32_t d = (uint32_t)deg;
+    uint32_t q = d;
+    if (d >= 16) {
+        const int lg = 31 - __clz((int)d);
+        q = 16u + 8u * (uint32_t)(lg - 4) + ((d >> (lg - 3)) & 7u);
+    }
+    return (q << 24) | (uint32_t)id;
+}
+// Heavy: a degree of 192 or more at load (class 44 starts there).
+constexpr uint32_t kHeavyKey = 44u << 24;
+__device__ __forceinline__ int32_t key_id(uint32_t key) { return (int32_t)(key & kIdMask); }
+
+// An entry of a vertex's list: hyperedge id (24 bits), demand and size (4
+// bits each, 15: that or more), signature folded to 32 bits.  Almost every
+// entry of a walk is ruled out by these alone, without a load of the
+// hyperedge's record.  Sizes and signatures may be those of an earlier round
+// (never smaller than the present ones, so nothing is ruled out wrongly).
+__device__ __forceinline__ u64 make_entry(int32_t e, int32_t f, int32_t len, uint32_t fold) {
+    return (u64)(uint32_t)e | ((u64)(uint32_t)min(f, 15) << 24) |
+           ((u64)(uint32_t)min(len, 15) << 28) | ((u64)fold << 32);
+}
+__device__ __forceinline__ int32_t entry_id(u64 x) { return (int32_t)((uint32_t)x & kIdMask); }
+constexpr u64 kNoEntry = ~0ull;  // (no hyperedge has id 2^24 - 1)
+__device__ __forceinline__ uint32_t fold_sig(u64 sig) { return (uint32_t)sig | (uint32_t)(sig >> 32); }
+__device__ __forceinline__ int4 make_rec(u64 sig, int32_t z, int32_t w) {
+    return make_int4((int32_t)(uint32_t)sig, (int32_t)(uint32_t)(sig >> 32), z, w);
+}
+__device__ __forceinline__ int32_t vload(const int32_t *p) {
+    return *reinterpret_cast<const volatile int32_t *>(p);
+}
+
+// The instance's arrays.
+struct View {
+    const int32_t *eptr;
+    uint32_t *row;
+    u64 *vedge;
+    int32_t *e_o2c, *v_o2c, *estamp, *vstamp, *tstamp;
+    int4 *erec, *vrec, *vaux;
+    SpAgg *agg;
+    uint32_t *gone;
+    SpCtl *ctl;
+    View() = default;
+    __device__ __forceinline__ explicit View(const InstState &s)
+        : eptr(s.eptr), row(s.sp_row), vedge(s.sp_vedge), e_o2c(s.e_o2c), v_o2c(s.v_o2c),
+          estamp(s.sp_estamp), vstamp(s.sp_vstamp), tstamp(s.sp_tstamp), erec(s.sp_erec),
+          vrec(s.sp_vrec), vaux(s.sp_vaux), agg(s.sp_vagg), gone(s.sp_gone), ctl(s.sp_ctl) {}
+};
+
+// The round state of an instance.
+struct Progress {
+    int32_t n, m, rounds, changed, dp, md, fe_passes, max_rounds, fe;
+    int32_t active, full;
+    int64_t k;
+    uint64_t t_dp, t_md, t_all;  // ns (kept by the team's first thread)
+};
+
+// A CTA's shared memory.  What a phase needs to start (the arrays, the
+// round) is kept here: every team barrier empties L1, and a pointer or a
+// stack slot fetched again from L2 costs as much as the work itself.
+struct Shared {
+    View view;
+    InstState *s;
+    const int32_t *heavy;
+    SpPair *pair_tab;
+    uint32_t pair_mask;
+    int4 *task;
+    int32_t task_cap, n0, m0, rule;
+    // The threads that reduce the instance: `size` CTAs, this one the `rank`-th.
+    int32_t rank, size;
+    uint32_t *bar;        // arrivals so far, over all launches (size > 1)
+    uint32_t target;      // arrivals that complete the last barrier begun
+    int32_t epoch;        // round being executed, from 1
+    int32_t par;          // counter parity
+    int32_t full;         // every hyperedge and vertex is a candidate
+    int32_t ok;           // the last barrier
+    SpRound got;          // counters read right after it
+    Progress g;           // the instance's rounds, as every CTA of the team knows them
+    int32_t del, del2;    // deletions of this phase
+    int32_t next;         // batch: the instance taken from the queue
+    int32_t mf, pos;      // md_lists: one high-degree vertex
+    u64 cost, sig, small;
+    int32_t ids[32][32];  // per warp: flagged ids of a chunk
+    int2 *pairs;          // this instance's pairs (i, j) to be decided exactly
+    int32_t pair_cap;
+    int2 buf[32][32 * (kTaskU + 1)];  // per warp: pairs not yet listed (decide_pairs: not yet decided)
+};
+extern __shared__ __align__(16) uint8_t sp_smem[];
+__device__ __forceinline__ Shared *shared() { return reinterpret_cast<Shared *>(sp_smem); }
+
+// Barrier over the team; false if it timed out.  The CTAs are resident
+// together (cooperative launch), and each wait gives up after kTeamWaitNs,
+// after which every CTA of the team leaves.  p: counters that are complete
+// once every CTA has arrived, read into `got`.
+__device__ __noinline__ bool team_sync(const SpRound *p = nullptr) {
+    Shared *sh = shared();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int32_t good = 1;
+        if (sh->size > 1) {
+            uint32_t *bar = sh->bar;
+            const uint32_t target = sh->target + (uint32_t)sh->size;
+            sh->target = target;
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+            uint64_t t0 = 0;
+            for (uint32_t it = 1;; ++it) {
+                uint32_t now;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(bar) : "memory");
+                if ((int32_t)(now - target) >= 0) break;
+                if ((it & 255u) == 0) {
+                    const uint64_t t = globaltimer();
+                    if (t0 == 0) t0 = t;
+                    else if (t - t0 > kTeamWaitNs) {
+                        atomicOr(&sh->s->status, kErrTimeout);
+                        good = 0;
+                        break;
+                    }
+                }
+            }
+        }
+        sh->ok = good;
+        if (p) {
+            sh->got.dp = vload(&p->dp);
+            sh->got.md = vload(&p->md);
+            sh->got.ntask = vload(&p->ntask);
+            sh->got.npair[0] = vload(&p->npair[0]);
+            sh->got.npair[1] = vload(&p->npair[1]);
+        }
+    }
+    __syncthreads();
+    return sh->ok != 0;
+}
+
+// A thread's place and the round, from shared memory.
+struct Ctx {
+    Shared *sh;
+    int lane, warp, sub, lead;  // lane in the warp, warp in the CTA, lane in the group, its first lane
+    int gw, nw;                 // warp of the team, and their number
+    int32_t epoch, par;
+    bool full;
+    __device__ __forceinline__ Ctx() {
+        sh = shared();
+        lane = threadIdx.x & 31;
+        warp = threadIdx.x >> 5;
+        sub = lane & (kG - 1);
+        lead = lane & ~(kG - 1);
+        gw = warp * sh->size + sh->rank;  // neighbours in the id range on different SMs
+        nw = (int)(blockDim.x >> 5) * sh->size;
+        epoch = sh->epoch;
+        par = sh->par;
+        full = sh->full != 0;
+    }
+};
+
+// Reductions over a group; every lane of the warp takes part.
+__device__ __forceinline__ u64 group_min(u64 x) {
+#pragma unroll
+    for (int o = kG / 2; o > 0; o >>= 1) {
+        const u64 y = __shfl_xor_sync(0xffffffffu, x, o);
+        x = y < x ? y : x;
+    }
+    return x;
+}
+__device__ __forceinline__ u64 group_or(u64 x) {
+#pragma unroll
+    for (int o = kG / 2; o > 0; o >>= 1) x |= __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+__device__ __forceinline__ int32_t group_max(int32_t x) {
+#pragma unroll
+    for (int o = kG / 2; o > 0; o >>= 1) x = max(x, __shfl_xor_sync(0xffffffffu, x, o));
+    return x;
+}
+__device__ __forceinline__ int32_t group_sum(int32_t x) {
+#pragma unroll
+    for (int o = kG / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+// The lanes of this group whose flag is set (bit 0: the group's first lane).
+__device__ __forceinline__ unsigned group_ballot(const Ctx &c, bool x) {
+    return (__ballot_sync(0xffffffffu, x) >> c.lead) & ((1u << kG) - 1u);
+}
+
+// Runs fn(id) for every id in [0, n) with flag(id): a group of lanes per id,
+// the warp's four groups in step (an idle group gets id -1), so that a list
+// that is longer in one group than in the others costs its excess only once.
+// A warp takes chunks of ids; the chunk shrinks to 4 (one per group) when
+// there are more warps than work.
+template <typename Flag, typename Fn>
+__device__ __forceinline__ void for_flagged(const Ctx &c, int32_t n, Flag &&flag, Fn &&fn) {
+    int chunk = 32;
+    while (chunk > 32 / kG && (int64_t)n < (int64_t)c.nw * chunk) chunk >>= 1;
+    int32_t *ids = c.sh->ids[c.warp];
+    const int g = c.lane / kG;
+#pragma unroll 1
+    for (int64_t base = (int64_t)c.gw * chunk; base < n; base += (int64_t)c.nw * chunk) {
+        const int32_t id = (int32_t)base + c.lane;
+        const bool on = c.lane < chunk && id < n && flag(id);
+        const unsigned mk = __ballot_sync(0xffffffffu, on);
+        if (!mk) continue;
+        if (on) ids[__popc(mk & ((1u << c.lane) - 1u))] = id;
+        __syncwarp();
+        const int cnt = __popc(mk);
+#pragma unroll 1
+        for (int q = 0; q < cnt; q += 32 / kG) fn(q + g < cnt ? ids[q + g] : -1);
+        __syncwarp();
+    }
+}
+
+// ------------------------------------------------------------------ bounds --
+
+// The slot of the pair of heavy vertices a < b, or the free one for it.
+constexpr int kProbes = 16;
+__device__ __forceinline__ SpPair *pair_slot(const Shared *sh, uint32_t a, uint32_t b, int probe) {
+    const uint32_t h = a * 0x9e3779b1u ^ (b * 0x85ebca77u + 0x165667b1u);
+    return sh->pair_tab + ((((h ^ (h >> 15)) * 0x2c1b3c6du >> 8) + (uint32_t)probe) & sh->pair_mask);
+}
+__device__ __forceinline__ u64 pair_key(uint32_t a, uint32_t b) { return ((u64)a << 24 | b) + 1; }
+
+// Hyperedge e's bound for the pair of its heavy vertices x and y.
+__device__ __forceinline__ void add_pair_bound(Shared *sh, int32_t e, int32_t f, int32_t len,
+                                               uint32_t x, uint32_t y) {
+    SpAgg *agg = sh->view.agg;
+    const uint32_t lo = min(x, y), hi = max(x, y);
+    const u64 key = pair_key(lo, hi);
+    SpPair *slot = nullptr;
+#pragma unroll 1
+    for (int q = 0; q < kProbes && !slot; ++q) {
+        SpPair *p = pair_slot(sh, lo, hi, q);
+        u64 cur = *reinterpret_cast<volatile u64 *>(&p->key);
+        if (cur == 0) cur = atomicCAS(&p->key, 0ull, key);
+        if (cur == 0 || cur == key) slot = p;
+    }
+    if (!slot) {
+        sh->view.ctl->pairs_full = 1;  // the walks must find what the bounds miss
+        return;
+    }
+    // (popular pairs have hundreds of writers: look before an atomic)
+    const int32_t bound = len == 2 ? f : f - len + 2;
+    const int32_t most = min(bound, 0x3ffffffe) << 1;  // (bit 0: for whole CTAs)
+    const int32_t hx = vload(&agg[x].heavy), hy = vload(&agg[y].heavy);
+    if ((hx & ~1) < most) atomicMax(&agg[x].heavy, most | (hx & 1));
+    if ((hy & ~1) < most) atomicMax(&agg[y].heavy, most | (hy & 1));
+    if (len == 2) {
+        const u64 s2 = ((u64)(uint32_t)f << 32) | (0xffffffffu - (uint32_t)e);
+        if (*reinterpret_cast<volatile u64 *>(&slot->s2) < s2) atomicMax(&slot->s2, s2);
+    } else if (vload(&slot->m2) < bound) {
+        atomicMax(&slot->m2, bound);
+    }
+}
+
+// True if e_j goes by the bound of its heavy vertices x and y.
+__device__ __forceinline__ bool pair_hit(const Shared *sh, uint32_t x, uint32_t y, int32_t j,
+                                         int32_t fj, int32_t lenj) {
+    const uint32_t lo = min(x, y), hi = max(x, y);
+    const u64 key = pair_key(lo, hi);
+#pragma unroll 1
+    for (int q = 0; q < kProbes; ++q) {
+        const SpPair *p = pair_slot(sh, lo, hi, q);
+        const u64 cur = p->key;
+        if (cur == 0) return false;
+        if (cur != key) continue;
+        if (p->m2 >= fj) return true;
+        const u64 s2 = p->s2;
+        return s2 && fj <= (int32_t)(s2 >> 32) &&
+               (lenj >= 3 || (int32_t)(0xffffffffu - (uint32_t)s2) != j);
+    }
+    return false;
+}
+
+// What hyperedge e (row: its keys) contributes to the tests with need <= 1,
+// and in full rounds to those of pairs of heavy vertices.  One group, without
+// the others.
+__device__ __noinline__ void contribute(int32_t e, int32_t f, int32_t len, const uint32_t *row) {
+    Shared *sh = shared();
+    const int sub = threadIdx.x & (kG - 1);
+    SpAgg *agg = sh->view.agg;
+    int32_t *tstamp = sh->view.tstamp;
+    SpCtl *ctl = sh->view.ctl;
+    const int32_t epoch = sh->epoch;
+    if (len <= 1) {
+        if (sub != 0) return;
+        const u64 key = ((u64)(uint32_t)f << 32) | (0xffffffffu - (uint32_t)e);
+        if (len == 0) {
+            if (atomicMax(&ctl->empty, key) < key) ctl->c[sh->par].scan_all = 1;
+            return;
+        }
+        const int32_t x = key_id(row[0]);
+        if (*reinterpret_cast<volatile u64 *>(&agg[x].s1) < key && atomicMax(&agg[x].s1, key) < key)
+            tstamp[x] = epoch;
+        if (!sh->rule && f > 1 && atomicMax(&ctl->loose, f - 1) < f - 1) ctl->c[sh->par].scan_all = 1;
+        return;
+    }
+    if (sh->rule || f < len - 1) return;
+    const int32_t m1 = f - len + 1;
+    if (m1 >= 1)
+#pragma unroll 1
+        for (int32_t k = sub; k < len; k += kG) {
+            const int32_t x = key_id(row[k]);
+            if (vload(&agg[x].m1) < m1 && atomicMax(&agg[x].m1, m1) < m1) tstamp[x] = epoch;
+        }
+    if (f > len && sub == 0 && atomicMax(&ctl->loose, f - len) < f - len)
+        ctl->c[sh->par].scan_all = 1;
+    if (!sh->full) return;
+#pragma unroll 1
+    for (int32_t a = 0; a < len - 1; ++a) {
+        const uint32_t ka = row[a];
+        if (ka < kHeavyKey) continue;  // (the heavy ones end the row)
+#pragma unroll 1
+        for (int32_t k = a + 1 + sub; k < len; k += kG)
+            add_pair_bound(sh, e, f, len, ka & kIdMask, row[k] & kIdMask);
+    }
+}
+
+// ---------------------------------------------------------------- DP pass --
+
+// Flag hyperedge x as deleted (once), and its vertices as MD candidates.
+// One thread.
+__device__ __noinline__ void delete_edge(int32_t x) {
+    Shared *sh = shared();
+    const View &v = sh->view;
+    if (atomicExch(&v.erec[x].z, kGone) == kGone) return;
+    atomicAdd(&sh->del, 1);
+    const int32_t epoch = sh->epoch;
+    v.e_o2c[x] = -1 - epoch;
+    atomicOr(&v.gone[x >> 5], 1u << (x & 31));
+    if (sh->full) return;  // every vertex is a candidate
+    const int32_t len = v.erec[x].w;
+    const uint32_t *row = v.row + v.eptr[x];
+#pragma unroll 1
+    for (int32_t k = 0; k < len; ++k) v.vstamp[key_id(row[k])] = epoch;
+}
+
+// True if e_j goes by the need <= 1 bounds of one of its vertices.
+__device__ __forceinline__ bool agg_hit(int4 a, int32_t j, int32_t fj, int32_t lenj) {
+    if (a.x >= fj) return true;                      // m1
+    if (a.w == 0) return false;                      // s1: demand a.w, ~index a.z
+    return fj <= a.w && (lenj >= 2 || (int32_t)(0xffffffffu - (uint32_t)a.z) != j);
+}
+// True if e_j goes by the instance-wide bounds.
+__device__ __forceinline__ bool global_hit(int32_t loose, u64 empty, int32_t j, int32_t fj,
+                                           int32_t lenj) {
+    if (fj <= loose) return true;
+    return empty && fj <= (int32_t)(empty >> 32) &&
+           (lenj > 0 || (int32_t)(0xffffffffu - (uint32_t)empty) != j);
+}
+__device__ __forceinline__ int4 load_agg(const SpAgg *p) {
+    return *reinterpret_cast<const int4 *>(p);
+}
+
+// Reserve tasks for the list of vertex x, in the lanes with want set (the
+// whole warp, one atomic); false if there is no room (the caller walks the
+// list itself).
+__device__ __noinline__ bool push_tasks(bool want, int32_t i, int32_t x, int32_t p, int32_t deg) {
+    if (!__any_sync(0xffffffffu, want)) return false;
+    Shared *sh = shared();
+    const int lane = threadIdx.x & 31;
+    const int32_t cap = sh->task_cap;
+    const int32_t parts = want ? (deg + kTaskLen - 1) / kTaskLen : 0;
+    int32_t inc = parts;
+#pragma unroll 1
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    int32_t at = 0;
+    if (lane == 31) at = atomicAdd(&sh->view.ctl->c[sh->par].ntask, inc);
+    at = __shfl_sync(0xffffffffu, at, 31) + inc - parts;
+    const bool fits = at >= 0 && at <= cap - parts;
+#pragma unroll 1
+    for (int32_t q = 0; q < parts; ++q)
+        if (at >= 0 && at + q < cap)
+            sh->task[at + q] = fits ? make_int4(i, x, p, q) : make_int4(kNoTask, 0, 0, 0);
+    return want && fits;
+}
+
+// The hyperedges of vertex x that its bounds delete: entries k0, k0 + step, ... < k1.
+__device__ __noinline__ void bound_list(int32_t x, int32_t k0, int32_t k1, int32_t step, int shard,
+                                        int nshards) {
+    const View &v = shared()->view;
+    const int4 a = load_agg(v.agg + x);
+    const u64 *list = v.vedge + v.vrec[x].w;
+#pragma unroll 1
+    for (int32_t k = k0; k < k1; k += step) {
+        const int32_t j = entry_id(list[k]);
+        if (nshards > 1 && (j >> 7) % nshards != shard) continue;
+        const int4 r = v.erec[j];
+        if (r.z != kGone && agg_hit(a, j, r.z, r.w)) delete_edge(j);
+    }
+}
+
+// The tests with need <= 1 (and of pairs of heavy vertices) for every
+// hyperedge: full rounds, or an instance-wide bound rose.
+__device__ __noinline__ void dp_bounds_all(int shard, int nshards) {
+    const Ctx c;
+    const View &v = c.sh->view;
+    const int32_t loose = vload(&v.ctl->loose);
+    const u64 empty = *reinterpret_cast<volatile u64 *>(&v.ctl->empty);
+    const int32_t *const e_o2c = v.e_o2c, *const eptr = v.eptr;
+    const int4 *const erec = v.erec;
+    const uint32_t *const rows = v.row;
+    const SpAgg *const agg = v.agg;
+    for_flagged(
+        c, c.sh->m0,
+        [&](int32_t j) { return e_o2c[j] >= 0 && (nshards == 1 || (j >> 7) % nshards == shard); },
+        [&](int32_t j) {
+            const int4 r = j >= 0 ? erec[j] : make_int4(0, 0, kGone, 0);
+            const uint32_t *row = j >= 0 ? rows + eptr[j] : nullptr;
+            const int32_t fj = r.z;
+            bool hit = fj != kGone && global_hit(loose, empty, j, fj, r.w);
+            int32_t heavy = 0;  // heavy vertices in pairs whose bound may reach f_j
+            const int32_t maxlen = c.full ? __reduce_max_sync(0xffffffffu, r.w) : 0;
+#pragma unroll 1
+            for (int32_t k0 = 0; k0 < maxlen; k0 += kU * kG) {
+                int32_t x[kU];
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    const int32_t k = k0 + u * kG + c.sub;
+                    x[u] = k < r.w ? key_id(row[k]) : -1;
+                }
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    if (x[u] < 0) continue;
+                    const int4 a = load_agg(agg + x[u]);
+                    hit |= agg_hit(a, j, fj, r.w);
+                    heavy += a.y > 1 && (a.y >> 1) >= fj;
+                }
+            }
+            hit = hit && fj != kGone;
+            // every two of them, unless decided
+            heavy = group_sum(heavy);
+            int32_t end = group_ballot(c, hit) == 0 && heavy > 1 ? r.w : 0;
+            end = __shfl_sync(0xffffffffu, end, c.lead);
+            const int32_t maxend = __reduce_max_sync(0xffffffffu, end);
+#pragma unroll 1
+            for (int32_t a = 0; a < maxend; ++a) {
+                const uint32_t ka = a < end ? row[a] : 0;
+                bool on = ka >= kHeavyKey;
+                if (!__any_sync(0xffffffffu, on)) continue;
+                on = on && (agg[ka & kIdMask].heavy >> 1) >= fj;
+                if (on)
+#pragma unroll 1
+                    for (int32_t k = a + 1 + c.sub; k < end && !hit; k += kG) {
+                        const uint32_t y = row[k] & kIdMask;
+                        if ((agg[y].heavy >> 1) >= fj) hit = pair_hit(c.sh, ka & kIdMask, y, j, fj, r.w);
+                    }
+                __syncwarp();
+                if (group_ballot(c, hit)) end = 0;
+            }
+            if (group_ballot(c, hit) && c.sub == 0 && fj != kGone) delete_edge(j);
+            __syncwarp();
+        });
+}
+
+// The same for the hyperedges of the vertices whose bounds rose.
+__device__ __noinline__ void dp_bounds_touched(int shard, int nshards) {
+    const Ctx c;
+    const View &v = c.sh->view;
+    const int32_t *const tstamp = v.tstamp, *const v_o2c = v.v_o2c;
+    const int4 *const vrec = v.vrec;
+    for_flagged(
+        c, c.sh->n0, [&](int32_t x) { return tstamp[x] == c.epoch && v_o2c[x] >= 0; },
+        [&](int32_t x) {
+            const int32_t deg = x >= 0 ? vrec[x].z : 0;
+            bool later = push_tasks(deg > kHeavyList && c.sub == 0, kBoundTask, x, 0, deg);
+            later = __shfl_sync(0xffffffffu, later, c.lead);
+            if (x >= 0 && !later) bound_list(x, c.sub, deg, kG, shard, nshards);
+            __syncwarp();
+        });
+}
+
+__device__ __forceinline__ void dp_bounds(int shard, int nshards) {
+    const Shared *sh = shared();
+    if (sh->full || vload(&sh->view.ctl->c[sh->par].scan_all)) dp_bounds_all(shard, nshards);
+    if (!sh->full) dp_bounds_touched(shard, nshards);
+}
+
+// Vertices of a row to be walked: need >= 2 leaves out the most popular.
+__device__ __forceinline__ int32_t walk_count(int32_t rule, int32_t f, int32_t len) {
+    if (len < 2) return 0;
+    return rule ? 1 : min(f, len - 1);
+}
+
+struct Walker {  // the superseder of a walk
+    int32_t i, f, len, rule;
+    uint32_t fold;
+};
+
+// May e_i supersede the hyperedge of entry x of its p-th rarest vertex's
+// list?  (Demands and sizes of 15 stand for larger ones: decide_pairs looks.)
+// p carries kNeed3 in the lists of heavy vertices that only pairs with
+// need >= 3 are taken from.
+constexpr int32_t kNeed3 = 1 << 30;
+__device__ __forceinline__ bool may_supersede(const uint32_t *gone, const Walker &w, int32_t p,
+                                              u64 x) {
+    const int32_t fj = (int32_t)((uint32_t)x >> 24) & 15, lenj = (int32_t)((uint32_t)x >> 28);
+    const int32_t t = w.rule ? 0 : w.f - fj;
+    // the strongest test first
+    if (__popc(w.fold & ~(uint32_t)(x >> 32)) > t) return false;
+    if (fj > w.f - (p & ~kNeed3) || entry_id(x) == w.i) return false;
+    // need <= 1 (2): dp_bounds
+    if (!w.rule && fj < 15 && w.len - t < (p & kNeed3 ? 3 : 2)) return false;
+    if (lenj < 15 && lenj < w.len - t) return false;
+    // lists keep the hyperedges deleted since they were last rewritten: most
+    // of what gets here in a first round (power-law: 3.07 of 3.25 million)
+    const int32_t j = entry_id(x);
+    return !((gone[j >> 5] >> (j & 31)) & 1u);
+}
+
+// Can the pair (i, j) fire, by the records as they are now?  Leaves the
+// slack in *t.
+__device__ __forceinline__ bool pair_open(int32_t rule, int4 ri, int4 rj, int32_t *t) {
+    if (ri.z == kGone || rj.z == kGone || rj.z > ri.z) return false;
+    *t = rule ? 0 : ri.z - rj.z;
+    return rj.w >= ri.w - *t && __popcll(rec_sig(ri) & ~rec_sig(rj)) <= *t;
+}
+
+// Place of `key` in a row of len keys, or of the next larger one.
+__device__ __forceinline__ int32_t find_key(const uint32_t *row, int32_t len, uint32_t key) {
+    int32_t lo = 0, hi = len;
+#pragma unroll 1
+    while (lo < hi) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (row[mid] < key) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
+// Decide the pair (i, j) of each group (i < 0: none) exactly: |e_i \ e_j| <= t.
+// Each lane looks for one vertex of e_i at a time (rows are in key order).
+// The whole warp.
+__device__ __noinline__ void decide_group(int2 ij) {
+    const Ctx c;
+    const View &v = c.sh->view;
+    const int32_t rule = c.sh->rule;
+    const int4 gone = make_int4(0, 0, kGone, 0);
+    const int4 ri = ij.x >= 0 ? v.erec[ij.x] : gone;
+    const int4 rj = ij.x >= 0 ? v.erec[ij.y] : gone;
+    const uint32_t *rowi = ij.x >= 0 ? v.row + v.eptr[ij.x] : nullptr;
+    const uint32_t *rowj = ij.x >= 0 ? v.row + v.eptr[ij.y] : nullptr;
+    int32_t t = 0;
+    const bool mine = pair_open(rule, ri, rj, &t);
+    // (one lane's view: the records may change under the others)
+    const bool open = __shfl_sync(0xffffffffu, mine, c.lead);
+    t = __shfl_sync(0xffffffffu, t, c.lead);
+    const int32_t leni = open ? ri.w : 0, lenj = rj.w;
+    const int32_t maxi = __reduce_max_sync(0xffffffffu, leni);
+    int32_t miss = 0;
+#pragma unroll 1
+    for (int32_t k0 = 0; k0 < maxi; k0 += kG) {
+        const int32_t k = k0 + c.sub;
+        bool lost = false;
+        if (k < leni && miss <= t) {
+            const uint32_t a = rowi[k];
+            const int32_t at = find_key(rowj, lenj, a);
+            lost = at >= lenj || rowj[at] != a;
+        }
+        __syncwarp();
+        miss += __popc(group_ballot(c, lost));
+        if (!__any_sync(0xffffffffu, miss <= t && k0 + kG < leni)) break;
+    }
+    if (open && miss <= t && c.sub == 0) {
+        // mutual (equal sets and demands): the lower index stays
+        const bool eq = miss == 0 && leni == lenj && ri.z == rj.z;
+        delete_edge(eq && ij.y < ij.x ? ij.x : ij.y);
+    }
+    __syncwarp();
+}
+
+// The pairs that may fire are few, and the walks find them very unevenly (a
+// warp hundreds, most none), so they are listed, and decided by all threads
+// of the team alike once the walks are done.  A warp gathers them in shared
+// memory and lists 32 or more at a time.
+__device__ __noinline__ void list_pairs(int32_t which, int32_t base, int32_t n) {
+    const Ctx c;
+    Shared *sh = c.sh;
+    const int2 *buf = sh->buf[c.warp];
+    __syncwarp();
+    int32_t at = 0;
+    if (c.lane == 0) at = atomicAdd(&sh->view.ctl->c[c.par].npair[which], n);
+    const int64_t to = (int64_t)base + __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll 1
+    for (int32_t k = c.lane; k < n; k += 32)
+        if (to + k < sh->pair_cap) sh->pairs[to + k] = buf[k];
+    __syncwarp();
+    if (to + n <= sh->pair_cap) return;
+#pragma unroll 1
+    for (int32_t k0 = 0; k0 < n; k0 += 32 / kG) {  // no room: decided here
+        const int32_t k = k0 + c.lane / kG;
+        decide_group(k < n && to + k >= sh->pair_cap ? buf[k] : make_int2(-1, -1));
+    }
+    __syncwarp();
+}
+struct Pairs {
+    int2 *buf;
+    int32_t which;  // the walks' list (0), or the tasks' behind it (1)
+    int32_t base;   // its first place
+    int32_t n = 0;  // pairs in the buffer, the same in every lane
+    __device__ __forceinline__ Pairs(const Ctx &c, int32_t w)
+        : buf(c.sh->buf[c.warp]), which(w), base(w ? min(c.sh->got.npair[0], c.sh->pair_cap) : 0) {}
+    // At most kTaskU times between two calls of list().
+    __device__ __forceinline__ void push(const Ctx &c, bool want, int32_t i, int32_t j) {
+        const unsigned mk = __ballot_sync(0xffffffffu, want);
+        if (want) buf[n + __popc(mk & ((1u << c.lane) - 1u))] = make_int2(i, j);
+        n += __popc(mk);
+    }
+    __device__ __forceinline__ void list(int32_t least) {
+        if (n < least) return;
+        list_pairs(which, base, n);
+        n = 0;
+    }
+};
+
+// After the barrier that ends a walk: decide the pairs of a list.  First
+// each lane looks at one pair's records (most pairs fall here: the hyperedge
+// is deleted by now, or its whole signature rules it out); the rest goes to
+// groups of lanes.  (One thread per pair to the end: 103 us for the 220,000
+// pairs of the 2,000 x 4,000 interval instance, in chains of 100 loads.)
+__device__ __noinline__ void decide_pairs(int32_t which) {
+    const Ctx c;
+    Shared *sh = c.sh;
+    const View &v = sh->view;
+    const int2 *pairs = sh->pairs;
+    const int32_t rule = sh->rule;
+    const int32_t from = which ? min(sh->got.npair[0], sh->pair_cap) : 0;
+    const int64_t to = min((int64_t)from + sh->got.npair[which], (int64_t)sh->pair_cap);
+    int2 *buf = sh->buf[c.warp];
+    int32_t n = 0;  // pairs in the buffer
+    int32_t chunk = 32;  // fewer per warp when there are more warps than work
+    while (chunk > 32 / kG && to - from < (int64_t)c.nw * chunk) chunk >>= 1;
+#pragma unroll 1
+    for (int64_t base = from + (int64_t)c.gw * chunk;; base += (int64_t)c.nw * chunk) {
+        const bool last = base >= to;
+        if (!last) {
+            const bool on = c.lane < chunk && base + c.lane < to;
+            const int2 ij = on ? pairs[base + c.lane] : make_int2(-1, -1);
+            int32_t t;
+            const bool open = on && pair_open(rule, v.erec[ij.x], v.erec[ij.y], &t);
+            const unsigned mk = __ballot_sync(0xffffffffu, open);
+            if (open) buf[n + __popc(mk & ((1u << c.lane) - 1u))] = ij;
+            n += __popc(mk);
+            __syncwarp();
+        }
+        // whole sets of four, then the rest at the end
+#pragma unroll 1
+        while (n >= (last ? 1 : 32 / kG)) {
+            const int32_t q = n - 1 - c.lane / kG;
+            decide_group(q >= 0 ? buf[q] : make_int2(-1, -1));
+            n = max(n - 32 / kG, 0);
+        }
+        if (last) break;
+    }
+}
+
+// The tests with need >= 2: short lists at once, long ones as tasks.
+__device__ __noinline__ void dp_walk(int shard, int nshards) {
+    const Ctx c;
+    const View &v = c.sh->view;
+    const int32_t rule = c.sh->rule;
+    const bool bounded = c.full && !rule && !vload(&v.ctl->pairs_full);
+    const int32_t *const e_o2c = v.e_o2c, *const estamp = v.estamp, *const eptr = v.eptr;
+    const int4 *const erec = v.erec, *const vrec = v.vrec;
+    const uint32_t *const rows = v.row, *const gone = v.gone;
+    const u64 *const vedge = v.vedge;
+    Pairs pairs(c, 0);
+    for_flagged(
+        c, c.sh->m0,
+        [&](int32_t i) {
+            return (c.full ? e_o2c[i] >= 0 : estamp[i] == c.epoch) &&
+                   (nshards == 1 || (i >> 7) % nshards == shard);
+        },
+        [&](int32_t i) {
+            const int4 r = i >= 0 ? erec[i] : make_int4(0, 0, kGone, 0);
+            const uint32_t *row = i >= 0 ? rows + eptr[i] : nullptr;
+            Walker w;
+            w.i = i;
+            // one lane's view of the flag: another might read it later
+            w.f = __shfl_sync(0xffffffffu, r.z, c.lead);
+            w.len = r.w;
+            w.fold = fold_sig(rec_sig(r));
+            w.rule = rule;
+            const int32_t np = w.f == kGone ? 0 : walk_count(rule, w.f, w.len);
+            const int32_t npmax = __reduce_max_sync(0xffffffffu, np);
+#pragma unroll 1
+            for (int32_t p0 = 0; p0 < npmax; p0 += kG) {
+                // one of the next 8 vertices' lists per lane, walked as one
+                int32_t p = p0 + c.sub;
+                const uint32_t key = p < np ? row[p] : 0;
+                int32_t x = p < np ? key_id(key) : -1;
+                if (bounded && key >= kHeavyKey) {  // its pairs with need 2 went by the bounds
+                    if (p > w.len - 3) x = -1;
+                    p |= kNeed3;
+                }
+                const int4 vr = x >= 0 ? vrec[x] : make_int4(0, 0, 0, 0);
+                int32_t deg = vr.z;
+                if (push_tasks(deg > kHeavyList, i, x, p, deg)) deg = 0;
+                int32_t inc = deg;  // inclusive prefix over the group
+#pragma unroll
+                for (int o = 1; o < kG; o <<= 1) {
+                    const int32_t y = __shfl_up_sync(0xffffffffu, inc, o, kG);
+                    if (c.sub >= o) inc += y;
+                }
+                const int32_t start = inc - deg;
+                const int32_t tot = __shfl_sync(0xffffffffu, inc, c.lead + kG - 1);
+                const int32_t maxtot = __reduce_max_sync(0xffffffffu, tot);
+                const int32_t base = vr.w - start;
+#pragma unroll 1
+                for (int32_t o = 0; o < maxtot; o += kU * kG) {
+                    u64 ent[kU];
+                    int32_t lp[kU];
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) {
+                        const int32_t k = o + u * kG + c.sub;
+                        int q = c.lead;  // the list of entry k: the last that starts at or before it
+#pragma unroll
+                        for (int st = kG / 2; st > 0; st >>= 1)
+                            if (__shfl_sync(0xffffffffu, start, q + st) <= k) q += st;
+                        const int32_t b = __shfl_sync(0xffffffffu, base, q);
+                        lp[u] = __shfl_sync(0xffffffffu, p, q);
+                        ent[u] = k < tot ? vedge[b + k] : kNoEntry;
+                    }
+#pragma unroll
+                    for (int u = 0; u < kU; ++u)
+                        pairs.push(c, ent[u] != kNoEntry && may_supersede(gone, w, lp[u], ent[u]), i,
+                                   entry_id(ent[u]));
+                    pairs.list(32);
+                }
+            }
+        });
+    pairs.list(1);
+}
+
+// The tasks: one warp per kTaskLen entries of a long list.
+__device__ __noinline__ void dp_tasks(int shard, int nshards) {
+    const Ctx c;
+    const View &v = c.sh->view;
+    const int32_t nt = min(c.sh->got.ntask, c.sh->task_cap);
+    const uint32_t *const gone = v.gone;
+    Pairs pairs(c, 1);
+#pragma unroll 1
+    for (int32_t t = c.gw; t < nt; t += c.nw) {
+        const int4 tk = c.sh->task[t];
+        if (tk.x == kNoTask) continue;
+        const int4 vr = v.vrec[tk.y];
+        const int4 r = tk.x >= 0 ? v.erec[tk.x] : make_int4(0, 0, 0, 0);
+        const int32_t k0 = tk.w * kTaskLen, k1 = min(k0 + kTaskLen, vr.z);
+        if (tk.x == kBoundTask) {
+            bound_list(tk.y, k0 + c.lane, k1, 32, shard, nshards);
+            __syncwarp();
+            continue;
+        }
+        Walker w;
+        w.i = tk.x;
+        w.f = __shfl_sync(0xffffffffu, r.z, 0);
+        if (w.f == kGone) continue;
+        w.len = r.w;
+        w.fold = fold_sig(rec_sig(r));
+        w.rule = c.sh->rule;
+        const u64 *list = v.vedge + vr.w;
+#pragma unroll 1
+        for (int32_t k = k0 + c.lane; k - c.lane < k1; k += kTaskU * 32) {
+            u64 ent[kTaskU];
+            unsigned may = 0;
+#pragma unroll
+            for (int u = 0; u < kTaskU; ++u) ent[u] = k + u * 32 < k1 ? list[k + u * 32] : kNoEntry;
+#pragma unroll
+            for (int u = 0; u < kTaskU; ++u)
+                may |= (ent[u] != kNoEntry && may_supersede(gone, w, tk.z, ent[u]) ? 1u : 0u) << u;
+            if (!__any_sync(0xffffffffu, may != 0)) continue;
+#pragma unroll
+            for (int u = 0; u < kTaskU; ++u) pairs.push(c, (may >> u) & 1u, tk.x, entry_id(ent[u]));
+            pairs.list(32);
+        }
+    }
+    pairs.list(1);
+}
+
+// Rows of the candidates without the vertices MD deleted, their signatures
+// and contributions.
+__device__ __noinline__ void dp_rows() {
+    const Ctx c;
+    const View &v = c.sh->view;
+    const int32_t *const e_o2c = v.e_o2c, *const estamp = v.estamp, *const v_o2c = v.v_o2c;
+    for_flagged(
+        c, c.sh->m0, [&](int32_t e) { return e_o2c[e] >= 0 && (c.full || estamp[e] == c.epoch); },
+        [&](int32_t e) {
+            const int4 r = e >= 0 ? v.erec[e] : make_int4(0, 0, 0, 0);
+            uint32_t *row = e >= 0 ? v.row + v.eptr[e] : nullptr;
+            u64 sig = 0;
+            int32_t w = 0;
+            const int32_t maxlen = __reduce_max_sync(0xffffffffu, r.w);
+#pragma unroll 1
+            for (int32_t k0 = 0; k0 < maxlen; k0 += kG) {
+                const int32_t k = k0 + c.sub;
+                const uint32_t x = k < r.w ? row[k] : 0;
+                const bool keep = k < r.w && v_o2c[key_id(x)] >= 0;
+                const unsigned b = group_ballot(c, keep);
+                if (keep) {
+                    sig |= sig_bit(key_id(x));
+                    row[w + __popc(b & ((1u << c.sub) - 1u))] = x;
+                }
+                w += __popc(b);
+            }
+            sig = group_or(sig);
+            __syncwarp();
+            if (e >= 0) {
+                if (c.sub == 0) v.erec[e] = make_rec(sig, r.z, w);
+                contribute(e, r.z, w, row);
+            }
+            __syncwarp();
+        });
+}
+
+// ---------------------------------------------------------------- MD pass --
+
+__device__ __forceinline__ bool vertex_candidate(const Ctx &c, const View &v, int32_t x) {
+    return v.v_o2c[x] >= 0 && (c.full || v.vstamp[x] == c.epoch);
+}
+
+// Lists of the candidates without the hyperedges DP deleted; degree,
+// signature, largest demand and smallest hyperedge.
+__device__ __noinline__ void md_lists() {
+    const Ctx c;
+    const View &v = c.sh->view;
+    const int4 *const erec = v.erec;
+    for_flagged(
+        c, c.sh->n0, [&](int32_t x) { return vertex_candidate(c, v, x) && !(v.agg[x].heavy & 1); },
+        [&](int32_t x) {
+            const int4 vr = x >= 0 ? v.vrec[x] : make_int4(0, 0, 0, 0);
+            u64 *list = v.vedge + vr.w;
+            u64 sig = 0, small = ~0ull;
+            int32_t w = 0, mf = 0;
+            const int32_t maxdeg = __reduce_max_sync(0xffffffffu, vr.z);
+#pragma unroll 1
+            for (int32_t k0 = 0; k0 < maxdeg; k0 += kU * kG) {
+                u64 ent[kU];
+                int4 r[kU];
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    const int32_t k = k0 + u * kG + c.sub;
+                    ent[u] = k < vr.z ? list[k] : kNoEntry;
+                }
+#pragma unroll
+                for (int u = 0; u < kU; ++u)
+                    r[u] = ent[u] != kNoEntry ? erec[entry_id(ent[u])] : make_int4(0, 0, kGone, 0);
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    const bool keep = r[u].z != kGone;
+                    const unsigned b = group_ballot(c, keep);
+                    if (keep) {
+                        const int32_t e = entry_id(ent[u]);
+                        sig |= sig_bit(e);
+                        mf = max(mf, r[u].z);
+                        const u64 key = ((u64)(uint32_t)r[u].w << 32) | (uint32_t)e;
+                        small = key < small ? key : small;
+                        list[w + __popc(b & ((1u << c.sub) - 1u))] =
+                            make_entry(e, r[u].z, r[u].w, fold_sig(rec_sig(r[u])));
+                    }
+                    w += __popc(b);
+                }
+            }
+            sig = group_or(sig);
+            small = group_min(small);
+            mf = group_max(mf);
+            if (x >= 0 && c.sub == 0) {
+                v.vrec[x] = make_rec(sig, w, vr.w);
+                const int32_t e0 = (int32_t)(uint32_t)small;
+                v.vaux[x] = make_int4(e0, mf, w > 0 ? v.eptr[e0] : 0, (int32_t)(small >> 32));
+            }
+        });
+    // the vertices whose degree at load was above kHeavyDeg: one CTA each
+    Shared *sh = c.sh;
+    const int32_t nh = vload(&v.ctl->n_heavy);
+#pragma unroll 1
+    for (int32_t h = sh->rank; h < nh; h += sh->size) {
+        const int32_t x = sh->heavy[h];
+        if (!vertex_candidate(c, v, x)) continue;
+        const int4 vr = v.vrec[x];
+        u64 *list = v.vedge + vr.w;
+        __syncthreads();  // every thread has the record before it is replaced
+        if (threadIdx.x == 0) { sh->pos = 0; sh->mf = 0; sh->sig = 0; sh->small = ~0ull; }
+        __syncthreads();
+        u64 sig = 0, small = ~0ull;
+        int32_t mf = 0;
+#pragma unroll 1
+        for (int32_t k0 = 0; k0 < vr.z; k0 += kU * blockDim.x) {
+            int32_t e[kU];
+            int4 r[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int32_t k = k0 + u * blockDim.x + threadIdx.x;
+                e[u] = k < vr.z ? entry_id(list[k]) : -1;
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u)
+                r[u] = e[u] >= 0 ? erec[e[u]] : make_int4(0, 0, kGone, 0);
+            __syncthreads();  // the chunk is read: the kept ones move to the front
+            int32_t kept = 0;
+#pragma unroll
+            for (int u = 0; u < kU; ++u) kept += __popc(__ballot_sync(0xffffffffu, r[u].z != kGone));
+            int32_t at = 0;
+            if (c.lane == 0 && kept) at = atomicAdd(&sh->pos, kept);
+            at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const bool keep = r[u].z != kGone;
+                const unsigned b = __ballot_sync(0xffffffffu, keep);
+                if (keep) {
+                    sig |= sig_bit(e[u]);
+                    mf = max(mf, r[u].z);
+                    const u64 key = ((u64)(uint32_t)r[u].w << 32) | (uint32_t)e[u];
+                    small = key < small ? key : small;
+                    list[at + __popc(b & ((1u << c.lane) - 1u))] =
+                        make_entry(e[u], r[u].z, r[u].w, fold_sig(rec_sig(r[u])));
+                }
+                at += __popc(b);
+            }
+            __syncthreads();
+        }
+        mf = __reduce_max_sync(0xffffffffu, mf);
+#pragma unroll 1
+        for (int o = 16; o > 0; o >>= 1) {
+            sig |= __shfl_xor_sync(0xffffffffu, sig, o);
+            const u64 y = __shfl_xor_sync(0xffffffffu, small, o);
+            small = y < small ? y : small;
+        }
+        if (c.lane == 0) {
+            atomicMax(&sh->mf, mf);
+            atomicOr(&sh->sig, sig);
+            atomicMin(&sh->small, small);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            v.vrec[x] = make_rec(sh->sig, sh->pos, vr.w);
+            const int32_t e0 = (int32_t)(uint32_t)sh->small;
+            v.vaux[x] = make_int4(e0, sh->mf, sh->pos > 0 ? v.eptr[e0] : 0,
+                                  (int32_t)(sh->small >> 32));
+        }
+        __syncthreads();
+    }
+}
+
+// The vertex of key i in the row of hyperedge e?
+__device__ __forceinline__ bool in_row(const View &v, int32_t e, uint32_t i) {
+    const uint32_t *r = v.row + v.eptr[e];
+    const int32_t len = v.erec[e].w;
+    const int32_t at = find_key(r, len, i);
+    return at < len && r[at] == i;
+}
+
+// Can vertex i dominate j, by degree, signature and tie-break?
+__device__ __forceinline__ bool may_dominate(int32_t i, int4 ri, int32_t j, int4 rj) {
+    if (i == j || ri.z < rj.z) return false;
+    if (rec_sig(rj) & ~rec_sig(ri)) return false;
+    return ri.z > rj.z || i < j;  // equal degrees: contained means equal, the lower index dominates
+}
+
+// Delete vertex j (lane `sub` of `step` lanes): its hyperedges are the next
+// round's candidates.
+__device__ __forceinline__ void delete_vertex(Shared *sh, int32_t j, int4 rj, int32_t sub,
+                                              int32_t step) {
+    const View &v = sh->view;
+    if (sub == 0) {
+        v.v_o2c[j] = -1;
+        atomicAdd(&sh->del2, 1);
+    }
+    const int32_t next = sh->epoch + 1;
+#pragma unroll 1
+    for (int32_t q = sub; q < rj.z; q += step) v.estamp[entry_id(v.vedge[rj.w + q])] = next;
+}
+
+// The dominators of the candidates (count: into v_cnt; else a vertex with
+// at least as many as its largest demand is deleted, and its hyperedges
+// become the next round's candidates).
+__device__ __noinline__ void md_test(bool count, int shard, int nshards) {
+    const Ctx c;
+    Shared *sh = c.sh;
+    const View &v = sh->view;
+    const int4 *const vrec = v.vrec;
+    int32_t *const v_cnt = sh->s->v_cnt;
+    for_flagged(
+        c, sh->n0,
+        [&](int32_t x) {
+            return vertex_candidate(c, v, x) && !(v.agg[x].heavy & 1) &&
+                   (!count || nshards == 1 || (x >> 7) % nshards == shard);
+        },
+        [&](int32_t j) {
+            const int4 rj = j >= 0 ? vrec[j] : make_int4(0, 0, 0, 0);
+            const int4 aux = j >= 0 ? v.vaux[j] : make_int4(0, 0, 0, 0);
+            const int32_t e0 = aux.x;
+            int32_t len0 = rj.z > 0 ? aux.w : 0;
+            if (!count && len0 - 1 < aux.y) len0 = 0;  // too few members to dominate
+            const uint32_t *row = v.row + aux.z;
+            const u64 *list = v.vedge + rj.w;
+            int32_t cnt = 0;
+            const int32_t maxlen = __reduce_max_sync(0xffffffffu, len0);
+#pragma unroll 1
+            for (int32_t k = c.sub; k - c.sub < maxlen; k += kG) {
+                const uint32_t i = k < len0 ? row[k] : 0;
+                bool ok = k < len0 && may_dominate(key_id(i), vrec[key_id(i)], j, rj);
+#pragma unroll 1
+                for (int32_t q = 0; q < rj.z && ok; ++q) {
+                    const int32_t e = entry_id(list[q]);
+                    ok = e == e0 || in_row(v, e, i);
+                }
+                cnt += ok;
+                __syncwarp();
+            }
+            cnt = group_sum(cnt);
+            if (j >= 0) {
+                if (count) {
+                    if (c.sub == 0) v_cnt[j] = cnt;
+                } else if (rj.z == 0 || cnt >= aux.y) {
+                    delete_vertex(sh, j, rj, c.sub, kG);
+                }
+            }
+            __syncwarp();
+        });
+    const int32_t nh = vload(&v.ctl->n_heavy);
+#pragma unroll 1
+    for (int32_t h = sh->rank; h < nh; h += sh->size) {
+        const int32_t j = sh->heavy[h];
+        const bool mine = vertex_candidate(c, v, j) &&
+                          (!count || nshards == 1 || (j >> 7) % nshards == shard);
+        __syncthreads();  // (v_o2c[j] is written below)
+        if (!mine) continue;
+        const int4 rj = vrec[j], aux = v.vaux[j];
+        const int32_t e0 = aux.x, len0 = rj.z > 0 ? aux.w : 0;
+        if (rj.z > 0 && !count && len0 - 1 < aux.y) continue;
+        const uint32_t *row = v.row + aux.z;
+        const u64 *list = v.vedge + rj.w;
+        if (threadIdx.x == 0) sh->pos = 0;
+        __syncthreads();
+        // one member per warp, 32 hyperedges at a time
+#pragma unroll 1
+        for (int32_t k = c.warp; k < len0; k += blockDim.x >> 5) {
+            const uint32_t i = row[k];
+            bool ok = may_dominate(key_id(i), vrec[key_id(i)], j, rj);  // (all lanes alike)
+#pragma unroll 1
+            for (int32_t q0 = 0; q0 < rj.z && ok; q0 += 32) {
+                const int32_t q = q0 + c.lane;
+                const int32_t e = q < rj.z ? entry_id(list[q]) : e0;
+                const bool in = e == e0 || in_row(v, e, i);
+                __syncwarp();
+                ok = !__any_sync(0xffffffffu, !in);
+            }
+            if (ok && c.lane == 0) atomicAdd(&sh->pos, 1);
+        }
+        __syncthreads();
+        const int32_t cnt = sh->pos;
+        __syncthreads();  // (reset for the next)
+        if (count) {
+            if (threadIdx.x == 0) v_cnt[j] = cnt;
+        } else if (rj.z == 0 || cnt >= aux.y) {
+            delete_vertex(sh, j, rj, threadIdx.x, blockDim.x);
+        }
+    }
+}
+
+// Sharded passes: the decision from the (merged) counts.
+__device__ __noinline__ void md_decide() {
+    const Ctx c;
+    const View &v = c.sh->view;
+    const int32_t *const v_cnt = c.sh->s->v_cnt;
+    for_flagged(
+        c, c.sh->n0, [&](int32_t x) { return vertex_candidate(c, v, x); },
+        [&](int32_t j) {
+            if (j >= 0) {
+                const int4 rj = v.vrec[j];
+                if (rj.z == 0 || v_cnt[j] >= v.vaux[j].y) delete_vertex(c.sh, j, rj, c.sub, kG);
+            }
+            __syncwarp();
+        });
+}
+
+// ---------------------------------------------------------------- rule FE --
+
+// Full hyperedges go, their vertices into the solution.
+__device__ __noinline__ void fe_mark() {
+    const Ctx c;
+    const View &v = c.sh->view;
+    uint8_t *const forced = c.sh->s->forced;
+    for_flagged(
+        c, c.sh->m0, [&](int32_t e) { return v.e_o2c[e] >= 0; },
+        [&](int32_t e) {
+            const int4 r = e >= 0 ? v.erec[e] : make_int4(0, 0, 0, -1);
+            __syncwarp();  // read by every lane before it is written
+            if (r.w == r.z) {
+                const uint32_t *row = v.row + v.eptr[e];
+#pragma unroll 1
+                for (int32_t k = c.sub; k < r.w; k += kG) {
+                    const int32_t x = key_id(row[k]);
+                    if (atomicExch(&v.v_o2c[x], -1) >= 0) {
+                        forced[x] = 1;
+                        atomicAdd(&c.sh->del2, 1);
+                    }
+                }
+                if (c.sub == 0) {
+                    v.erec[e].z = kGone;
+                    v.e_o2c[e] = -1;
+                    atomicOr(&v.gone[e >> 5], 1u << (e & 31));
+                    atomicAdd(&c.sh->del, 1);
+                }
+            }
+            __syncwarp();
+        });
+}
+
+// The others lose one unit of demand per vertex taken; the bounds restart.
+__device__ __noinline__ void fe_apply() {
+    const Ctx c;
+    const View &v = c.sh->view;
+    int32_t *const f = c.sh->s->f;
+    for_flagged(
+        c, c.sh->m0, [&](int32_t e) { return v.e_o2c[e] >= 0; },
+        [&](int32_t e) {
+            const int4 r = e >= 0 ? v.erec[e] : make_int4(0, 0, 0, 0);
+            const uint32_t *row = e >= 0 ? v.row + v.eptr[e] : nullptr;
+            int32_t lost = 0;
+#pragma unroll 1
+            for (int32_t k = c.sub; k < r.w; k += kG) lost += v.v_o2c[key_id(row[k])] < 0;
+            __syncwarp();
+            lost = group_sum(lost);
+            if (lost > 0 && c.sub == 0) {
+                const int32_t left = r.z - lost;
+                f[e] = left;
+                v.erec[e].z = left > 0 ? left : kGone;
+                if (left <= 0) {
+                    v.e_o2c[e] = -1;
+                    atomicOr(&v.gone[e >> 5], 1u << (e & 31));
+                    atomicAdd(&c.sh->del, 1);
+                }
+            }
+            __syncwarp();
+        });
+    const int32_t t0 = c.sh->rank * blockDim.x + threadIdx.x, ts = c.sh->size * blockDim.x;
+#pragma unroll 1
+    for (int32_t x = t0; x < c.sh->n0; x += ts) {
+        v.agg[x].m1 = 0;
+        v.agg[x].heavy &= 1;
+        v.agg[x].s1 = 0;
+    }
+#pragma unroll 1
+    for (uint32_t q = t0; q <= c.sh->pair_mask; q += ts) c.sh->pair_tab[q] = SpPair{};
+    if (t0 == 0) {
+        v.ctl->loose = 0;
+        v.ctl->empty = 0;
+        v.ctl->pairs_full = 0;
+    }
+}
+
+// ------------------------------------------------------------------ build --
+
+// Hyperedge e of the input: its checks, the vertices' degrees and the
+// incidences' places in their lists.  A row that is not strictly ascending is
+// sorted, without repeats, into v.row (its ids; noted in the record).
+// Returns the error bits found.  The whole warp.
+__device__ __forceinline__ int32_t count_row(const Ctx &c, const View &v, const int32_t *evtx,
+                                             const int32_t *f, int32_t *place, int32_t n0,
+                                             int64_t nnz0, int32_t e) {
+    int32_t p0 = 0, len = 0, fe = 1, bad = 0;
+    if (e >= 0) {
+        p0 = v.eptr[e];
+        len = v.eptr[e + 1] - p0;
+        fe = f[e];
+        if (fe < 1) bad |= kErrBadDemand;
+        if (p0 < 0 || len < 0 || (int64_t)p0 + len > nnz0) { bad |= kErrBadPtr; len = 0; }
+    }
+    const int32_t *in = evtx + p0;
+    int32_t *row = reinterpret_cast<int32_t *>(v.row) + p0;
+    const int32_t maxlen = __reduce_max_sync(0xffffffffu, len);
+    // first the entries, in order? (each against its right neighbour)
+    bool asc = true;
+#pragma unroll 1
+    for (int32_t k = c.sub; k + 1 < len; k += kG) asc = asc && in[k] < in[k + 1];
+    __syncwarp();
+    const bool sorted = group_ballot(c, !asc) == 0;
+    if (__any_sync(0xffffffffu, !sorted)) {
+        // rank sort (ties by place), then drop repeats
+        if (!sorted)
+#pragma unroll 1
+            for (int32_t k = c.sub; k < len; k += kG) {
+                const int32_t y = in[k];
+                int32_t rank = 0;
+#pragma unroll 1
+                for (int32_t l = 0; l < len; ++l) rank += in[l] < y || (in[l] == y && l < k);
+                row[rank] = y;
+            }
+        __syncwarp();
+        int32_t w = len;
+        if (!sorted && c.sub == 0) {
+            int32_t last = row[0];
+            w = 1;
+#pragma unroll 1
+            for (int32_t k = 1; k < len; ++k) {
+                const int32_t y = row[k];
+                if (y != last) row[w++] = y;
+                last = y;
+            }
+        }
+        len = __shfl_sync(0xffffffffu, w, c.lead);
+        __syncwarp();
+    }
+    const int32_t *ids = sorted ? in : row;
+#pragma unroll 1
+    for (int32_t k0 = 0; k0 < maxlen; k0 += kRowU * kG) {
+        int32_t x[kRowU], at[kRowU];
+#pragma unroll
+        for (int u = 0; u < kRowU; ++u) {
+            const int32_t k = k0 + u * kG + c.sub;
+            x[u] = k < len ? ids[k] : 0;
+        }
+        // (the atomics of a batch are under way together)
+#pragma unroll
+        for (int u = 0; u < kRowU; ++u) {
+            const bool on = k0 + u * kG + c.sub < len;
+            const bool ok = x[u] >= 0 && x[u] < n0;
+            if (on && !ok) bad |= kErrBadVertex;
+            at[u] = on && ok ? atomicAdd(&v.vrec[x[u]].z, 1) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < kRowU; ++u)
+            if (k0 + u * kG + c.sub < len) place[p0 + k0 + u * kG + c.sub] = at[u];
+    }
+    if (e >= 0 && c.sub == 0) v.erec[e] = make_int4(sorted ? 0 : 1, 0, fe, len);
+    return bad;
+}
+
+// The row of hyperedge e in key order, and its entries in its vertices'
+// lists, by kW lanes (8 or 32; `lane` of them, from the warp's lane `lead`)
+// that hold the row (len <= kRowU * kW) in registers and rank each key by
+// counting.  Adds to *cost the lengths of the lists of its np rarest
+// vertices; returns the signature.  The whole warp calls it.
+template <int kW>
+__device__ __forceinline__ u64 fill_row(const Ctx &c, const View &v, const int32_t *ids,
+                                        const int32_t *place, uint32_t *row, int32_t e, int32_t f,
+                                        int32_t len, int32_t np, int lane, int lead, u64 *cost) {
+    const int32_t maxlen = kW == 32 ? len : __reduce_max_sync(0xffffffffu, len);
+    uint32_t key[kRowU];
+    int32_t at[kRowU], deg[kRowU], rank[kRowU];
+    u64 sig = 0;
+#pragma unroll
+    for (int u = 0; u < kRowU; ++u) {
+        const int32_t k = u * kW + lane;
+        const int32_t x = k < len ? ids[k] : -1;
+        const int4 vr = x >= 0 ? v.vrec[x] : make_int4(0, 0, 0, 0);
+        key[u] = x >= 0 ? row_key(x, vr.z) : 0xffffffffu;
+        at[u] = x >= 0 ? vr.w + place[k] : 0;
+        deg[u] = vr.z;
+        rank[u] = 0;
+        if (x >= 0) sig |= sig_bit(x);
+    }
+    sig = group_or(sig);
+    if (kW == 32) {
+        sig |= __shfl_xor_sync(0xffffffffu, sig, 8);
+        sig |= __shfl_xor_sync(0xffffffffu, sig, 16);
+    }
+#pragma unroll
+    for (int w = 0; w < kRowU; ++w) {
+        const int32_t n = min(kW, maxlen - w * kW);
+#pragma unroll 1
+        for (int l = 0; l < n; ++l) {
+            const uint32_t y = __shfl_sync(0xffffffffu, key[w], lead + l);
+#pragma unroll
+            for (int u = 0; u < kRowU; ++u) rank[u] += y < key[u];
+        }
+    }
+    __syncwarp();  // (ids may lie where the row goes)
+    const uint32_t fold = fold_sig(sig);
+#pragma unroll
+    for (int u = 0; u < kRowU; ++u) {
+        if (u * kW + lane >= len) continue;
+        row[rank[u]] = key[u];
+        v.vedge[at[u]] = make_entry(e, f, len, fold);
+        if (rank[u] < np) *cost += (uint32_t)deg[u];
+    }
+    return sig;
+}
+
+// The same for any length, by the warp: keys into tmp, then class by class
+// of the degree, rarest first (ids ascend inside a class).
+__device__ __noinline__ u64 fill_long_row(const int32_t *ids, const int32_t *place, uint32_t *tmp,
+                                          uint32_t *row, int32_t e, int32_t f, int32_t len,
+                                          int32_t np, u64 *cost) {
+    const View &v = shared()->view;
+    const int lane = threadIdx.x & 31;
+    u64 sig = 0;
+#pragma unroll 1
+    for (int32_t k = lane; k < len; k += 32) {
+        const int32_t x = ids[k];
+        tmp[k] = row_key(x, v.vrec[x].z);
+        sig |= sig_bit(x);
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) sig |= __shfl_xor_sync(0xffffffffu, sig, o);
+    const uint32_t fold = fold_sig(sig);
+#pragma unroll 1
+    for (int32_t k = lane; k < len; k += 32)
+        v.vedge[v.vrec[key_id(tmp[k])].w + place[k]] = make_entry(e, f, len, fold);
+    uint32_t from = 0;  // keys below are placed
+#pragma unroll 1
+    for (int32_t w = 0; w < len;) {
+        uint32_t low = 0xffffffffu;
+#pragma unroll 1
+        for (int32_t k = lane; k < len; k += 32) {
+            const uint32_t y = tmp[k];
+            if (y >= from) low = min(low, y);
+        }
+        __syncwarp();
+        low = __reduce_min_sync(0xffffffffu, low) & ~kIdMask;
+        const uint32_t end = low | kIdMask;
+#pragma unroll 1
+        for (int32_t k0 = 0; k0 < len; k0 += 32) {
+            const int32_t k = k0 + lane;
+            const uint32_t y = k < len ? tmp[k] : 0xffffffffu;
+            const bool in = k < len && y >= low && y <= end;
+            const unsigned b = __ballot_sync(0xffffffffu, in);
+            if (in) {
+                const int32_t to = w + __popc(b & ((1u << lane) - 1u));
+                row[to] = y;
+                if (to < np) *cost += (uint32_t)v.vrec[key_id(y)].z;
+            }
+            w += __popc(b);
+        }
+        from = end + 1;  // (the top class, 0xff, cannot occur)
+    }
+    return sig;
+}
+
+// ------------------------------------------------------------ round driver --
+
+// Add this CTA's deletions of a phase to the instance's counter.
+__device__ __forceinline__ void flush(int32_t *sh_ctr, int32_t *to) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (*sh_ctr) atomicAdd(to, *sh_ctr);
+        *sh_ctr = 0;
+    }
+}
+
+// Shared memory for one instance.
+__device__ __noinline__ void start(InstState *s, int rank, int size) {
+    Shared *sh = shared();
+    if (threadIdx.x == 0) {
+        sh->view = View(*s);
+        sh->s = s;
+        sh->heavy = s->sp_heavy;
+        sh->pair_tab = s->sp_pair_tab;
+        sh->pair_mask = s->sp_pair_mask;
+        sh->task = s->sp_task;
+        sh->task_cap = s->sp_task_cap;
+        sh->n0 = s->n0;
+        sh->m0 = s->m0;
+        sh->rule = s->edge_rule;
+        sh->rank = rank;
+        sh->size = size;
+        sh->epoch = 1;
+        sh->par = 0;
+        sh->full = 1;
+        sh->del = sh->del2 = 0;
+        sh->cost = 0;
+        sh->pairs = s->sp_pairs;
+        sh->pair_cap = s->sp_pair_cap;
+        sh->bar = &s->sp_ctl->bar;
+        // no barrier can complete without this CTA, so the arrivals seen
+        // beyond a multiple of the team's size are this launch's first
+        const uint32_t now = *reinterpret_cast<volatile uint32_t *>(sh->bar);
+        sh->target = now / (uint32_t)size * (uint32_t)size;
+    }
+    __syncthreads();
+}
+
+// Structural checks, rows and lists of one instance.
+__device__ __noinline__ void build_instance(int32_t max_rounds, SpTotals *out) {
+    const Ctx c;
+    InstState &s = *c.sh->s;
+    const View v = c.sh->view;
+    const int32_t n0 = s.n0, m0 = s.m0;
+    const int64_t nnz0 = s.nnz0;
+    const int32_t *const evtx = s.evtx;
+    const int32_t *const f = s.f;
+    int32_t *const place = s.sp_pos;
+    uint32_t *const tmp = s.sp_tmp;
+    const int32_t t0 = c.sh->rank * blockDim.x + threadIdx.x, ts = c.sh->size * blockDim.x;
+    if (t0 == 0) {
+        s.n = s.n0; s.m = s.m0; s.m_dp = s.m0; s.n_next = s.n0;
+        s.rounds = 0; s.active = 1; s.max_rounds = max_rounds; s.changed = 0;
+        s.dp_deleted = 0; s.md_deleted = 0; s.fe_stage = 0; s.fe_passes = 0;
+        v.ctl->full = 1;
+        if (s.eptr[0] != 0 || (int64_t)s.eptr[s.m0] != s.nnz0) atomicOr(&s.status, kErrBadPtr);
+    }
+    // (the records, bounds and stamps are zero: cleared with the control words)
+    int32_t bad = 0;
+    uint8_t *const forced = s.forced;
+#pragma unroll 1
+    for (int32_t x = t0; x < n0; x += ts) {
+        v.v_o2c[x] = x;
+        if (forced) forced[x] = 0;
+    }
+#pragma unroll 1
+    for (int32_t e = t0; e < m0; e += ts) v.e_o2c[e] = e;
+    for_flagged(
+        c, m0, [](int32_t) { return true; },
+        [&](int32_t e) { bad |= count_row(c, v, evtx, f, place, n0, nnz0, e); });
+    if (bad) atomicOr(&s.status, bad);
+    if (!team_sync()) return;
+    if (const int32_t st = vload(&s.status)) {
+        if (t0 == 0) atomicOr(&out->status, st);
+        return;
+    }
+    // a place for every vertex's list (in any order): one atomic per warp
+    int32_t *const heavy = s.sp_heavy;
+#pragma unroll 1
+    for (int32_t x0 = t0 - c.lane; x0 < n0; x0 += ts) {
+        const int32_t x = x0 + c.lane;
+        const int32_t d = x < n0 ? v.vrec[x].z : 0;
+        int32_t inc = d;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (c.lane >= o) inc += y;
+        }
+        int32_t at = 0;
+        if (c.lane == 31) at = (int32_t)atomicAdd(&v.ctl->cursor, (uint32_t)inc);
+        at = __shfl_sync(0xffffffffu, at, 31);
+        if (x < n0) v.vrec[x].w = at + inc - d;
+        if (d > kHeavyDeg) {
+            v.agg[x].heavy = 1;
+            heavy[atomicAdd(&v.ctl->n_heavy, 1)] = x;
+        }
+    }
+    if (!team_sync()) return;
+    const int32_t rule = s.edge_rule;
+    for_flagged(
+        c, m0, [](int32_t) { return true; },
+        [&](int32_t e) {
+            const int4 r = e >= 0 ? v.erec[e] : make_int4(0, 0, 0, 0);
+            const int32_t p0 = e >= 0 ? v.eptr[e] : 0, len = r.w;
+            const int32_t *ids = r.x ? reinterpret_cast<const int32_t *>(v.row) + p0 : evtx + p0;
+            uint32_t *row = v.row + p0;
+            const int32_t np = e >= 0 ? walk_count(rule, r.z, len) : 0;
+            u64 sig = 0, cost = 0;  // cost: the entries walking this hyperedge may visit
+            // rows up to 32: the group ranks each key among the row's
+            const bool small = len <= kRowU * kG;
+            if (__any_sync(0xffffffffu, small && len > 0)) {
+                sig = fill_row<kG>(c, v, ids, place + p0, row, e, r.z, small ? len : 0, np, c.sub,
+                                   c.lead, &cost);
+                if (small && c.sub == 0 && e >= 0) v.erec[e] = make_rec(sig, r.z, len);
+            }
+            // longer ones, one after the other: the whole warp
+            unsigned longs = __ballot_sync(0xffffffffu, !small && c.sub == 0);
+#pragma unroll 1
+            while (longs) {
+                const int l = __ffs(longs) - 1;
+                longs &= longs - 1;
+                const int32_t le = __shfl_sync(0xffffffffu, e, l);
+                const int32_t lp = __shfl_sync(0xffffffffu, p0, l);
+                const int32_t llen = __shfl_sync(0xffffffffu, len, l);
+                const int32_t lf = __shfl_sync(0xffffffffu, r.z, l);
+                const int32_t lnp = __shfl_sync(0xffffffffu, np, l);
+                const bool sorted = __shfl_sync(0xffffffffu, r.x, l) == 0;
+                const int32_t *lids =
+                    sorted ? evtx + lp : reinterpret_cast<const int32_t *>(v.row) + lp;
+                u64 ls;
+                if (llen <= kRowU * 32)
+                    ls = fill_row<32>(c, v, lids, place + lp, v.row + lp, le, lf, llen, lnp, c.lane,
+                                      0, &cost);
+                else
+                    ls = fill_long_row(lids, place + lp, tmp + lp, v.row + lp, le, lf, llen, lnp, &cost);
+                if (c.lane == 0) v.erec[le] = make_rec(ls, lf, llen);
+                __syncwarp();
+            }
+            cost += (u64)(uint32_t)(c.sub == 0 ? np : 0);
+            __syncwarp();
+            if (e >= 0) contribute(e, r.z, len, row);
+            __syncwarp();
+#pragma unroll
+            for (int o = kG / 2; o > 0; o >>= 1) cost += __shfl_xor_sync(0xffffffffu, cost, o);
+            if (c.sub == 0 && cost) atomicAdd(&c.sh->cost, cost);
+        });
+    __syncthreads();
+    if (threadIdx.x == 0 && c.sh->cost) atomicAdd(&out->cost, c.sh->cost);
+}
+
+// Thread 0 of every CTA: the state at the start of a launch.
+__device__ void load_progress(Progress &g, const InstState &s) {
+    g.n = s.n; g.m = s.m; g.rounds = s.rounds; g.changed = s.changed;
+    g.dp = s.dp_deleted; g.md = s.md_deleted; g.fe_passes = s.fe_passes;
+    g.max_rounds = s.max_rounds; g.fe = s.full_edges; g.k = s.k;
+    g.active = s.active && !s.status;
+    g.full = s.sp_ctl->full;
+    g.t_dp = g.t_md = 0;
+    g.t_all = globaltimer();
+}
+
+// One thread of the team: the state at its end.
+__device__ void store_progress(const Progress &g, InstState &s, BatchCounters *ctr) {
+    s.n = g.n; s.n_next = g.n; s.m = g.m; s.m_dp = g.m; s.rounds = g.rounds;
+    s.changed = g.changed; s.dp_deleted = g.dp; s.md_deleted = g.md;
+    s.fe_passes = g.fe_passes; s.k = g.k; s.active = g.active;
+    s.sp_ctl->full = g.full;
+    if (!ctr) return;
+    atomicAdd(&ctr->active, g.active);
+    atomicAdd(&ctr->n_alive, g.n);
+    atomicAdd(&ctr->m_alive, g.m);
+    atomicAdd(&ctr->dp_deleted, g.dp);
+    atomicAdd(&ctr->md_deleted, g.md);
+    atomicMax(&ctr->max_rounds_seen, g.rounds);
+    atomicOr(&ctr->changed_any, g.changed);
+    atomicOr(&ctr->status_any, vload(&s.status));
+}
+
+__device__ __forceinline__ void begin_round() {
+    Shared *sh = shared();
+    if (threadIdx.x == 0) {
+        sh->epoch = sh->g.rounds + 1;
+        sh->par = sh->g.rounds & 1;
+        sh->full = sh->g.full;
+    }
+    __syncthreads();
+}
+
+// The end of a round that deleted dp hyperedges and md vertices: the books,
+// rule FE at a fixpoint, and whether there is more to do.  False if a
+// barrier timed out.
+__device__ __noinline__ bool finish_round(int32_t dp, int32_t md) {
+    Shared *sh = shared();
+    SpCtl *ctl = sh->view.ctl;
+    Progress &g = sh->g;
+    const bool fe = dp + md == 0 && g.fe && g.max_rounds == 0;
+    __syncthreads();  // g is read above by every thread
+    if (threadIdx.x == 0) {
+        if (sh->rank == 0 && g.rounds < kTraceRounds) {
+            int32_t *row = sh->s->trace[g.rounds];
+            row[0] = g.m;
+            row[1] = g.n;
+            row[2] = g.m - dp;
+        }
+        g.dp = dp;
+        g.md = md;
+        g.m -= dp;
+        g.n -= md;
+        g.full = 0;
+        g.changed = dp + md > 0;
+        ++g.rounds;
+        if (!fe && (!g.changed || (g.max_rounds > 0 && g.rounds >= g.max_rounds))) g.active = 0;
+    }
+    __syncthreads();
+    if (!fe) return true;
+    fe_mark();
+    flush(&sh->del, &ctl->fe.dp);
+    flush(&sh->del2, &ctl->fe.md);
+    if (!team_sync()) return false;
+    fe_apply();
+    flush(&sh->del, &ctl->fe.dp);
+    if (!team_sync(&ctl->fe)) return false;
+    const int32_t de = sh->got.dp, dv = sh->got.md;
+    if (!team_sync()) return false;  // every CTA has read them
+    if (threadIdx.x == 0) {
+        if (sh->rank == 0) ctl->fe = SpRound{};
+        ++g.fe_passes;
+        g.m -= de;
+        g.n -= dv;
+        g.k -= dv;
+        // lowered demands make every hyperedge and vertex a candidate again
+        if (de + dv > 0) g.full = g.changed = 1;
+        else g.active = 0;
+    }
+    __syncthreads();
+    return true;
+}
+
+// Rounds of Algorithm 3 (and FE at its fixpoints) until the fixpoint or
+// `limit` rounds (0: no limit).
+__device__ __noinline__ void run_instance(int32_t limit, BatchCounters *ctr, SpTimes *times) {
+    Shared *sh = shared();
+    if (threadIdx.x == 0) load_progress(sh->g, *sh->s);
+    // one CTA must not publish the final state before all have read this one
+    if (!team_sync()) return;
+    for (int32_t done = 0; sh->g.active && (limit <= 0 || done < limit); ++done) {
+        begin_round();
+        SpRound *rc = &sh->view.ctl->c[sh->par], *nx = &sh->view.ctl->c[sh->par ^ 1];
+        const bool lead = sh->rank == 0 && threadIdx.x == 0;
+        int32_t dp = 0, md = 0;
+        if (sh->full || sh->g.md > 0) {
+            if (sh->epoch > 1) {  // (the first round's rows are the load's)
+                dp_rows();
+                if (!team_sync()) return;
+                if (sh->full) {  // FE lowered demands, which the lists repeat
+                    md_lists();
+                    if (!team_sync()) return;
+                }
+            }
+            if (lead) sh->g.t_dp -= globaltimer();
+            dp_bounds(0, 1);
+            // full rounds: the walks skip what the bounds deleted (a matter of
+            // time only: 40 M list entries become 14 M on the power-law instance)
+            if (sh->full && !team_sync()) return;
+            dp_walk(0, 1);
+            flush(&sh->del, &rc->dp);
+            if (!team_sync(rc)) return;
+            // (each list has a counter that is final at the barrier before it is
+            // read: the CTAs must agree on the barriers that follow)
+            if (sh->got.npair[0] > 0) {
+                decide_pairs(0);
+                flush(&sh->del, &rc->dp);
+                if (!team_sync(rc)) return;
+            }
+            if (sh->got.ntask > 0) {  // (after the pairs: a hyperedge found deleted needs no walk)
+                dp_tasks(0, 1);
+                flush(&sh->del, &rc->dp);
+                if (!team_sync(rc)) return;
+                if (sh->got.npair[1] > 0) {
+                    decide_pairs(1);
+                    flush(&sh->del, &rc->dp);
+                    if (!team_sync(rc)) return;
+                }
+            }
+            if (lead) sh->g.t_dp += globaltimer();
+            dp = sh->got.dp;
+            // every CTA is past the previous round: its counters serve the next one
+            if (lead) *nx = SpRound{};
+            if (sh->full || dp > 0) {
+                md_lists();
+                if (!team_sync()) return;
+                if (lead) sh->g.t_md -= globaltimer();
+                md_test(false, 0, 1);
+                flush(&sh->del2, &rc->md);
+                if (!team_sync(rc)) return;
+                if (lead) sh->g.t_md += globaltimer();
+                md = sh->got.md;
+            }
+        } else if (lead) {
+            // no hyperedge lost a vertex: both passes are empty.  (The last
+            // round's md is 0, so resetting its counters loses nothing.)
+            *nx = SpRound{};
+        }
+        if (!finish_round(dp, md)) return;
+    }
+    if (sh->rank == 0 && threadIdx.x == 0) {
+        const Progress &g = sh->g;
+        store_progress(g, *sh->s, ctr);
+        atomicAdd(&times->dp, (u64)g.t_dp);
+        atomicAdd(&times->md, (u64)g.t_md);
+        atomicAdd(&times->all, (u64)(globaltimer() - g.t_all));
+    }
+}
+
+// One part of a sharded round (mhs_pass_*).
+__device__ void run_pass(int op, int shard, int nshards, BatchCounters *ctr, void *buf) {
+    Shared *sh = shared();
+    InstState &s = *sh->s;
+    if (threadIdx.x == 0) load_progress(sh->g, s);
+    if (!team_sync()) return;
+    begin_round();
+    const bool lead = sh->rank == 0 && threadIdx.x == 0;
+    const int32_t t0 = sh->rank * blockDim.x + threadIdx.x, ts = sh->size * blockDim.x;
+    if (!sh->g.active && op != kSpExport0 && op != kSpExport1) {
+        if (lead && op == kSpEnd1) store_progress(sh->g, s, ctr);
+        return;
+    }
+    const Ctx c;
+    const View v = sh->view;
+    SpRound *rc = &v.ctl->c[sh->par], *nx = &v.ctl->c[sh->par ^ 1];
+    switch (op) {
+        case kSpBegin0:
+            if (lead) *nx = SpRound{};
+            if (c.epoch > 1) {
+                dp_rows();
+                if (c.full) {  // FE lowered demands, which the lists repeat
+                    if (!team_sync()) return;
+                    md_lists();
+                }
+            }
+            break;
+        case kSpContract0:
+            if (lead) rc->ntask = rc->npair[0] = rc->npair[1] = 0;
+            if (!team_sync()) return;
+            dp_bounds(shard, nshards);
+            if (!team_sync()) return;
+            dp_walk(shard, nshards);
+            if (!team_sync(rc)) return;
+            dp_tasks(shard, nshards);
+            if (!team_sync(rc)) return;
+            decide_pairs(0);
+            decide_pairs(1);
+            flush(&sh->del, &rc->dp);
+            break;
+        case kSpExport0:
+#pragma unroll 1
+            for (int32_t e = t0; e < s.m0; e += ts)
+                static_cast<uint8_t *>(buf)[e] = v.e_o2c[e] == -1 - c.epoch;
+            break;
+        case kSpImport0:
+#pragma unroll 1
+            for (int32_t e = t0; e < s.m0; e += ts)
+                if (static_cast<const uint8_t *>(buf)[e] && v.e_o2c[e] >= 0) delete_edge(e);
+            flush(&sh->del, &rc->dp);
+            break;
+        case kSpBegin1:
+#pragma unroll 1
+            for (int32_t x = t0; x < s.n0; x += ts) s.v_cnt[x] = 0;
+            md_lists();
+            break;
+        case kSpContract1:
+            md_test(true, shard, nshards);
+            break;
+        case kSpExport1:
+#pragma unroll 1
+            for (int32_t x = t0; x < s.n0; x += ts)
+                static_cast<int32_t *>(buf)[x] = v.v_o2c[x] >= 0 ? s.v_cnt[x] : 0;
+            break;
+        case kSpImport1:
+#pragma unroll 1
+            for (int32_t x = t0; x < s.n0; x += ts) s.v_cnt[x] = static_cast<const int32_t *>(buf)[x];
+            break;
+        case kSpEnd1: {
+            md_decide();
+            flush(&sh->del2, &rc->md);
+            if (!team_sync(rc)) return;
+            const int32_t dp = sh->got.dp, md = sh->got.md;
+            if (!finish_round(dp, md)) return;
+            if (lead) store_progress(sh->g, s, ctr);
+            break;
+        }
+        default:
+            break;
+    }
+}
+
+// Team of CTAs per instance (team > 0, all CTAs resident: a cooperative
+// launch), or one CTA per instance taken from a queue (team = 0).
+template <int kThreads, int kMinBlocks>
+__global__ void __launch_bounds__(kThreads, kMinBlocks)
+    k_sparse_build(InstState *st, int count, int team, int32_t max_rounds, int32_t *queue,
+                   SpTotals *out) {
+    Shared *sh = shared();
+    if (team > 0) {
+        const int b = blockIdx.x / team;
+        if (b >= count) return;
+        start(st + b, blockIdx.x % team, team);
+        build_instance(max_rounds, out);
+        return;
+    }
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) sh->next = atomicAdd(queue, 1);
+        __syncthreads();
+        if (sh->next >= count) return;
+        start(st + sh->next, 0, 1);
+        build_instance(max_rounds, out);
+    }
+}
+
+template <int kThreads, int kMinBlocks>
+__global__ void __launch_bounds__(kThreads, kMinBlocks)
+    k_sparse_rounds(InstState *st, int count, int team, int32_t limit, BatchCounters *ctr,
+                    int32_t *queue, SpTimes *times) {
+    Shared *sh = shared();
+    if (team > 0) {
+        const int b = blockIdx.x / team;
+        if (b >= count) return;
+        start(st + b, blockIdx.x % team, team);
+        run_instance(limit, ctr, times);
+        return;
+    }
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) sh->next = atomicAdd(queue, 1);
+        __syncthreads();
+        if (sh->next >= count) return;
+        start(st + sh->next, 0, 1);
+        run_instance(limit, ctr, times);
+    }
+}
+
+__global__ void __launch_bounds__(kSpThreads, 1)
+    k_sparse_pass(InstState *st, int team, int op, int shard, int nshards, BatchCounters *ctr,
+                  void *buf) {
+    start(st, blockIdx.x, team);
+    run_pass(op, shard, nshards, ctr, buf);
+}
+
+}  // namespace
+
+// ------------------------------------------------------- host launchers --
+
+int sparse_team(int count, int64_t nnz, int64_t items, int sms) {
+    // one CTA of kSpThreads threads per SM at most; about one hyperedge or
+    // vertex, and a few incidences, per group of lanes
+    const int64_t want = std::max<int64_t>((nnz + kSpTeamNnz - 1) / kSpTeamNnz,
+                                           (items + kSpTeamItems - 1) / kSpTeamItems);
+    const int64_t cap = sms / std::max(count, 1);
+    if (count > 1 && cap < 2) return 0;  // a batch: one CTA each, from a queue
+    return (int)std::max<int64_t>(1, std::min(want, cap));
+}
+
+template <typename... A, typename... B>
+static cudaError_t launch_team(void (*k)(A...), int ctas, cudaStream_t s, B... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(kSpThreads);
+    cfg.dynamicSmemBytes = sizeof(Shared);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, A(args)...);
+}
+
+cudaError_t launch_sparse_build(InstState *st, int count, int team, int32_t max_rounds,
+                                int32_t *queue, SpTotals *out, int sms, cudaStream_t s) {
+    if (team > 0)
+        return launch_team(k_sparse_build<kSpThreads, 1>, count * team, s, st, count, team,
+                           max_rounds, queue, out);
+    k_sparse_build<kSpBatchThreads, kSpBatchBlocks>
+        <<<std::min(count, sms * kSpBatchBlocks), kSpBatchThreads, sizeof(Shared), s>>>(st, count, 0, max_rounds,
+                                                                           queue, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sparse_rounds(InstState *st, int count, int team, int32_t limit,
+                                 BatchCounters *ctr, int32_t *queue, SpTimes *times, int sms,
+                                 cudaStream_t s) {
+    if (team > 0)
+        return launch_team(k_sparse_rounds<kSpThreads, 1>, count * team, s, st, count, team, limit,
+                           ctr, queue, times);
+    k_sparse_rounds<kSpBatchThreads, kSpBatchBlocks>
+        <<<std::min(count, sms * kSpBatchBlocks), kSpBatchThreads, sizeof(Shared), s>>>(st, count, 0, limit, ctr,
+                                                                           queue, times);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sparse_pass(InstState *st, int team, int op, int shard, int nshards,
+                               BatchCounters *ctr, void *buf, cudaStream_t s) {
+    return launch_team(k_sparse_pass, team, s, st, team, op, shard, nshards, ctr, buf);
+}
+
+}  // namespace mhs
