@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <vector>
 
 #include "mhs.h"
 
@@ -33,6 +34,31 @@ const char *tile_table_path();
 inline int32_t layout_code(int32_t layout) {
     return layout == MHS_LAYOUT_INPUT ? 0 : layout == MHS_LAYOUT_SORTED ? 1 : 2;
 }
+
+// Are the len >= 1 ids strictly ascending and within [0, n)?  Then they are
+// distinct.  (No early exit: the loop is short and vectorises.)
+inline bool ascending_row(const int32_t *ids, int64_t len, int32_t n) {
+    int32_t bad = (ids[0] < 0) | (ids[len - 1] >= n);
+    for (int64_t k = 1; k < len; ++k) bad |= ids[k - 1] >= ids[k];
+    return !bad;
+}
+
+// One request of a group that solve_sparse_group reduces together.
+struct GroupItem {
+    int32_t n, m;
+    int64_t k;                       // in: the budget; out: what rule FE left of it
+    const int32_t *ptr, *vtx, *dem;  // host CSR and demands, already checked
+    std::vector<int32_t> *vout, *eout, *dout, *forced;  // the result lists
+    int32_t rounds;
+    mhs_status status;               // of this request
+};
+// Reduces the group on the sparse path, all requests in the same launches, on
+// `stream` (synchronises it).  *again: the path does not pay for this group;
+// nothing has been written.  opt: contraction auto.
+mhs_status solve_sparse_group(const mhs_options &opt, cudaStream_t stream,
+                              std::vector<GroupItem> &group, bool *again);
+// Would MHS_CONTRACT_AUTO try the sparse path with these options?
+bool auto_takes_sparse(const mhs_options &opt);
 
 // Blocks of kPinnedBlock bytes of page-locked host memory from a
 // process-wide slab.  cudaMallocHost / cudaFreeHost cost tens of

@@ -365,12 +365,14 @@ mhs_status validate_host(int32_t n, int32_t m, const int64_t *eptr64, const int3
     if (n >= (1 << 24) || m >= (1 << 24))
         return bad(MHS_EINVAL, "%s: n and m must be < 2^24 (exact FP32 counts)", what);
     auto ptr = [&](int64_t i) -> int64_t { return eptr64 ? eptr64[i] : eptr32[i]; };
-    if ((size_t)n > mark.size()) mark.assign((size_t)n, -1);
     for (int32_t e = 0; e < m; ++e) {
         int64_t a = ptr(e), b = ptr(e + 1);
         if (b < a) return bad(MHS_EINVAL, "%s: edge_ptr decreases at hyperedge %d", what, e);
         if (b - a > (1ll << 24)) return bad(MHS_EINVAL, "%s: hyperedge %d too large", what, e);
         if (demand[e] < 1) return bad(MHS_EINVAL, "%s: demand of hyperedge %d is < 1", what, e);
+        // an ascending row within [0, n) needs no marks
+        if (a == b || ascending_row(evtx + a, b - a, n)) continue;
+        if ((size_t)n > mark.size()) mark.assign((size_t)n, -1);
         for (int64_t p = a; p < b; ++p) {
             int32_t v = evtx[p];
             if (v < 0 || v >= n)
@@ -1165,6 +1167,133 @@ mhs_status run_rounds(mhs_instance *h, int32_t limit, mhs_round_stats *stats) {
 }
 
 }  // namespace
+
+bool mhs::auto_takes_sparse(const mhs_options &opt) { return auto_sparse(&opt); }
+
+mhs_status mhs::solve_sparse_group(const mhs_options &opt, cudaStream_t stream,
+                                   std::vector<GroupItem> &group, bool *again) {
+    const int count = (int)group.size();
+    *again = false;
+    if (count == 0) return MHS_OK;
+    std::vector<int32_t> n(count), m(count);
+    std::vector<int64_t> nnz(count), k(count);
+    int64_t sum_n = 0, sum_m = 0, sum_z = 0;
+    for (int b = 0; b < count; ++b) {
+        const GroupItem &g = group[b];
+        n[b] = g.n;
+        m[b] = g.m;
+        nnz[b] = g.ptr[g.m];
+        k[b] = g.k;
+        sum_n += n[b];
+        sum_m += m[b];
+        sum_z += nnz[b];
+    }
+    if (!sparse_may_pay(count, n.data(), m.data(), nnz.data())) {
+        *again = true;
+        return MHS_OK;
+    }
+    std::vector<Layout> lay;
+    int64_t tmoff = 0;
+    mhs_instance *h = nullptr;
+    mhs_status st =
+        create(count, n.data(), m.data(), nnz.data(), k.data(), &opt, stream, &h, lay, tmoff, true);
+    if (st) return st;
+    // page-locked staging: the inputs, array by array as in the arena, then
+    // room for the masks
+    const int64_t sum_m1 = sum_m + count;
+    const int64_t in_bytes = 4 * (sum_m1 + sum_z + sum_m);
+    h->in_stage = static_cast<uint8_t *>(
+        pinned_take((size_t)std::max(in_bytes, sum_n + sum_m), &h->in_stage_cls));
+    uint8_t *masks = nullptr;  // device: alive masks of all vertices, then of all hyperedges
+    auto body = [&]() -> mhs_status {
+        if (!h->in_stage) return fail(MHS_ENOMEM, "pinned host allocation failed");
+        int32_t *s_ptr = reinterpret_cast<int32_t *>(h->in_stage);
+        int32_t *s_vtx = s_ptr + sum_m1, *s_f = s_vtx + sum_z;
+        for (int b = 0; b < count; ++b) {
+            const GroupItem &g = group[b];
+            std::memcpy(s_ptr, g.ptr, 4 * ((size_t)g.m + 1));
+            if (nnz[b] > 0) std::memcpy(s_vtx, g.vtx, 4 * (size_t)nnz[b]);
+            if (g.m > 0) std::memcpy(s_f, g.dem, 4 * (size_t)g.m);
+            s_ptr += g.m + 1;
+            s_vtx += nnz[b];
+            s_f += g.m;
+        }
+        const uint8_t *in = h->in_stage;
+        CUDA_TRY(cudaMemcpyAsync(h->arena + h->in_eptr, in, 4 * (size_t)sum_m1,
+                                 cudaMemcpyHostToDevice, h->stream));
+        if (sum_z > 0)
+            CUDA_TRY(cudaMemcpyAsync(h->arena + h->in_evtx, in + 4 * sum_m1, 4 * (size_t)sum_z,
+                                     cudaMemcpyHostToDevice, h->stream));
+        if (sum_m > 0)
+            CUDA_TRY(cudaMemcpyAsync(h->arena + h->in_f, in + 4 * (sum_m1 + sum_z),
+                                     4 * (size_t)sum_m, cudaMemcpyHostToDevice, h->stream));
+        CUDA_TRY(upload_states(h));
+        mhs_status st2 = finish_sparse(h, again);
+        if (st2 || *again) return st2;
+        st2 = run_sparse(h, 0, nullptr);
+        if (st2) return st2;
+        cudaMemPool_t pool;
+        CUDA_TRY(pool_for(h->device, &pool));
+        CUDA_TRY(cudaMallocFromPoolAsync(reinterpret_cast<void **>(&masks),
+                                         (size_t)std::max<int64_t>(sum_n + sum_m, 1), pool,
+                                         h->stream));
+        CUDA_TRY(launch_alive_masks_batch(h->dstate, count, masks, masks + sum_n, h->stream));
+        std::vector<InstState> states(count);
+        CUDA_TRY(cudaMemcpyAsync(states.data(), h->dstate, sizeof(InstState) * count,
+                                 cudaMemcpyDeviceToHost, h->stream));
+        if (sum_n + sum_m > 0)
+            CUDA_TRY(cudaMemcpyAsync(h->in_stage, masks, (size_t)(sum_n + sum_m),
+                                     cudaMemcpyDeviceToHost, h->stream));
+        std::vector<int32_t> f;
+        std::vector<uint8_t> taken;
+        if (opt.full_edges) {  // FE lowered demands and took vertices
+            f.resize(std::max<int64_t>(sum_m, 1));
+            taken.resize(std::max<int64_t>(sum_n, 1));
+            if (sum_m > 0)
+                CUDA_TRY(cudaMemcpyAsync(f.data(), h->arena + h->in_f, 4 * (size_t)sum_m,
+                                         cudaMemcpyDeviceToHost, h->stream));
+            int64_t at = 0;
+            for (int b = 0; b < count; at += n[b], ++b)
+                if (n[b] > 0)
+                    CUDA_TRY(cudaMemcpyAsync(taken.data() + at, h->hstate[b].forced, (size_t)n[b],
+                                             cudaMemcpyDeviceToHost, h->stream));
+        }
+        CUDA_TRY(cudaStreamSynchronize(h->stream));
+        const uint8_t *av = h->in_stage, *ae = av + sum_n;
+        const int32_t *fb = f.data();
+        const uint8_t *tk = taken.data();
+        for (int b = 0; b < count; ++b) {
+            GroupItem &g = group[b];
+            const InstState &s = states[b];
+            g.status = s.status ? MHS_EDEVICE : MHS_OK;
+            g.rounds = s.rounds;
+            g.k = s.k;
+            g.vout->reserve(s.n);
+            g.eout->reserve(s.m);
+            g.dout->reserve(s.m);
+            for (int32_t v = 0; v < g.n; ++v)
+                if (av[v]) g.vout->push_back(v);
+            for (int32_t e = 0; e < g.m; ++e)
+                if (ae[e]) {
+                    g.eout->push_back(e);
+                    g.dout->push_back(opt.full_edges ? fb[e] : g.dem[e]);
+                }
+            if (opt.full_edges) {
+                for (int32_t v = 0; v < g.n; ++v)
+                    if (tk[v]) g.forced->push_back(v);
+                fb += g.m;
+                tk += g.n;
+            }
+            av += g.n;
+            ae += g.m;
+        }
+        return MHS_OK;
+    };
+    st = body();
+    if (masks) cudaFreeAsync(masks, h->stream);
+    destroy(h);
+    return st;
+}
 
 extern "C" {
 

@@ -183,6 +183,7 @@ struct Lane {
 struct mhs_server {
     mhs_server_options opt{};
     int contraction = kFp8;
+    bool sparse = false;      // contraction auto: requests are tried on the sparse path first
     int device = 0, sms = 0;
     cudaMemPool_t pool = nullptr;
     int64_t small_items = 0;  // n + m at most for the small-request lane
@@ -196,6 +197,7 @@ struct mhs_server {
     mhs_status fatal = MHS_OK;
     int64_t in_use = 0, peak = 0;
     int64_t submitted = 0, admitted = 0, completed = 0;
+    int64_t group_rounds = 0;  // rounds of the groups solved on the sparse path
 };
 
 namespace {
@@ -298,6 +300,54 @@ mhs_status admit(Lane &Ln, int si, std::shared_ptr<Request> req) {
     std::lock_guard<std::mutex> lk(S->mu);
     ++Ln.active_count;
     return MHS_OK;
+}
+
+// Contraction auto: reduce the admitted requests together on the sparse path,
+// on the load stream and beside the lane's loop.  Returns the ones it does
+// not pay for, which take slots of the loop.  (The footprint reserved for a
+// request is that of the loop's dense form, which it may need.)
+std::vector<std::shared_ptr<Request>> solve_group(Lane &Ln,
+                                                  std::vector<std::shared_ptr<Request>> reqs) {
+    mhs_server *S = Ln.S;
+    mhs_options opt;
+    mhs_default_options(&opt);
+    opt.edge_rule = S->opt.edge_rule;
+    opt.full_edges = S->opt.full_edges;
+    std::vector<GroupItem> group;
+    for (auto &r : reqs)
+        group.push_back({r->n, r->m, r->k, r->ptr.data(), r->vtx.data(), r->dem.data(), &r->vout,
+                         &r->eout, &r->dout, &r->forced, 0, MHS_OK});
+    {
+        std::lock_guard<std::mutex> lk(S->mu);
+        Ln.active_count += (int32_t)reqs.size();
+    }
+    bool again = false;
+    const mhs_status st = solve_sparse_group(opt, Ln.load, group, &again);
+    const int64_t t = now_ns();
+    std::lock_guard<std::mutex> lk(S->mu);
+    Ln.active_count -= (int32_t)reqs.size();
+    if (again) return reqs;
+    int32_t rounds = 0;
+    for (size_t i = 0; i < reqs.size(); ++i) {
+        Request &r = *reqs[i];
+        if (r.done) continue;  // (failed by a shutdown)
+        r.status = st ? st : group[i].status;
+        r.rounds = group[i].rounds;
+        r.k = group[i].k;
+        rounds = std::max(rounds, r.rounds);
+        r.t_done = t;
+        r.done = true;
+        r.ptr.clear();
+        r.vtx.clear();
+        r.dem.clear();
+        ++S->completed;
+        S->in_use -= r.footprint;
+        Ln.tiles_in_use -= r.tiles;
+    }
+    S->group_rounds += rounds;
+    S->cv_done.notify_all();
+    for (auto &ln : S->lanes) ln.cv_work.notify_one();
+    return {};
 }
 
 // Fail every request that has not finished (device error or shutdown).
@@ -449,6 +499,12 @@ void worker_loop(Lane *L) {
             }
         }
         std::vector<int> loaded;
+        if (S->sparse && !to_admit.empty()) {
+            std::vector<std::shared_ptr<Request>> reqs;
+            for (auto &p : to_admit) reqs.push_back(p.second);
+            progress = true;
+            if (solve_group(Ln, std::move(reqs)).empty()) to_admit.clear();
+        }
         for (auto &p : to_admit) {
             mhs_status st = admit(Ln, p.first, p.second);
             if (st != MHS_OK) {
@@ -746,6 +802,13 @@ mhs_status mhs_server_create(const mhs_server_options *opt_in, void *cuda_stream
     auto *S = new mhs_server();
     S->opt = opt;
     S->contraction = opt.contraction == MHS_CONTRACT_POPCOUNT ? kPopcount : kFp8;
+    {
+        mhs_options o;
+        mhs_default_options(&o);
+        o.contraction = opt.contraction;
+        o.sparsity = opt.sparsity;
+        S->sparse = auto_takes_sparse(o);
+    }
     // < 0: one lane for every request; 0: default split
     S->small_items = opt.small_items < 0 ? INT64_MAX : (opt.small_items == 0 ? 8192 : opt.small_items);
     auto bail = [&](mhs_status st) {
@@ -789,12 +852,15 @@ mhs_status mhs_submit(mhs_server *S, int32_t n, int32_t m, const int32_t *edge_p
     const int32_t nnz = edge_ptr[m];
     if (nnz > 0 && !edge_vtx) return set_error(MHS_EINVAL, "edge_vtx is NULL");
     // structural checks on the host, before anything is queued
-    std::vector<int32_t> mark((size_t)n, -1);
+    std::vector<int32_t> mark;
     for (int32_t e = 0; e < m; ++e) {
         if (edge_ptr[e + 1] < edge_ptr[e])
             return set_error(MHS_EINVAL, "edge_ptr decreases at hyperedge %d", e);
         if (demand[e] < 1) return set_error(MHS_EINVAL, "demand of hyperedge %d is < 1", e);
-        for (int32_t p = edge_ptr[e]; p < edge_ptr[e + 1]; ++p) {
+        const int32_t a = edge_ptr[e], b = edge_ptr[e + 1];
+        if (a == b || ascending_row(edge_vtx + a, b - a, n)) continue;
+        if (mark.empty()) mark.assign((size_t)n, -1);
+        for (int32_t p = a; p < b; ++p) {
             const int32_t v = edge_vtx[p];
             if (v < 0 || v >= n)
                 return set_error(MHS_EINVAL, "hyperedge %d has vertex id %d outside [0,%d)", e, v, n);
@@ -915,6 +981,7 @@ mhs_status mhs_server_get_stats(mhs_server *S, mhs_server_stats *out) {
     out->submitted = S->submitted;
     out->admitted = S->admitted;
     out->completed = S->completed;
+    out->rounds = S->group_rounds;
     for (auto &ln : S->lanes)
         if (ln.hflags) out->rounds += reinterpret_cast<volatile ServerFlags *>(ln.hflags)->rounds;
     out->pending = (int32_t)(S->lanes[0].pending.size() + S->lanes[1].pending.size());
