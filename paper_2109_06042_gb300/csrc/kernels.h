@@ -127,8 +127,8 @@ struct SpTimes {
 // instance of a batch, from a queue.  nnz, items (n + m): of the largest one.
 int sparse_team(int count, int64_t nnz, int64_t items, int sms);
 // Structural checks (status bits), rows, vertex lists and the cost of every
-// instance.  The caller has zeroed every sp_ctl, sp_vrec, sp_vagg and stamp
-// array, *queue (used for team = 0) and *out.
+// instance.  The caller has zeroed every sp_ctl, sp_vrec, sp_vagg, sp_bound and
+// stamp array, *queue (used for team = 0) and *out.
 cudaError_t launch_sparse_build(InstState *st, int count, int team, int32_t max_rounds,
                                 int32_t *queue, SpTotals *out, int sms, cudaStream_t s);
 // At most `limit` rounds (0: to the fixpoint); adds to *ctr and *times

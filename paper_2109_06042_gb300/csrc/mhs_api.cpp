@@ -441,7 +441,7 @@ struct Layout {  // byte offsets inside the arena for one instance
     int64_t v_o2c, v_c2o, e_o2c, e_c2o, e_f, e_s, v_deg, v_maxf, v_cnt, e_del, v_del, forced;
     int64_t e_dirty_rb, v_dirty, v_dirty_rb, e_prev, e_rec, scan;
     int64_t A, At, Ab, Atb;
-    int64_t gone, row, pos, tmp, vedge, erec, vrec, vagg, vaux, estamp, vstamp, tstamp, task, heavy;
+    int64_t bound, gone, row, pos, tmp, vedge, erec, vrec, vagg, vaux, estamp, vstamp, tstamp, task, heavy;
     int64_t pairs, pair_tab;
     int32_t task_cap, pair_cap;
 };
@@ -637,6 +637,7 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
         lay[b].vrec = ar.take(16 * (int64_t)n[b]);
         lay[b].vagg = ar.take(16 * (int64_t)n[b]);
         lay[b].pair_tab = ar.take((int64_t)sizeof(SpPair) * pair_slots(m[b]));
+        lay[b].bound = ar.take(4 * (int64_t)n[b]);
         lay[b].gone = ar.take(4 * (((int64_t)m[b] + 31) / 32));
         lay[b].estamp = ar.take(4 * (int64_t)m[b]);
         lay[b].vstamp = ar.take(4 * (int64_t)n[b]);
@@ -721,6 +722,7 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
             s.sp_vrec = reinterpret_cast<int4 *>(base + L.vrec);
             s.sp_vagg = reinterpret_cast<SpAgg *>(base + L.vagg);
             s.sp_vaux = reinterpret_cast<int4 *>(base + L.vaux);
+            s.sp_bound = reinterpret_cast<int32_t *>(base + L.bound);
             s.sp_gone = reinterpret_cast<uint32_t *>(base + L.gone);
             s.sp_estamp = reinterpret_cast<int32_t *>(base + L.estamp);
             s.sp_vstamp = reinterpret_cast<int32_t *>(base + L.vstamp);

@@ -173,6 +173,7 @@ struct InstState {
     int4 *sp_erec;         // [m0] {signature (2 words), f or "gone", |e|}
     int4 *sp_vrec;         // [n0] {signature (2 words), degree, place of the list}
     SpAgg *sp_vagg;        // [n0]
+    int32_t *sp_bound;     // [n0] max of sp_vagg's m1 and the demand in s1
     int4 *sp_vaux;         // [n0] {smallest hyperedge, largest demand, its row's place and length}
     uint32_t *sp_gone;     // [m0 / 32] bit: the hyperedge is deleted
     int32_t *sp_estamp;    // [m0] round for which the hyperedge is a DP candidate
