@@ -42,8 +42,8 @@
  *  - Lowest-index tie-breaking makes results deterministic: ids are the
  *    input ids, and the result lists them in ascending order.
  *  - Counts are exact: incidences are 0/1 values in FP8 E4M3 (exact) with
- *    FP32 accumulation (exact below 2^24), or bit-packed with integer
- *    popcounts; n and m must be < 2^24.
+ *    FP32 accumulation (exact below 2^24), or bits on the integer units;
+ *    n and m must be < 2^24.
  *  - All device work of an instance runs on the stream given at load time
  *    (NULL: the library creates a non-blocking stream for the instance).
  */
@@ -75,7 +75,7 @@ typedef enum {
                                   others, and those whose tile shape or sparsity the options
                                   name, as MHS_CONTRACT_FP8 */
     MHS_CONTRACT_FP8 = 1,      /* tcgen05 tensor cores, E4M3 0/1, FP32 accumulate */
-    MHS_CONTRACT_POPCOUNT = 2  /* bit-packed AND + popcount on the integer units */
+    MHS_CONTRACT_POPCOUNT = 2  /* bit-packed, on the integer units */
 } mhs_contraction;
 
 /* Order of the rows (and K columns) of the dense operands.  Results never

@@ -1,14 +1,14 @@
-// kernels.cu -- encode, compaction, planning and the bit-packed popcount
-// contraction with the fused DP / MD epilogue.
+// kernels.cu -- encode, compaction, planning and the bit-packed DP / MD passes.
 //
 // Round structure (Algorithm 3, Section 4.1), all on the device:
 //   plan(phase 0) -> encode A -> contract(DP or SE) -> compact_edges
 //   plan(phase 1) -> clear A + encode A^T -> contract(MD) -> clear A^T -> compact_vertices
 //   [rule FE at a fixpoint, fe.cu]
-// The contraction of either kind (this file: popcount; contract_tc.cu:
-// tcgen05 FP8) computes the pair counts of Eq. (1) / Eq. (2) tile by tile
-// and never writes them out: the epilogue turns each count into the
-// deletion flags of Algorithm 1 or the dominator counts of Algorithm 2.
+// (bit-packed: both operands are set before DP and cleared after MD.)  The
+// contraction (contract_tc.cu: tcgen05 FP8) computes the pair counts of Eq. (1)
+// / Eq. (2) tile by tile, the bit-packed passes (this file) 32 pairs to a
+// word; neither writes them out: they turn them into the deletion flags of
+// Algorithm 1 or the dominator counts of Algorithm 2.
 #include <algorithm>
 
 #include <cuda_runtime.h>
@@ -335,7 +335,7 @@ __global__ void k_layout_commit(InstState *st, int count) {
         s.e_c2o[s.e_o2c[e]] = (int32_t)e;
 }
 
-// Hyperedge rows of round 1, by position.
+// Hyperedge rows of round 1, by position; bit-packed operands: no degrees yet.
 __global__ void k_edge_rows(InstState *st, int count) {
     const int b = blockIdx.y;
     if (b >= count) return;
@@ -347,12 +347,16 @@ __global__ void k_edge_rows(InstState *st, int count) {
         s.e_s[r] = -1;  // never tested: every hyperedge is a DP candidate
         s.e_del[r] = 0;
     }
+    if (s.Ab)
+        for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < s.n0;
+             r += (int64_t)gridDim.x * blockDim.x)
+            s.v_deg[r] = 0;
 }
 
 // ------------------------------------------------------------- planning --
 
 // phase 0: rows = current hyperedges (DP); phase 1: rows = current vertices (MD).
-// tc: 0 popcount tiles, 1 tcgen05 tiles (128 x plan->tile_n).
+// tc: 0 units of the bit-packed passes, 1 tcgen05 tiles (128 x plan->tile_n).
 __global__ void k_plan(InstState *st, Plan *plan, int phase, int tc, BatchCounters *ctr) {
     __shared__ int32_t sh[33];
     __shared__ int64_t sh64[33];
@@ -392,7 +396,7 @@ __global__ void k_plan(InstState *st, Plan *plan, int phase, int tc, BatchCounte
                 const bool none = phase == 0 ? skip : skip && s.skip_a;
                 rows = !tc ? s.m : none ? 0 : (s.m + 31) & ~31;
                 const int32_t R = phase == 0 ? s.m : s.n;
-                tiles = tc ? tc_tiles(R, plan->tile_n) : pop_tiles(R);
+                tiles = tc ? tc_tiles(R, plan->tile_n) : pop_units(phase, R);
                 act_any = 1;
             }
         }
@@ -426,123 +430,76 @@ __global__ void k_plan(InstState *st, Plan *plan, int phase, int tc, BatchCounte
 
 // --------------------------------------------------------------- encode --
 
-// Bit-packed operands (popcount path).  One hyperedge row per lane, a warp
-// walking the original vertex lists of its 32 hyperedges together.  Phase 0
-// (rows = current hyperedges) sets A[e'][v'] (K = current vertices) and
-// counts |e| (= I^E_ii).  Phase 1 walks the rows the DP pass saw (e_prev):
-// its set pass clears their entries of A (the DP pass's clear, fused in since
-// it walks the same incidences), marks the vertices of the hyperedges DP
-// deleted as MD candidates, and for the kept ones sets At[v'][e''] (rows =
-// current vertices, K = the hyperedges' positions after DP) and counts deg(v)
-// (= I^V_jj) and the maximum demand; its clear pass clears At after the MD
-// contraction.  So the operands are all-zero between rounds, and A^T between
-// phases.  A set counts only incidences that were not already set, so a
-// repeated id inside one hyperedge counts once.
+// Bit-packed operands (popcount path), from the original vertex lists.  Phase
+// 0 (rows = current hyperedges) sets A[e'][v'] (K = current vertices) and
+// At[v'][e'] (K = current hyperedges) and counts |e| (= I^E_ii) and deg(v).
+// Phase 1 walks the rows the DP pass saw (e_prev), at their positions of
+// then: its set pass takes the hyperedges that DP deleted out of At and
+// deg(v) (= I^V_jj) and marks their vertices as MD candidates, and collects
+// the maximum demand over the kept ones; its clear pass clears both after the
+// MD pass, so the operands are all-zero between rounds.  Only incidences whose
+// bit changed are counted, so a repeated id inside one hyperedge counts once.
 template <int kPhase, bool kSet>
 __global__ void __launch_bounds__(256) k_scatter(InstState *st, const Plan *plan) {
-    // Each warp takes 32 consecutive rows and walks the incidences of all of
-    // them together, 32 at a time, so a hyperedge of 64 vertices does not
-    // hold its warp 64 dependent atomics long.
-    __shared__ int32_t wfresh[8][32];  // fresh incidences per row of each warp
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    // Eight lanes per row: what bounds this is the chain of a row's dependent
+    // loads and atomics, not their number (a row per lane, walked by the warp
+    // together, left 250 warps for 8,000 rows of 9: 25 us instead of 12).
+    constexpr int kLanes = 8;
+    const int lane = threadIdx.x & 31, sub = lane % kLanes;
     const int32_t total = plan->total_rows;
-    const int32_t nw = gridDim.x * (blockDim.x >> 5);
-    for (int32_t g0 = (blockIdx.x * (blockDim.x >> 5) + wib) * 32; g0 < total; g0 += nw * 32) {
-        const int32_t g = g0 + lane;
-        int b = 0;
-        int32_t ce = 0, e = 0, p0 = 0, len = 0;
-        bool mark = false;
-        int32_t cnew = 0;  // phase 1: the row's position after DP, -1 if DP deleted it
+    const int32_t step = gridDim.x * (blockDim.x / kLanes);
+    for (int32_t g0 = (int32_t)((blockIdx.x * blockDim.x + threadIdx.x - lane) / kLanes); g0 < total;
+         g0 += step) {
+        const int32_t g = g0 + lane / kLanes;
+        int32_t fresh = 0, ce = 0, e = 0;  // incidences that changed a bit
+        InstState *sp = nullptr;
         if (g < total) {
-            b = find_owner(plan->row_off, plan->count, g);
-            const InstState &s = st[b];
+            const int b = find_owner(plan->row_off, plan->count, g);
+            sp = st + b;
+            InstState &s = *sp;
             ce = g - plan->row_off[b];
             e = kPhase == 0 ? s.e_c2o[ce] : s.e_prev[ce];
-            if (kPhase == 1) cnew = s.e_o2c[e];
-            p0 = s.eptr[e];
-            len = s.eptr[e + 1] - p0;
-            // phase 1 set: a hyperedge the DP pass deleted makes its
-            // vertices MD candidates of this round
-            mark = kPhase == 1 && kSet && s.v_dirty && cnew < 0;
-            // phase 1 clear: A^T holds only the rows DP kept
-            if (kPhase == 1 && !kSet && cnew < 0) len = 0;
-        }
-        int32_t incl = len;  // inclusive prefix of the row lengths over the warp
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        const int32_t start = incl - len;
-        const int32_t tot = __shfl_sync(0xffffffffu, incl, 31);
-        if (kSet && kPhase == 0) wfresh[wib][lane] = 0;
-        __syncwarp();
-        for (int32_t f0 = 0; f0 < tot; f0 += 32) {
-            const int32_t f = f0 + lane;
-            // owner row: the last lane whose run starts at or before f
-            int r = 0;
-#pragma unroll
-            for (int step = 16; step > 0; step >>= 1) {
-                const int c = r + step;
-                const int32_t sc = __shfl_sync(0xffffffffu, start, c & 31);
-                if (c < 32 && sc <= f) r = c;
-            }
-            const int rb = __shfl_sync(0xffffffffu, b, r);
-            const int32_t rce = __shfl_sync(0xffffffffu, ce, r);
-            const int32_t rnew = __shfl_sync(0xffffffffu, cnew, r);
-            const int32_t re = __shfl_sync(0xffffffffu, e, r);
-            const int32_t rp = __shfl_sync(0xffffffffu, p0, r) + f - __shfl_sync(0xffffffffu, start, r);
-            const bool rmark = __shfl_sync(0xffffffffu, mark, r);
-            if (f >= tot) continue;
-            InstState &s = st[rb];
-            const int32_t cv = s.v_o2c[s.evtx[rp]];
-            if (cv < 0) continue;
-            if (rmark && cv < s.n) {
-                s.v_dirty[cv] = 1;
-                s.v_dirty_rb[cv >> 7] = 1;
-            }
-            if (kPhase == 1 && kSet) {  // the DP pass's clear of A, fused in
-                s.Ab[(int64_t)rce * s.Ab_pitch + (cv >> 5)] = 0;
-                if (rnew < 0) continue;  // deleted by DP: nothing in A^T
-            }
-            const int32_t R = kPhase == 0 ? s.m : s.n;
-            const int32_t K = kPhase == 0 ? s.n : s.m_dp;
-            const int32_t rr = kPhase == 0 ? rce : cv;
-            const int32_t cc = kPhase == 0 ? cv : rnew;
-            if (rr >= R || cc >= K) { atomicOr(&s.status, kErrCapacity); continue; }
-            bool fresh = false;
-            uint32_t *row = (kPhase == 0 ? s.Ab : s.Atb) +
-                            (int64_t)rr * (kPhase == 0 ? s.Ab_pitch : s.Atb_pitch);
-            if (kSet) {
-                const uint32_t bit = 1u << (cc & 31);
-                fresh = (atomicOr(&row[cc >> 5], bit) & bit) == 0;
-            } else {
-                row[cc >> 5] = 0;  // every set bit of this word is cleared by some thread
-            }
-            if (kSet && fresh) {
-                if (kPhase == 0) {
-                    atomicAdd(&wfresh[wib][r], 1);
+            const bool gone = kPhase == 1 && s.e_o2c[e] < 0;  // DP deleted it
+            const int32_t end = s.eptr[e + 1];
+            const int32_t f = kPhase == 1 && kSet ? s.f[e] : 0;
+            for (int32_t p = s.eptr[e] + sub; p < end; p += kLanes) {
+                const int32_t cv = s.v_o2c[s.evtx[p]];
+                if (cv < 0) continue;
+                if (ce >= s.m || cv >= s.n) { atomicOr(&s.status, kErrCapacity); continue; }
+                uint32_t *a = &s.Ab[(int64_t)ce * s.Ab_pitch + (cv >> 5)];
+                uint32_t *at = &s.Atb[(int64_t)cv * s.Atb_pitch + (ce >> 5)];
+                const uint32_t a_bit = 1u << (cv & 31), at_bit = 1u << (ce & 31);
+                if (!kSet) {  // every set bit of these words is cleared by some thread
+                    *a = 0;
+                    *at = 0;
+                } else if (kPhase == 0) {
+                    if ((atomicOr(a, a_bit) & a_bit) == 0) {
+                        atomicOr(at, at_bit);
+                        atomicAdd(&s.v_deg[cv], 1);
+                        ++fresh;
+                    }
+                } else if (gone) {
+                    if (s.v_dirty) {
+                        s.v_dirty[cv] = 1;
+                        s.v_dirty_rb[cv >> 7] = 1;
+                    }
+                    if (atomicAnd(at, ~at_bit) & at_bit) atomicSub(&s.v_deg[cv], 1);
                 } else {
-                    atomicAdd(&s.v_deg[cv], 1);
-                    atomicMax(&s.v_maxf[cv], s.f[re]);
+                    atomicMax(&s.v_maxf[cv], f);
                 }
             }
         }
         if (kSet && kPhase == 0) {
             __syncwarp();
-            if (g < total) {
-                InstState &s = st[b];
-                const int32_t fresh_cnt = wfresh[wib][lane];
+#pragma unroll
+            for (int o = kLanes / 2; o > 0; o >>= 1) fresh += __shfl_xor_sync(0xffffffffu, fresh, o);
+            if (sp && sub == 0) {
+                InstState &s = *sp;
                 // a hyperedge whose size changed since the previous DP pass (or
                 // never tested) makes its row block a DP candidate
-                if (s.e_dirty_rb && s.e_s[ce] != fresh_cnt) s.e_dirty_rb[ce >> 7] = 1;
-                s.e_s[ce] = fresh_cnt;  // one lane owns the row
-                if (s.e_rec) {  // the tcgen05 epilogue stages this one record per row
-                    const int32_t fe = s.e_f[ce];
-                    s.e_rec[ce] = make_int4(fe, s.edge_rule ? fresh_cnt : fe - fresh_cnt, e, 0);
-                }
+                if (s.e_dirty_rb && s.e_s[ce] != fresh) s.e_dirty_rb[ce >> 7] = 1;
+                s.e_s[ce] = fresh;
             }
-            __syncwarp();  // wfresh is reused by the next group of rows
         }
     }
 }
@@ -1034,7 +991,7 @@ __global__ void k_compact_edges(InstState *st, int count) {
     const int32_t nv = s.n;
     zero_occupancy(s, 1, nv, first, stride);
     for (int32_t r = first; r < nv; r += stride) {
-        s.v_deg[r] = 0;
+        if (!s.Ab) s.v_deg[r] = 0;  // (bit-packed: counted before the DP pass)
         s.v_maxf[r] = 0;
         s.v_cnt[r] = 0;
         s.v_del[r] = 0;
@@ -1139,6 +1096,8 @@ __global__ void k_compact_vertices(InstState *st, int count, BatchCounters *ctr,
                 for (int32_t r = first; r < nv; r += stride) s.v_dirty[r] = 0;
                 for (int32_t w = first; w < (nv + 127) / 128; w += stride) s.v_dirty_rb[w] = 0;
             }
+            if (s.Ab)
+                for (int32_t r = first; r < nv; r += stride) s.v_deg[r] = 0;
             for (int32_t r = first; r < m_dp; r += stride) {
                 s.e_f[r] = s.f[s.e_c2o[r]];
                 s.e_del[r] = 0;
@@ -1163,139 +1122,320 @@ __global__ void k_compact_vertices(InstState *st, int count, BatchCounters *ctr,
     }
 }
 
-// ------------------------------------------------ popcount contraction --
+// ---------------------------------------------------- bit-packed passes --
+//
+// Both passes take the rows' intersections from bitmaps of the OTHER side,
+// 32 pairs per instruction, instead of counting each pair's bits:
+//  * DP, superseder e_i: for every v in e_i the bitmap of v's hyperedges says
+//    which e_j do not miss it, so a few bitwise operations per word keep, for
+//    32 columns j at once, whether more than t vertices of e_i are missed
+//    (t = 0..3; demands above 4 count the misses in bit planes).
+//  * MD, candidate v_j: the vertices in all of its hyperedges are the AND of
+//    those hyperedges' bitmaps.
+// A warp stops as soon as no column of its block is left, after some three
+// vertices of a hyperedge or two hyperedges of a vertex.  Bounded by the
+// latency of chains of three loads (a row's bitmap, its members' bitmaps, what
+// is known of the pairs found); the AND + POPC of all pairs, 64 x 64 to a
+// tile, was bounded by POPC (16 a clock and SM).  On one GB300, uniform 4,000 x
+// 8,000, |e| 2..16: both passes of two rounds 53 us, load to result 317 us,
+// 1,704 with the tiles; power law 20,000 x 40,000: the rounds 2.5 ms, 138 with
+// the tiles; 2,000 x 3,000, |e| 200..400, demands up to 200: 0.98 ms, 1.93 with
+// the tiles.
 
-// Map a tile index of the upper triangle of an nt x nt tile grid (ti <= tj,
-// row-major) to (ti, tj).
-__device__ __forceinline__ void tri_tile(int64_t t, int32_t nt, int32_t *ti, int32_t *tj) {
-    // off(i) = i*nt - i*(i-1)/2 ; find the largest i with off(i) <= t
-    double a = 2.0 * nt + 1.0;
-    double disc = a * a - 8.0 * (double)t;
-    int32_t i = (int32_t)((a - sqrt(disc > 0 ? disc : 0)) * 0.5);
-    if (i < 0) i = 0;
-    if (i > nt - 1) i = nt - 1;
-    auto off = [nt](int64_t x) { return x * nt - x * (x - 1) / 2; };
-    while (i > 0 && off(i) > t) --i;
-    while (i + 1 < nt && off(i + 1) <= t) ++i;
-    *ti = i;
-    *tj = i + (int32_t)(t - off(i));
+constexpr int kPopWarps = 8;
+// Blocks per SM.  (4 for DP spill 64 bytes a thread; 3 take 524 us instead of
+// 447 for the DP passes of uniform 16,000 x 32,000.)
+constexpr int kPopDpBlocks = 4, kPopMdBlocks = 4;
+constexpr int kPopIds = 512;    // members of a row gathered at a time
+constexpr int kPopT = 4;        // demands up to this: misses counted in unary
+constexpr int kPopPlanes = 24;  // above: in binary (sizes are < 2^24)
+
+// Members of a row of W words, from word *k0 on, into ids: as many as fit.
+// The whole warp.
+__device__ __forceinline__ int32_t pop_ids(const uint32_t *row, int32_t W, int32_t *k0,
+                                           int32_t *ids, int lane) {
+    int32_t n = 0;
+    __syncwarp();  // ids is free
+    while (*k0 < W) {
+        const int32_t k = *k0 + 4 * lane;  // (the pitch is a multiple of 4 words, zero behind W)
+        uint4 x = make_uint4(0, 0, 0, 0);
+        if (k < W) x = *reinterpret_cast<const uint4 *>(row + k);
+        int32_t c = __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
+        int32_t step = 128;
+        if (n + __reduce_add_sync(0xffffffffu, c) > kPopIds) {
+            if (n > 0) break;
+            step = kPopIds / 32;  // a dense row: what always fits
+            if (4 * lane >= step) {
+                x = make_uint4(0, 0, 0, 0);
+                c = 0;
+            }
+        }
+        int32_t inc = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        int32_t at = n + inc - c;
+        n += __shfl_sync(0xffffffffu, inc, 31);
+        const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            for (uint32_t b = w[u]; b; b &= b - 1) ids[at++] = (k + u) * 32 + __ffs(b) - 1;
+        *k0 += step;
+    }
+    __syncwarp();
+    return n;
 }
 
-constexpr int kPopKW = 32;  // K words staged per step
+// Four words of a lane.
+struct Quad {
+    uint32_t w[4];
+    __device__ __forceinline__ bool any() const { return (w[0] | w[1] | w[2] | w[3]) != 0; }
+};
+__device__ __forceinline__ Quad quad_fill(uint32_t x) { return {{x, x, x, x}}; }
+__device__ __forceinline__ Quad quad_load(const uint32_t *p) {
+    const uint4 x = *reinterpret_cast<const uint4 *>(p);
+    return {{x.x, x.y, x.z, x.w}};
+}
+// Bits of rows < R other than `self`, from row r0 on.
+__device__ __forceinline__ Quad quad_rows(int32_t r0, int32_t R, int32_t self) {
+    Quad q;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int32_t left = R - (r0 + 32 * u), at = self - (r0 + 32 * u);
+        q.w[u] = left >= 32 ? ~0u : left > 0 ? (1u << left) - 1u : 0u;
+        if (at >= 0 && at < 32) q.w[u] &= ~(1u << at);
+    }
+    return q;
+}
 
-// phase 0: DP on Ab (rows = hyperedges); phase 1: MD on Atb (rows = vertices).
-// With nshards > 1 only the tiles whose rows lie in a 128-row block b with
-// b % nshards == shard are contracted (one share of a sharded pass).
-__global__ void __launch_bounds__(256) k_pop_contract(InstState *st, const Plan *plan, int phase,
-                                                      int shard, int nshards) {
-    __shared__ uint32_t As[kPopTile][kPopKW + 1];
-    __shared__ uint32_t Bs[kPopTile][kPopKW + 1];
-    __shared__ int32_t rcnt[kPopTile], ccnt[kPopTile];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+struct PopRow {  // a superseder
+    int32_t i, f, size, id;
+};
+
+// e_j goes unless the two are equal and e_j's index is the lower one.
+__device__ __forceinline__ void pop_delete(const InstState &s, const PopRow &r, int32_t j,
+                                           bool missed, int32_t fj) {
+    if (missed || fj != r.f || s.e_s[j] != r.size || r.id < s.e_c2o[j]) s.e_del[j] = 1;
+}
+
+// Demands above kPopT: the misses of 32 columns a lane, in binary, seven
+// vertices to an addition (four full adders, then one ripple), until every
+// column has missed too many (looked at after every 28 vertices).
+__device__ __noinline__ void pop_dp_planes(const InstState &s, PopRow r, int32_t jb, int32_t *ids,
+                                           int lane) {
+    const int32_t W = (s.n + 31) / 32, K = (s.m + 31) / 32;
+    const int np = max(3, 32 - __clz(r.size));
+    const int32_t t = s.edge_rule ? 0 : min(r.f - 1, r.size);
+    for (int32_t k0 = jb * 128; k0 < min(K, jb * 128 + 128); k0 += 32) {
+        const int32_t k = k0 + lane, left = s.m - k * 32;
+        uint32_t may = left >= 32 ? ~0u : left > 0 ? (1u << left) - 1u : 0u;
+        if (r.i >> 5 == k) may &= ~(1u << (r.i & 31));
+        uint32_t cnt[kPopPlanes];
+#pragma unroll
+        for (int p = 0; p < kPopPlanes; ++p) cnt[p] = 0;
+        auto at_most_t = [&] {
+            uint32_t less = 0, same = ~0u;  // misses below, equal to t
+#pragma unroll
+            for (int p = kPopPlanes - 1; p >= 0; --p) {
+                if (p >= np) continue;
+                if (t >> p & 1) {
+                    less |= same & ~cnt[p];
+                    same &= cnt[p];
+                } else {
+                    same &= ~cnt[p];
+                }
+            }
+            return less | same;
+        };
+        bool any = true;
+        for (int32_t at = 0, group = 0; at < W && any;) {
+            const int32_t n = pop_ids(s.Ab + (int64_t)r.i * s.Ab_pitch, W, &at, ids, lane);
+#pragma unroll 1
+            for (int32_t q = 0; q < n && any; q += 7, ++group) {
+                uint32_t x[7];
+#pragma unroll
+                for (int u = 0; u < 7; ++u)
+                    x[u] = q + u < n && k < K ? ~s.Atb[(int64_t)ids[q + u] * s.Atb_pitch + k] : 0;
+                auto add = [](uint32_t a, uint32_t b, uint32_t c, uint32_t *carry) {
+                    *carry = (a & b) | (c & (a | b));
+                    return a ^ b ^ c;
+                };
+                uint32_t c0, c1, c2, four, two, carry;
+                const uint32_t s0 = add(x[0], x[1], x[2], &c0), s1 = add(x[3], x[4], x[5], &c1);
+                const uint32_t one = add(s0, s1, x[6], &c2);
+                two = add(c0, c1, c2, &four);
+                cnt[0] = add(cnt[0], one, 0, &carry);
+                cnt[1] = add(cnt[1], two, carry, &carry);
+                cnt[2] = add(cnt[2], four, carry, &carry);
+#pragma unroll
+                for (int p = 3; p < kPopPlanes; ++p)
+                    if (p < np) cnt[p] = add(cnt[p], 0, carry, &carry);
+                if ((group & 3) == 3) {
+                    may &= at_most_t();
+                    any = __any_sync(0xffffffffu, may != 0);
+                }
+            }
+        }
+        may &= at_most_t();
+        for (; may; may &= may - 1) {
+            const int b = __ffs(may) - 1;
+            const int32_t j = k * 32 + b, fj = s.e_f[j];
+            int32_t miss = 0;
+#pragma unroll
+            for (int p = 0; p < kPopPlanes; ++p) miss |= (int32_t)(cnt[p] >> b & 1u) << p;
+            if (fj <= r.f - miss) pop_delete(s, r, j, miss > 0, fj);
+        }
+    }
+}
+
+// Algorithm 1, D_ij = [f_i - |e_i \ e_j| >= f_j]; delete j iff D_ij and (not
+// D_ji or i < j), i < j comparing input indices (D_ij and D_ji: equal sets
+// and demands).  Rule SE instead: D_ij = [e_i within e_j and f_i >= f_j].
+// A block takes kPopDpRows superseders against 4,096 columns.  Incremental
+// rounds: only row blocks with a hyperedge that lost a vertex.  With
+// nshards > 1 only rows of 128-row blocks b with b % nshards == shard.
+__global__ void __launch_bounds__(32 * kPopWarps, kPopDpBlocks)
+    k_pop_dp(InstState *st, const Plan *plan, int shard, int nshards) {
+    __shared__ int32_t ids_all[kPopWarps][kPopIds];
+    __shared__ __align__(16) uint32_t fle[kPopT][128];  // [d - 1]: columns of demand <= d
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int32_t *ids = ids_all[warp];
     const int64_t total = plan->total_tiles;
-    for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
-        const int b = find_owner(plan->tile_off, plan->count, t);
+    for (int64_t unit = blockIdx.x; unit < total; unit += gridDim.x) {
+        const int b = find_owner(plan->tile_off, plan->count, unit);
+        const InstState &s = st[b];
+        const int32_t m = s.m, blocks = (m + 4095) / 4096;
+        const int64_t local = unit - plan->tile_off[b];
+        const int32_t i0 = (int32_t)(local / blocks) * kPopDpRows, jb = (int32_t)(local % blocks);
+        if (nshards > 1 && (i0 / kTcM) % nshards != shard) continue;
+        if (s.e_dirty_rb && !s.e_dirty_rb[i0 >> 7]) continue;
+        __syncthreads();  // fle is free
+#pragma unroll 4
+        for (int w = warp; w < 128; w += kPopWarps) {
+            const int32_t j = jb * 4096 + 32 * w + lane;
+            const int32_t f = j < m ? s.e_f[j] : 0x7fffffff;
+#pragma unroll
+            for (int d = 0; d < kPopT; ++d) {
+                const uint32_t bits = __ballot_sync(0xffffffffu, f <= d + 1);
+                if (lane == d) fle[d][w] = bits;
+            }
+        }
+        __syncthreads();
+        const int32_t W = (s.n + 31) / 32, K = (m + 31) / 32, k = jb * 128 + 4 * lane;
+        const uint32_t *const col = s.Atb + k;  // this lane's words of a vertex's bitmap
+        bool large = false;  // the warp has a demand above kPopT
+        for (int32_t i = i0 + warp; i < min(i0 + kPopDpRows, m); i += kPopWarps) {
+            const PopRow r = {i, s.e_f[i], s.e_s[i], s.e_c2o[i]};
+            if (r.f > kPopT) {
+                large = true;
+                continue;
+            }
+            const int t = s.edge_rule ? 0 : r.f - 1;
+            const Quad valid = quad_rows(k * 32, m, i);
+            Quad miss[kPopT], left = valid;  // [t]: columns that miss more than t; at most t
+#pragma unroll
+            for (int d = 0; d < kPopT; ++d) miss[d] = quad_fill(0);
+            bool any = true;
+            for (int32_t at = 0; at < W && any;) {
+                const int32_t n = pop_ids(s.Ab + (int64_t)i * s.Ab_pitch, W, &at, ids, lane);
+                for (int32_t q = 0; q < n && any; q += 4) {
+                    Quad x[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        x[u] = quad_fill(~0u);
+                        if (q + u < n && k < K)
+                            x[u] = quad_load(col + (int64_t)ids[q + u] * s.Atb_pitch);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+#pragma unroll
+                            for (int d = kPopT - 1; d > 0; --d)
+                                miss[d].w[c] |= miss[d - 1].w[c] & ~x[u].w[c];
+                            miss[0].w[c] |= ~x[u].w[c];
+                        }
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        left.w[c] = valid.w[c] & ~(t == 0   ? miss[0].w[c]
+                                                   : t == 1 ? miss[1].w[c]
+                                                   : t == 2 ? miss[2].w[c]
+                                                            : miss[3].w[c]);
+                    any = __any_sync(0xffffffffu, left.any());
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                if (!left.w[c]) continue;
+                uint32_t go = 0;
+#pragma unroll
+                for (int d = 0; d < kPopT; ++d)
+                    if (d <= t && r.f - d >= 1) go |= ~miss[d].w[c] & fle[r.f - d - 1][4 * lane + c];
+                for (go &= valid.w[c]; go; go &= go - 1) {
+                    const int bit = __ffs(go) - 1;
+                    const int32_t j = (k + c) * 32 + bit;
+                    const bool missed = miss[0].w[c] >> bit & 1u;
+                    pop_delete(s, r, j, missed, missed ? 0 : s.e_f[j]);
+                }
+            }
+        }
+        if (!large) continue;
+        for (int32_t i = i0 + warp; i < min(i0 + kPopDpRows, m); i += kPopWarps)
+            if (s.e_f[i] > kPopT) pop_dp_planes(s, {i, s.e_f[i], s.e_s[i], s.e_c2o[i]}, jb, ids, lane);
+    }
+}
+
+// Algorithm 2, D_ij = [x = d_j and (x != d_i or i < j)], i < j comparing
+// input indices: C_j counts the other vertices of all of v_j's hyperedges,
+// without those of equal incidence and a higher index.  A warp per vertex;
+// incremental rounds: only vertices that lost a hyperedge.  (A vertex of no
+// hyperedge goes whatever its count.)  Shares as in k_pop_dp.
+__global__ void __launch_bounds__(32 * kPopWarps, kPopMdBlocks)
+    k_pop_md(InstState *st, const Plan *plan, int shard, int nshards) {
+    __shared__ int32_t ids_all[kPopWarps][kPopIds];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int32_t *ids = ids_all[warp];
+    const int64_t total = plan->total_tiles;
+    for (int64_t unit = blockIdx.x; unit < total; unit += gridDim.x) {
+        const int b = find_owner(plan->tile_off, plan->count, unit);
         InstState &s = st[b];
-        const int64_t local = t - plan->tile_off[b];
-        const int32_t R = phase == 0 ? s.m : s.n;
-        const int32_t W = phase == 0 ? (s.n + 31) / 32 : (s.m_dp + 31) / 32;
-        const uint32_t *X = phase == 0 ? s.Ab : s.Atb;
-        const int64_t pitch = phase == 0 ? s.Ab_pitch : s.Atb_pitch;
-        const int32_t nt = (R + kPopTile - 1) / kPopTile;
-        int32_t ti, tj;
-        tri_tile(local, nt, &ti, &tj);
-        const int32_t i0 = ti * kPopTile, j0 = tj * kPopTile;
-        if (nshards > 1 && (i0 / kTcM) % nshards != shard) continue;  // another share's tile
-        {  // incremental rounds: only tiles that hold a candidate row or column
-            const uint8_t *drb = phase == 0 ? s.e_dirty_rb : s.v_dirty_rb;
-            if (drb && !(phase == 1 && s.md_full) && !drb[i0 >> 7] && !drb[j0 >> 7]) continue;
-        }
-        int32_t acc[4][4];
+        const int32_t n = s.n;
+        const int32_t j0 = (int32_t)(unit - plan->tile_off[b]) * kPopMdRows;
+        if (nshards > 1 && (j0 / kTcM) % nshards != shard) continue;
+        const int32_t W = (s.m + 31) / 32, K = (n + 31) / 32;
+        for (int32_t j = j0 + warp; j < min(j0 + kPopMdRows, n); j += kPopWarps) {
+            if (s.v_dirty && !s.md_full && !s.v_dirty[j]) continue;
+            const int32_t dj = s.v_deg[j], oj = s.v_c2o[j];
+            if (dj == 0) continue;
+            int32_t count = 0;
+            for (int32_t k0 = 0; k0 < K; k0 += 128) {
+                const int32_t k = k0 + 4 * lane;
+                Quad in = quad_rows(k * 32, n, j);
+                bool any = true;
+                for (int32_t at = 0; at < W && any;) {
+                    const int32_t cnt = pop_ids(s.Atb + (int64_t)j * s.Atb_pitch, W, &at, ids, lane);
+                    for (int32_t q = 0; q < cnt && any; q += 4) {
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+                        for (int u = 0; u < 4; ++u) {
+                            if (q + u >= cnt || k >= K) continue;
+                            const Quad x = quad_load(s.Ab + (int64_t)ids[q + u] * s.Ab_pitch + k);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[a][c] = 0;
-        for (int32_t k0 = 0; k0 < W; k0 += kPopKW) {
-            for (int idx = threadIdx.x; idx < kPopTile * kPopKW; idx += blockDim.x) {
-                int row = idx / kPopKW, w = idx % kPopKW;
-                int32_t kw = k0 + w;
-                uint32_t va = 0, vb = 0;
-                if (kw < W) {
-                    if (i0 + row < R) va = X[(int64_t)(i0 + row) * pitch + kw];
-                    if (j0 + row < R) vb = X[(int64_t)(j0 + row) * pitch + kw];
+                            for (int c = 0; c < 4; ++c) in.w[c] &= x.w[c];
+                        }
+                        any = __any_sync(0xffffffffu, in.any());
+                    }
                 }
-                As[row][w] = va;
-                Bs[row][w] = vb;
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    for (uint32_t x = in.w[c]; x; x &= x - 1) {
+                        const int32_t i = (k + c) * 32 + __ffs(x) - 1;
+                        count += s.v_deg[i] != dj || s.v_c2o[i] < oj;
+                    }
             }
-            __syncthreads();
-#pragma unroll 8
-            for (int w = 0; w < kPopKW; ++w) {
-                uint32_t av[4], bv[4];
-#pragma unroll
-                for (int a = 0; a < 4; ++a) av[a] = As[ty + 16 * a][w];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) bv[c] = Bs[tx + 16 * c][w];
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[a][c] += __popc(av[a] & bv[c]);
-            }
-            __syncthreads();
-        }
-        // ---- fused epilogue: pairs i < j < R ----
-        if (phase == 0) {
-            // Algorithm 1: D_ij = [f_i - (s_i - x) >= f_j]; delete j iff
-            // D_ij and (not D_ji or i < j), i < j comparing input indices.
-            // Rule SE instead: D_ij = [x = s_i and f_i >= f_j] (e_i within e_j).
-            const bool se = s.edge_rule != 0;
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                const int32_t i = i0 + ty + 16 * a;
-                if (i >= R) continue;
-                const int32_t fi = s.e_f[i], si = s.e_s[i], oi = s.e_c2o[i];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const int32_t j = j0 + tx + 16 * c;
-                    if (j <= i || j >= R) continue;
-                    const int32_t x = acc[a][c];
-                    const int32_t fj = s.e_f[j], sj = s.e_s[j];
-                    const bool dij = se ? (x == si && fi >= fj) : fi - (si - x) >= fj;
-                    const bool dji = se ? (x == sj && fj >= fi) : fj - (sj - x) >= fi;
-                    const bool i_first = oi < s.e_c2o[j];  // tie-break by input index
-                    if (dij && (!dji || i_first)) s.e_del[j] = 1;   // same-value stores
-                    if (dji && (!dij || !i_first)) s.e_del[i] = 1;
-                }
-            }
-        } else {
-            // Algorithm 2: D_ij = [x = d_j and (x != d_i or i < j)], i < j
-            // comparing input indices.
-            if (threadIdx.x < kPopTile) { rcnt[threadIdx.x] = 0; ccnt[threadIdx.x] = 0; }
-            __syncthreads();
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                const int32_t i = i0 + ty + 16 * a;
-                if (i >= R) continue;
-                const int32_t di = s.v_deg[i], oi = s.v_c2o[i];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const int32_t j = j0 + tx + 16 * c;
-                    if (j <= i || j >= R) continue;
-                    const int32_t x = acc[a][c];
-                    const int32_t dj = s.v_deg[j];
-                    const bool i_first = oi < s.v_c2o[j];  // tie-break by input index
-                    if (x == dj && (x != di || i_first)) atomicAdd(&ccnt[tx + 16 * c], 1);
-                    if (x == di && (x != dj || !i_first)) atomicAdd(&rcnt[ty + 16 * a], 1);
-                }
-            }
-            __syncthreads();
-            if (threadIdx.x < kPopTile) {
-                int32_t v = ccnt[threadIdx.x];
-                if (v) atomicAdd(&s.v_cnt[j0 + threadIdx.x], v);
-            } else if (threadIdx.x < 2 * kPopTile) {
-                int32_t v = rcnt[threadIdx.x - kPopTile];
-                if (v) atomicAdd(&s.v_cnt[i0 + threadIdx.x - kPopTile], v);
-            }
-            __syncthreads();
+            count = __reduce_add_sync(0xffffffffu, count);
+            if (lane == 0) s.v_cnt[j] = count;
         }
     }
 }
@@ -1527,6 +1667,13 @@ static void launch_scatter(InstState *st, const Plan *plan, bool set, bool dense
     else k_scatter<kPhase, false><<<grid, 256, 0, s>>>(st, plan);
 }
 
+static void launch_pop(InstState *st, const Plan *plan, int phase, int shard, int nshards,
+                       int sms, cudaStream_t s) {
+    const int threads = 32 * kPopWarps;
+    if (phase == 0) k_pop_dp<<<grid_for(sms, kPopDpBlocks), threads, 0, s>>>(st, plan, shard, nshards);
+    else k_pop_md<<<grid_for(sms, kPopMdBlocks), threads, 0, s>>>(st, plan, shard, nshards);
+}
+
 cudaError_t launch_phase_prologue(InstState *st, Plan *plan, BatchCounters *ctr, int phase,
                                   int contraction, int sms, cudaStream_t s) {
     const bool tc = contraction == kFp8;
@@ -1549,7 +1696,7 @@ cudaError_t launch_phase_contract(InstState *st, Plan *plan, BatchCounters *ctr,
         if (e != cudaSuccess) return e;
         return launch_tc_contract(st, plan, ctr, phase, sms, tile_n, kerr, s);
     }
-    k_pop_contract<<<grid_for(sms, 6), 256, 0, s>>>(st, plan, phase, shard, nshards);
+    launch_pop(st, plan, phase, shard, nshards, sms, s);
     return cudaGetLastError();
 }
 
@@ -1625,7 +1772,7 @@ cudaError_t launch_round_phase(InstState *st, Plan *plan, BatchCounters *ctr, in
         cudaError_t e = launch_tc_contract(st, plan, ctr, phase, sms, tile_n, kerr, s);
         if (e != cudaSuccess) return e;
     } else {
-        k_pop_contract<<<grid_for(sms, 6), 256, 0, s>>>(st, plan, phase, 0, 1);
+        launch_pop(st, plan, phase, 0, 1, sms, s);
     }
     if (ev_contract_end) record(ev_contract_end);
     return launch_phase_epilogue(st, plan, ctr, count, phase, contraction, sms, s, done_list,

@@ -21,7 +21,8 @@
 namespace mhs {
 
 // Tile shapes.
-constexpr int kPopTile = 64;     // popcount contraction: 64 x 64 pair tiles
+constexpr int kPopDpRows = 16;   // bit-packed passes: rows of a block, x 4,096 columns (DP)
+constexpr int kPopMdRows = 8;    // (MD: x all columns)
 constexpr int kTcM = 128;        // tcgen05 contraction: 128 rows (i) x 128 or 256 columns (j)
 constexpr int kTcNDefault = 256; // per tile; the wider tile unless chosen otherwise
 constexpr int kTcK = 128;        // K bytes per pipeline stage (FP8)
@@ -215,10 +216,10 @@ struct Plan {
     int32_t two_queues;       // 0: every tile in the front queue (one queue)
 };
 
-// Number of pair tiles of an R x R upper triangle.
-__host__ __device__ inline int64_t pop_tiles(int32_t R) {
-    int64_t t = (R + kPopTile - 1) / kPopTile;
-    return R > 1 ? t * (t + 1) / 2 : 0;
+// Blocks of the bit-packed pass over R rows (phase 0: DP; 1: MD).
+__host__ __device__ inline int64_t pop_units(int phase, int32_t R) {
+    if (phase) return (R + kPopMdRows - 1) / kPopMdRows;
+    return (int64_t)((R + kPopDpRows - 1) / kPopDpRows) * ((R + 4095) / 4096);
 }
 
 // Packed tile-list entries.
