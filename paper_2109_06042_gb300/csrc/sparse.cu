@@ -48,7 +48,7 @@
 // more than kHeavyDeg hyperedges are handled by whole CTAs.
 // Measured on one GB300, the rounds alone (load, kernelization and result
 // through the C ABI beside the FP8 contraction's):
-//   power law 20,000 x 40,000: 280 us (474 / 1,690)
+//   power law 20,000 x 40,000: 223 us (407 / 1,690)
 //   interval 50,000 x 100,000: 358 us (628 / 11,357)
 //   uniform 16,000 x 32,000, |e| 2..16: 68 us (197 / 6,145)
 #include <algorithm>
@@ -73,8 +73,19 @@ constexpr int kG = 8;                  // lanes per hyperedge / vertex
 constexpr int kU = 2;
 constexpr int kTaskU = 4;
 constexpr int kRowU = 2;
-constexpr int kHeavyList = 192;        // longer lists are walked by whole warps (see kHeavyKey)
-constexpr int kTaskLen = 1024;         // entries per such task
+// Longer lists become tasks of whole warps, in parts: eight lanes take 0.6 us
+// per 16 entries, up to four lists in turn.  At 192 and parts of 1,024, the
+// walk of a round with 880 tasks took 32 us, the tasks 18 (power law; 24 and
+// below gain nothing).  Where lists are that long on average, tasks only cost
+// their barrier (|e| 64 over 2,000 x 4,000: DP 179 us, 200 with tasks from 96
+// entries on), so a list also has to be twice as long as the mean, or 4 times
+// kHeavyList (Shared::heavy_list).
+constexpr int kHeavyList = 48;
+constexpr int kTaskLen = 256;
+// The same for a vertex's bounds, whose entries are read four in flight, like
+// the members of a deleted hyperedge (rule SE: tasks of 72 us in a second
+// round with 1,024 entries, one at a time; 20 now).
+constexpr int kBoundList = 32, kBoundLen = 128;
 constexpr int kHeavyDeg = 256;         // vertices of a higher degree: whole CTAs
 constexpr int32_t kNoTask = -1, kBoundTask = -2;  // Task.x: unused; a vertex's bounds
 constexpr int32_t kGone = 0x7fffffff;  // demand of a deleted hyperedge: no test passes it
@@ -174,6 +185,7 @@ struct Shared {
     int32_t full;         // every hyperedge and vertex is a candidate
     int32_t ok;           // the last barrier
     int32_t local;        // there is room for degrees (build of a batch)
+    int32_t heavy_list;   // longer lists are walked as tasks
     SpRound got;          // counters read right after it
     Progress g;           // the instance's rounds, as every CTA of the team knows them
     int32_t del, del2;    // deletions of this phase
@@ -451,7 +463,9 @@ __device__ __noinline__ void delete_edge(int32_t x) {
     if (sh->full) return;  // every vertex is a candidate
     const int32_t len = v.erec[x].w;
     const uint32_t *row = v.row + v.eptr[x];
-#pragma unroll 1
+    // (a store waits for its own load, a serial chain of L2 latencies, unless
+    // several are in flight)
+#pragma unroll 4
     for (int32_t k = 0; k < len; ++k) v.vstamp[key_id(row[k])] = epoch;
 }
 
@@ -475,12 +489,13 @@ __device__ __forceinline__ int4 load_agg(const SpAgg *p) {
 // Reserve tasks for the list of vertex x, in the lanes with want set (the
 // whole warp, one atomic); false if there is no room (the caller walks the
 // list itself).
-__device__ __noinline__ bool push_tasks(bool want, int32_t i, int32_t x, int32_t p, int32_t deg) {
+__device__ __noinline__ bool push_tasks(bool want, int32_t i, int32_t x, int32_t p, int32_t deg,
+                                        int32_t part) {
     if (!__any_sync(0xffffffffu, want)) return false;
     Shared *sh = shared();
     const int lane = threadIdx.x & 31;
     const int32_t cap = sh->task_cap;
-    const int32_t parts = want ? (deg + kTaskLen - 1) / kTaskLen : 0;
+    const int32_t parts = want ? (deg + part - 1) / part : 0;
     int32_t inc = parts;
 #pragma unroll 1
     for (int o = 1; o < 32; o <<= 1) {
@@ -505,11 +520,19 @@ __device__ __noinline__ void bound_list(int32_t x, int32_t k0, int32_t k1, int32
     const int4 a = load_agg(v.agg + x);
     const u64 *list = v.vedge + v.vrec[x].w;
 #pragma unroll 1
-    for (int32_t k = k0; k < k1; k += step) {
-        const int32_t j = entry_id(list[k]);
-        if (nshards > 1 && (j >> 7) % nshards != shard) continue;
-        const int4 r = v.erec[j];
-        if (r.z != kGone && agg_hit(a, j, r.z, r.w)) delete_edge(j);
+    for (int32_t k = k0; k < k1; k += kTaskU * step) {
+        int32_t j[kTaskU];
+        int4 r[kTaskU];
+#pragma unroll
+        for (int u = 0; u < kTaskU; ++u) {
+            j[u] = k + u * step < k1 ? entry_id(list[k + u * step]) : -1;
+            if (nshards > 1 && j[u] >= 0 && (j[u] >> 7) % nshards != shard) j[u] = -1;
+        }
+#pragma unroll
+        for (int u = 0; u < kTaskU; ++u) r[u] = j[u] >= 0 ? v.erec[j[u]] : make_int4(0, 0, kGone, 0);
+#pragma unroll
+        for (int u = 0; u < kTaskU; ++u)
+            if (r[u].z != kGone && agg_hit(a, j[u], r[u].z, r[u].w)) delete_edge(j[u]);
     }
 }
 
@@ -591,7 +614,7 @@ __device__ __noinline__ void dp_bounds_touched(int shard, int nshards) {
         c, c.sh->n0, [&](int32_t x) { return tstamp[x] == c.epoch && v_o2c[x] >= 0; },
         [&](int32_t x) {
             const int32_t deg = x >= 0 ? vrec[x].z : 0;
-            bool later = push_tasks(deg > kHeavyList && c.sub == 0, kBoundTask, x, 0, deg);
+            bool later = push_tasks(deg > kBoundList && c.sub == 0, kBoundTask, x, 0, deg, kBoundLen);
             later = __shfl_sync(0xffffffffu, later, c.lead);
             if (x >= 0 && !later) bound_list(x, c.sub, deg, kG, shard, nshards);
             __syncwarp();
@@ -791,6 +814,7 @@ __device__ __noinline__ void dp_walk(int shard, int nshards) {
     const int4 *const erec = v.erec, *const vrec = v.vrec;
     const uint32_t *const rows = v.row, *const gone = v.gone;
     const u64 *const vedge = v.vedge;
+    const int32_t heavy_list = c.sh->heavy_list;
     Pairs pairs(c, 0);
     for_flagged(
         c, c.sh->m0,
@@ -822,7 +846,7 @@ __device__ __noinline__ void dp_walk(int shard, int nshards) {
                 }
                 const int4 vr = x >= 0 ? vrec[x] : make_int4(0, 0, 0, 0);
                 int32_t deg = vr.z;
-                if (push_tasks(deg > kHeavyList, i, x, p, deg)) deg = 0;
+                if (push_tasks(deg > heavy_list, i, x, p, deg, kTaskLen)) deg = 0;
                 const int32_t lists = min(npmax - p0, kG);
 #pragma unroll 1
                 for (int q = 0; q < lists; ++q) {
@@ -867,7 +891,8 @@ __device__ __noinline__ void dp_tasks(int shard, int nshards) {
         if (tk.x == kNoTask) continue;
         const int4 vr = v.vrec[tk.y];
         const int4 r = tk.x >= 0 ? v.erec[tk.x] : make_int4(0, 0, 0, 0);
-        const int32_t k0 = tk.w * kTaskLen, k1 = min(k0 + kTaskLen, vr.z);
+        const int32_t part = tk.x == kBoundTask ? kBoundLen : kTaskLen;
+        const int32_t k0 = tk.w * part, k1 = min(k0 + part, vr.z);
         if (tk.x == kBoundTask) {
             bound_list(tk.y, k0 + c.lane, k1, 32, shard, nshards);
             __syncwarp();
@@ -1480,6 +1505,7 @@ __device__ __noinline__ void start(InstState *s, int rank, int size, bool local 
         sh->rule = s->edge_rule;
         sh->rank = rank;
         sh->local = local;
+        sh->heavy_list = max(kHeavyList, min(2 * (int32_t)(s->nnz0 / max(s->n0, 1)), 4 * kHeavyList));
         sh->size = size;
         sh->epoch = 1;
         sh->par = 0;

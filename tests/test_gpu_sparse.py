@@ -184,6 +184,22 @@ def test_batch_around_the_limit_of_shared_degrees(mhs, n):
             _same(h.result(b), refs[b % 3], f"{n}: {b}")
 
 
+@pytest.mark.parametrize("rule", ["dp", "se"])
+@pytest.mark.parametrize("deg", [31, 33, 47, 48, 49, 128, 129, 191, 193, 256, 257])
+def test_lists_around_the_lengths_of_tasks(mhs, deg, rule):
+    """Lists of `deg` hyperedges, alone among short ones and as the mean
+    length; several rounds, with hyperedges of one vertex (bounds)."""
+    rng = np.random.Generator(np.random.PCG64(deg))
+    hubs = 6
+    edges = [sorted({h, hubs + int(x), hubs + int(y)}) for h in range(hubs)
+             for x, y in rng.integers(0, 90, (deg, 2))]
+    edges += [[hubs + i] for i in range(0, 90, 7)]
+    dense = [np.sort(rng.choice(40, 8, replace=False)).tolist() for _ in range(deg * 5)]
+    for n, e in ((hubs + 90, edges), (40, dense)):
+        inst = I.from_edges(n, e, rng.integers(1, 4, len(e)), k=3)
+        _same(mhs.kernelize(inst, rule=rule), O.reduce_variant(inst, rule, False))
+
+
 def test_dense_hypergraphs_are_contracted(mhs):
     """Long lists throughout: the load leaves this path, with the same result."""
     rng = np.random.Generator(np.random.PCG64(3))
