@@ -375,7 +375,8 @@ mhs_status mhs_last_timing(const mhs_instance *inst, float *ms4);
  * must stay valid until the call returns.  Outputs: alive_v (uint8[n]) and
  * alive_e (uint8[m]) DEVICE buffers receive 1 for surviving vertices /
  * hyperedges (input ids); *rounds_out (host, may be NULL) the round count.
- * Same rules and result as mhs_kernelize (bit-packed popcount contraction).
+ * Same rules and result as mhs_kernelize (candidate lists, or the
+ * bit-packed passes where those would walk too much).
  * Every array must be device (or managed) memory of the current device; any
  * other pointer gives MHS_EINVAL before a kernel runs.  A malformed instance
  * (bad edge_ptr, vertex id out of range) gives MHS_EINVAL; a kernel error

@@ -446,17 +446,6 @@ struct Layout {  // byte offsets inside the arena for one instance
     int32_t task_cap, pair_cap;
 };
 
-// Vertices of more than 256 hyperedges (sparse.cu's limit for a group of lanes).
-inline int64_t heavy_cap(int64_t nnz) { return nnz / 257 + 1; }
-
-// Slots of the pair table: a power of two, about one per 4 hyperedges (power
-// law 20,000 x 40,000: 2,020 pairs).
-inline int64_t pair_slots(int64_t m) {
-    int64_t s = 16;
-    while (s < m / 4 && s < (1 << 20)) s <<= 1;
-    return s;
-}
-
 // Can MHS_CONTRACT_AUTO take the sparse path?  Options that name the operands
 // of the contraction ask for the contraction.
 bool auto_sparse(const mhs_options *opt) {
@@ -572,7 +561,7 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
             L.task = ar.take(16 * (int64_t)L.task_cap);
             L.pair_cap = (int32_t)std::min<int64_t>(count == 1 ? 65536 + 64 * m0 : 256 + 2 * m0, 1 << 22);
             L.pairs = ar.take(8 * (int64_t)L.pair_cap);
-            L.heavy = ar.take(4 * heavy_cap(z));
+            L.heavy = ar.take(4 * sp_heavy_cap(z));
             continue;
         }
         L.v_c2o = ar.take(4 * n0);
@@ -636,7 +625,7 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
     for (int b = 0; b < count && sparse; ++b) {  // what starts at zero, with the words above
         lay[b].vrec = ar.take(16 * (int64_t)n[b]);
         lay[b].vagg = ar.take(16 * (int64_t)n[b]);
-        lay[b].pair_tab = ar.take((int64_t)sizeof(SpPair) * pair_slots(m[b]));
+        lay[b].pair_tab = ar.take((int64_t)sizeof(SpPair) * sp_pair_slots(m[b]));
         lay[b].bound = ar.take(4 * (int64_t)n[b]);
         lay[b].gone = ar.take(4 * (((int64_t)m[b] + 31) / 32));
         lay[b].estamp = ar.take(4 * (int64_t)m[b]);
@@ -730,7 +719,7 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
             s.sp_task = reinterpret_cast<int4 *>(base + L.task);
             s.sp_task_cap = L.task_cap;
             s.sp_pair_tab = reinterpret_cast<SpPair *>(base + L.pair_tab);
-            s.sp_pair_mask = (uint32_t)pair_slots(s.m0) - 1;
+            s.sp_pair_mask = (uint32_t)sp_pair_slots(s.m0) - 1;
             s.sp_pairs = reinterpret_cast<int2 *>(base + L.pairs);
             s.sp_pair_cap = L.pair_cap;
             s.sp_heavy = reinterpret_cast<int32_t *>(base + L.heavy);

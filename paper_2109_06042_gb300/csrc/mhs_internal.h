@@ -57,6 +57,17 @@ struct alignas(32) SpPair {
     int32_t m2;                 // largest f_i - |e_i| + 2 over its hyperedges of |e_i| >= 3
     int32_t pad[3];
 };
+// Vertices of more than 256 hyperedges (sparse.cu's limit for a group of lanes).
+inline int64_t sp_heavy_cap(int64_t nnz) { return nnz / 257 + 1; }
+
+// Slots of the pair table: a power of two, about one per 4 hyperedges (power
+// law 20,000 x 40,000: 2,020 pairs).
+inline int64_t sp_pair_slots(int64_t m) {
+    int64_t s = 16;
+    while (s < m / 4 && s < (1 << 20)) s <<= 1;
+    return s;
+}
+
 // Counters of one round; rounds alternate between two.
 struct SpRound {
     int32_t dp, md;             // deletions

@@ -12,8 +12,9 @@
 // The array is kScratchBytes (6 MiB) and every GPU that loads this library
 // holds it until the process exits.  It fits instances with n <= 4096,
 // m <= 4096 and at most 65,536 incidences; larger ones are rejected with
-// MHS_EINVAL.  It uses the bit-packed popcount contraction and the same
-// encode / compaction kernels as the main path.
+// MHS_EINVAL.  It takes the candidate lists (sparse.cu: one launch to load, one
+// for all rounds), or, where their first round would walk too much, the
+// bit-packed passes with the encode / compaction kernels of the main path.
 //
 // All calls share the one array and it keeps the last call's contents, so
 // everything that must start from zero is cleared by each call.  Calls whose
@@ -51,6 +52,27 @@ static __device__ __align__(256) uint8_t kScratch[kScratchBytes];
 
 inline int64_t up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 inline int64_t words(int64_t K) { return up(((K + 31) / 32) > 0 ? (K + 31) / 32 : 1, 4); }
+
+// The candidate lists are taken for rows of this mean length at most, and while
+// their first round visits no more list entries than this.  Measured, a call
+// by lists / by bits alone (us); bits after a build that did not pay: + 50.
+//   n 1,000, m 2,000, |e| 2..16:       cost 55 K     96 / 254
+//   n 256, m 4,096, |e| 14..16:        cost 1.8 M   131 / 180
+//   n 32, m 4,096, |e| 14..16:         cost 15 M    322 / 292
+//   n 8, m 4,096, |e| 1..8:            cost 20 M    102 / 381
+//   n 16, m 4,096, |e| 8..16:          cost 25 M   1293 / 370
+//   n 1,000, m 300, |e| 150..200:      mean 175     184 / 201
+//   n 2,000, m 200, |e| 300..320:      mean 310     289 / 237
+constexpr unsigned long long kNoAllocCost = 20000000;
+constexpr int64_t kNoAllocMeanSize = 200;
+
+// What the candidate lists' two launches start with at zero.
+struct Words {
+    SpTotals totals;
+    SpTimes times;
+    BatchCounters ctr;
+    int32_t queue;
+};
 
 struct Take {
     int64_t bytes = 0;
@@ -120,22 +142,37 @@ extern "C" mhs_status mhs_kernelize_noalloc(int32_t n, int32_t m, const int32_t 
     // layout inside the scratch (same roles as the main path's arena)
     Take take;
     const int64_t o_state = take(sizeof(InstState));
-    const int64_t o_plan = take(sizeof(Plan));
-    const int64_t o_rowoff = take(2 * sizeof(int32_t));
-    const int64_t o_tileoff = take(2 * sizeof(int64_t));
-    const int64_t o_ctr = take(sizeof(BatchCounters));
-    const int64_t o_kerr = take(sizeof(int32_t));
-    const int64_t o_vo2c = take(4 * (int64_t)n), o_vc2o = take(4 * (int64_t)n);
-    const int64_t o_eo2c = take(4 * (int64_t)m), o_ec2o = take(4 * (int64_t)m);
-    const int64_t o_eprev = take(4 * (int64_t)m);
-    const int64_t o_ef = take(4 * (int64_t)m), o_es = take(4 * (int64_t)m);
-    const int64_t o_vdeg = take(4 * ((int64_t)n + 1)), o_vmaxf = take(4 * (int64_t)n);
+    const int64_t o_vo2c = take(4 * (int64_t)n), o_eo2c = take(4 * (int64_t)m);
     const int64_t o_vcnt = take(4 * ((int64_t)n + 1));
-    const int64_t o_edel = take(m), o_vdel = take(n);
+    // the two forms of the rest lie over one another
+    Take bits = take;
+    const int64_t o_plan = bits(sizeof(Plan));
+    const int64_t o_rowoff = bits(2 * sizeof(int32_t));
+    const int64_t o_tileoff = bits(2 * sizeof(int64_t));
+    const int64_t o_ctr = bits(sizeof(BatchCounters));
+    const int64_t o_kerr = bits(sizeof(int32_t));
+    const int64_t o_vc2o = bits(4 * (int64_t)n), o_ec2o = bits(4 * (int64_t)m);
+    const int64_t o_eprev = bits(4 * (int64_t)m);
+    const int64_t o_ef = bits(4 * (int64_t)m), o_es = bits(4 * (int64_t)m);
+    const int64_t o_vdeg = bits(4 * ((int64_t)n + 1)), o_vmaxf = bits(4 * (int64_t)n);
+    const int64_t o_edel = bits(m), o_vdel = bits(n);
     const int64_t arows = up(m > 0 ? m : 1, kRowAlign), atrows = up(n > 0 ? n : 1, kRowAlign);
-    const int64_t o_ab = take(arows * words(n) * 4);
-    const int64_t o_atb = take(atrows * words(m) * 4);
-    if (take.bytes > (int64_t)kScratchBytes)
+    const int64_t o_ab = bits(arows * words(n) * 4);
+    const int64_t o_atb = bits(atrows * words(m) * 4);
+    const int64_t o_row = take(4 * (int64_t)nnz), o_pos = take(4 * (int64_t)nnz);
+    const int64_t o_tmp = take(4 * (int64_t)nnz), o_vedge = take(8 * (int64_t)nnz);
+    const int64_t o_erec = take(16 * (int64_t)m), o_vaux = take(16 * (int64_t)n);
+    const int64_t o_heavy = take(4 * sp_heavy_cap(nnz));
+    const int32_t task_cap = 8192, pair_cap = 131072;
+    const int64_t o_task = take(16 * (int64_t)task_cap), o_pairs = take(8 * (int64_t)pair_cap);
+    const int64_t o_words = take(sizeof(Words));  // from here on zero at the start
+    const int64_t o_ctl = take(sizeof(SpCtl)), o_vrec = take(16 * (int64_t)n);
+    const int64_t o_vagg = take(16 * (int64_t)n);
+    const int64_t slots = sp_pair_slots(m), o_tab = take((int64_t)sizeof(SpPair) * slots);
+    const int64_t o_bound = take(4 * (int64_t)n), o_gone = take(4 * (((int64_t)m + 31) / 32));
+    const int64_t o_estamp = take(4 * (int64_t)m);
+    const int64_t o_vstamp = take(4 * (int64_t)n), o_tstamp = take(4 * (int64_t)n);
+    if (take.bytes > (int64_t)kScratchBytes || bits.bytes > (int64_t)kScratchBytes)
         return err(err_buf, err_cap, MHS_EINVAL, "instance does not fit the static scratch");
 
     InstState st;
@@ -165,6 +202,28 @@ extern "C" mhs_status mhs_kernelize_noalloc(int32_t n, int32_t m, const int32_t 
     st.A_rows = (int32_t)arows;
     st.At_rows = (int32_t)atrows;
 
+    st.sp_row = reinterpret_cast<uint32_t *>(base + o_row);
+    st.sp_pos = reinterpret_cast<int32_t *>(base + o_pos);
+    st.sp_tmp = reinterpret_cast<uint32_t *>(base + o_tmp);
+    st.sp_vedge = reinterpret_cast<unsigned long long *>(base + o_vedge);
+    st.sp_erec = reinterpret_cast<int4 *>(base + o_erec);
+    st.sp_vrec = reinterpret_cast<int4 *>(base + o_vrec);
+    st.sp_vagg = reinterpret_cast<SpAgg *>(base + o_vagg);
+    st.sp_vaux = reinterpret_cast<int4 *>(base + o_vaux);
+    st.sp_bound = reinterpret_cast<int32_t *>(base + o_bound);
+    st.sp_gone = reinterpret_cast<uint32_t *>(base + o_gone);
+    st.sp_estamp = reinterpret_cast<int32_t *>(base + o_estamp);
+    st.sp_vstamp = reinterpret_cast<int32_t *>(base + o_vstamp);
+    st.sp_tstamp = reinterpret_cast<int32_t *>(base + o_tstamp);
+    st.sp_task = reinterpret_cast<int4 *>(base + o_task);
+    st.sp_task_cap = task_cap;
+    st.sp_pair_tab = reinterpret_cast<SpPair *>(base + o_tab);
+    st.sp_pair_mask = (uint32_t)slots - 1;
+    st.sp_pairs = reinterpret_cast<int2 *>(base + o_pairs);
+    st.sp_pair_cap = pair_cap;
+    st.sp_heavy = reinterpret_cast<int32_t *>(base + o_heavy);
+    st.sp_ctl = reinterpret_cast<SpCtl *>(base + o_ctl);
+
     Plan pl;
     std::memset(&pl, 0, sizeof(pl));
     pl.count = 1;
@@ -177,24 +236,56 @@ extern "C" mhs_status mhs_kernelize_noalloc(int32_t n, int32_t m, const int32_t 
     int32_t *dkerr = reinterpret_cast<int32_t *>(base + o_kerr);
 
     // pageable sources: each copy returns once the source has been staged
+    Words *dw = reinterpret_cast<Words *>(base + o_words);
+    const int team = sparse_team(1, nnz, (int64_t)n + m, sms);
     cudaError_t e = cudaMemcpyAsync(dst, &st, sizeof(st), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dplan, &pl, sizeof(pl), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dkerr, 0, sizeof(int32_t), s);
-    if (e == cudaSuccess) e = launch_validate(dst, 1, s);
-    int32_t status = 0;
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&status, &dst->status, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+    BatchCounters ctr;
+    std::memset(&ctr, 0, sizeof(ctr));
+    bool lists = nnz <= kNoAllocMeanSize * m;
+    SpTotals found = {};
+    if (lists) {
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync(base + o_words, 0, (size_t)(take.bytes - o_words), s);
+        if (e == cudaSuccess)
+            e = launch_sparse_build(dst, 1, team, 0, &dw->queue, &dw->totals, sms, s);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(&found, &dw->totals, sizeof(found), cudaMemcpyDeviceToHost, s);
+    } else {
+        if (e == cudaSuccess) e = launch_validate(dst, 1, s);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(&found.status, &dst->status, sizeof(int32_t),
+                                cudaMemcpyDeviceToHost, s);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return err(err_buf, err_cap, MHS_ECUDA, cudaGetErrorString(e));
-    if (status) return err(err_buf, err_cap, MHS_EINVAL, "malformed instance (bad edge_ptr or vertex id)");
+    if (found.status & (kErrTimeout | kErrCapacity))
+        return err(err_buf, err_cap, MHS_EDEVICE, "kernel reported an error status");
+    if (found.status)
+        return err(err_buf, err_cap, MHS_EINVAL, "malformed instance (bad edge_ptr or vertex id)");
+    if (lists && found.cost <= kNoAllocCost) {
+        e = launch_sparse_rounds(dst, 1, team, 0, &dw->ctr, &dw->queue, &dw->times, sms, s);
+        if (e == cudaSuccess && (n > 0 || m > 0))
+            e = launch_alive_masks(dst, n > 0 ? alive_v : nullptr, m > 0 ? alive_e : nullptr, s);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(&ctr, &dw->ctr, sizeof(ctr), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return err(err_buf, err_cap, MHS_ECUDA, cudaGetErrorString(e));
+        if (ctr.status_any || ctr.active)
+            return err(err_buf, err_cap, MHS_EDEVICE, "kernel reported an error status");
+        if (rounds_out) *rounds_out = ctr.max_rounds_seen;
+        return MHS_OK;
+    }
 
+    // the bit-packed passes, from the input again
+    e = cudaMemcpyAsync(dst, &st, sizeof(st), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dplan, &pl, sizeof(pl), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(dkerr, 0, sizeof(int32_t), s);
+    if (e != cudaSuccess) return err(err_buf, err_cap, MHS_ECUDA, cudaGetErrorString(e));
     // the bit-packed operands must start all-zero (a call that stopped early
     // may have left incidences set)
     e = cudaMemsetAsync(base + o_ab, 0, (size_t)(o_atb - o_ab + atrows * words(m) * 4), s);
     if (e == cudaSuccess) e = launch_build(dst, 1, 0, nnz, m, n, s);
     if (e != cudaSuccess) return err(err_buf, err_cap, MHS_ECUDA, cudaGetErrorString(e));
-    BatchCounters ctr;
-    std::memset(&ctr, 0, sizeof(ctr));
     int32_t kerr = 0;
     // every changing round deletes an item, so n + m + 1 rounds always suffice
     for (int32_t r = 0; r <= n + m + 1; ++r) {

@@ -200,6 +200,26 @@ def test_lists_around_the_lengths_of_tasks(mhs, deg, rule):
         _same(mhs.kernelize(inst, rule=rule), O.reduce_variant(inst, rule, False))
 
 
+@pytest.mark.parametrize("n,m,lo,hi,alpha", [
+    (1000, 2000, 2, 16, 3), (32, 4096, 14, 16, 3), (16, 4096, 16, 16, 3), (8, 4096, 1, 8, 5),
+    (300, 300, 195, 205, 4), (1000, 60, 900, 1000, 9), (4096, 4096, 1, 16, 3)])
+def test_noalloc_by_lists_and_by_bits(mhs, n, m, lo, hi, alpha):
+    """mhs_kernelize_noalloc on both sides of the rule between its two forms."""
+    import torch
+    inst = I.uniform_random(n, m, lo, hi, alpha, 0, seed=n + m + lo)
+    d = [torch.from_numpy(np.ascontiguousarray(a, np.int32)).cuda()
+         for a in (inst.edge_ptr, inst.edge_vtx, inst.demand)]
+    ref = O.reduce(inst)
+    for _ in range(2):
+        av = torch.full((n,), 7, dtype=torch.uint8, device="cuda")
+        ae = torch.full((m,), 7, dtype=torch.uint8, device="cuda")
+        rounds = mhs.kernelize_noalloc(n, m, *d, inst.nnz, av, ae)
+        assert rounds == ref["rounds"]
+        assert torch.nonzero(av).flatten().tolist() == ref["vertices"].tolist()
+        assert torch.nonzero(ae).flatten().tolist() == ref["edges"].tolist()
+        assert int(av.max()) <= 1 and int(ae.max()) <= 1
+
+
 def test_dense_hypergraphs_are_contracted(mhs):
     """Long lists throughout: the load leaves this path, with the same result."""
     rng = np.random.Generator(np.random.PCG64(3))
