@@ -551,8 +551,11 @@ def run_ours(args, rank, world, dist):
     # the DP contraction, k_compact_edges, k_plan, the fused A clear / A^T set
     # scatter, [k_tile_list], the MD contraction, the A^T clear scatter,
     # k_compact_vertices and the loop-condition kernel ([] tcgen05 only), plus
-    # the three FE kernels with --full-edges.
+    # the three FE kernels with --full-edges.  FP8 from 8,000 hyperedges on: the
+    # three kernels of the vertex bounds, once.
     load_kernels = 11 + (2 if batch else 0)
+    if args.contraction == "fp8" and (sum if batch else max)(i.m for i in insts) >= 8000:
+        load_kernels += 3
     per_round = (12 if args.contraction == "fp8" else 10) + (3 if args.full_edges else 0)
     line = {
         "metric": METRIC, "value": round(value, 4), "unit": UNIT, "n_gpus": world,

@@ -39,6 +39,10 @@ cudaError_t launch_build(InstState *st, int count, int32_t max_rounds, int64_t m
 // done_list (may be NULL): receives the index of every instance that stops
 // in this round (phase 1); ctr->n_done counts them.
 // tile_n: columns per tcgen05 tile (128 or 256; the value in plan->tile_n).
+// tcgen05 path, before the first round: the hyperedges that a vertex's bound
+// deletes leave its DP pass before the operand is built (they count as deleted
+// by it).
+cudaError_t launch_bounds(InstState *st, int count, int sms, cudaStream_t s, int compact_blocks);
 cudaError_t launch_round_phase(InstState *st, Plan *plan, BatchCounters *ctr, int count,
                                int phase, int contraction, int sms, int32_t *kerr,
                                cudaStream_t s, cudaEvent_t ev_contract_begin,

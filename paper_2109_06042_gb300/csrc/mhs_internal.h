@@ -114,6 +114,7 @@ struct InstState {
     int32_t max_rounds;    // 0 = unbounded
     int32_t changed;       // last round deleted something
     int32_t dp_deleted, md_deleted;
+    int32_t bounds_deleted; // of the running DP pass: deleted before its operand was built
     int32_t status;        // kErr* bits
     int32_t layout_sorted; // 0: input order; 1: hyperedges by smallest vertex id;
                            // 2: vertices by degree class, hyperedges by smallest vertex position
