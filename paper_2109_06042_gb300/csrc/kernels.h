@@ -130,16 +130,22 @@ struct SpTimes {
 // CTAs per instance (all of the launch resident together), or 0: one CTA per
 // instance of a batch, from a queue.  nnz, items (n + m): of the largest one.
 int sparse_team(int count, int64_t nnz, int64_t items, int sms);
+// The next instance of a batch (team = 0), and the CTAs that are done.
+struct SpQueue {
+    int32_t next, done;
+};
 // Structural checks (status bits), rows, vertex lists and the cost of every
 // instance.  The caller has zeroed every sp_ctl, sp_vrec, sp_vagg, sp_bound and
-// stamp array, *queue (used for team = 0) and *out.
+// stamp array, *queue and *out.  host (page-locked) receives *out, which is
+// zero again afterwards, like *queue; null: they are left as they end.
 cudaError_t launch_sparse_build(InstState *st, int count, int team, int32_t max_rounds,
-                                int32_t *queue, SpTotals *out, int sms, cudaStream_t s);
-// At most `limit` rounds (0: to the fixpoint); adds to *ctr and *times
-// (which the caller has zeroed, like *queue).
+                                SpQueue *queue, SpTotals *out, SpTotals *host, int sms,
+                                cudaStream_t s);
+// At most `limit` rounds (0: to the fixpoint); adds to *ctr and *times (zero
+// before, like *queue).  host: as above, for *ctr.
 cudaError_t launch_sparse_rounds(InstState *st, int count, int team, int32_t limit,
-                                 BatchCounters *ctr, int32_t *queue, SpTimes *times, int sms,
-                                 cudaStream_t s);
+                                 BatchCounters *ctr, SpQueue *queue, SpTimes *times,
+                                 BatchCounters *host, int sms, cudaStream_t s);
 // One part of a sharded round of a single instance.
 enum SpPass : int {
     kSpBegin0, kSpContract0, kSpExport0, kSpImport0,

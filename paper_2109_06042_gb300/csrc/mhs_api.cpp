@@ -223,11 +223,8 @@ struct Arena {
 struct SpWords {
     BatchCounters ctr;
     SpTimes times;
-    int32_t queue;     // next instance of a batch
-    int32_t pad;
     SpTotals totals;   // written by the build
-    int32_t build_queue;
-    int32_t pad2;
+    SpQueue queue;
 };
 
 struct HostInst {  // per-instance host bookkeeping
@@ -291,6 +288,7 @@ struct mhs_instance {
     // and its words in the arena
     int sp_team = 0;
     SpWords *sp = nullptr;
+    bool sp_counted = false;     // a sharded pass left its counts in them
     // sharded passes (mhs_pass_*): 0 between rounds, 1 DP pass open,
     // 2 DP pass ended, 3 MD pass open
     int32_t pass_state = 0;
@@ -898,11 +896,9 @@ mhs_status finish_load(mhs_instance *h, int64_t tmap_off) {
 // kernel, and what it found.  Synchronises.  *pays: the instance stays on
 // this path.
 mhs_status build_sparse(mhs_instance *h, SpTotals *found, bool *pays) {
-    CUDA_TRY(launch_sparse_build(h->dstate, h->count, h->sp_team, h->opt.max_rounds,
-                                 &h->sp->build_queue, &h->sp->totals, h->sms, h->stream));
     SpTotals *host = reinterpret_cast<SpTotals *>(h->pin + 128);
-    CUDA_TRY(cudaMemcpyAsync(host, &h->sp->totals, sizeof(SpTotals), cudaMemcpyDeviceToHost,
-                             h->stream));
+    CUDA_TRY(launch_sparse_build(h->dstate, h->count, h->sp_team, h->opt.max_rounds, &h->sp->queue,
+                                 &h->sp->totals, host, h->sms, h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     *found = *host;
     double pairs = 0;
@@ -1074,13 +1070,15 @@ mhs_status run_sparse(mhs_instance *h, int32_t limit, mhs_round_stats *stats) {
     if (h->timing)
         for (auto &e : h->ev)
             if (!e) CUDA_TRY(cudaEventCreate(&e));
-    CUDA_TRY(cudaMemsetAsync(h->sp, 0, offsetof(SpWords, totals), h->stream));
-    if (h->timing) CUDA_TRY(cudaEventRecord(h->ev[4], h->stream));
+    if (h->sp_counted) CUDA_TRY(cudaMemsetAsync(&h->sp->ctr, 0, sizeof(BatchCounters), h->stream));
+    h->sp_counted = false;
+    if (h->timing) {
+        CUDA_TRY(cudaMemsetAsync(&h->sp->times, 0, sizeof(SpTimes), h->stream));
+        CUDA_TRY(cudaEventRecord(h->ev[4], h->stream));
+    }
     CUDA_TRY(launch_sparse_rounds(h->dstate, h->count, h->sp_team, limit, &h->sp->ctr,
-                                  &h->sp->queue, &h->sp->times, h->sms, h->stream));
+                                  &h->sp->queue, &h->sp->times, h->hctr, h->sms, h->stream));
     if (h->timing) CUDA_TRY(cudaEventRecord(h->ev[5], h->stream));
-    CUDA_TRY(cudaMemcpyAsync(h->hctr, &h->sp->ctr, sizeof(BatchCounters), cudaMemcpyDeviceToHost,
-                             h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     if (h->timing) {  // the launch's time, split by where its lead threads spent theirs
         SpTimes t;
@@ -1832,6 +1830,7 @@ cudaError_t pass_finish(mhs_instance *h, int phase) {
         if (phase == 0) return cudaSuccess;  // DP's deletions are booked with MD's
         cudaError_t e = cudaMemsetAsync(&h->sp->ctr, 0, sizeof(BatchCounters), h->stream);
         if (e != cudaSuccess) return e;
+        h->sp_counted = true;
         return launch_sparse_pass(h->dstate, h->sp_team, kSpEnd1, 0, 1, &h->sp->ctr, nullptr,
                                   h->stream);
     }

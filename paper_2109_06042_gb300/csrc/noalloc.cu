@@ -71,7 +71,7 @@ struct Words {
     SpTotals totals;
     SpTimes times;
     BatchCounters ctr;
-    int32_t queue;
+    SpQueue queue;
 };
 
 struct Take {
@@ -247,7 +247,7 @@ extern "C" mhs_status mhs_kernelize_noalloc(int32_t n, int32_t m, const int32_t 
         if (e == cudaSuccess)
             e = cudaMemsetAsync(base + o_words, 0, (size_t)(take.bytes - o_words), s);
         if (e == cudaSuccess)
-            e = launch_sparse_build(dst, 1, team, 0, &dw->queue, &dw->totals, sms, s);
+            e = launch_sparse_build(dst, 1, team, 0, &dw->queue, &dw->totals, nullptr, sms, s);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(&found, &dw->totals, sizeof(found), cudaMemcpyDeviceToHost, s);
     } else {
@@ -263,7 +263,8 @@ extern "C" mhs_status mhs_kernelize_noalloc(int32_t n, int32_t m, const int32_t 
     if (found.status)
         return err(err_buf, err_cap, MHS_EINVAL, "malformed instance (bad edge_ptr or vertex id)");
     if (lists && found.cost <= kNoAllocCost) {
-        e = launch_sparse_rounds(dst, 1, team, 0, &dw->ctr, &dw->queue, &dw->times, sms, s);
+        e = launch_sparse_rounds(dst, 1, team, 0, &dw->ctr, &dw->queue, &dw->times, nullptr,
+                                 sms, s);
         if (e == cudaSuccess && (n > 0 || m > 0))
             e = launch_alive_masks(dst, n > 0 ? alive_v : nullptr, m > 0 ? alive_e : nullptr, s);
         if (e == cudaSuccess)

@@ -1889,48 +1889,68 @@ __device__ void run_pass(int op, int shard, int nshards, BatchCounters *ctr, voi
 
 // Team of CTAs per instance (team > 0, all CTAs resident: a cooperative
 // launch), or one CTA per instance taken from a queue (team = 0).
+// The last CTA of the launch hands `words` words over to the host and zeroes
+// them for the next launch (a copy and a memset in the stream took 5 us of a
+// call with a small instance).  host null: they stay.  Thread 0.
+__device__ __noinline__ void report(SpQueue *q, int32_t *from, volatile int32_t *host, int words) {
+    if (!host) return;
+    __threadfence();
+    if (atomicAdd(&q->done, 1) != (int32_t)gridDim.x - 1) return;
+    __threadfence();
+#pragma unroll 1
+    for (int w = 0; w < words; ++w) {
+        host[w] = __ldcg(from + w);
+        from[w] = 0;
+    }
+    q->next = q->done = 0;
+}
+
 template <int kThreads, int kMinBlocks>
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
-    k_sparse_build(InstState *st, int count, int team, int32_t max_rounds, int32_t *queue,
-                   SpTotals *out) {
+    k_sparse_build(InstState *st, int count, int team, int32_t max_rounds, SpQueue *queue,
+                   SpTotals *out, SpTotals *host) {
     Shared *sh = shared();
     if (team > 0) {
-        const int b = blockIdx.x / team;
-        if (b >= count) return;
-        start(st + b, blockIdx.x % team, team);
+        start(st + blockIdx.x / team, blockIdx.x % team, team);
         build_instance(max_rounds, out);
-        return;
+    } else {
+        for (;;) {
+            __syncthreads();
+            if (threadIdx.x == 0) sh->next = atomicAdd(&queue->next, 1);
+            __syncthreads();
+            if (sh->next >= count) break;
+            start(st + sh->next, 0, 1, true);
+            build_instance(max_rounds, out);
+        }
     }
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) sh->next = atomicAdd(queue, 1);
-        __syncthreads();
-        if (sh->next >= count) return;
-        start(st + sh->next, 0, 1, true);
-        build_instance(max_rounds, out);
-    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        report(queue, reinterpret_cast<int32_t *>(out), reinterpret_cast<int32_t *>(host),
+               sizeof(SpTotals) / 4);
 }
 
 template <int kThreads, int kMinBlocks>
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
     k_sparse_rounds(InstState *st, int count, int team, int32_t limit, BatchCounters *ctr,
-                    int32_t *queue, SpTimes *times) {
+                    SpQueue *queue, SpTimes *times, BatchCounters *host) {
     Shared *sh = shared();
     if (team > 0) {
-        const int b = blockIdx.x / team;
-        if (b >= count) return;
-        start(st + b, blockIdx.x % team, team);
+        start(st + blockIdx.x / team, blockIdx.x % team, team);
         run_instance(limit, ctr, times);
-        return;
+    } else {
+        for (;;) {
+            __syncthreads();
+            if (threadIdx.x == 0) sh->next = atomicAdd(&queue->next, 1);
+            __syncthreads();
+            if (sh->next >= count) break;
+            start(st + sh->next, 0, 1);
+            run_instance(limit, ctr, times);
+        }
     }
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) sh->next = atomicAdd(queue, 1);
-        __syncthreads();
-        if (sh->next >= count) return;
-        start(st + sh->next, 0, 1);
-        run_instance(limit, ctr, times);
-    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        report(queue, reinterpret_cast<int32_t *>(ctr), reinterpret_cast<int32_t *>(host),
+               sizeof(BatchCounters) / 4);
 }
 
 __global__ void __launch_bounds__(kSpThreads, 1)
@@ -1970,26 +1990,27 @@ static cudaError_t launch_team(void (*k)(A...), int ctas, cudaStream_t s, B... a
 }
 
 cudaError_t launch_sparse_build(InstState *st, int count, int team, int32_t max_rounds,
-                                int32_t *queue, SpTotals *out, int sms, cudaStream_t s) {
+                                SpQueue *queue, SpTotals *out, SpTotals *host, int sms,
+                                cudaStream_t s) {
     if (team > 0)
         return launch_team(k_sparse_build<kSpThreads, 1>, count * team, s, st, count, team,
-                           max_rounds, queue, out);
+                           max_rounds, queue, out, host);
     const size_t smem = shared_bytes(kSpBatchThreads) + 4 * kLocalVertices;
     k_sparse_build<kSpBatchThreads, kSpBatchBlocks>
-        <<<std::min(count, sms * kSpBatchBlocks), kSpBatchThreads, smem, s>>>(st, count, 0, max_rounds,
-                                                                              queue, out);
+        <<<std::min(count, sms * kSpBatchBlocks), kSpBatchThreads, smem, s>>>(
+            st, count, 0, max_rounds, queue, out, host);
     return cudaGetLastError();
 }
 
 cudaError_t launch_sparse_rounds(InstState *st, int count, int team, int32_t limit,
-                                 BatchCounters *ctr, int32_t *queue, SpTimes *times, int sms,
-                                 cudaStream_t s) {
+                                 BatchCounters *ctr, SpQueue *queue, SpTimes *times,
+                                 BatchCounters *host, int sms, cudaStream_t s) {
     if (team > 0)
         return launch_team(k_sparse_rounds<kSpThreads, 1>, count * team, s, st, count, team, limit,
-                           ctr, queue, times);
+                           ctr, queue, times, host);
     k_sparse_rounds<kSpBatchThreads, kSpBatchBlocks>
         <<<std::min(count, sms * kSpBatchBlocks), kSpBatchThreads, shared_bytes(kSpBatchThreads), s>>>(
-            st, count, 0, limit, ctr, queue, times);
+            st, count, 0, limit, ctr, queue, times, host);
     return cudaGetLastError();
 }
 
