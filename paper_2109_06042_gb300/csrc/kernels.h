@@ -134,6 +134,14 @@ int sparse_team(int count, int64_t nnz, int64_t items, int sms);
 struct SpQueue {
     int32_t next, done;
 };
+// A single instance whose rounds are launched before the host has seen what the
+// build found (built set): they run if it found no error and a cost of at most
+// max_cost, and leave the alive masks of the input ids.
+struct SpMasks {
+    const SpTotals *built;
+    unsigned long long max_cost;
+    uint8_t *v, *e;
+};
 // Structural checks (status bits), rows, vertex lists and the cost of every
 // instance.  The caller has zeroed every sp_ctl, sp_vrec, sp_vagg, sp_bound and
 // stamp array, *queue and *out.  host (page-locked) receives *out, which is
@@ -145,7 +153,8 @@ cudaError_t launch_sparse_build(InstState *st, int count, int team, int32_t max_
 // before, like *queue).  host: as above, for *ctr.
 cudaError_t launch_sparse_rounds(InstState *st, int count, int team, int32_t limit,
                                  BatchCounters *ctr, SpQueue *queue, SpTimes *times,
-                                 BatchCounters *host, int sms, cudaStream_t s);
+                                 BatchCounters *host, const SpMasks &masks, int sms,
+                                 cudaStream_t s);
 // One part of a sharded round of a single instance.
 enum SpPass : int {
     kSpBegin0, kSpContract0, kSpExport0, kSpImport0,

@@ -1077,7 +1077,7 @@ mhs_status run_sparse(mhs_instance *h, int32_t limit, mhs_round_stats *stats) {
         CUDA_TRY(cudaEventRecord(h->ev[4], h->stream));
     }
     CUDA_TRY(launch_sparse_rounds(h->dstate, h->count, h->sp_team, limit, &h->sp->ctr,
-                                  &h->sp->queue, &h->sp->times, h->hctr, h->sms, h->stream));
+                                  &h->sp->queue, &h->sp->times, h->hctr, {}, h->sms, h->stream));
     if (h->timing) CUDA_TRY(cudaEventRecord(h->ev[5], h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     if (h->timing) {  // the launch's time, split by where its lead threads spent theirs

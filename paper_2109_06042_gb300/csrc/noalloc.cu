@@ -33,6 +33,7 @@
 // before any kernel touches it; anything else is MHS_EINVAL.
 #include <cuda_runtime.h>
 
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 
@@ -56,23 +57,32 @@ inline int64_t words(int64_t K) { return up(((K + 31) / 32) > 0 ? (K + 31) / 32 
 // The candidate lists are taken for rows of this mean length at most, and while
 // their first round visits no more list entries than this.  Measured, a call
 // by lists / by bits alone (us); bits after a build that did not pay: + 50.
-//   n 1,000, m 2,000, |e| 2..16:       cost 55 K     96 / 254
-//   n 256, m 4,096, |e| 14..16:        cost 1.8 M   131 / 180
-//   n 32, m 4,096, |e| 14..16:         cost 15 M    322 / 292
-//   n 8, m 4,096, |e| 1..8:            cost 20 M    102 / 381
-//   n 16, m 4,096, |e| 8..16:          cost 25 M   1293 / 370
-//   n 1,000, m 300, |e| 150..200:      mean 175     184 / 201
-//   n 2,000, m 200, |e| 300..320:      mean 310     289 / 237
+//   n 1,000, m 2,000, |e| 2..16:       cost 55 K     83 / 254
+//   n 256, m 4,096, |e| 14..16:        cost 1.8 M   117 / 180
+//   n 32, m 4,096, |e| 14..16:         cost 15 M    308 / 292
+//   n 8, m 4,096, |e| 1..8:            cost 20 M     87 / 381
+//   n 16, m 4,096, |e| 8..16:          cost 25 M   1280 / 370
+//   n 1,000, m 300, |e| 150..200:      mean 175     169 / 201
+//   n 2,000, m 200, |e| 300..320:      mean 310     275 / 237
 constexpr unsigned long long kNoAllocCost = 20000000;
 constexpr int64_t kNoAllocMeanSize = 200;
+// Not even built above this: a list of mean length per hyperedge (n 16, m 4,096,
+// |e| 8..16: 12.6 M, 400 us with the build, 370 without; n 8: 9.3 M).
+constexpr int64_t kNoAllocEstimate = 10000000;
 
-// What the candidate lists' two launches start with at zero.
+// What the candidate lists' two launches start with at zero, and what the host
+// reads back (the first two).
 struct Words {
     SpTotals totals;
-    SpTimes times;
     BatchCounters ctr;
+    SpTimes times;
     SpQueue queue;
 };
+struct Found {
+    SpTotals totals;
+    BatchCounters ctr;
+};
+static_assert(offsetof(Words, ctr) == offsetof(Found, ctr), "one copy");
 
 struct Take {
     int64_t bytes = 0;
@@ -239,38 +249,34 @@ extern "C" mhs_status mhs_kernelize_noalloc(int32_t n, int32_t m, const int32_t 
     Words *dw = reinterpret_cast<Words *>(base + o_words);
     const int team = sparse_team(1, nnz, (int64_t)n + m, sms);
     cudaError_t e = cudaMemcpyAsync(dst, &st, sizeof(st), cudaMemcpyHostToDevice, s);
-    BatchCounters ctr;
-    std::memset(&ctr, 0, sizeof(ctr));
-    bool lists = nnz <= kNoAllocMeanSize * m;
-    SpTotals found = {};
+    const bool lists = nnz <= kNoAllocMeanSize * m && (int64_t)nnz * m <= kNoAllocEstimate * n;
+    Found found;
+    std::memset(&found, 0, sizeof(found));
+    BatchCounters &ctr = found.ctr;
     if (lists) {
         if (e == cudaSuccess)
             e = cudaMemsetAsync(base + o_words, 0, (size_t)(take.bytes - o_words), s);
         if (e == cudaSuccess)
             e = launch_sparse_build(dst, 1, team, 0, &dw->queue, &dw->totals, nullptr, sms, s);
+        // (whether they are to run is decided on the device: one wait, not two)
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(&found, &dw->totals, sizeof(found), cudaMemcpyDeviceToHost, s);
+            e = launch_sparse_rounds(dst, 1, team, 0, &dw->ctr, &dw->queue, &dw->times, nullptr,
+                                     {&dw->totals, kNoAllocCost, alive_v, alive_e}, sms, s);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(&found, dw, sizeof(found), cudaMemcpyDeviceToHost, s);
     } else {
         if (e == cudaSuccess) e = launch_validate(dst, 1, s);
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(&found.status, &dst->status, sizeof(int32_t),
+            e = cudaMemcpyAsync(&found.totals.status, &dst->status, sizeof(int32_t),
                                 cudaMemcpyDeviceToHost, s);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return err(err_buf, err_cap, MHS_ECUDA, cudaGetErrorString(e));
-    if (found.status & (kErrTimeout | kErrCapacity))
+    if (found.totals.status & (kErrTimeout | kErrCapacity))
         return err(err_buf, err_cap, MHS_EDEVICE, "kernel reported an error status");
-    if (found.status)
+    if (found.totals.status)
         return err(err_buf, err_cap, MHS_EINVAL, "malformed instance (bad edge_ptr or vertex id)");
-    if (lists && found.cost <= kNoAllocCost) {
-        e = launch_sparse_rounds(dst, 1, team, 0, &dw->ctr, &dw->queue, &dw->times, nullptr,
-                                 sms, s);
-        if (e == cudaSuccess && (n > 0 || m > 0))
-            e = launch_alive_masks(dst, n > 0 ? alive_v : nullptr, m > 0 ? alive_e : nullptr, s);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(&ctr, &dw->ctr, sizeof(ctr), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) return err(err_buf, err_cap, MHS_ECUDA, cudaGetErrorString(e));
+    if (lists && found.totals.cost <= kNoAllocCost) {
         if (ctr.status_any || ctr.active)
             return err(err_buf, err_cap, MHS_EDEVICE, "kernel reported an error status");
         if (rounds_out) *rounds_out = ctr.max_rounds_seen;

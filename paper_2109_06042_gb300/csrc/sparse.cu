@@ -1932,11 +1932,19 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
 template <int kThreads, int kMinBlocks>
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
     k_sparse_rounds(InstState *st, int count, int team, int32_t limit, BatchCounters *ctr,
-                    SpQueue *queue, SpTimes *times, BatchCounters *host) {
+                    SpQueue *queue, SpTimes *times, BatchCounters *host, SpMasks masks) {
     Shared *sh = shared();
+    if (masks.built && (masks.built->status || masks.built->cost > masks.max_cost)) return;
     if (team > 0) {
         start(st + blockIdx.x / team, blockIdx.x % team, team);
         run_instance(limit, ctr, times);
+        if (masks.built) {  // (every CTA is past the last round's barrier)
+            const int32_t t0 = sh->rank * blockDim.x + threadIdx.x, ts = sh->size * blockDim.x;
+#pragma unroll 1
+            for (int32_t x = t0; x < sh->n0; x += ts) masks.v[x] = sh->view.v_o2c[x] >= 0;
+#pragma unroll 1
+            for (int32_t e = t0; e < sh->m0; e += ts) masks.e[e] = sh->view.e_o2c[e] >= 0;
+        }
     } else {
         for (;;) {
             __syncthreads();
@@ -2004,13 +2012,14 @@ cudaError_t launch_sparse_build(InstState *st, int count, int team, int32_t max_
 
 cudaError_t launch_sparse_rounds(InstState *st, int count, int team, int32_t limit,
                                  BatchCounters *ctr, SpQueue *queue, SpTimes *times,
-                                 BatchCounters *host, int sms, cudaStream_t s) {
+                                 BatchCounters *host, const SpMasks &masks, int sms,
+                                 cudaStream_t s) {
     if (team > 0)
         return launch_team(k_sparse_rounds<kSpThreads, 1>, count * team, s, st, count, team, limit,
-                           ctr, queue, times, host);
+                           ctr, queue, times, host, masks);
     k_sparse_rounds<kSpBatchThreads, kSpBatchBlocks>
         <<<std::min(count, sms * kSpBatchBlocks), kSpBatchThreads, shared_bytes(kSpBatchThreads), s>>>(
-            st, count, 0, limit, ctr, queue, times, host);
+            st, count, 0, limit, ctr, queue, times, host, masks);
     return cudaGetLastError();
 }
 

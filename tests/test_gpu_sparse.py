@@ -202,6 +202,7 @@ def test_lists_around_the_lengths_of_tasks(mhs, deg, rule):
 
 @pytest.mark.parametrize("n,m,lo,hi,alpha", [
     (1000, 2000, 2, 16, 3), (32, 4096, 14, 16, 3), (16, 4096, 16, 16, 3), (8, 4096, 1, 8, 5),
+    (40, 4096, 14, 16, 8),
     (300, 300, 195, 205, 4), (1000, 60, 900, 1000, 9), (4096, 4096, 1, 16, 3)])
 def test_noalloc_by_lists_and_by_bits(mhs, n, m, lo, hi, alpha):
     """mhs_kernelize_noalloc on both sides of the rule between its two forms."""
