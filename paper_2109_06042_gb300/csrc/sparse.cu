@@ -204,16 +204,17 @@ constexpr size_t kSharedBytes = (sizeof(Shared) + 15) / 16 * 16;
 constexpr size_t shared_bytes(int threads) { return kSharedBytes + threads / 32 * sizeof(WarpShared); }
 extern __shared__ __align__(16) uint8_t sp_smem[];
 __device__ __forceinline__ Shared *shared() { return reinterpret_cast<Shared *>(sp_smem); }
-// And behind that, in the build of a batch, degrees of up to kLocalVertices
-// vertices: a CTA that has an instance to itself counts them there (on a batch
-// of 4,096 instances with 56 M incidences the load takes 2.91 ms, 3.80 with
-// returning atomics on L2).  4,096: the CTAs' shared memory stays below 48 KB.
-constexpr int32_t kLocalVertices = 4096;
+// And behind that, in the build of a batch, the degrees of up to kLocalVertices
+// vertices, and the places of their lists: a CTA that has an instance to
+// itself counts them there (a batch of 4,096 instances with 56 M incidences:
+// the load takes 2.9 ms, 3.8 with returning atomics on L2; the places 0.08).
+// 3,072: the CTAs' shared memory stays below 48 KB.
+constexpr int32_t kLocalVertices = 3072;
 __device__ __forceinline__ int32_t *local_degrees() {
     return reinterpret_cast<int32_t *>(sp_smem + shared_bytes(blockDim.x));
 }
 static_assert(shared_bytes(kSpThreads) <= 48 * 1024 &&
-                  shared_bytes(kSpBatchThreads) + 4 * kLocalVertices <= 48 * 1024,
+                  shared_bytes(kSpBatchThreads) + 8 * kLocalVertices <= 48 * 1024,
               "more needs cudaFuncAttributeMaxDynamicSharedMemorySize");
 __device__ __forceinline__ WarpShared *warp_shared() {
     return reinterpret_cast<WarpShared *>(sp_smem + kSharedBytes) + (threadIdx.x >> 5);
@@ -438,10 +439,12 @@ __device__ __noinline__ void contribute(int32_t e, int32_t f, int32_t len, const
     if (f > len && sub == 0 && atomicMax(&ctl->loose, f - len) < f - len)
         ctl->c[sh->par].scan_all = 1;
     if (!sh->full) return;
+    // every two heavy ones: they end the row, and most rows have fewer
+    int32_t a = len - 1;
+    while (a > 0 && row[a - 1] >= kHeavyKey) --a;
 #pragma unroll 1
-    for (int32_t a = 0; a < len - 1; ++a) {
+    for (; a < len - 1; ++a) {
         const uint32_t ka = row[a];
-        if (ka < kHeavyKey) continue;  // (the heavy ones end the row)
 #pragma unroll 1
         for (int32_t k = a + 1 + sub; k < len; k += kG)
             add_pair_bound(sh, e, f, len, ka & kIdMask, row[k] & kIdMask);
@@ -850,9 +853,9 @@ __device__ __noinline__ void dp_walk(int shard, int nshards) {
                 const int32_t lists = min(npmax - p0, kG);
 #pragma unroll 1
                 for (int q = 0; q < lists; ++q) {
-                    const int32_t d = __shfl_sync(0xffffffffu, deg, c.lead + q);
-                    const int32_t b = __shfl_sync(0xffffffffu, vr.w, c.lead + q);
-                    const int32_t lp = __shfl_sync(0xffffffffu, p, c.lead + q);
+                    const int32_t dq = __shfl_sync(0xffffffffu, deg | (p & kNeed3), q, kG);
+                    const int32_t b = __shfl_sync(0xffffffffu, vr.w, q, kG);
+                    const int32_t d = dq & ~kNeed3, lp = (p0 + q) | (dq & kNeed3);
                     const int32_t maxd = __reduce_max_sync(0xffffffffu, d);
 #pragma unroll 1
                     for (int32_t o = c.sub; o - c.sub < maxd; o += kU * kG) {
@@ -1377,14 +1380,15 @@ __device__ __forceinline__ int32_t count_row(const Ctx &c, const View &v, const 
 }
 
 // The row of hyperedge e in key order, and its entries in its vertices'
-// lists, by kW lanes (8 or 32; `lane` of them, from the warp's lane `lead`)
+// lists, by kW lanes (8 or 32; `lane` of them)
 // that hold the row (len <= kRowU * kW) in registers and rank each key by
 // counting.  Adds to *cost the lengths of the lists of its np rarest
 // vertices; returns the signature.  The whole warp calls it.
 template <int kW>
-__device__ __forceinline__ u64 fill_row(const Ctx &c, const View &v, const int32_t *ids,
-                                        const int32_t *place, uint32_t *row, int32_t e, int32_t f,
-                                        int32_t len, int32_t np, int lane, int lead, u64 *cost) {
+__device__ __forceinline__ u64 fill_row(const Ctx &c, const View &v, const int32_t *local,
+                                        const int32_t *ids, const int32_t *place, uint32_t *row,
+                                        int32_t e, int32_t f, int32_t len, int32_t np, int lane,
+                                        u64 *cost) {
     const int32_t maxlen = kW == 32 ? len : __reduce_max_sync(0xffffffffu, len);
     uint32_t key[kRowU];
     int32_t at[kRowU], deg[kRowU], rank[kRowU];
@@ -1393,10 +1397,13 @@ __device__ __forceinline__ u64 fill_row(const Ctx &c, const View &v, const int32
     for (int u = 0; u < kRowU; ++u) {
         const int32_t k = u * kW + lane;
         const int32_t x = k < len ? ids[k] : -1;
-        const int4 vr = x >= 0 ? v.vrec[x] : make_int4(0, 0, 0, 0);
-        key[u] = x >= 0 ? row_key(x, vr.z) : 0xffffffffu;
-        at[u] = x >= 0 ? vr.w + place[k] : 0;
-        deg[u] = vr.z;
+        int2 vr = make_int2(0, 0);  // degree, place of the list
+        if (x >= 0)
+            vr = local ? make_int2(local[x], local[kLocalVertices + x])
+                       : *reinterpret_cast<const int2 *>(&v.vrec[x].z);
+        key[u] = x >= 0 ? row_key(x, vr.x) : 0xffffffffu;
+        at[u] = x >= 0 ? vr.y + place[k] : 0;
+        deg[u] = vr.x;
         rank[u] = 0;
         if (x >= 0) sig |= sig_bit(x);
     }
@@ -1407,10 +1414,23 @@ __device__ __forceinline__ u64 fill_row(const Ctx &c, const View &v, const int32
     }
 #pragma unroll
     for (int w = 0; w < kRowU; ++w) {
+        // (eight lanes: without loop control.  A batch is bound by what its
+        // warps issue; this and the sum of costs kept in registers take 0.3
+        // of its load's 2.8 ms)
+        if (kW == kG) {
+            if (w * kW >= maxlen) break;
+#pragma unroll
+            for (int l = 0; l < kW; ++l) {
+                const uint32_t y = __shfl_sync(0xffffffffu, key[w], l, kW);
+#pragma unroll
+                for (int u = 0; u < kRowU; ++u) rank[u] += y < key[u];
+            }
+            continue;
+        }
         const int32_t n = min(kW, maxlen - w * kW);
 #pragma unroll 1
         for (int l = 0; l < n; ++l) {
-            const uint32_t y = __shfl_sync(0xffffffffu, key[w], lead + l);
+            const uint32_t y = __shfl_sync(0xffffffffu, key[w], l);
 #pragma unroll
             for (int u = 0; u < kRowU; ++u) rank[u] += y < key[u];
         }
@@ -1582,7 +1602,10 @@ __device__ __noinline__ void build_instance(int32_t max_rounds, SpTotals *out) {
         int32_t at = 0;
         if (c.lane == 31) at = (int32_t)atomicAdd(&v.ctl->cursor, (uint32_t)inc);
         at = __shfl_sync(0xffffffffu, at, 31);
-        if (x < n0) v.vrec[x] = make_int4(0, 0, d, at + inc - d);
+        if (x < n0) {
+            v.vrec[x] = make_int4(0, 0, d, at + inc - d);
+            if (local) local[kLocalVertices + x] = at + inc - d;
+        }
         if (d > kHeavyDeg) {
             v.agg[x].heavy = 1;
             heavy[atomicAdd(&v.ctl->n_heavy, 1)] = x;
@@ -1590,6 +1613,7 @@ __device__ __noinline__ void build_instance(int32_t max_rounds, SpTotals *out) {
     }
     if (!team_sync()) return;
     const int32_t rule = s.edge_rule;
+    u64 cost = 0;  // the entries that walking this lane's hyperedges may visit
     for_flagged(
         c, m0, [](int32_t) { return true; },
         [&](int32_t e) {
@@ -1598,12 +1622,12 @@ __device__ __noinline__ void build_instance(int32_t max_rounds, SpTotals *out) {
             const int32_t *ids = r.x ? reinterpret_cast<const int32_t *>(v.row) + p0 : evtx + p0;
             uint32_t *row = v.row + p0;
             const int32_t np = e >= 0 ? walk_count(rule, r.z, len) : 0;
-            u64 sig = 0, cost = 0;  // cost: the entries walking this hyperedge may visit
+            u64 sig = 0;
             // rows up to 32: the group ranks each key among the row's
             const bool small = len <= kRowU * kG;
             if (__any_sync(0xffffffffu, small && len > 0)) {
-                sig = fill_row<kG>(c, v, ids, place + p0, row, e, r.z, small ? len : 0, np, c.sub,
-                                   c.lead, &cost);
+                sig = fill_row<kG>(c, v, local, ids, place + p0, row, e, r.z, small ? len : 0, np, c.sub,
+                                   &cost);
                 if (small && c.sub == 0 && e >= 0) v.erec[e] = make_rec(sig, r.z, len);
             }
             // longer ones, one after the other: the whole warp
@@ -1622,8 +1646,8 @@ __device__ __noinline__ void build_instance(int32_t max_rounds, SpTotals *out) {
                     sorted ? evtx + lp : reinterpret_cast<const int32_t *>(v.row) + lp;
                 u64 ls;
                 if (llen <= kRowU * 32)
-                    ls = fill_row<32>(c, v, lids, place + lp, v.row + lp, le, lf, llen, lnp, c.lane,
-                                      0, &cost);
+                    ls = fill_row<32>(c, v, local, lids, place + lp, v.row + lp, le, lf, llen, lnp, c.lane,
+                                      &cost);
                 else
                     ls = fill_long_row(lids, place + lp, tmp + lp, v.row + lp, le, lf, llen, lnp, &cost);
                 if (c.lane == 0) v.erec[le] = make_rec(ls, lf, llen);
@@ -1633,10 +1657,10 @@ __device__ __noinline__ void build_instance(int32_t max_rounds, SpTotals *out) {
             __syncwarp();
             if (e >= 0) contribute(e, r.z, len, row);
             __syncwarp();
-#pragma unroll
-            for (int o = kG / 2; o > 0; o >>= 1) cost += __shfl_xor_sync(0xffffffffu, cost, o);
-            if (c.sub == 0 && cost) atomicAdd(&c.sh->cost, cost);
         });
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) cost += __shfl_xor_sync(0xffffffffu, cost, o);
+    if (c.lane == 0 && cost) atomicAdd(&c.sh->cost, cost);
     __syncthreads();
     if (threadIdx.x == 0 && c.sh->cost) atomicAdd(&out->cost, c.sh->cost);
 }
@@ -2003,7 +2027,7 @@ cudaError_t launch_sparse_build(InstState *st, int count, int team, int32_t max_
     if (team > 0)
         return launch_team(k_sparse_build<kSpThreads, 1>, count * team, s, st, count, team,
                            max_rounds, queue, out, host);
-    const size_t smem = shared_bytes(kSpBatchThreads) + 4 * kLocalVertices;
+    const size_t smem = shared_bytes(kSpBatchThreads) + 8 * kLocalVertices;
     k_sparse_build<kSpBatchThreads, kSpBatchBlocks>
         <<<std::min(count, sms * kSpBatchBlocks), kSpBatchThreads, smem, s>>>(
             st, count, 0, max_rounds, queue, out, host);

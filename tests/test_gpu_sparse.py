@@ -171,10 +171,10 @@ def test_batch_of_uneven_instances(mhs):
                 _same(h.result(b), refs[b], f"{len(part)}: {b}")
 
 
-@pytest.mark.parametrize("n", [4095, 4096, 4097])
-def test_batch_around_the_limit_of_shared_degrees(mhs, n):
-    """The build of a batch counts the degrees of at most 4,096 vertices in
-    shared memory, and one CTA takes instances of both kinds in turn."""
+@pytest.mark.parametrize("n", [3071, 3072, 3073])
+def test_batch_around_the_limit_of_shared_vertices(mhs, n):
+    """The build of a batch keeps the degrees and places of at most 3,072
+    vertices in shared memory, and one CTA takes instances of both kinds in turn."""
     insts = [I.uniform_random(n + (s % 3 - 1) * 2, 3000 + s, 1, 6, 3, 5, seed=s) for s in range(3)]
     refs = [O.reduce(i) for i in insts]
     batch = [insts[b % 3] for b in range(700)]
