@@ -81,7 +81,8 @@ typedef enum {
 /* Order of the rows (and K columns) of the dense operands.  Results never
  * depend on it (ties are broken by input index); performance does. */
 typedef enum {
-    MHS_LAYOUT_AUTO = 0,    /* library choice (currently MHS_LAYOUT_DEGREE) */
+    MHS_LAYOUT_AUTO = 0,    /* library choice (currently MHS_LAYOUT_DEGREE; bit-packed, up to
+                               10,000 hyperedges: MHS_LAYOUT_INPUT) */
     MHS_LAYOUT_INPUT = 1,   /* input order */
     MHS_LAYOUT_SORTED = 2,  /* hyperedges by their smallest vertex id: interval-like
                                (low Dilworth number) inputs become banded */

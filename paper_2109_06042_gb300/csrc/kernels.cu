@@ -308,19 +308,30 @@ __global__ void k_layout_place(InstState *st, int count) {
 // start plus the number of hyperedges of the bucket with a smaller input id
 // (after step 3, v_deg[key] is the bucket's end and v_cnt[key] its size).
 // The cost is the sum of the squared bucket sizes; buckets hold the
-// hyperedges sharing their smallest vertex (id or position).
+// hyperedges sharing their smallest vertex (id or position).  Eight lanes per
+// hyperedge: a lane per hyperedge took 32 us on the power-law instance (the
+// largest bucket, entry by entry), eight take 20.
+constexpr int kRankLanes = 8;
 __global__ void k_layout_rank(InstState *st, int count) {
     const int b = blockIdx.y;
     if (b >= count) return;
     InstState &s = st[b];
     if (!s.layout_sorted || s.status) return;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < s.m0;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t key = s.e_s[e];
-        const int32_t hi = s.v_deg[key], lo = hi - s.v_cnt[key];
-        int32_t rank = 0;
-        for (int32_t p = lo; p < hi; ++p) rank += s.e_c2o[p] < (int32_t)e;
-        s.e_o2c[e] = lo + rank;
+    const int sub = threadIdx.x % kRankLanes;
+    for (int64_t e0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x - threadIdx.x % 32) / kRankLanes;
+         e0 < s.m0; e0 += (int64_t)gridDim.x * blockDim.x / kRankLanes) {
+        const int64_t e = e0 + threadIdx.x % 32 / kRankLanes;
+        int32_t lo = 0, hi = 0, rank = 0;
+        if (e < s.m0) {
+            const int32_t key = s.e_s[e];
+            hi = s.v_deg[key];
+            lo = hi - s.v_cnt[key];
+        }
+        for (int32_t p = lo + sub; p < hi; p += kRankLanes) rank += s.e_c2o[p] < (int32_t)e;
+        __syncwarp();
+#pragma unroll
+        for (int o = kRankLanes / 2; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+        if (sub == 0 && e < s.m0) s.e_o2c[e] = lo + rank;
     }
 }
 
@@ -1748,19 +1759,24 @@ cudaError_t launch_gather_bounds(const int64_t *gptr, const int64_t *e0, int64_t
 }
 
 cudaError_t launch_build(InstState *st, int count, int32_t max_rounds, int64_t max_nnz,
-                         int64_t max_m, int64_t max_n, cudaStream_t s) {
+                         int64_t max_m, int64_t max_n, cudaStream_t s, int layout) {
     const int gx = per_instance_grid(max_m, count);
     const int gz = per_instance_grid(max_nnz, count);
+    const int gr = per_instance_grid(max_m * kRankLanes, count);
     // a single instance splits its initial ranges over blocks
     const int gi = count > 1 ? 1 : (int)std::min<int64_t>((std::max(max_m, max_n) + 4095) / 4096, 152);
     k_init<<<dim3(gi > 0 ? gi : 1, count), 1024, 0, s>>>(st, count, max_rounds);
-    k_vertex_degrees<<<dim3(gz, count), 256, 0, s>>>(st, count);
-    k_vertex_layout<<<count, 1024, 0, s>>>(st, count);
-    k_layout_keys<<<dim3(gx, count), 256, 0, s>>>(st, count);
-    k_layout_scan<<<count, 1024, 0, s>>>(st, count);
-    k_layout_place<<<dim3(gx, count), 256, 0, s>>>(st, count);
-    k_layout_rank<<<dim3(gx, count), 256, 0, s>>>(st, count);
-    k_layout_commit<<<dim3(gx, count), 256, 0, s>>>(st, count);
+    if (layout == 2) {
+        k_vertex_degrees<<<dim3(gz, count), 256, 0, s>>>(st, count);
+        k_vertex_layout<<<count, 1024, 0, s>>>(st, count);
+    }
+    if (layout) {
+        k_layout_keys<<<dim3(gx, count), 256, 0, s>>>(st, count);
+        k_layout_scan<<<count, 1024, 0, s>>>(st, count);
+        k_layout_place<<<dim3(gx, count), 256, 0, s>>>(st, count);
+        k_layout_rank<<<dim3(gr, count), 256, 0, s>>>(st, count);
+        k_layout_commit<<<dim3(gx, count), 256, 0, s>>>(st, count);
+    }
     k_edge_rows<<<dim3(gx, count), 256, 0, s>>>(st, count);
     return cudaGetLastError();
 }

@@ -33,8 +33,9 @@ cudaError_t launch_localize_ptr(InstState *st, int count, const int64_t *gptr, c
                                 cudaStream_t s);
 cudaError_t launch_gather_bounds(const int64_t *gptr, const int64_t *e0, int64_t *out, int count,
                                  cudaStream_t s);
+// layout: InstState::layout_sorted of every instance.
 cudaError_t launch_build(InstState *st, int count, int32_t max_rounds, int64_t max_nnz,
-                         int64_t max_m, int64_t max_n, cudaStream_t s);
+                         int64_t max_m, int64_t max_n, cudaStream_t s, int layout);
 // One phase of a round: phase 0 = DP (Algorithm 1), phase 1 = MD (Algorithm 2).
 // done_list (may be NULL): receives the index of every instance that stops
 // in this round (phase 1); ctr->n_done counts them.

@@ -690,7 +690,7 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
         s.m0 = m[b];
         s.nnz0 = nnz[b];
         s.k = k[b];
-        s.layout_sorted = layout_code(opt.layout);
+        s.layout_sorted = layout_code(opt.layout, h->contraction, h->max_m);
         s.no_skip = opt.sparsity == MHS_SPARSITY_DENSE;
         s.edge_rule = opt.edge_rule;
         s.full_edges = opt.full_edges;
@@ -888,7 +888,7 @@ mhs_status finish_load(mhs_instance *h, int64_t tmap_off) {
         h->dense_zeroed = true;
     }
     CUDA_TRY(launch_build(h->dstate, h->count, h->opt.max_rounds, h->max_nnz, h->max_m,
-                          h->max_n, h->stream));
+                          h->max_n, h->stream, h->hstate[0].layout_sorted));
     return MHS_OK;
 }
 

@@ -291,7 +291,7 @@ extern "C" mhs_status mhs_kernelize_noalloc(int32_t n, int32_t m, const int32_t 
     // the bit-packed operands must start all-zero (a call that stopped early
     // may have left incidences set)
     e = cudaMemsetAsync(base + o_ab, 0, (size_t)(o_atb - o_ab + atrows * words(m) * 4), s);
-    if (e == cudaSuccess) e = launch_build(dst, 1, 0, nnz, m, n, s);
+    if (e == cudaSuccess) e = launch_build(dst, 1, 0, nnz, m, n, s, 0);
     if (e != cudaSuccess) return err(err_buf, err_cap, MHS_ECUDA, cudaGetErrorString(e));
     int32_t kerr = 0;
     // every changing round deletes an item, so n + m + 1 rounds always suffice

@@ -219,7 +219,7 @@ mhs_status admit(Lane &Ln, int si, std::shared_ptr<Request> req) {
     s.m0 = req->m;
     s.nnz0 = nnz;
     s.k = req->k;
-    s.layout_sorted = layout_code(S->opt.layout);
+    s.layout_sorted = layout_code(S->opt.layout, S->contraction, req->m);
     s.no_skip = S->opt.sparsity == MHS_SPARSITY_DENSE;
     s.edge_rule = S->opt.edge_rule;
     s.full_edges = S->opt.full_edges;
@@ -286,7 +286,8 @@ mhs_status admit(Lane &Ln, int si, std::shared_ptr<Request> req) {
     if (e == cudaSuccess) e = cudaMemsetAsync(a + L.dense, 0, (size_t)L.dense_bytes, Ln.load);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(Ln.dstage + si, &s, sizeof(s), cudaMemcpyHostToDevice, Ln.load);
-    if (e == cudaSuccess) e = launch_build(Ln.dstage + si, 1, 0, nnz, req->m, req->n, Ln.load);
+    if (e == cudaSuccess) e = launch_build(Ln.dstage + si, 1, 0, nnz, req->m, req->n, Ln.load,
+                                          s.layout_sorted);
     if (e != cudaSuccess) {
         cudaFreeAsync(a, Ln.load);
         return set_error(MHS_ECUDA, "server: admission failed: %s", cudaGetErrorString(e));
