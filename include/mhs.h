@@ -111,7 +111,8 @@ typedef enum {
 typedef struct {
     int32_t contraction; /* mhs_contraction */
     int32_t max_rounds;  /* mhs_kernelize stops after this many rounds; 0 = fixpoint */
-    int32_t use_graphs;  /* 1: replay captured CUDA graphs (the whole fixpoint in one launch) */
+    int32_t use_graphs;  /* 1: replay captured CUDA graphs (the whole fixpoint in one launch;
+                            bit-packed: what is left of it after three rounds) */
     int32_t layout;      /* mhs_layout */
     int32_t sparsity;    /* mhs_sparsity */
     int32_t edge_rule;   /* mhs_edge_rule */

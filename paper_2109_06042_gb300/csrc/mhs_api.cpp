@@ -1113,6 +1113,31 @@ mhs_status run_rounds(mhs_instance *h, int32_t limit, mhs_round_stats *stats) {
         CUDA_TRY(launch_bounds(h->dstate, h->count, h->sms, h->stream, h->compact_blocks));
     h->started = true;
     if (limit <= 0 && h->opt.use_graphs && !h->timing) {
+        // The bit-packed form's rounds are short and, without FE, usually two:
+        // they are launched as they are, and only then the graph is built, in
+        // the shadow of a third.  (Building and freeing it takes 85 us.)  Load
+        // to free, us, so / with the graph at once:
+        //   uniform 4,000 x 8,000, 2 rounds    250 / 317   (with FE, 4: 519 / 493)
+        //   power law 2,000 x 4,000, 4 rounds  542 / 510
+        //   interval 2,000 x 4,000, 7 rounds   629 / 606
+        // The FP8 form, 14 kernels a round, loses: power law 20,000 x 40,000,
+        // 4 rounds, 1357 / 1277.
+        const bool direct = h->contraction == kPopcount && !h->opt.full_edges;
+        for (int32_t r = 0; direct && !h->loop_graph; ++r) {
+            CUDA_TRY(enqueue_round(h, false));
+            if (r == 0) CUDA_TRY(enqueue_round(h, false));
+            if (r == 1) {
+                mhs_status st = build_loop_graph(h);
+                if (st) return st;
+            }
+            CUDA_TRY(cudaStreamSynchronize(h->stream));
+            mhs_status st = check_device_status(h);
+            if (st) return st;
+            if (h->hctr->active == 0) {
+                if (stats) stats_from(*h->hctr, stats);
+                return MHS_OK;
+            }
+        }
         if (!h->loop_graph) {
             mhs_status st = build_loop_graph(h);
             if (st) return st;
