@@ -455,13 +455,13 @@ bool auto_sparse(const mhs_options *opt) {
 // Does the sparse path pay?  cost: list entries its first round may visit;
 // pairs: m^2 + n^2 summed over the instances, what the contraction's
 // epilogue tests.  Measured (load and kernelization, sparse / FP8, us):
-//   n 200, m 20,000, |e| 16..32: cost 118 M, pairs 0.4 G    1240 /  768
-//   n 64, m 20,000, |e| 3..6:    cost  62 M, pairs 0.4 G     298 /  497
-//   n 16,000, m 24,000, |e| 32..64: cost 3.5 M, pairs 0.8 G  258 / 5248
+//   n 200, m 20,000, |e| 16..32: cost 118 M, pairs 0.4 G     921 /  749
+//   n 64, m 20,000, |e| 3..6:    cost  62 M, pairs 0.4 G     292 /  455
+//   n 16,000, m 24,000, |e| 32..64: cost 3.5 M, pairs 0.8 G  235 / 5273
 // and by the mean size, where the searches in rows and the work per
 // incidence grow:
-//   n 2,000, m 4,000, |e| 256..512: mean 384                1567 / 1302
-//   n 2,000, m 4,000, |e| 128..256: mean 192                 726 /  804
+//   n 2,000, m 4,000, |e| 256..512: mean 384                1664 / 1286
+//   n 2,000, m 4,000, |e| 128..256: mean 192                 774 /  790
 constexpr double kSparseBase = 64e6, kSparsePerPair = 1.0 / 20;
 constexpr double kSparseMeanSize = 256;
 bool sparse_pays(double cost, double pairs) { return cost <= kSparseBase + kSparsePerPair * pairs; }

@@ -44,13 +44,13 @@
 // team of CTAs per instance with a barrier between the phases (a cooperative
 // launch), or one CTA per instance of a batch.  Eight lanes share a
 // hyperedge or vertex, a warp's four groups in step; lists longer than
-// kHeavyList become tasks of kTaskLen entries for whole warps, vertices with
-// more than kHeavyDeg hyperedges are handled by whole CTAs.
+// kHeavyList become tasks for whole warps, vertices with more than kHeavyDeg
+// hyperedges are handled by whole CTAs.
 // Measured on one GB300, the rounds alone (load, kernelization and result
 // through the C ABI beside the FP8 contraction's):
-//   power law 20,000 x 40,000: 223 us (407 / 1,690)
-//   interval 50,000 x 100,000: 358 us (628 / 11,357)
-//   uniform 16,000 x 32,000, |e| 2..16: 68 us (197 / 6,145)
+//   power law 20,000 x 40,000: 225 us (400 / 1,240)
+//   interval 50,000 x 100,000: 358 us (600 / 5,900)
+//   uniform 16,000 x 32,000, |e| 2..16: 70 us (200 / 4,150)
 #include <algorithm>
 
 #include <cuda_runtime.h>
@@ -79,7 +79,9 @@ constexpr int kRowU = 2;
 // below gain nothing).  Where lists are that long on average, tasks only cost
 // their barrier (|e| 64 over 2,000 x 4,000: DP 179 us, 200 with tasks from 96
 // entries on), so a list also has to be twice as long as the mean, or 4 times
-// kHeavyList (Shared::heavy_list).
+// kHeavyList (Shared::heavy_list).  Parts grow with the mean too, up to 1,024:
+// with 256, the tasks of 20,000 hyperedges over 64 vertices do not all find
+// room, and eight lanes walk the rest (load and kernelization 531 us; 292 now).
 constexpr int kHeavyList = 48;
 constexpr int kTaskLen = 256;
 // The same for a vertex's bounds, whose entries are read four in flight, like
@@ -185,7 +187,8 @@ struct Shared {
     int32_t full;         // every hyperedge and vertex is a candidate
     int32_t ok;           // the last barrier
     int32_t local;        // there is room for degrees (build of a batch)
-    int32_t heavy_list;   // longer lists are walked as tasks
+    int32_t heavy_list;   // longer lists are walked as tasks,
+    int32_t task_len;     // of so many entries
     SpRound got;          // counters read right after it
     Progress g;           // the instance's rounds, as every CTA of the team knows them
     int32_t del, del2;    // deletions of this phase
@@ -817,7 +820,7 @@ __device__ __noinline__ void dp_walk(int shard, int nshards) {
     const int4 *const erec = v.erec, *const vrec = v.vrec;
     const uint32_t *const rows = v.row, *const gone = v.gone;
     const u64 *const vedge = v.vedge;
-    const int32_t heavy_list = c.sh->heavy_list;
+    const int32_t heavy_list = c.sh->heavy_list, task_len = c.sh->task_len;
     Pairs pairs(c, 0);
     for_flagged(
         c, c.sh->m0,
@@ -849,7 +852,7 @@ __device__ __noinline__ void dp_walk(int shard, int nshards) {
                 }
                 const int4 vr = x >= 0 ? vrec[x] : make_int4(0, 0, 0, 0);
                 int32_t deg = vr.z;
-                if (push_tasks(deg > heavy_list, i, x, p, deg, kTaskLen)) deg = 0;
+                if (push_tasks(deg > heavy_list, i, x, p, deg, task_len)) deg = 0;
                 const int32_t lists = min(npmax - p0, kG);
 #pragma unroll 1
                 for (int q = 0; q < lists; ++q) {
@@ -881,7 +884,7 @@ __device__ __noinline__ void dp_walk(int shard, int nshards) {
     pairs.list(1);
 }
 
-// The tasks: one warp per kTaskLen entries of a long list.
+// The tasks: one warp per task_len entries of a long list.
 __device__ __noinline__ void dp_tasks(int shard, int nshards) {
     const Ctx c;
     const View &v = c.sh->view;
@@ -894,7 +897,7 @@ __device__ __noinline__ void dp_tasks(int shard, int nshards) {
         if (tk.x == kNoTask) continue;
         const int4 vr = v.vrec[tk.y];
         const int4 r = tk.x >= 0 ? v.erec[tk.x] : make_int4(0, 0, 0, 0);
-        const int32_t part = tk.x == kBoundTask ? kBoundLen : kTaskLen;
+        const int32_t part = tk.x == kBoundTask ? kBoundLen : c.sh->task_len;
         const int32_t k0 = tk.w * part, k1 = min(k0 + part, vr.z);
         if (tk.x == kBoundTask) {
             bound_list(tk.y, k0 + c.lane, k1, 32, shard, nshards);
@@ -1525,7 +1528,9 @@ __device__ __noinline__ void start(InstState *s, int rank, int size, bool local 
         sh->rule = s->edge_rule;
         sh->rank = rank;
         sh->local = local;
-        sh->heavy_list = max(kHeavyList, min(2 * (int32_t)(s->nnz0 / max(s->n0, 1)), 4 * kHeavyList));
+        const int32_t twice = 2 * (int32_t)min(s->nnz0 / max(s->n0, 1), (int64_t)1 << 29);
+        sh->heavy_list = max(kHeavyList, min(twice, 4 * kHeavyList));
+        sh->task_len = max(kTaskLen, min(twice, 4 * kTaskLen));
         sh->size = size;
         sh->epoch = 1;
         sh->par = 0;
