@@ -184,6 +184,29 @@ def test_batch_around_the_limit_of_shared_vertices(mhs, n):
             _same(h.result(b), refs[b % 3], f"{n}: {b}")
 
 
+@pytest.mark.parametrize("size", [16, 17, 63, 64, 65, 96, 97, 700])
+def test_rows_around_the_widths_of_the_build(mhs, size):
+    """Rows of about `size` vertices of very uneven degrees, in order and not,
+    with repeats (a group's registers, a warp's, the counting sort)."""
+    import torch
+    rng = np.random.Generator(np.random.PCG64(size))
+    n, rows = 900, []
+    weight = 1.0 / np.arange(1, n + 1) ** 1.2
+    for i in range(300):
+        r = rng.choice(n, size + int(rng.integers(-1, 2)), replace=False, p=weight / weight.sum())
+        rows.append(r if i % 3 else np.concatenate([r, r[:rng.integers(0, 3)]]))
+    rows = [np.sort(r) if i % 2 else r for i, r in enumerate(rows)] + rows[:5] + [r[1:] for r in rows[:9]]
+    inst = I.from_edges(n, [sorted(set(r.tolist())) for r in rows], rng.integers(1, 5, len(rows)), k=2)
+    ptr = np.concatenate([[0], np.cumsum([len(r) for r in rows])])
+    d = [torch.from_numpy(np.ascontiguousarray(x, np.int32)).cuda()
+         for x in (ptr, np.concatenate(rows), inst.demand)]
+    ref = O.reduce(inst)
+    with mhs.Instance.load_device(inst.n, inst.m, *d, inst.k) as h:
+        h.kernelize()
+        _same(h.result(), ref)
+    _same(mhs.kernelize(inst), ref)
+
+
 @pytest.mark.parametrize("rule", ["dp", "se"])
 @pytest.mark.parametrize("deg", [31, 33, 47, 48, 49, 128, 129, 191, 193, 256, 257])
 def test_lists_around_the_lengths_of_tasks(mhs, deg, rule):
