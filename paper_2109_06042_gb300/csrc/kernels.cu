@@ -531,9 +531,9 @@ __global__ void __launch_bounds__(256) k_scatter(InstState *st, const Plan *plan
 //    builds those sectors from its hyperedges' incidences.
 //  * A clear writes the zero sector: every nonzero byte in it belongs to the
 //    row being cleared (A) or to the same all-clearing pass (A^T).
-// Warps take groups of 32 rows; the plan rounds every instance's rows up to
-// a multiple of 32, so a group lies in one instance at a 32-aligned
-// position.  A group whose incidences exceed its table sets its bytes with
+// Warps take groups of 32 rows (A, few rows: 8); the plan rounds every
+// instance's rows up to a multiple of 32, so a group lies in one instance at a
+// 32-aligned position.  A group whose incidences exceed its table sets its bytes with
 // atomics instead, for all of its sectors, so no sector is written both
 // ways.  The table also deduplicates: a vertex listed twice in a hyperedge
 // sets one bit, so sizes and degrees count it once.
@@ -541,6 +541,11 @@ __global__ void __launch_bounds__(256) k_scatter(InstState *st, const Plan *plan
 constexpr int kSecWarps = 4;          // warps per block
 constexpr int kSecTab = 512;          // table entries per warp (a power of two)
 constexpr int kSecTabLog = 9;
+// Up to this, the A set pass gives a warp 8 rows and half of its table: 24,000
+// rows are 760 warps of 32 on 152 SMs (power law 20,000 x 40,000: 35 us a pass,
+// 22 with 8; all of FP8, 1287 and 1260).  A batch fills the chip either way, and
+// empties half as many tables with 32.
+constexpr int32_t kFewRows = 65536;
 
 // One entry per sector: key << 32 | byte mask (bit b: byte b is 1.0).
 struct SecTable {
@@ -551,11 +556,12 @@ constexpr unsigned long long kSecFree = ~0ull;
 // Sets `bit` in the entry of `key`, inserting the key if absent: one shared
 // atomic in the common cases (the key present: an OR; its slot free: a
 // compare-and-swap).  False if the table is full (callers insert at most
-// kSecTab keys, so it never is).
-__device__ __forceinline__ bool sec_set(SecTable &t, uint32_t key, uint32_t bit) {
-    uint32_t h = (key * 2654435761u) >> (32 - kSecTabLog);
+// `slots` keys, a power of two, so it never is).
+__device__ __forceinline__ bool sec_set(SecTable &t, uint32_t key, uint32_t bit,
+                                        int slots = kSecTab) {
+    uint32_t h = (key * 2654435761u) >> (32 - kSecTabLog) & (uint32_t)(slots - 1);
     const unsigned long long mine = (unsigned long long)key << 32;
-    for (int p = 0; p < kSecTab; ++p) {
+    for (int p = 0; p < slots; ++p) {
         const unsigned long long cur = *reinterpret_cast<volatile unsigned long long *>(&t.e[h]);
         if (cur != kSecFree && (cur >> 32) == key) {
             atomicOr(&t.e[h], (unsigned long long)bit);
@@ -569,7 +575,7 @@ __device__ __forceinline__ bool sec_set(SecTable &t, uint32_t key, uint32_t bit)
                 return true;
             }
         }
-        h = (h + 1) & (kSecTab - 1);
+        h = (h + 1) & (uint32_t)(slots - 1);
     }
     return false;
 }
@@ -670,9 +676,9 @@ __device__ __forceinline__ void walk_live(const InstState &s, int lane, int32_t 
 // it sets.  The lanes of one pass over 32 slots set each distinct word with
 // one atomic.
 template <typename F>
-__device__ __forceinline__ void drain_table(SecTable &t, int lane, F &&fn) {
+__device__ __forceinline__ void drain_table(SecTable &t, int lane, int slots, F &&fn) {
     __syncwarp();
-    for (int base = 0; base < kSecTab; base += 32) {
+    for (int base = 0; base < slots; base += 32) {
         const int i = base + lane;
         const unsigned long long ent = t.e[i];
         uint32_t *ow = nullptr;
@@ -712,12 +718,15 @@ __global__ void __launch_bounds__(32 * kSecWarps) k_set_a_tc(InstState *st, cons
     init_table(t, lane);
     const int32_t total = plan->total_rows;
     const int32_t nw = gridDim.x * kSecWarps;
-    for (int32_t g0 = (blockIdx.x * kSecWarps + wib) * 32; g0 < total; g0 += nw * 32) {
+    // few rows: 8 to a warp, and half of its table
+    const int32_t rows = total <= kFewRows ? 8 : 32;
+    const int slots = total <= kFewRows ? kSecTab / 2 : kSecTab;
+    for (int32_t g0 = (blockIdx.x * kSecWarps + wib) * rows; g0 < total; g0 += nw * rows) {
         const int b = find_owner(plan->row_off, plan->count, g0);
         InstState &s = st[b];
         const int32_t ce0 = g0 - plan->row_off[b];
         const int32_t ce = ce0 + lane;
-        const bool row = ce < s.m;
+        const bool row = lane < rows && ce < s.m;
         int32_t e = 0, p0 = 0, len = 0;
         if (row) {
             e = __ldg(s.e_c2o + ce);
@@ -726,7 +735,7 @@ __global__ void __launch_bounds__(32 * kSecWarps) k_set_a_tc(InstState *st, cons
         }
         int32_t start;
         const int32_t tot = rows_prefix(lane, len, &start);
-        const bool table = tot <= kSecTab;
+        const bool table = tot <= slots;
         const int32_t K = s.n;
         uint8_t *const A = s.A;
         const int64_t pitch = s.A_pitch;
@@ -735,7 +744,7 @@ __global__ void __launch_bounds__(32 * kSecWarps) k_set_a_tc(InstState *st, cons
         walk_live(s, lane, p0, start, tot, 0, [&](int r, int32_t cv, int32_t) {
             if (cv >= K) { atomicOr(&s.status, kErrCapacity); return; }
             if (table) {
-                if (!sec_set(t, ((uint32_t)r << 26) | (uint32_t)(cv >> 5), 1u << (cv & 31)))
+                if (!sec_set(t, ((uint32_t)r << 26) | (uint32_t)(cv >> 5), 1u << (cv & 31), slots))
                     atomicOr(&s.status, kErrCapacity);
             } else {
                 const int32_t rr = ce0 + r;
@@ -744,7 +753,7 @@ __global__ void __launch_bounds__(32 * kSecWarps) k_set_a_tc(InstState *st, cons
             }
         });
         if (table) {
-            drain_table(t, lane, [&](uint32_t key, uint32_t m, uint32_t **ow, uint32_t *ob) {
+            drain_table(t, lane, slots, [&](uint32_t key, uint32_t m, uint32_t **ow, uint32_t *ob) {
                 const int r = (int)(key >> 26);
                 const int32_t c0 = (int32_t)(key & 0x3ffffffu) * 32;
                 const int32_t rr = ce0 + r;
@@ -845,7 +854,7 @@ __global__ void __launch_bounds__(32 * kSecWarps) k_set_md_tc(InstState *st, con
                 }
             });
             if (table) {
-                drain_table(t, lane, [&](uint32_t cv, uint32_t m, uint32_t **ow, uint32_t *ob) {
+                drain_table(t, lane, kSecTab, [&](uint32_t cv, uint32_t m, uint32_t **ow, uint32_t *ob) {
                     int32_t mf = 0;  // the largest demand among the sector's hyperedges
                     for (uint32_t bits = m; bits; bits &= bits - 1)
                         mf = max(mf, wdem[wib][__ffs(bits) - 1]);

@@ -79,3 +79,18 @@ def test_sizes_per_round_equal_the_bit_packed_form(mhs):
                     stats.append(h.reduce_round())
                 rec.append((stats, h.trace()[0].tolist()))
         assert rec[0] == rec[1]
+
+
+@pytest.mark.parametrize("count", [64, 65])
+def test_operand_groups_of_8_and_of_32_rows(mhs, count):
+    """Loads of up to and above 65,536 rows set the operand by 8 and by 32 rows
+    a warp; rows of 30 to 40 vertices overflow the warp's table in both."""
+    insts = [I.uniform_random(300, 1024, 1, 6, 3, 0, seed=1), I.uniform_random(300, 1024, 30, 40, 3, 0, seed=2),
+             I.uniform_random(290, 1024, 1, 40, 3, 0, seed=3)]
+    refs = [O.reduce(i) for i in insts]
+    with mhs.Instance.load_batch([insts[b % 3] for b in range(count)], contraction="fp8") as h:
+        h.kernelize()
+        for b in range(count):
+            got, ref = h.result(b), refs[b % 3]
+            assert got["vertices"].tolist() == ref["vertices"].tolist(), b
+            assert got["edges"].tolist() == ref["edges"].tolist() and got["rounds"] == ref["rounds"]
