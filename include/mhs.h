@@ -390,8 +390,9 @@ mhs_status mhs_last_timing(const mhs_instance *inst, float *ms4);
  * reuses the same array (the call clears what must start at zero), so calls
  * whose GPU work overlaps race and must be serialised by the caller.  Each
  * call looks up the array's address (cudaGetSymbolAddress) on the current
- * device; the first call on a device may load the library's device code and
- * should come before any stream capture.  The call runs on cuda_stream
+ * device; the first call on a device (and the first that takes the other of
+ * its two forms) may load the library's device code and should come before any
+ * stream capture.  The call runs on cuda_stream
  * (NULL: the default stream) and returns after the work is done.  Errors
  * are reported through the return value and, if err_buf is non-NULL, a
  * message in err_buf[err_cap] (mhs_last_error is not used, so that no host

@@ -24,9 +24,9 @@
 // Set-up: every call looks up the array's device address with
 // cudaGetSymbolAddress, with the caller's device current.  No address is
 // cached, so a context torn down and created again (cudaDeviceReset) cannot
-// leave a stale one behind.  The first call on a device may load the
-// library's device code into the context; make that first call before any
-// stream capture.
+// leave a stale one behind.  The first call on a device, and the first that
+// takes the other form, may load the library's device code into the context;
+// make them before any stream capture.
 //
 // Pointers: every device array the caller passes is checked with
 // cudaPointerGetAttributes (device or managed memory of the current device)
