@@ -541,10 +541,11 @@ __global__ void __launch_bounds__(256) k_scatter(InstState *st, const Plan *plan
 constexpr int kSecWarps = 4;          // warps per block
 constexpr int kSecTab = 512;          // table entries per warp (a power of two)
 constexpr int kSecTabLog = 9;
-// Up to this, the A set pass gives a warp 8 rows and half of its table: 24,000
-// rows are 760 warps of 32 on 152 SMs (power law 20,000 x 40,000: 35 us a pass,
-// 22 with 8; all of FP8, 1287 and 1260).  A batch fills the chip either way, and
-// empties half as many tables with 32.
+// Up to this, the A set pass gives a warp 8 rows and half of its table, and the
+// MD set pass gives a group's vertices to four warps: 24,000 rows are 760 warps
+// of 32 on 152 SMs (power law 20,000 x 40,000: 35 us for A, 22 with 8; MD 32 and
+// 29, later rounds 25 and 20; uniform 2,000 x 4,000, all of FP8, 390 and 363).  A
+// batch fills the chip either way, and walks and empties less with 32.
 constexpr int32_t kFewRows = 65536;
 
 // One entry per sector: key << 32 | byte mask (bit b: byte b is 1.0).
@@ -780,11 +781,11 @@ __global__ void __launch_bounds__(32 * kSecWarps) k_set_a_tc(InstState *st, cons
     }
 }
 
-// Phase 1 set, two walks per group of 32 positions [c0, c0 + 32):
+// Phase 1 set, two walks over groups of positions:
 //  (a) the rows the DP pass saw there (e_prev): zero their sectors of A (the
 //      DP pass's clear), and mark the vertices of the hyperedges DP deleted
 //      as MD candidates;
-//  (b) the hyperedges DP kept there (e_c2o after DP): sector c0 / 32 of
+//  (b) the hyperedges DP kept in [c0, c0 + 32) (e_c2o after DP): sector c0 / 32 of
 //      A^T's vertex rows, deg(v) (= I^V_jj), the maximum demand over E(v),
 //      and the occupancy bits of A^T.
 __global__ void __launch_bounds__(32 * kSecWarps) k_set_md_tc(InstState *st, const Plan *plan) {
@@ -795,7 +796,9 @@ __global__ void __launch_bounds__(32 * kSecWarps) k_set_md_tc(InstState *st, con
     init_table(t, lane);
     const int32_t total = plan->total_rows;
     const int32_t nw = gridDim.x * kSecWarps;
-    for (int32_t g0 = (blockIdx.x * kSecWarps + wib) * 32; g0 < total; g0 += nw * 32) {
+    const bool few = total <= kFewRows;
+    const int32_t rows = few ? 8 : 32;
+    for (int32_t g0 = (blockIdx.x * kSecWarps + wib) * rows; g0 < total; g0 += nw * rows) {
         const int b = find_owner(plan->row_off, plan->count, g0);
         InstState &s = st[b];
         const int32_t c0 = g0 - plan->row_off[b];
@@ -803,7 +806,7 @@ __global__ void __launch_bounds__(32 * kSecWarps) k_set_md_tc(InstState *st, con
         if (!s.skip_a) {  // (a)
             const int32_t ce = c0 + lane;
             int32_t p0 = 0, len = 0, mark = 0;
-            if (ce < s.m) {
+            if (lane < rows && ce < s.m) {
                 const int32_t e = __ldg(s.e_prev + ce);
                 p0 = __ldg(s.eptr + e);
                 len = __ldg(s.eptr + e + 1) - p0;
@@ -823,6 +826,14 @@ __global__ void __launch_bounds__(32 * kSecWarps) k_set_md_tc(InstState *st, con
                 zero_sector(A + (int64_t)(c0 + r) * pitch + (cv & ~31));
             });
         }
+    }
+    const int32_t parts = few ? 4 : 1;  // of a group's vertices, by position
+    for (int32_t u = blockIdx.x * kSecWarps + wib; u < total / 32 * parts; u += nw) {
+        const int32_t g0 = u / parts * 32, part = u % parts;
+        const int b = find_owner(plan->row_off, plan->count, g0);
+        InstState &s = st[b];
+        const int32_t c0 = g0 - plan->row_off[b];
+        const int32_t n = s.n;
         if (!s.skip_at) {  // (b)
             const int32_t cn = c0 + lane;
             int32_t p0 = 0, len = 0, fe = 0;
@@ -843,6 +854,7 @@ __global__ void __launch_bounds__(32 * kSecWarps) k_set_md_tc(InstState *st, con
             int32_t *const maxf = s.v_maxf;
             walk_live(s, lane, p0, start, tot, fe, [&](int r, int32_t cv, int32_t rfe) {
                 if (cv >= n) { atomicOr(&s.status, kErrCapacity); return; }
+                if ((cv & (parts - 1)) != part) return;
                 if (table) {
                     if (!sec_set(t, (uint32_t)cv, 1u << r)) atomicOr(&s.status, kErrCapacity);
                 } else {
