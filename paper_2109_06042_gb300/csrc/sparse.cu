@@ -90,7 +90,7 @@ constexpr int kTaskLen = 256;
 constexpr int kBoundList = 32, kBoundLen = 128;
 constexpr int kHeavyDeg = 256;         // vertices of a higher degree: whole CTAs
 constexpr int32_t kNoTask = -1, kBoundTask = -2;  // Task.x: unused; a vertex's bounds
-constexpr int32_t kGone = 0x7fffffff;  // demand of a deleted hyperedge: no test passes it
+constexpr int32_t kGone = 0;           // demand of a deleted hyperedge: no legal one (they are >= 1)
 constexpr int kSpThreads = 1024;       // threads of a CTA of a team
 constexpr int kSpBatchThreads = 512;   // threads of a CTA of a batch
 constexpr int kSpBatchBlocks = 2;      // such CTAs per SM
@@ -560,17 +560,17 @@ __device__ __noinline__ void dp_bounds_all(int shard, int nshards) {
         [&](int32_t j) {
             const int4 r = j >= 0 ? erec[j] : make_int4(0, 0, kGone, 0);
             const uint32_t *row = j >= 0 ? rows + eptr[j] : nullptr;
-            const int32_t fj = r.z;
+            const int32_t fj = r.z, len = fj == kGone ? 0 : r.w;
             bool hit = fj != kGone && global_hit(loose, empty, j, fj, r.w);
             int32_t heavy = 0;  // heavy vertices
-            const int32_t maxlen = c.full ? __reduce_max_sync(0xffffffffu, r.w) : 0;
+            const int32_t maxlen = c.full ? __reduce_max_sync(0xffffffffu, len) : 0;
 #pragma unroll 1
             for (int32_t k0 = 0; k0 < maxlen; k0 += kU * kG) {
                 uint32_t x[kU];
 #pragma unroll
                 for (int u = 0; u < kU; ++u) {
                     const int32_t k = k0 + u * kG + c.sub;
-                    x[u] = k < r.w ? row[k] : 0xffffffffu;
+                    x[u] = k < len ? row[k] : 0xffffffffu;
                 }
 #pragma unroll
                 for (int u = 0; u < kU; ++u) {
@@ -586,7 +586,7 @@ __device__ __noinline__ void dp_bounds_all(int shard, int nshards) {
             int32_t end = 0;
             if (__any_sync(0xffffffffu, heavy != 0)) {
                 heavy = group_sum(heavy);
-                end = group_ballot(c, hit) == 0 && heavy > 1 ? r.w : 0;
+                end = group_ballot(c, hit) == 0 && heavy > 1 ? len : 0;
                 end = __shfl_sync(0xffffffffu, end, c.lead);
             }
             const int32_t maxend = __reduce_max_sync(0xffffffffu, end);

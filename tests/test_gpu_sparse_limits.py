@@ -1,0 +1,73 @@
+"""Inputs at the limits of what the loads accept, by the forms that a caller
+gets without naming one (candidate lists alone, in a batch, on a server and
+without allocations) and bit-packed, against the oracle."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2109_06042_gb300 import instances as I
+
+pytestmark = pytest.mark.gpu
+
+VARIANTS = [("dp", False), ("se", False), ("dp", True), ("se", True)]
+TOP = 2**31 - 1  # the largest demand
+
+
+@pytest.fixture(scope="module")
+def mhs():
+    from paper_2109_06042_gb300 import build
+    build.build()
+    from paper_2109_06042_gb300 import mhs as M
+    return M
+
+
+def _same(got, ref, ctx=""):
+    for key in ("vertices", "edges", "demands"):
+        assert got[key].tolist() == ref[key].tolist(), (key, ctx)
+    assert got["k"] == ref["k"] and got["rounds"] == ref["rounds"], ctx
+
+
+def _dev(*arrays):
+    import torch
+    return [torch.from_numpy(np.ascontiguousarray(a, np.int32)).cuda() for a in arrays]
+
+
+def _noalloc(mhs, inst, ref, ctx=""):
+    import torch
+    av = torch.full((max(inst.n, 1),), 7, dtype=torch.uint8, device="cuda")
+    ae = torch.full((max(inst.m, 1),), 7, dtype=torch.uint8, device="cuda")
+    d = _dev(inst.edge_ptr, np.append(inst.edge_vtx, 0), inst.demand)
+    assert mhs.kernelize_noalloc(inst.n, inst.m, *d, inst.nnz, av, ae) == ref["rounds"], ctx
+    assert torch.nonzero(av[:inst.n]).flatten().tolist() == ref["vertices"].tolist(), ctx
+    assert torch.nonzero(ae[:inst.m]).flatten().tolist() == ref["edges"].tolist(), ctx
+
+
+def _every_form(mhs, insts, rule="dp", fe=False):
+    refs = [O.reduce_variant(i, rule, fe) for i in insts]
+    opts = {"rule": rule, "full_edges": fe}
+    with mhs.Instance.load_batch(insts, **opts) as h:
+        h.kernelize()
+        for b, ref in enumerate(refs):
+            _same(h.result(b), ref, f"batch {b}")
+    with mhs.Server(**opts) as srv:
+        tickets = [srv.submit(i) for i in insts]
+        for b, t in enumerate(tickets):
+            _same(srv.poll(t), refs[b], f"server {b}")
+    for b, inst in enumerate(insts):
+        _same(mhs.kernelize(inst, **opts), refs[b], f"alone {b}")
+        _same(mhs.kernelize(inst, contraction="popcount", **opts), refs[b], f"popcount {b}")
+        if rule == "dp" and not fe:
+            _noalloc(mhs, inst, refs[b], f"noalloc {b}")
+
+
+@pytest.mark.parametrize("rule,fe", VARIANTS)
+def test_the_largest_demands(mhs, rule, fe):
+    """Any demand from 1 to 2^31 - 1 is legal: none stands for a deleted hyperedge."""
+    rng = np.random.Generator(np.random.PCG64(31))
+    insts = [I.from_edges(2, [[0, 1]], [TOP]),
+             I.from_edges(5, [[0, 1], [0, 1, 2], [3, 4], [3], []], [TOP, TOP - 1, TOP, 5, TOP])]
+    for s in range(24):
+        i = I.tiny_random(s, nmax=16, mmax=16)
+        i.demand[:] = rng.choice([TOP, TOP - 1, TOP - 2, 2**30, 2**24 + 1, 1, 2, 3], i.m)
+        insts.append(i)
+    _every_form(mhs, insts, rule, fe)
