@@ -47,7 +47,7 @@ enum : int32_t {
 // holding it, and whether whole CTAs handle it.
 struct alignas(16) SpAgg {
     int32_t m1;                 // largest f_i - |e_i| + 1 over its hyperedges of |e_i| >= 2
-    int32_t heavy;              // bit 0: whole CTAs handle it; above: its pairs' largest bound
+    uint32_t heavy;             // bit 0: whole CTAs handle it; above: its pairs' largest bound
     unsigned long long s1;      // hyperedges of this vertex alone: largest f << 32 | ~index
 };
 // Bounds of a pair of vertices (a hash table, linear probing).

@@ -372,10 +372,11 @@ __device__ __forceinline__ void add_pair_bound(Shared *sh, int32_t e, int32_t f,
     }
     // (popular pairs have hundreds of writers: look before an atomic)
     const int32_t bound = len == 2 ? f : f - len + 2;
-    const int32_t most = min(bound, 0x3ffffffe) << 1;  // (bit 0: for whole CTAs)
-    const int32_t hx = vload(&agg[x].heavy), hy = vload(&agg[y].heavy);
-    if ((hx & ~1) < most) atomicMax(&agg[x].heavy, most | (hx & 1));
-    if ((hy & ~1) < most) atomicMax(&agg[y].heavy, most | (hy & 1));
+    const uint32_t most = (uint32_t)bound << 1;  // (bit 0: for whole CTAs)
+    const uint32_t hx = *reinterpret_cast<volatile uint32_t *>(&agg[x].heavy);
+    const uint32_t hy = *reinterpret_cast<volatile uint32_t *>(&agg[y].heavy);
+    if ((hx & ~1u) < most) atomicMax(&agg[x].heavy, most | (hx & 1u));
+    if ((hy & ~1u) < most) atomicMax(&agg[y].heavy, most | (hy & 1u));
     if (len == 2) {
         const u64 s2 = ((u64)(uint32_t)f << 32) | (0xffffffffu - (uint32_t)e);
         if (*reinterpret_cast<volatile u64 *>(&slot->s2) < s2) atomicMax(&slot->s2, s2);
@@ -595,12 +596,12 @@ __device__ __noinline__ void dp_bounds_all(int shard, int nshards) {
                 const uint32_t ka = a < end ? row[a] : 0;
                 bool on = ka >= kHeavyKey;
                 if (!__any_sync(0xffffffffu, on)) continue;
-                on = on && (agg[ka & kIdMask].heavy >> 1) >= fj;
+                on = on && (int32_t)(agg[ka & kIdMask].heavy >> 1) >= fj;
                 if (on)
 #pragma unroll 1
                     for (int32_t k = a + 1 + c.sub; k < end && !hit; k += kG) {
                         const uint32_t y = row[k] & kIdMask;
-                        if ((agg[y].heavy >> 1) >= fj) hit = pair_hit(c.sh, ka & kIdMask, y, j, fj, r.w);
+                        if ((int32_t)(agg[y].heavy >> 1) >= fj) hit = pair_hit(c.sh, ka & kIdMask, y, j, fj, r.w);
                     }
                 __syncwarp();
                 if (group_ballot(c, hit)) end = 0;

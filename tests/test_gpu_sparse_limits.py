@@ -71,3 +71,15 @@ def test_the_largest_demands(mhs, rule, fe):
         i.demand[:] = rng.choice([TOP, TOP - 1, TOP - 2, 2**30, 2**24 + 1, 1, 2, 3], i.m)
         insts.append(i)
     _every_form(mhs, insts, rule, fe)
+
+
+@pytest.mark.parametrize("f", [2**30 - 2, 2**30 - 1, 2**30 + 5, TOP])
+def test_large_demands_on_a_pair_of_heavy_vertices(mhs, f):
+    """The bound that a hyperedge of two vertices of high degree sets is as
+    large as its demand; supersets of that demand and below go, others stay."""
+    edges = [[0, 1]] + [[0, 1, 2 + k] for k in range(300)] + [[0, 1, 2 + k, 3 + k] for k in range(299)]
+    dem = [f] + [f] * 300 + [f - k % 7 for k in range(298)] + [TOP]
+    same = I.from_edges(302, edges, dem, k=1)
+    dem[0] = f - 3
+    _every_form(mhs, [same, I.from_edges(302, edges, dem, k=1)])
+    _every_form(mhs, [same], fe=True)
