@@ -963,8 +963,10 @@ __device__ int32_t chain_exclusive(unsigned long long *status, uint32_t epoch, i
 // Bounded by the latency of the walks' loads (eight lanes per row).  Power law
 // 20,000 x 40,000: 16 of the pass's 27 thousand deletions; the DP passes take
 // 483 us with them, 880 without (uniform 16,000 x 32,000: 2.0 and 4.3 ms).
+// The first round only: later ones, full again after an FE pass, find the
+// largest demands of the last MD pass in v_maxf, not zeros.
 __device__ __forceinline__ bool bounds_apply(const InstState &s) {
-    return s.active && !s.status && s.md_full && !s.no_skip;
+    return s.active && !s.status && s.rounds == 0 && !s.no_skip;
 }
 
 // kTest false: collect the bounds; true: flag the rows they delete.

@@ -263,7 +263,7 @@ struct mhs_instance {
     BatchCounters *hctr = nullptr;
     int32_t *hkerr = nullptr;
     int64_t max_nnz = 0, max_m = 0, max_n = 0;
-    bool started = false;        // a round was launched
+    bool started = false;        // a round, or a pass of one, was launched
     int32_t compact_blocks = 1;  // compaction blocks per instance (> 1: chained scan)
     TileChoice tiles{kTcNDefault, 16, 1, 0};  // tcgen05 tile shape of this load
     // arena offsets of the batch-wide input arrays
@@ -1879,6 +1879,7 @@ mhs_status mhs_pass_begin(mhs_instance *inst, int32_t phase) {
         CUDA_TRY(launch_phase_prologue(inst->dstate, inst->dplan, inst->dctr, phase,
                                        inst->contraction, inst->sms, inst->stream));
     inst->pass_state = phase == 0 ? 1 : 3;
+    inst->started = true;
     return MHS_OK;
 }
 

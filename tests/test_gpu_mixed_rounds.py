@@ -1,0 +1,51 @@
+"""Sharded rounds (mhs_pass_*) and mhs_kernelize on one handle, in turn."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2109_06042_gb300 import instances as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mhs():
+    from paper_2109_06042_gb300 import build
+    build.build()
+    from paper_2109_06042_gb300 import mhs as M
+    return M
+
+
+def _fixpoint(n, m):
+    """A large instance that the rules leave as it is, with full hyperedges."""
+    inst = I.uniform_random(n, m, 3, 8, 4, 5, seed=1)
+    res = O.reduce(inst)
+    new = np.full(inst.n, -1)
+    new[res["vertices"]] = np.arange(len(res["vertices"]))
+    rows = inst.edges()
+    edges = [[int(x) for x in new[rows[e]] if x >= 0] for e in res["edges"]]
+    return I.from_edges(len(res["vertices"]), edges, res["demands"], k=5)
+
+
+@pytest.mark.parametrize("contraction", ["fp8", "popcount", "auto"])
+@pytest.mark.parametrize("rounds", [1, 2])
+def test_kernelize_after_sharded_rounds(mhs, contraction, rounds):
+    """The first round deletes nothing and rule FE fires; what the passes
+    left behind (largest demands per vertex) is not taken for bounds."""
+    inst = _fixpoint(12000, 12000)
+    assert inst.m >= 8000 and any(len(e) == f for e, f in zip(inst.edges(), inst.demand))
+    ref = O.reduce_variant(inst, "dp", True)
+    with mhs.Instance.load(inst, contraction=contraction, full_edges=True) as h:
+        for r in range(rounds):
+            for phase in (0, 1):
+                h.pass_begin(phase)
+                h.pass_contract(phase, 0, 1)
+                st = h.pass_end(phase)
+            if r == 0:
+                assert st["dp_deleted"] == st["md_deleted"] == 0 and st["active"]
+        h.kernelize()
+        got = h.result()
+        for key in ("vertices", "edges", "demands"):
+            assert got[key].tolist() == ref[key].tolist(), key
+        assert got["k"] == ref["k"] and got["rounds"] == ref["rounds"]
+        assert h.forced()[0].tolist() == ref["forced"].tolist()
