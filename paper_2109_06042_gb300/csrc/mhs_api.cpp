@@ -926,6 +926,9 @@ mhs_status finish_sparse(mhs_instance *h, bool *again) {
     bool pays = true;
     mhs_status st = build_sparse(h, &found, &pays);
     if (st) return st;
+    if (found.status & kErrTimeout)
+        return fail(MHS_EDEVICE, "load: status 0x%x: %s", found.status,
+                    status_text(kErrTimeout));
     if (found.status) {
         if (h->count == 1)
             return fail(MHS_EINVAL, "malformed device instance (status 0x%x: %s)", found.status,

@@ -6,10 +6,14 @@
 // write the timeout status and return, and the CUDA context must stay
 // usable.  This exercises failure detection without faulting or hanging a
 // GPU.
+//
+// mhs_selftest_team_wait does the same for the barriers of the candidate lists'
+// kernels: every one of them waits for a CTA too many.
 #include <cuda_runtime.h>
 
 #include "bounded_wait.cuh"
 #include "host_internal.h"
+#include "kernels.h"
 #include "mhs.h"
 #include "mhs_internal.h"
 
@@ -55,5 +59,13 @@ extern "C" mhs_status mhs_selftest_bounded_wait(int64_t limit_ns, int32_t *statu
     if (e != cudaSuccess) return set_error(MHS_ECUDA, "selftest: %s", cudaGetErrorString(e));
     if (status_out) *status_out = h_status;
     if (waited_ns_out) *waited_ns_out = h_waited;
+    return MHS_OK;
+}
+
+extern "C" mhs_status mhs_selftest_team_wait(int64_t limit_ns) {
+    using namespace mhs;
+    if (limit_ns < 0 || limit_ns > 2000000000ll)
+        return set_error(MHS_EINVAL, "limit_ns must be in [0, 2e9]");
+    set_team_absent((uint64_t)limit_ns);
     return MHS_OK;
 }

@@ -97,6 +97,9 @@ constexpr int kSpBatchBlocks = 2;      // such CTAs per SM
 constexpr int64_t kSpTeamNnz = 512;    // incidences per CTA of a team
 constexpr int64_t kSpTeamItems = 256;  // hyperedges and vertices per CTA of a team
 constexpr uint64_t kTeamWaitNs = 4000000000ull;  // 4 s bound on a team barrier
+// Self-test (mhs_selftest_team_wait): this thread's launches wait so long for a
+// CTA that never comes; 0: off.
+thread_local uint64_t t_absent_ns = 0;
 
 __device__ __forceinline__ u64 sig_bit(int32_t id) {
     return 1ull << (((uint32_t)id * 2654435761u) >> 26);
@@ -182,6 +185,8 @@ struct Shared {
     int32_t rank, size;
     uint32_t *bar;        // arrivals so far, over all launches (size > 1)
     uint32_t target;      // arrivals that complete the last barrier begun
+    uint32_t absent;      // self-test: arrivals waited for in vain
+    uint64_t wait_ns;     // bound on a barrier
     int32_t epoch;        // round being executed, from 1
     int32_t par;          // counter parity
     int32_t full;         // every hyperedge and vertex is a candidate
@@ -225,8 +230,8 @@ __device__ __forceinline__ WarpShared *warp_shared() {
 
 // Barrier over the team; false if it timed out.  The CTAs are resident
 // together (cooperative launch), and each wait gives up after kTeamWaitNs,
-// after which every CTA of the team leaves.  p: counters that are complete
-// once every CTA has arrived, read into `got`.
+// after which every CTA of the team leaves and the kernel tells the host.  p:
+// counters that are complete once every CTA has arrived, read into `got`.
 __device__ __noinline__ bool team_sync(const SpRound *p = nullptr) {
     Shared *sh = shared();
     __syncthreads();
@@ -241,11 +246,11 @@ __device__ __noinline__ bool team_sync(const SpRound *p = nullptr) {
             for (uint32_t it = 1;; ++it) {
                 uint32_t now;
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(bar) : "memory");
-                if ((int32_t)(now - target) >= 0) break;
+                if ((int32_t)(now - target - sh->absent) >= 0) break;
                 if ((it & 255u) == 0) {
                     const uint64_t t = globaltimer();
                     if (t0 == 0) t0 = t;
-                    else if (t - t0 > kTeamWaitNs) {
+                    else if (t - t0 > sh->wait_ns) {
                         atomicOr(&sh->s->status, kErrTimeout);
                         good = 0;
                         break;
@@ -1533,7 +1538,8 @@ __device__ __forceinline__ void flush(int32_t *sh_ctr, int32_t *to) {
 }
 
 // Shared memory for one instance.
-__device__ __noinline__ void start(InstState *s, int rank, int size, bool local = false) {
+__device__ __noinline__ void start(InstState *s, int rank, int size, uint64_t absent_ns,
+                                   bool local = false) {
     Shared *sh = shared();
     if (threadIdx.x == 0) {
         sh->view = View(*s);
@@ -1552,6 +1558,8 @@ __device__ __noinline__ void start(InstState *s, int rank, int size, bool local 
         sh->heavy_list = max(kHeavyList, min(twice, 4 * kHeavyList));
         sh->task_len = max(kTaskLen, min(twice, 4 * kTaskLen));
         sh->size = size;
+        sh->absent = absent_ns != 0;
+        sh->wait_ns = absent_ns ? absent_ns : kTeamWaitNs;
         sh->epoch = 1;
         sh->par = 0;
         sh->full = 1;
@@ -1568,8 +1576,8 @@ __device__ __noinline__ void start(InstState *s, int rank, int size, bool local 
     __syncthreads();
 }
 
-// Structural checks, rows and lists of one instance.
-__device__ __noinline__ void build_instance(int32_t max_rounds, SpTotals *out) {
+// Structural checks, rows and lists of one instance.  False if a barrier timed out.
+__device__ __noinline__ bool build_instance(int32_t max_rounds, SpTotals *out) {
     const Ctx c;
     InstState &s = *c.sh->s;
     const View v = c.sh->view;
@@ -1607,10 +1615,10 @@ __device__ __noinline__ void build_instance(int32_t max_rounds, SpTotals *out) {
         c, m0, [](int32_t) { return true; },
         [&](int32_t e) { bad |= count_row(c, v, evtx, f, place, local, n0, nnz0, e); });
     if (bad) atomicOr(&s.status, bad);
-    if (!team_sync()) return;
+    if (!team_sync()) return false;
     if (const int32_t st = vload(&s.status)) {
         if (t0 == 0) atomicOr(&out->status, st);
-        return;
+        return true;
     }
     // a place for every vertex's list (in any order): one atomic per warp
     int32_t *const heavy = s.sp_heavy;
@@ -1636,7 +1644,7 @@ __device__ __noinline__ void build_instance(int32_t max_rounds, SpTotals *out) {
             heavy[atomicAdd(&v.ctl->n_heavy, 1)] = x;
         }
     }
-    if (!team_sync()) return;
+    if (!team_sync()) return false;
     const int32_t rule = s.edge_rule;
     u64 cost = 0;  // the entries that walking this lane's hyperedges may visit
     for_flagged(
@@ -1688,6 +1696,7 @@ __device__ __noinline__ void build_instance(int32_t max_rounds, SpTotals *out) {
     if (c.lane == 0 && cost) atomicAdd(&c.sh->cost, cost);
     __syncthreads();
     if (threadIdx.x == 0 && c.sh->cost) atomicAdd(&out->cost, c.sh->cost);
+    return true;
 }
 
 // Thread 0 of every CTA: the state at the start of a launch.
@@ -1779,12 +1788,12 @@ __device__ __noinline__ bool finish_round(int32_t dp, int32_t md) {
 }
 
 // Rounds of Algorithm 3 (and FE at its fixpoints) until the fixpoint or
-// `limit` rounds (0: no limit).
-__device__ __noinline__ void run_instance(int32_t limit, BatchCounters *ctr, SpTimes *times) {
+// `limit` rounds (0: no limit).  False if a barrier timed out.
+__device__ __noinline__ bool run_instance(int32_t limit, BatchCounters *ctr, SpTimes *times) {
     Shared *sh = shared();
     if (threadIdx.x == 0) load_progress(sh->g, *sh->s);
     // one CTA must not publish the final state before all have read this one
-    if (!team_sync()) return;
+    if (!team_sync()) return false;
     for (int32_t done = 0; sh->g.active && (limit <= 0 || done < limit); ++done) {
         begin_round();
         SpRound *rc = &sh->view.ctl->c[sh->par], *nx = &sh->view.ctl->c[sh->par ^ 1];
@@ -1793,35 +1802,35 @@ __device__ __noinline__ void run_instance(int32_t limit, BatchCounters *ctr, SpT
         if (sh->full || sh->g.md > 0) {
             if (sh->epoch > 1) {  // (the first round's rows are the load's)
                 dp_rows();
-                if (!team_sync()) return;
+                if (!team_sync()) return false;
                 if (sh->full) {  // FE lowered demands, which the lists repeat
                     md_lists();
-                    if (!team_sync()) return;
+                    if (!team_sync()) return false;
                 }
             }
             if (lead) sh->g.t_dp -= globaltimer();
             dp_bounds(0, 1);
             // full rounds: the walks skip what the bounds deleted (a matter of
             // time only: 40 M list entries become 14 M on the power-law instance)
-            if (sh->full && !team_sync()) return;
+            if (sh->full && !team_sync()) return false;
             dp_walk(0, 1);
             flush(&sh->del, &rc->dp);
-            if (!team_sync(rc)) return;
+            if (!team_sync(rc)) return false;
             // (each list has a counter that is final at the barrier before it is
             // read: the CTAs must agree on the barriers that follow)
             if (sh->got.npair[0] > 0) {
                 decide_pairs(0);
                 flush(&sh->del, &rc->dp);
-                if (!team_sync(rc)) return;
+                if (!team_sync(rc)) return false;
             }
             if (sh->got.ntask > 0) {  // (after the pairs: a hyperedge found deleted needs no walk)
                 dp_tasks(0, 1);
                 flush(&sh->del, &rc->dp);
-                if (!team_sync(rc)) return;
+                if (!team_sync(rc)) return false;
                 if (sh->got.npair[1] > 0) {
                     decide_pairs(1);
                     flush(&sh->del, &rc->dp);
-                    if (!team_sync(rc)) return;
+                    if (!team_sync(rc)) return false;
                 }
             }
             if (lead) sh->g.t_dp += globaltimer();
@@ -1830,11 +1839,11 @@ __device__ __noinline__ void run_instance(int32_t limit, BatchCounters *ctr, SpT
             if (lead) *nx = SpRound{};
             if (sh->full || dp > 0) {
                 md_lists();
-                if (!team_sync()) return;
+                if (!team_sync()) return false;
                 if (lead) sh->g.t_md -= globaltimer();
                 md_test(false, 0, 1);
                 flush(&sh->del2, &rc->md);
-                if (!team_sync(rc)) return;
+                if (!team_sync(rc)) return false;
                 if (lead) sh->g.t_md += globaltimer();
                 md = sh->got.md;
             }
@@ -1843,7 +1852,7 @@ __device__ __noinline__ void run_instance(int32_t limit, BatchCounters *ctr, SpT
             // round's md is 0, so resetting its counters loses nothing.)
             *nx = SpRound{};
         }
-        if (!finish_round(dp, md)) return;
+        if (!finish_round(dp, md)) return false;
     }
     if (sh->rank == 0 && threadIdx.x == 0) {
         const Progress &g = sh->g;
@@ -1852,20 +1861,21 @@ __device__ __noinline__ void run_instance(int32_t limit, BatchCounters *ctr, SpT
         atomicAdd(&times->md, (u64)g.t_md);
         atomicAdd(&times->all, (u64)(globaltimer() - g.t_all));
     }
+    return true;
 }
 
-// One part of a sharded round (mhs_pass_*).
-__device__ void run_pass(int op, int shard, int nshards, BatchCounters *ctr, void *buf) {
+// One part of a sharded round (mhs_pass_*).  False if a barrier timed out.
+__device__ bool run_pass(int op, int shard, int nshards, BatchCounters *ctr, void *buf) {
     Shared *sh = shared();
     InstState &s = *sh->s;
     if (threadIdx.x == 0) load_progress(sh->g, s);
-    if (!team_sync()) return;
+    if (!team_sync()) return false;
     begin_round();
     const bool lead = sh->rank == 0 && threadIdx.x == 0;
     const int32_t t0 = sh->rank * blockDim.x + threadIdx.x, ts = sh->size * blockDim.x;
     if (!sh->g.active && op != kSpExport0 && op != kSpExport1) {
         if (lead && op == kSpEnd1) store_progress(sh->g, s, ctr);
-        return;
+        return true;
     }
     const Ctx c;
     const View v = sh->view;
@@ -1876,20 +1886,20 @@ __device__ void run_pass(int op, int shard, int nshards, BatchCounters *ctr, voi
             if (c.epoch > 1) {
                 dp_rows();
                 if (c.full) {  // FE lowered demands, which the lists repeat
-                    if (!team_sync()) return;
+                    if (!team_sync()) return false;
                     md_lists();
                 }
             }
             break;
         case kSpContract0:
             if (lead) rc->ntask = rc->npair[0] = rc->npair[1] = 0;
-            if (!team_sync()) return;
+            if (!team_sync()) return false;
             dp_bounds(shard, nshards);
-            if (!team_sync()) return;
+            if (!team_sync()) return false;
             dp_walk(shard, nshards);
-            if (!team_sync(rc)) return;
+            if (!team_sync(rc)) return false;
             dp_tasks(shard, nshards);
-            if (!team_sync(rc)) return;
+            if (!team_sync(rc)) return false;
             decide_pairs(0);
             decide_pairs(1);
             flush(&sh->del, &rc->dp);
@@ -1925,15 +1935,16 @@ __device__ void run_pass(int op, int shard, int nshards, BatchCounters *ctr, voi
         case kSpEnd1: {
             md_decide();
             flush(&sh->del2, &rc->md);
-            if (!team_sync(rc)) return;
+            if (!team_sync(rc)) return false;
             const int32_t dp = sh->got.dp, md = sh->got.md;
-            if (!finish_round(dp, md)) return;
+            if (!finish_round(dp, md)) return false;
             if (lead) store_progress(sh->g, s, ctr);
             break;
         }
         default:
             break;
     }
+    return true;
 }
 
 // Team of CTAs per instance (team > 0, all CTAs resident: a cooperative
@@ -1957,22 +1968,24 @@ __device__ __noinline__ void report(SpQueue *q, int32_t *from, volatile int32_t 
 template <int kThreads, int kMinBlocks>
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
     k_sparse_build(InstState *st, int count, int team, int32_t max_rounds, SpQueue *queue,
-                   SpTotals *out, SpTotals *host) {
+                   SpTotals *out, SpTotals *host, uint64_t absent_ns) {
     Shared *sh = shared();
+    bool ok = true;
     if (team > 0) {
-        start(st + blockIdx.x / team, blockIdx.x % team, team);
-        build_instance(max_rounds, out);
+        start(st + blockIdx.x / team, blockIdx.x % team, team, absent_ns);
+        ok = build_instance(max_rounds, out);
     } else {
         for (;;) {
             __syncthreads();
             if (threadIdx.x == 0) sh->next = atomicAdd(&queue->next, 1);
             __syncthreads();
             if (sh->next >= count) break;
-            start(st + sh->next, 0, 1, true);
+            start(st + sh->next, 0, 1, 0, true);
             build_instance(max_rounds, out);
         }
     }
     __syncthreads();
+    if (threadIdx.x == 0 && !ok) atomicOr(&out->status, kErrTimeout);
     if (threadIdx.x == 0)
         report(queue, reinterpret_cast<int32_t *>(out), reinterpret_cast<int32_t *>(host),
                sizeof(SpTotals) / 4);
@@ -1981,13 +1994,15 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
 template <int kThreads, int kMinBlocks>
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
     k_sparse_rounds(InstState *st, int count, int team, int32_t limit, BatchCounters *ctr,
-                    SpQueue *queue, SpTimes *times, BatchCounters *host, SpMasks masks) {
+                    SpQueue *queue, SpTimes *times, BatchCounters *host, SpMasks masks,
+                    uint64_t absent_ns) {
     Shared *sh = shared();
+    bool ok = true;
     if (masks.built && (masks.built->status || masks.built->cost > masks.max_cost)) return;
     if (team > 0) {
-        start(st + blockIdx.x / team, blockIdx.x % team, team);
-        run_instance(limit, ctr, times);
-        if (masks.built) {  // (every CTA is past the last round's barrier)
+        start(st + blockIdx.x / team, blockIdx.x % team, team, absent_ns);
+        ok = run_instance(limit, ctr, times);
+        if (masks.built && ok) {  // (every CTA is past the last round's barrier)
             const int32_t t0 = sh->rank * blockDim.x + threadIdx.x, ts = sh->size * blockDim.x;
 #pragma unroll 1
             for (int32_t x = t0; x < sh->n0; x += ts) masks.v[x] = sh->view.v_o2c[x] >= 0;
@@ -2000,11 +2015,13 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
             if (threadIdx.x == 0) sh->next = atomicAdd(&queue->next, 1);
             __syncthreads();
             if (sh->next >= count) break;
-            start(st + sh->next, 0, 1);
+            start(st + sh->next, 0, 1, 0);
             run_instance(limit, ctr, times);
         }
     }
     __syncthreads();
+    // (a CTA that gave up has not stored the state, and no other may)
+    if (threadIdx.x == 0 && !ok) atomicOr(&ctr->status_any, kErrTimeout);
     if (threadIdx.x == 0)
         report(queue, reinterpret_cast<int32_t *>(ctr), reinterpret_cast<int32_t *>(host),
                sizeof(BatchCounters) / 4);
@@ -2012,9 +2029,11 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
 
 __global__ void __launch_bounds__(kSpThreads, 1)
     k_sparse_pass(InstState *st, int team, int op, int shard, int nshards, BatchCounters *ctr,
-                  void *buf) {
-    start(st, blockIdx.x, team);
-    run_pass(op, shard, nshards, ctr, buf);
+                  void *buf, uint64_t absent_ns) {
+    start(st, blockIdx.x, team, absent_ns);
+    // (a pass that ends early leaves its status for the round's last)
+    if (!run_pass(op, shard, nshards, ctr, buf) && ctr && threadIdx.x == 0)
+        atomicOr(&ctr->status_any, kErrTimeout);
 }
 
 }  // namespace
@@ -2051,11 +2070,11 @@ cudaError_t launch_sparse_build(InstState *st, int count, int team, int32_t max_
                                 cudaStream_t s) {
     if (team > 0)
         return launch_team(k_sparse_build<kSpThreads, 1>, count * team, s, st, count, team,
-                           max_rounds, queue, out, host);
+                           max_rounds, queue, out, host, t_absent_ns);
     const size_t smem = shared_bytes(kSpBatchThreads) + 8 * kLocalVertices;
     k_sparse_build<kSpBatchThreads, kSpBatchBlocks>
         <<<std::min(count, sms * kSpBatchBlocks), kSpBatchThreads, smem, s>>>(
-            st, count, 0, max_rounds, queue, out, host);
+            st, count, 0, max_rounds, queue, out, host, 0);
     return cudaGetLastError();
 }
 
@@ -2065,16 +2084,18 @@ cudaError_t launch_sparse_rounds(InstState *st, int count, int team, int32_t lim
                                  cudaStream_t s) {
     if (team > 0)
         return launch_team(k_sparse_rounds<kSpThreads, 1>, count * team, s, st, count, team, limit,
-                           ctr, queue, times, host, masks);
+                           ctr, queue, times, host, masks, t_absent_ns);
     k_sparse_rounds<kSpBatchThreads, kSpBatchBlocks>
         <<<std::min(count, sms * kSpBatchBlocks), kSpBatchThreads, shared_bytes(kSpBatchThreads), s>>>(
-            st, count, 0, limit, ctr, queue, times, host, masks);
+            st, count, 0, limit, ctr, queue, times, host, masks, 0);
     return cudaGetLastError();
 }
 
 cudaError_t launch_sparse_pass(InstState *st, int team, int op, int shard, int nshards,
                                BatchCounters *ctr, void *buf, cudaStream_t s) {
-    return launch_team(k_sparse_pass, team, s, st, team, op, shard, nshards, ctr, buf);
+    return launch_team(k_sparse_pass, team, s, st, team, op, shard, nshards, ctr, buf, t_absent_ns);
 }
+
+void set_team_absent(uint64_t ns) { t_absent_ns = ns; }
 
 }  // namespace mhs

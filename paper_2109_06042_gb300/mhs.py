@@ -124,6 +124,7 @@ _SIGS = {
     "mhs_server_get_stats": (_i32, [_vp, ctypes.POINTER(ServerStats)]),
     "mhs_server_destroy": (None, [_vp]),
     "mhs_selftest_bounded_wait": (_i32, [_i64, _P32, _P64]),
+    "mhs_selftest_team_wait": (_i32, [_i64]),
     "mhs_free": (None, [_vp]),
     "mhs_last_error": (ctypes.c_char_p, []),
     "mhs_version": (ctypes.c_char_p, []),
@@ -608,6 +609,12 @@ def selftest_bounded_wait(limit_ns=20_000_000):
     w = ctypes.c_int64()
     _check(lib().mhs_selftest_bounded_wait(int(limit_ns), ctypes.byref(st), ctypes.byref(w)))
     return int(st.value), int(w.value)
+
+
+def selftest_team_wait(limit_ns):
+    """This thread's candidate-list kernels wait limit_ns for a CTA that never
+    comes (calls fail with EDEVICE); 0: off."""
+    _check(lib().mhs_selftest_team_wait(int(limit_ns)))
 
 
 def version() -> str:

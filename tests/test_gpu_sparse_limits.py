@@ -83,3 +83,51 @@ def test_large_demands_on_a_pair_of_heavy_vertices(mhs, f):
     dem[0] = f - 3
     _every_form(mhs, [same, I.from_edges(302, edges, dem, k=1)])
     _every_form(mhs, [same], fe=True)
+
+
+def test_a_barrier_that_times_out_is_an_error(mhs):
+    """Every kernel of the candidate lists whose CTAs wait for one that never
+    comes gives up and the call says so; the next call is right again."""
+    import torch
+    inst = I.uniform_random(2000, 4000, 2, 8, 3, 5, seed=9)
+    ref = O.reduce(inst)
+    d = _dev(inst.edge_ptr, inst.edge_vtx, inst.demand)
+
+    def fails(call):
+        mhs.selftest_team_wait(1_000_000)
+        try:
+            with pytest.raises(mhs.MhsError) as ei:
+                call()
+        finally:
+            mhs.selftest_team_wait(0)
+        assert ei.value.status == mhs.MHS_EDEVICE
+
+    fails(lambda: mhs.Instance.load(inst))
+    fails(lambda: mhs.Instance.load_device(inst.n, inst.m, *d, inst.k))
+    fails(lambda: mhs.Instance.load_batch([inst, inst]))
+    av, ae = (torch.zeros(x, dtype=torch.uint8, device="cuda") for x in (inst.n, inst.m))
+    fails(lambda: mhs.kernelize_noalloc(inst.n, inst.m, *d, inst.nnz, av, ae))
+    for insts in ([inst], [inst, inst]):
+        for step in ("kernelize", "reduce_round"):
+            with mhs.Instance.load_batch(insts) as h:
+                fails(getattr(h, step))
+                with pytest.raises(mhs.MhsError):
+                    h.result()
+    for late in ("contract", "end"):
+        with mhs.Instance.load(inst) as h:
+            h.pass_begin(0)
+            if late == "contract":
+                mhs.selftest_team_wait(1_000_000)
+            h.pass_contract(0, 0, 1)
+            mhs.selftest_team_wait(0)
+            h.pass_end(0)
+            h.pass_begin(1)
+            h.pass_contract(1, 0, 1)
+            if late == "end":
+                fails(lambda: h.pass_end(1))
+            else:
+                with pytest.raises(mhs.MhsError) as ei:
+                    h.pass_end(1)
+                assert ei.value.status == mhs.MHS_EDEVICE
+    _same(mhs.kernelize(inst), ref)
+    _noalloc(mhs, inst, ref)
