@@ -558,7 +558,7 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
             L.vaux = ar.take(16 * n0);
             L.task_cap = (int32_t)std::min<int64_t>(count == 1 ? 16384 + 4 * m0 : 64 + m0 / 8, 1 << 20);
             L.task = ar.take(16 * (int64_t)L.task_cap);
-            L.pair_cap = (int32_t)std::min<int64_t>(count == 1 ? 65536 + 64 * m0 : 256 + 2 * m0, 1 << 22);
+            L.pair_cap = (int32_t)std::min<int64_t>(count == 1 ? 65536 + 64 * m0 : 256 + 2 * m0, kMaxListed);
             L.pairs = ar.take(8 * (int64_t)L.pair_cap);
             L.heavy = ar.take(4 * sp_heavy_cap(z));
             continue;

@@ -57,6 +57,8 @@ struct alignas(32) SpPair {
     int32_t m2;                 // largest f_i - |e_i| + 2 over its hyperedges of |e_i| >= 3
     int32_t pad[3];
 };
+// Places of an instance's list of tasks, or of pairs, at most.
+constexpr int64_t kMaxListed = 1 << 22;
 // Vertices of more than 256 hyperedges (sparse.cu's limit for a group of lanes).
 inline int64_t sp_heavy_cap(int64_t nnz) { return nnz / 257 + 1; }
 

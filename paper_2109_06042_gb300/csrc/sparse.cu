@@ -92,6 +92,7 @@ constexpr int kHeavyDeg = 256;         // vertices of a higher degree: whole CTA
 constexpr int32_t kNoTask = -1, kBoundTask = -2;  // Task.x: unused; a vertex's bounds
 constexpr int32_t kGone = 0;           // demand of a deleted hyperedge: no legal one (they are >= 1)
 constexpr int kSpThreads = 1024;       // threads of a CTA of a team
+constexpr int kMaxTeam = 256;          // CTAs of a team, at most
 constexpr int kSpBatchThreads = 512;   // threads of a CTA of a batch
 constexpr int kSpBatchBlocks = 2;      // such CTAs per SM
 constexpr int64_t kSpTeamNnz = 512;    // incidences per CTA of a team
@@ -498,6 +499,15 @@ __device__ __forceinline__ int4 load_agg(const SpAgg *p) {
     return *reinterpret_cast<const int4 *>(p);
 }
 
+// The counters of the task and pair lists must not wrap, however much finds no
+// room: a reservation wholly behind the end is given back, so that beside the
+// one that crossed it at most one per warp of the team is counted at a time.
+// (Looking at the counter before each addition costs a chain of two L2
+// latencies: power law 396 -> 410 us, with SE and FE 1,134 -> 1,217.)
+constexpr int32_t kMaxReserve = 1 << 17;  // places a warp reserves at once, at most
+static_assert((int64_t)kMaxTeam * (kSpThreads / 32) * kMaxReserve + kMaxListed < (1ll << 31),
+              "the lists' counters cannot wrap");
+
 // Reserve tasks for the list of vertex x, in the lanes with want set (the
 // whole warp, one atomic); false if there is no room (the caller walks the
 // list itself).
@@ -514,13 +524,21 @@ __device__ __noinline__ bool push_tasks(bool want, int32_t i, int32_t x, int32_t
         const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += y;
     }
+    // (the lanes before the first that does not fit are a prefix; 65,536 parts, the
+    // most of one lane, fit)
+    const int32_t total = __reduce_max_sync(0xffffffffu, inc <= kMaxReserve ? inc : 0);
+    int32_t *const ntask = &sh->view.ctl->c[sh->par].ntask;
     int32_t at = 0;
-    if (lane == 31) at = atomicAdd(&sh->view.ctl->c[sh->par].ntask, inc);
+    if (lane == 31) {
+        at = atomicAdd(ntask, total);
+        if (at >= cap) atomicSub(ntask, total);
+    }
     at = __shfl_sync(0xffffffffu, at, 31) + inc - parts;
-    const bool fits = at >= 0 && at <= cap - parts;
+    if (inc > kMaxReserve) return false;
+    const bool fits = at <= cap - parts;
 #pragma unroll 1
     for (int32_t q = 0; q < parts; ++q)
-        if (at >= 0 && at + q < cap)
+        if (at + q < cap)
             sh->task[at + q] = fits ? make_int4(i, x, p, q) : make_int4(kNoTask, 0, 0, 0);
     return want && fits;
 }
@@ -740,8 +758,12 @@ __device__ __noinline__ void list_pairs(int32_t which, int32_t base, int32_t n) 
     Shared *sh = c.sh;
     const int2 *buf = warp_shared()->buf;
     __syncwarp();
+    int32_t *const npair = &sh->view.ctl->c[c.par].npair[which];
     int32_t at = 0;
-    if (c.lane == 0) at = atomicAdd(&sh->view.ctl->c[c.par].npair[which], n);
+    if (c.lane == 0) {
+        at = atomicAdd(npair, n);
+        if (at >= sh->pair_cap - base) atomicSub(npair, n);
+    }
     const int64_t to = (int64_t)base + __shfl_sync(0xffffffffu, at, 0);
 #pragma unroll 1
     for (int32_t k = c.lane; k < n; k += 32)
@@ -2045,7 +2067,7 @@ int sparse_team(int count, int64_t nnz, int64_t items, int sms) {
     // vertex, and a few incidences, per group of lanes
     const int64_t want = std::max<int64_t>((nnz + kSpTeamNnz - 1) / kSpTeamNnz,
                                            (items + kSpTeamItems - 1) / kSpTeamItems);
-    const int64_t cap = sms / std::max(count, 1);
+    const int64_t cap = std::min(sms, kMaxTeam) / std::max(count, 1);
     if (count > 1 && cap < 2) return 0;  // a batch: one CTA each, from a queue
     return (int)std::max<int64_t>(1, std::min(want, cap));
 }

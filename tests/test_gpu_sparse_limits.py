@@ -131,3 +131,23 @@ def test_a_barrier_that_times_out_is_an_error(mhs):
                 assert ei.value.status == mhs.MHS_EDEVICE
     _same(mhs.kernelize(inst), ref)
     _noalloc(mhs, inst, ref)
+
+
+@pytest.mark.parametrize("rule", ["dp", "se"])
+def test_full_lists_of_tasks_and_pairs(mhs, rule):
+    """Many more long lists and open pairs than an instance of a batch has room
+    for: what finds none is walked and decided in place."""
+    rng = np.random.Generator(np.random.PCG64(17))
+    insts = []
+    for m, n, size in [(700, 14, 7), (400, 24, 20), (300, 70, 60), (500, 20, 10)]:
+        edges = [np.sort(rng.choice(n, size + int(rng.integers(0, 2)), replace=False)) for _ in range(m)]
+        insts.append(I.from_edges(n, edges, rng.integers(1, 6, m), k=3))
+    refs = [O.reduce_variant(i, rule, False) for i in insts]
+    for times in (20, 3):  # a CTA for each, teams of CTAs
+        with mhs.Instance.load_batch(insts * times, rule=rule) as h:
+            h.kernelize()
+            assert h.work_stats() == (0, 0)  # by candidate lists
+            for b in range(0, len(insts) * times, 7):
+                _same(h.result(b), refs[b % len(insts)], b)
+    for inst, ref in zip(insts, refs):
+        _same(mhs.kernelize(inst, rule=rule), ref)
