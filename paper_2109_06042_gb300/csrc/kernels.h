@@ -118,11 +118,12 @@ cudaError_t launch_alive_masks_batch(const InstState *st, int count, uint8_t *al
 
 // ---- candidate lists instead of a contraction (sparse.cu) ----
 // What a load reads back: the list entries the first round's walks may visit
-// (summed over a batch) and the OR of the status words.
+// (summed over a batch), the OR of the status words, and whether some instance
+// has a row that is not for this path (nothing is built then).
 struct SpTotals {
     unsigned long long cost;
     int32_t status;
-    int32_t pad;
+    int32_t leave;
 };
 // Time spent in the DP and MD tests and in all, summed over the instances (ns).
 struct SpTimes {
@@ -136,8 +137,8 @@ struct SpQueue {
     int32_t next, done;
 };
 // A single instance whose rounds are launched before the host has seen what the
-// build found (built set): they run if it found no error and a cost of at most
-// max_cost, and leave the alive masks of the input ids.
+// build found (built set): they run if it found no error, all rows for this path and
+// a cost of at most max_cost, and leave the alive masks of the input ids.
 struct SpMasks {
     const SpTotals *built;
     unsigned long long max_cost;

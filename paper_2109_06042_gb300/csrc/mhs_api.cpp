@@ -904,7 +904,7 @@ mhs_status build_sparse(mhs_instance *h, SpTotals *found, bool *pays) {
     double pairs = 0;
     for (const HostInst &i : h->hinst)
         pairs += (double)i.m0 * i.m0 + (double)i.n0 * i.n0;
-    *pays = sparse_pays((double)host->cost, pairs);
+    *pays = !host->leave && sparse_pays((double)host->cost, pairs);
     return MHS_OK;
 }
 

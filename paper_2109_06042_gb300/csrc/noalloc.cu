@@ -276,7 +276,7 @@ extern "C" mhs_status mhs_kernelize_noalloc(int32_t n, int32_t m, const int32_t 
         return err(err_buf, err_cap, MHS_EDEVICE, "kernel reported an error status");
     if (found.totals.status)
         return err(err_buf, err_cap, MHS_EINVAL, "malformed instance (bad edge_ptr or vertex id)");
-    if (lists && found.totals.cost <= kNoAllocCost) {
+    if (lists && !found.totals.leave && found.totals.cost <= kNoAllocCost) {
         if (ctr.status_any || ctr.active)
             return err(err_buf, err_cap, MHS_EDEVICE, "kernel reported an error status");
         if (rounds_out) *rounds_out = ctr.max_rounds_seen;

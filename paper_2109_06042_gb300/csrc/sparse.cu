@@ -1335,13 +1335,117 @@ __device__ __noinline__ void fe_apply() {
 
 // ------------------------------------------------------------------ build --
 
+// 256 counters of a warp become the first places of their classes.
+__device__ __forceinline__ void first_places(int32_t *at, int lane) {
+    constexpr int kPer = 256 / 32;
+    int32_t sum = 0;
+#pragma unroll 1
+    for (int c = 0; c < kPer; ++c) sum += at[lane * kPer + c];
+    int32_t inc = sum;
+#pragma unroll 1
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    int32_t first = inc - sum;
+    __syncwarp();
+#pragma unroll 1
+    for (int c = 0; c < kPer; ++c) {
+        const int32_t n = at[lane * kPer + c];
+        at[lane * kPer + c] = first;
+        first += n;
+    }
+    __syncwarp();
+}
+
+// Rows that are not strictly ascending: up to kRankRow ids their eight lanes rank
+// each id by counting, up to kSortRow the warp sorts them by bytes of the id, and
+// with a longer one the load leaves this path (kLeave), as for one that does not
+// pay.  One such row among 20,000 of 10 ids over 40,000 vertices, load and
+// kernelization (us), all by counting / so / by the contraction:
+//   2,000 ids  21,035 / 640 / 21,237     32,768 ids  (not run) / 3,944 / 21,472
+// 10,000 ids among 300 rows over 10,000 vertices: 1,196 / 1,225 by the contraction.
+constexpr int32_t kRankRow = 64;
+constexpr int32_t kSortRow = 65536;
+constexpr int32_t kLeave = 1 << 30;  // (beside the kErr* bits)
+constexpr int32_t kInOrder = -1;
+
+// A row of more than kRankRow ids, by the warp: kInOrder if `in` ascends, else
+// its ids in order, without repeats, into row, and their number (ids outside
+// [0, n0) may come out anywhere; one of each remains).  Too long for that:
+// kLeave, and kErrBadVertex if it has such an id.
+__device__ __noinline__ int32_t long_row(const int32_t *in, int32_t *tmp, int32_t *row, int32_t len,
+                                         int32_t n0) {
+    const int lane = threadIdx.x & 31;
+    int32_t back = 0, out = 0;  // entries not below their right neighbour; outside
+#pragma unroll 4
+    for (int32_t k = lane; k < len; k += 32) {
+        const int32_t x = in[k];
+        back |= k + 1 < len && x >= in[k + 1 < len ? k + 1 : k];
+        out |= x < 0 || x >= n0;
+    }
+    if (!__any_sync(0xffffffffu, back)) return kInOrder;
+    if (len > kSortRow) return kLeave | (__any_sync(0xffffffffu, out) ? kErrBadVertex : 0);
+    int32_t *const at = reinterpret_cast<int32_t *>(warp_shared()->buf);
+    constexpr int kAhead = 4;  // loads in flight
+    const int passes = n0 <= 1 << 8 ? 1 : n0 <= 1 << 16 ? 2 : 3;
+    const int32_t *from = in;
+    int32_t *to = passes == 2 ? tmp : row;
+#pragma unroll 1
+    for (int p = 0; p < passes; ++p) {
+        const int shift = 8 * p;
+        for (int c = lane; c < 256; c += 32) at[c] = 0;
+        __syncwarp();
+#pragma unroll 4
+        for (int32_t k = lane; k < len; k += 32) atomicAdd(&at[((uint32_t)from[k] >> shift) & 255u], 1);
+        __syncwarp();
+        first_places(at, lane);
+#pragma unroll 1
+        for (int32_t k0 = 0; k0 < len; k0 += kAhead * 32) {
+            int32_t x[kAhead];
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                const int32_t k = k0 + u * 32 + lane;
+                x[u] = k < len ? from[k] : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                const bool on = k0 + u * 32 + lane < len;
+                const uint32_t digit = on ? ((uint32_t)x[u] >> shift) & 255u : 256u;
+                const unsigned peers = __match_any_sync(0xffffffffu, digit);
+                const int32_t q = on ? at[digit] + __popc(peers & ((1u << lane) - 1u)) : 0;
+                __syncwarp();
+                if (on) {
+                    if (lane == 31 - __clz(peers)) at[digit] = q + 1;
+                    to[q] = x[u];
+                }
+                __syncwarp();
+            }
+        }
+        from = to;
+        to = to == row ? tmp : row;
+    }
+    int32_t w = 0;
+#pragma unroll 1
+    for (int32_t k0 = 0; k0 < len; k0 += 32) {
+        const int32_t k = k0 + lane;
+        const int32_t x = k < len ? row[k] : 0;
+        const bool keep = k < len && (k == 0 || row[k - 1] != x);
+        const unsigned mk = __ballot_sync(0xffffffffu, keep);  // (read before it is written)
+        if (keep) row[w + __popc(mk & ((1u << lane) - 1u))] = x;
+        w += __popc(mk);
+        __syncwarp();
+    }
+    return w;
+}
+
 // Hyperedge e of the input: its checks, the vertices' degrees and the
 // incidences' places in their lists.  A row that is not strictly ascending is
 // sorted, without repeats, into v.row (its ids; noted in the record).
-// Returns the error bits found.  The whole warp.
+// Returns the error bits found, and kLeave.  The whole warp.
 __device__ __forceinline__ int32_t count_row(const Ctx &c, const View &v, const int32_t *evtx,
-                                             const int32_t *f, int32_t *place, int32_t *local,
-                                             int32_t n0, int64_t nnz0, int32_t e) {
+                                             const int32_t *f, int32_t *place, uint32_t *tmp,
+                                             int32_t *local, int32_t n0, int64_t nnz0, int32_t e) {
     int32_t p0 = 0, len = 0, fe = 1, bad = 0;
     if (e >= 0) {
         p0 = v.eptr[e];
@@ -1355,13 +1459,33 @@ __device__ __forceinline__ int32_t count_row(const Ctx &c, const View &v, const 
     const int32_t maxlen = __reduce_max_sync(0xffffffffu, len);
     // first the entries, in order? (each against its right neighbour)
     bool asc = true;
+    const bool large = len > kRankRow;
 #pragma unroll 1
-    for (int32_t k = c.sub; k + 1 < len; k += kG) asc = asc && in[k] < in[k + 1];
+    for (int32_t k = c.sub; k + 1 < len && !large; k += kG) asc = asc && in[k] < in[k + 1];
     __syncwarp();
-    const bool sorted = group_ballot(c, !asc) == 0;
-    if (__any_sync(0xffffffffu, !sorted)) {
+    bool sorted = group_ballot(c, !asc) == 0;
+    // long rows: the warp, one after the other
+    unsigned longs = __ballot_sync(0xffffffffu, large && c.sub == 0);
+#pragma unroll 1
+    while (longs) {
+        const int l = __ffs(longs) - 1;
+        longs &= longs - 1;
+        const int32_t lp = __shfl_sync(0xffffffffu, p0, l), ln = __shfl_sync(0xffffffffu, len, l);
+        const int32_t n = long_row(evtx + lp, reinterpret_cast<int32_t *>(tmp) + lp,
+                                   reinterpret_cast<int32_t *>(v.row) + lp, ln, n0);
+        if (c.lead != l || n == kInOrder) continue;
+        if (n & kLeave) {
+            bad |= n;
+            len = 0;
+        } else {
+            sorted = false;
+            len = n;
+        }
+    }
+    if (__any_sync(0xffffffffu, !sorted && !large)) {
         // rank sort (ties by place), then drop repeats
-        if (!sorted)
+        const bool ranked = !sorted && !large;
+        if (ranked)
 #pragma unroll 1
             for (int32_t k = c.sub; k < len; k += kG) {
                 const int32_t y = in[k];
@@ -1372,7 +1496,7 @@ __device__ __forceinline__ int32_t count_row(const Ctx &c, const View &v, const 
             }
         __syncwarp();
         int32_t w = len;
-        if (!sorted && c.sub == 0) {
+        if (ranked && c.sub == 0) {
             int32_t last = row[0];
             w = 1;
 #pragma unroll 1
@@ -1511,25 +1635,7 @@ __device__ __noinline__ u64 fill_long_row(const int32_t *ids, int32_t *place, ui
 #pragma unroll 1
     for (int o = 16; o > 0; o >>= 1) sig |= __shfl_xor_sync(0xffffffffu, sig, o);
     const u64 entry = make_entry(e, f, len, fold_sig(sig));
-    // the first place of every class
-    int32_t sum = 0;
-#pragma unroll 1
-    for (int c = 0; c < kPer; ++c) sum += at[lane * kPer + c];
-    int32_t inc = sum;
-#pragma unroll 1
-    for (int o = 1; o < 32; o <<= 1) {
-        const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += y;
-    }
-    int32_t first = inc - sum;
-    __syncwarp();
-#pragma unroll 1
-    for (int c = 0; c < kPer; ++c) {
-        const int32_t n = at[lane * kPer + c];
-        at[lane * kPer + c] = first;
-        first += n;
-    }
-    __syncwarp();
+    first_places(at, lane);
 #pragma unroll 1
     for (int32_t k0 = 0; k0 < len; k0 += 32) {
         const int32_t k = k0 + lane;
@@ -1635,11 +1741,16 @@ __device__ __noinline__ bool build_instance(int32_t max_rounds, SpTotals *out) {
     for (int32_t e = t0; e < m0; e += ts) v.e_o2c[e] = e;
     for_flagged(
         c, m0, [](int32_t) { return true; },
-        [&](int32_t e) { bad |= count_row(c, v, evtx, f, place, local, n0, nnz0, e); });
-    if (bad) atomicOr(&s.status, bad);
+        [&](int32_t e) { bad |= count_row(c, v, evtx, f, place, tmp, local, n0, nnz0, e); });
+    if (bad & ~kLeave) atomicOr(&s.status, bad & ~kLeave);
+    if (bad & kLeave) v.ctl->leave = 1;
     if (!team_sync()) return false;
     if (const int32_t st = vload(&s.status)) {
         if (t0 == 0) atomicOr(&out->status, st);
+        return true;
+    }
+    if (vload(&v.ctl->leave)) {
+        if (t0 == 0) out->leave = 1;
         return true;
     }
     // a place for every vertex's list (in any order): one atomic per warp
@@ -2020,7 +2131,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
                     uint64_t absent_ns) {
     Shared *sh = shared();
     bool ok = true;
-    if (masks.built && (masks.built->status || masks.built->cost > masks.max_cost)) return;
+    if (masks.built &&
+        (masks.built->status || masks.built->leave || masks.built->cost > masks.max_cost))
+        return;
     if (team > 0) {
         start(st + blockIdx.x / team, blockIdx.x % team, team, absent_ns);
         ok = run_instance(limit, ctr, times);

@@ -151,3 +151,48 @@ def test_full_lists_of_tasks_and_pairs(mhs, rule):
                 _same(h.result(b), refs[b % len(insts)], b)
     for inst, ref in zip(insts, refs):
         _same(mhs.kernelize(inst, rule=rule), ref)
+
+
+def _unsorted(n, sizes, seed):
+    """Rows in no order, with a few repeats, and the instance that they are."""
+    rng = np.random.Generator(np.random.PCG64(seed))
+    rows = []
+    for s in sizes:
+        r = rng.choice(n, s, replace=False)
+        rows.append(rng.permutation(np.concatenate([r, r[:rng.integers(0, 4)]])))
+    rows += [r[1:] for r in rows[:6]]
+    inst = I.from_edges(n, [sorted(set(r.tolist())) for r in rows], rng.integers(1, 5, len(rows)), k=2)
+    ptr = np.concatenate([[0], np.cumsum([len(r) for r in rows])])
+    return inst, _dev(ptr, np.concatenate(rows), inst.demand)
+
+
+@pytest.mark.parametrize("n,longest", [(256, 256), (257, 257), (4000, 65), (4000, 1500), (65536, 8100),
+                                       (65537, 8100), (70000, 65536), (70000, 65537)])
+def test_unsorted_rows_of_any_length(mhs, n, longest):
+    """One long row among many short ones: ranked (up to 64 ids), sorted by bytes
+    of the id (1, 2 or 3 of them), or (above 65,536) not for this path."""
+    inst, d = _unsorted(n, [longest, 63, 64, 65, 128] + [3, 17, 30] * 700, seed=n + longest)
+    ref = O.reduce(inst)
+    with mhs.Instance.load_device(inst.n, inst.m, *d, inst.k) as h:
+        h.kernelize()
+        _same(h.result(), ref)
+    rows = np.split(d[1].cpu().numpy(), d[0].cpu().numpy()[1:-1])
+    host = I.Instance(n=inst.n, m=inst.m, edge_ptr=np.concatenate([[0], np.cumsum(
+        [len(set(r.tolist())) for r in rows])]).astype(np.int32), edge_vtx=np.concatenate(
+        [np.array(list(dict.fromkeys(r.tolist())), np.int32) for r in rows]),
+        demand=inst.demand, k=inst.k)  # host loads refuse repeats
+    _same(mhs.kernelize(host), ref)
+
+
+@pytest.mark.parametrize("length", [64, 65, 4096, 50000])
+def test_noalloc_unsorted_rows_with_many_repeats(mhs, length):
+    import torch
+    rng = np.random.Generator(np.random.PCG64(length))
+    n, rows = 4000, [rng.integers(0, 3000, length)] + [rng.choice(4000, 9, replace=False) for _ in range(900)]
+    inst = I.from_edges(n, [sorted(set(r.tolist())) for r in rows], rng.integers(1, 4, len(rows)), k=2)
+    ref = O.reduce(inst)
+    av, ae = (torch.zeros(x, dtype=torch.uint8, device="cuda") for x in (inst.n, inst.m))
+    d = _dev(np.concatenate([[0], np.cumsum([len(r) for r in rows])]), np.concatenate(rows), inst.demand)
+    assert mhs.kernelize_noalloc(n, inst.m, *d, d[1].numel(), av, ae) == ref["rounds"]
+    assert torch.nonzero(av).flatten().tolist() == ref["vertices"].tolist()
+    assert torch.nonzero(ae).flatten().tolist() == ref["edges"].tolist()
