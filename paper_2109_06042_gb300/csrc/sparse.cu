@@ -410,6 +410,19 @@ __device__ __forceinline__ bool pair_hit(const Shared *sh, uint32_t x, uint32_t 
     return false;
 }
 
+// Rows of many heavy vertices, whose pairs grow with the square: above kPairRow
+// a superseder sets no pair bounds and walks its heavy lists whole; above
+// kPairTest a hyperedge is not tested against them, and every walk is whole.
+// Every pair of every row, as far as the table had room, took (load and
+// kernelization, us; so / now / by the contraction):
+//   one hyperedge of 600, demand 600, among 20,000 of 10 over 700 vertices
+//                                                          124,935 /  811 / 549
+//   20,000 of 30 over 1,000 vertices, of demand |e|          3,650 /  881 / 652
+constexpr int32_t kPairRow = 16, kPairTest = 256;
+__device__ __forceinline__ bool many_heavy(const uint32_t *row, int32_t len, int32_t most) {
+    return len > most && row[len - 1 - most] >= kHeavyKey;  // (they end the row)
+}
+
 // What hyperedge e (row: its keys) contributes to the tests with need <= 1,
 // and in full rounds to those of pairs of heavy vertices.  One group, without
 // the others.
@@ -435,7 +448,9 @@ __device__ __noinline__ void contribute(int32_t e, int32_t f, int32_t len, const
         if (!sh->rule && f > 1 && atomicMax(&ctl->loose, f - 1) < f - 1) ctl->c[sh->par].scan_all = 1;
         return;
     }
-    if (sh->rule || f < len - 1) return;
+    if (sh->rule) return;
+    if (sh->full && many_heavy(row, len, kPairTest)) ctl->pairs_full = 1;
+    if (f < len - 1) return;
     const int32_t m1 = f - len + 1;
     if (m1 >= 1)
 #pragma unroll 1
@@ -448,12 +463,12 @@ __device__ __noinline__ void contribute(int32_t e, int32_t f, int32_t len, const
         }
     if (f > len && sub == 0 && atomicMax(&ctl->loose, f - len) < f - len)
         ctl->c[sh->par].scan_all = 1;
-    if (!sh->full) return;
+    if (!sh->full || many_heavy(row, len, kPairRow)) return;
     // every two heavy ones: they end the row, and most rows have fewer
     int32_t a = len - 1;
     while (a > 0 && row[a - 1] >= kHeavyKey) --a;
 #pragma unroll 1
-    for (; a < len - 1; ++a) {
+    for (; a < len - 1 && !vload(&ctl->pairs_full); ++a) {
         const uint32_t ka = row[a];
 #pragma unroll 1
         for (int32_t k = a + 1 + sub; k < len; k += kG)
@@ -573,6 +588,7 @@ __device__ __noinline__ void dp_bounds_all(int shard, int nshards) {
     const View &v = c.sh->view;
     const int32_t loose = vload(&v.ctl->loose);
     const u64 empty = *reinterpret_cast<volatile u64 *>(&v.ctl->empty);
+    const bool pairs = c.full && !vload(&v.ctl->pairs_full);  // (else the walks find theirs)
     const int32_t *const e_o2c = v.e_o2c, *const eptr = v.eptr;
     const int4 *const erec = v.erec;
     const uint32_t *const rows = v.row;
@@ -608,7 +624,7 @@ __device__ __noinline__ void dp_bounds_all(int shard, int nshards) {
             hit = hit && fj != kGone;
             // every two heavy ones, unless decided
             int32_t end = 0;
-            if (__any_sync(0xffffffffu, heavy != 0)) {
+            if (pairs && __any_sync(0xffffffffu, heavy != 0)) {
                 heavy = group_sum(heavy);
                 end = group_ballot(c, hit) == 0 && heavy > 1 ? len : 0;
                 end = __shfl_sync(0xffffffffu, end, c.lead);
@@ -868,13 +884,14 @@ __device__ __noinline__ void dp_walk(int shard, int nshards) {
             w.rule = rule;
             const int32_t np = w.f == kGone ? 0 : walk_count(rule, w.f, w.len);
             const int32_t npmax = __reduce_max_sync(0xffffffffu, np);
+            const bool mine = bounded && !(np > 0 && many_heavy(row, w.len, kPairRow));
 #pragma unroll 1
             for (int32_t p0 = 0; p0 < npmax; p0 += kG) {
                 // one of the next 8 vertices per lane
                 int32_t p = p0 + c.sub;
                 const uint32_t key = p < np ? row[p] : 0;
                 int32_t x = p < np ? key_id(key) : -1;
-                if (bounded && key >= kHeavyKey) {  // its pairs with need 2 went by the bounds
+                if (mine && key >= kHeavyKey) {  // its pairs with need 2 went by the bounds
                     if (p > w.len - 3) x = -1;
                     p |= kNeed3;
                 }

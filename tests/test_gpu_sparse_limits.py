@@ -196,3 +196,36 @@ def test_noalloc_unsorted_rows_with_many_repeats(mhs, length):
     assert mhs.kernelize_noalloc(n, inst.m, *d, d[1].numel(), av, ae) == ref["rounds"]
     assert torch.nonzero(av).flatten().tolist() == ref["vertices"].tolist()
     assert torch.nonzero(ae).flatten().tolist() == ref["edges"].tolist()
+
+
+@pytest.mark.parametrize("heavy", [2, 15, 16, 17, 255, 256, 257, 300])
+def test_hyperedges_of_many_heavy_vertices(mhs, heavy):
+    """Superseders of demand |e| - 1 .. |e| + 1 over `heavy` vertices of 192
+    hyperedges and more, which delete by pairs of them: up to 16 by bounds,
+    above by walks, and all by walks where some row has more than 256."""
+    rng = np.random.Generator(np.random.PCG64(heavy))
+    hubs = heavy + 6
+    each = max(1, 260 // hubs)
+    edges, dem = [], []
+    for q in range(3):
+        e = np.sort(rng.choice(hubs, heavy, replace=False)).tolist()
+        edges.append(e)
+        dem.append(max(1, len(e) - 1 + q))
+    for a in range(hubs):
+        for b in rng.choice([x for x in range(hubs) if x != a], min(hubs - 1, 40), replace=False):
+            for q in range(each):
+                edges.append(sorted({a, int(b), hubs + int(rng.integers(0, 900))}))
+                dem.append(int(rng.integers(1, 4)))
+        for q in range(200):
+            edges.append(sorted({a} | {hubs + int(x) for x in rng.integers(0, 900, 2)}))
+            dem.append(int(rng.integers(1, 3)))
+    inst = I.from_edges(hubs + 900, edges, dem, k=3)
+    deg = np.bincount(inst.edge_vtx, minlength=inst.n)
+    assert deg[:hubs].min() >= 192
+    with mhs.Instance.load(inst) as h:
+        h.kernelize()
+        assert h.work_stats() == (0, 0)  # by candidate lists
+        got = h.result()
+    _same(got, O.reduce(inst) if inst.m < 10000 else mhs.kernelize(inst, contraction="popcount"))
+    _same(mhs.kernelize(inst, full_edges=True),
+          mhs.kernelize(inst, contraction="popcount", full_edges=True))
