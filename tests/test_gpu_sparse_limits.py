@@ -229,3 +229,35 @@ def test_hyperedges_of_many_heavy_vertices(mhs, heavy):
     _same(got, O.reduce(inst) if inst.m < 10000 else mhs.kernelize(inst, contraction="popcount"))
     _same(mhs.kernelize(inst, full_edges=True),
           mhs.kernelize(inst, contraction="popcount", full_edges=True))
+
+
+def test_batch_of_instances_with_and_without_long_rows(mhs):
+    """One CTA builds instances of both kinds in turn, below and above the 3,072
+    vertices whose degrees it keeps in shared memory; malformed ones are named."""
+    import torch
+    insts, parts = [], []
+    for s, (n, long) in enumerate([(300, 0), (300, 65), (3072, 200), (3073, 0), (3500, 900), (40, 40), (4000, 64)]):
+        inst, d = _unsorted(n, [long] * (long > 0) + [5, 9, 16, 17] * 40, seed=s)
+        insts.append(inst)
+        parts.append([x.cpu().numpy() for x in d])
+    refs = [O.reduce(i) for i in insts]
+    order = [b % len(insts) for b in range(420)]
+    n = np.array([insts[b].n for b in order], np.int32)
+    m = np.array([insts[b].m for b in order], np.int32)
+    k = np.array([insts[b].k for b in order], np.int64)
+    sizes = np.concatenate([np.diff(parts[b][0]) for b in order])
+    ptr = torch.from_numpy(np.concatenate([[0], np.cumsum(sizes)])).cuda()
+    vtx, dem = _dev(np.concatenate([parts[b][1] for b in order]),
+                    np.concatenate([parts[b][2] for b in order]))
+    with mhs.Instance.load_batch_device(n, m, k, ptr, vtx, dem) as h:
+        h.kernelize()
+        assert h.work_stats() == (0, 0)  # by candidate lists
+        for b in range(0, len(order), 5):
+            _same(h.result(b), refs[order[b]], b)
+    for b in (1, 2, 9):  # (long rows in instances 1 and 2, 8 and 9)
+        start = int(ptr[int(m[:b].sum())])
+        bad = vtx.clone()
+        bad[start + 3] = int(n[b])
+        with pytest.raises(mhs.MhsError) as ei:
+            mhs.Instance.load_batch_device(n, m, k, ptr, bad, dem)
+        assert ei.value.status == mhs.MHS_EINVAL and f"instance {b} " in str(ei.value)
