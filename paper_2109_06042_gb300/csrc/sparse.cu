@@ -418,7 +418,7 @@ __device__ __forceinline__ bool pair_hit(const Shared *sh, uint32_t x, uint32_t 
 //   one hyperedge of 600, demand 600, among 20,000 of 10 over 700 vertices
 //                                                          124,935 /  811 / 549
 //   20,000 of 30 over 1,000 vertices, of demand |e|          3,650 /  881 / 652
-constexpr int32_t kPairRow = 16, kPairTest = 256;
+constexpr int32_t kPairRow = 6, kPairTest = 256;
 __device__ __forceinline__ bool many_heavy(const uint32_t *row, int32_t len, int32_t most) {
     return len > most && row[len - 1 - most] >= kHeavyKey;  // (they end the row)
 }
@@ -463,12 +463,12 @@ __device__ __noinline__ void contribute(int32_t e, int32_t f, int32_t len, const
         }
     if (f > len && sub == 0 && atomicMax(&ctl->loose, f - len) < f - len)
         ctl->c[sh->par].scan_all = 1;
-    if (!sh->full || many_heavy(row, len, kPairRow)) return;
+    if (!sh->full || many_heavy(row, len, kPairRow) || vload(&ctl->pairs_full)) return;
     // every two heavy ones: they end the row, and most rows have fewer
     int32_t a = len - 1;
     while (a > 0 && row[a - 1] >= kHeavyKey) --a;
 #pragma unroll 1
-    for (; a < len - 1 && !vload(&ctl->pairs_full); ++a) {
+    for (; a < len - 1; ++a) {
         const uint32_t ka = row[a];
 #pragma unroll 1
         for (int32_t k = a + 1 + sub; k < len; k += kG)
@@ -884,7 +884,8 @@ __device__ __noinline__ void dp_walk(int shard, int nshards) {
             w.rule = rule;
             const int32_t np = w.f == kGone ? 0 : walk_count(rule, w.f, w.len);
             const int32_t npmax = __reduce_max_sync(0xffffffffu, np);
-            const bool mine = bounded && !(np > 0 && many_heavy(row, w.len, kPairRow));
+            // (a smaller demand leaves need >= 3 in any case)
+            const bool mine = bounded && !(np > 0 && w.f >= w.len - 1 && many_heavy(row, w.len, kPairRow));
 #pragma unroll 1
             for (int32_t p0 = 0; p0 < npmax; p0 += kG) {
                 // one of the next 8 vertices per lane
