@@ -117,11 +117,12 @@ cudaError_t launch_alive_masks_batch(const InstState *st, int count, uint8_t *al
                                      uint8_t *alive_e, cudaStream_t s);
 
 // ---- candidate lists instead of a contraction (sparse.cu) ----
-// What a load reads back: the list entries the first round's walks may visit
-// (summed over a batch), the OR of the status words, and whether some instance
+// What a load reads back: the list entries the first round's walks may visit and,
+// in their units, what the pairs found in them may cost (both summed over a
+// batch), the OR of the status words, and whether some instance
 // has a row that is not for this path (nothing is built then).
 struct SpTotals {
-    unsigned long long cost;
+    unsigned long long cost, open;
     int32_t status;
     int32_t leave;
 };
@@ -138,7 +139,7 @@ struct SpQueue {
 };
 // A single instance whose rounds are launched before the host has seen what the
 // build found (built set): they run if it found no error, all rows for this path and
-// a cost of at most max_cost, and leave the alive masks of the input ids.
+// at most max_cost for both costs, and leave the alive masks of the input ids.
 struct SpMasks {
     const SpTotals *built;
     unsigned long long max_cost;

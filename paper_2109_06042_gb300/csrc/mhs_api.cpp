@@ -453,18 +453,27 @@ bool auto_sparse(const mhs_options *opt) {
 }
 
 // Does the sparse path pay?  cost: list entries its first round may visit;
-// pairs: m^2 + n^2 summed over the instances, what the contraction's
-// epilogue tests.  Measured (load and kernelization, sparse / FP8, us):
+// open: what the pairs found there may cost (sparse.cu); pairs: m^2 + n^2 summed
+// over the instances, what the contraction's epilogue tests.  Measured (load
+// and kernelization, sparse / FP8, us):
 //   n 200, m 20,000, |e| 16..32: cost 118 M, pairs 0.4 G     921 /  749
 //   n 64, m 20,000, |e| 3..6:    cost  62 M, pairs 0.4 G     292 /  455
 //   n 16,000, m 24,000, |e| 32..64: cost 3.5 M, pairs 0.8 G  235 / 5273
+// by demands (open: 370 M, 690 M, 9 M, 280 M, 320 M):
+//   n 2,000, m 4,000, |e| 24..96, f up to 24               2,272 /   495
+//   n 300, m 4,000, |e| 20..60, f up to 20                 1,807 /   430
+//   n 300, m 400, |e| 20..60, f up to 20                     235 /   393
+//   n 1,000, m 20,000, |e| 8..16, f up to |e|                850 /   607
+//   n 16,000, m 32,000, |e| 8..32, f up to |e|             1,564 / 7,425
 // and by the mean size, where the searches in rows and the work per
 // incidence grow:
 //   n 2,000, m 4,000, |e| 256..512: mean 384                1664 / 1286
 //   n 2,000, m 4,000, |e| 128..256: mean 192                 774 /  790
-constexpr double kSparseBase = 64e6, kSparsePerPair = 1.0 / 20;
+constexpr double kSparseBase = 64e6, kSparsePerPair = 1.0 / 20, kOpenPerPair = 1.0 / 4;
 constexpr double kSparseMeanSize = 256;
-bool sparse_pays(double cost, double pairs) { return cost <= kSparseBase + kSparsePerPair * pairs; }
+bool sparse_pays(double cost, double open, double pairs) {
+    return cost <= kSparseBase + kSparsePerPair * pairs && open <= kSparseBase + kOpenPerPair * pairs;
+}
 // A lower estimate of the cost before anything is loaded: every hyperedge
 // walks one list of mean length.
 bool sparse_may_pay(int32_t count, const int32_t *n, const int32_t *m, const int64_t *nnz) {
@@ -475,7 +484,7 @@ bool sparse_may_pay(int32_t count, const int32_t *n, const int32_t *m, const int
         edges += m[b];
         inc += (double)nnz[b];
     }
-    return inc <= kSparseMeanSize * edges && sparse_pays(cost / 4, pairs);
+    return inc <= kSparseMeanSize * edges && sparse_pays(cost / 4, 0, pairs);
 }
 
 mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64_t *nnz,
@@ -904,7 +913,7 @@ mhs_status build_sparse(mhs_instance *h, SpTotals *found, bool *pays) {
     double pairs = 0;
     for (const HostInst &i : h->hinst)
         pairs += (double)i.m0 * i.m0 + (double)i.n0 * i.n0;
-    *pays = !host->leave && sparse_pays((double)host->cost, pairs);
+    *pays = !host->leave && sparse_pays((double)host->cost, (double)host->open, pairs);
     return MHS_OK;
 }
 

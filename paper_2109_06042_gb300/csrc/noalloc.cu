@@ -55,7 +55,8 @@ inline int64_t up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 inline int64_t words(int64_t K) { return up(((K + 31) / 32) > 0 ? (K + 31) / 32 : 1, 4); }
 
 // The candidate lists are taken for rows of this mean length at most, and while
-// their first round visits no more list entries than this.  Measured, a call
+// their first round visits no more list entries than this (with what the pairs
+// found in them cost, in such units).  Measured, a call
 // by lists / by bits alone (us); bits after a build that did not pay: + 50.
 //   n 1,000, m 2,000, |e| 2..16:       cost 55 K     83 / 254
 //   n 256, m 4,096, |e| 14..16:        cost 1.8 M   117 / 180
@@ -276,7 +277,7 @@ extern "C" mhs_status mhs_kernelize_noalloc(int32_t n, int32_t m, const int32_t 
         return err(err_buf, err_cap, MHS_EDEVICE, "kernel reported an error status");
     if (found.totals.status)
         return err(err_buf, err_cap, MHS_EINVAL, "malformed instance (bad edge_ptr or vertex id)");
-    if (lists && !found.totals.leave && found.totals.cost <= kNoAllocCost) {
+    if (lists && !found.totals.leave && found.totals.cost + found.totals.open <= kNoAllocCost) {
         if (ctr.status_any || ctr.active)
             return err(err_buf, err_cap, MHS_EDEVICE, "kernel reported an error status");
         if (rounds_out) *rounds_out = ctr.max_rounds_seen;

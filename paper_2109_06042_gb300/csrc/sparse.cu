@@ -193,6 +193,7 @@ struct Shared {
     int32_t full;         // every hyperedge and vertex is a candidate
     int32_t ok;           // the last barrier
     int32_t local;        // there is room for degrees (build of a batch)
+    int32_t demands;      // (build) some demand is above kFewMisses
     int32_t heavy_list;   // longer lists are walked as tasks,
     int32_t task_len;     // of so many entries
     SpRound got;          // counters read right after it
@@ -200,7 +201,7 @@ struct Shared {
     int32_t del, del2;    // deletions of this phase
     int32_t next;         // batch: the instance taken from the queue
     int32_t mf, pos;      // md_lists: one high-degree vertex
-    u64 cost, sig, small;
+    u64 cost, open, sig, small;
     int2 *pairs;          // this instance's pairs (i, j) to be decided exactly
     int32_t pair_cap;
 };
@@ -678,6 +679,23 @@ __device__ __forceinline__ int32_t walk_count(int32_t rule, int32_t f, int32_t l
     if (len < 2) return 0;
     return rule ? 1 : min(f, len - 1);
 }
+
+// What a walk of `entries` list entries counts as open (SpTotals).  Where the demand allows as many missed vertices as the 64-bit signatures show of
+// two unrelated sets (less a standard deviation), most entries become pairs that
+// are searched row by row: 45 ps each at |e| 12, 950 at 60 (8 to 14 ps an entry
+// that is ruled out at once).  Demands up to 4 never do.
+constexpr int32_t kFewMisses = 4;
+__device__ __forceinline__ float open_walk(float entries, int32_t f, int32_t len) {
+    const float unset = __expf((float)len * (-1.f / 64.f));  // share of a signature's bits
+    const float missed = 64.f * unset * (1.f - unset);
+    const float dev = sqrtf(missed * (1.f - unset));
+    return (float)f - 1.f >= missed - dev ? entries * 1.5f * (float)len : 0.f;
+}
+// And a walk of many lists, which one group takes one after the other (one
+// hyperedge of demand and size 300 among 20,000 of 10 over 3,000 vertices: 1.4 ms
+// in all, 0.86 by the contraction; 3,000: 14 and 1.0).
+constexpr int32_t kManyLists = 128;
+constexpr float kPerListSquared = 4096.f;
 
 struct Walker {  // the superseder of a walk
     int32_t i, f, len, rule;
@@ -1487,6 +1505,7 @@ __device__ __forceinline__ int32_t count_row(const Ctx &c, const View &v, const 
         len = v.eptr[e + 1] - p0;
         fe = f[e];
         if (fe < 1) bad |= kErrBadDemand;
+        if (fe > kFewMisses) c.sh->demands = 1;
         if (p0 < 0 || len < 0 || (int64_t)p0 + len > nnz0) { bad |= kErrBadPtr; len = 0; }
         if (len > kRankRow) { bad |= kLongRow; len = 0; }
     }
@@ -1764,7 +1783,8 @@ __device__ __noinline__ void start(InstState *s, int rank, int size, uint64_t ab
         sh->par = 0;
         sh->full = 1;
         sh->del = sh->del2 = 0;
-        sh->cost = 0;
+        sh->cost = sh->open = 0;
+        sh->demands = 0;
         sh->pairs = s->sp_pairs;
         sh->pair_cap = s->sp_pair_cap;
         sh->bar = &s->sp_ctl->bar;
@@ -1774,6 +1794,35 @@ __device__ __noinline__ void start(InstState *s, int rank, int size, uint64_t ab
         sh->target = now / (uint32_t)size * (uint32_t)size;
     }
     __syncthreads();
+}
+
+// What the walks of the hyperedges with demands above kFewMisses count as open
+// (rows and degrees are in place).  Apart from the fill, whose loop keeps fewer
+// registers with it (the batch of 4,096: 2.52 ms instead of 2.47).
+__device__ __noinline__ void open_walks() {
+    const Ctx c;
+    Shared *sh = c.sh;
+    const View &v = sh->view;
+    if (sh->rule) return;
+    const int32_t *const f = sh->s->f;
+    float open = 0.f;
+    for_flagged(
+        c, sh->m0, [&](int32_t e) { return f[e] > kFewMisses; },
+        [&](int32_t e) {
+            if (e >= 0) {
+                const int4 r = v.erec[e];
+                const int32_t np = walk_count(0, r.z, r.w);
+                const uint32_t *row = v.row + v.eptr[e];
+                float entries = 0.f;
+#pragma unroll 1
+                for (int32_t k = c.sub; k < np && np <= kManyLists; k += kG)
+                    entries += (float)v.vrec[key_id(row[k])].z;
+                open += open_walk(entries, r.z, r.w);
+                if (np > kManyLists && c.sub == 0) open += kPerListSquared * (float)np * (float)np;
+            }
+            __syncwarp();
+        });
+    if (open > 0.f) atomicAdd(&sh->open, (u64)open);
 }
 
 // Structural checks, rows and lists of one instance; !kLong: if it has no row above
@@ -1865,7 +1914,7 @@ __device__ __noinline__ bool build_instance(int32_t max_rounds, SpTotals *out) {
             uint32_t *row = v.row + p0;
             const int32_t np = e >= 0 ? walk_count(rule, r.z, len) : 0;
             u64 sig = 0;
-            // rows up to 32: the group ranks each key among the row's
+            // rows up to 16: the group ranks each key among the row's
             const bool small = len <= kRowU * kG;
             if (__any_sync(0xffffffffu, small && len > 0)) {
                 sig = fill_row<kG>(c, v, local, ids, place + p0, row, e, r.z, small ? len : 0, np, c.sub,
@@ -1903,8 +1952,10 @@ __device__ __noinline__ bool build_instance(int32_t max_rounds, SpTotals *out) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) cost += __shfl_xor_sync(0xffffffffu, cost, o);
     if (c.lane == 0 && cost) atomicAdd(&c.sh->cost, cost);
+    if (c.sh->demands) open_walks();
     __syncthreads();
     if (threadIdx.x == 0 && c.sh->cost) atomicAdd(&out->cost, c.sh->cost);
+    if (threadIdx.x == 0 && c.sh->open) atomicAdd(&out->open, c.sh->open);
     return true;
 }
 
@@ -2224,7 +2275,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
     Shared *sh = shared();
     bool ok = true;
     if (masks.built &&
-        (masks.built->status || masks.built->leave || masks.built->cost > masks.max_cost))
+        (masks.built->status || masks.built->leave ||
+         masks.built->cost + masks.built->open > masks.max_cost))
         return;
     if (team > 0) {
         start(st + blockIdx.x / team, blockIdx.x % team, team, absent_ns);

@@ -261,3 +261,30 @@ def test_batch_of_instances_with_and_without_long_rows(mhs):
         with pytest.raises(mhs.MhsError) as ei:
             mhs.Instance.load_batch_device(n, m, k, ptr, bad, dem)
         assert ei.value.status == mhs.MHS_EINVAL and f"instance {b} " in str(ei.value)
+
+
+@pytest.mark.parametrize("n,m,lo,hi,fmin,fmax,leaves", [
+    (2000, 4000, 24, 96, 1, 24, True), (1000, 1000, 150, 200, 1, 40, True),
+    (1000, 4000, 150, 200, 1, 4, False), (300, 400, 20, 60, 1, 20, False),
+    (4000, 8000, 2, 16, 100, 100, False), (1000, 20000, 8, 16, 1, 8, False)])
+def test_large_demands_choose_the_path_that_pays(mhs, n, m, lo, hi, fmin, fmax, leaves):
+    """Walks that find many pairs to be decided row by row count for more."""
+    rng = np.random.Generator(np.random.PCG64(n + m + fmax))
+    inst = I.from_edges(n, [np.sort(rng.choice(n, rng.integers(lo, hi + 1), replace=False)) for _ in range(m)],
+                        rng.integers(fmin, fmax + 1, m), k=4)
+    with mhs.Instance.load(inst) as h:
+        h.kernelize()
+        assert (h.work_stats()[1] > 0) == leaves
+        got = h.result()
+    _same(got, mhs.kernelize(inst, contraction="popcount"))
+
+
+def test_one_hyperedge_of_a_large_demand_leaves_the_lists(mhs):
+    rng = np.random.Generator(np.random.PCG64(600))
+    rows = [np.sort(rng.choice(3000, 10, replace=False)) for _ in range(9000)] + [np.arange(600)]
+    inst = I.from_edges(3000, rows, [2] * 9000 + [600], k=4)
+    with mhs.Instance.load(inst) as h:
+        h.kernelize()
+        assert h.work_stats()[1] > 0
+        got = h.result()
+    _same(got, mhs.kernelize(inst, contraction="popcount"))
