@@ -969,7 +969,11 @@ __device__ __forceinline__ bool bounds_apply(const InstState &s) {
     return s.active && !s.status && s.rounds == 0 && !s.no_skip;
 }
 
-// kTest false: collect the bounds; true: flag the rows they delete.
+// kTest false: collect the bounds; true: flag the rows they delete.  Rows above
+// kBoundRow are left to the contraction: a bound needs f >= |e|, and eight lanes
+// walk such a row while the rest waits (one of 3,000 among 20,000 of 10: 1,206 us
+// in all; 979 without the bounds).
+constexpr int32_t kBoundRow = 64;
 template <bool kTest>
 __global__ void __launch_bounds__(256) k_bounds(InstState *st, int count) {
     constexpr int kLanes = 8;  // per row
@@ -991,6 +995,7 @@ __global__ void __launch_bounds__(256) k_bounds(InstState *st, int count) {
             const int32_t e = s.e_c2o[r];
             p0 = s.eptr[e];
             p1 = s.eptr[e + 1];
+            if (p1 - p0 > kBoundRow) p1 = p0;
         }
         for (int32_t p = p0 + sub; p < p1; p += kLanes) {
             const int32_t cv = s.v_o2c[s.evtx[p]];

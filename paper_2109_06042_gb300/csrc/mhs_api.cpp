@@ -1114,14 +1114,17 @@ mhs_status run_sparse(mhs_instance *h, int32_t limit, mhs_round_stats *stats) {
 //   uniform 2,000 x 4,000     386 / 389     4,000 x 8,000    514 / 489
 //   power law 2,000 x 4,000   557 / 569     5,000 x 10,000   546 / 542
 //   interval 8,000 x 16,000  1107 / 971     power law 10,000 x 20,000  742 / 687
-constexpr int64_t kBoundsRows = 8000;
+// and the mean size up to which they do:
+//   1,000 x 20,000, |e| 30   679 / 723      5,000 x 10,000, |e| 8..24   688 / 614
+constexpr int64_t kBoundsRows = 8000, kBoundsMeanSize = 24;
 
 mhs_status run_rounds(mhs_instance *h, int32_t limit, mhs_round_stats *stats) {
     if (h->pass_state != 0)
         return fail(MHS_EINVAL, "a sharded round is in progress (finish it with mhs_pass_end)");
     if (h->contraction == kSparse) return run_sparse(h, limit, stats);
     // (a sharded pass exports its deletion flags, all of them: it goes without)
-    if (!h->started && h->contraction == kFp8 && h->sum_m >= kBoundsRows)
+    if (!h->started && h->contraction == kFp8 && h->sum_m >= kBoundsRows &&
+        h->sum_nnz <= kBoundsMeanSize * h->sum_m)
         CUDA_TRY(launch_bounds(h->dstate, h->count, h->sms, h->stream, h->compact_blocks));
     h->started = true;
     if (limit <= 0 && h->opt.use_graphs && !h->timing) {

@@ -49,3 +49,19 @@ def test_kernelize_after_sharded_rounds(mhs, contraction, rounds):
             assert got[key].tolist() == ref[key].tolist(), key
         assert got["k"] == ref["k"] and got["rounds"] == ref["rounds"]
         assert h.forced()[0].tolist() == ref["forced"].tolist()
+
+
+@pytest.mark.parametrize("long", [64, 65, 900])
+@pytest.mark.parametrize("rule", ["dp", "se"])
+def test_vertex_bounds_leave_long_rows_to_the_contraction(mhs, rule, long):
+    """Rows above 64 ids set no bounds and are not tested against them."""
+    rng = np.random.Generator(np.random.PCG64(long))
+    rows = [np.sort(rng.choice(2000, rng.integers(1, 6), replace=False)) for _ in range(8200)]
+    rows += [np.sort(rng.choice(2000, long, replace=False)) for _ in range(30)]
+    inst = I.from_edges(2000, rows, rng.integers(1, 5, len(rows)), k=3)
+    inst.demand[8200:8215] = long
+    ref = O.reduce_variant(inst, rule, False)
+    got = mhs.kernelize(inst, contraction="fp8", rule=rule)
+    for key in ("vertices", "edges", "demands"):
+        assert got[key].tolist() == ref[key].tolist(), key
+    assert got["rounds"] == ref["rounds"]
