@@ -1237,10 +1237,11 @@ __device__ __noinline__ void md_test(bool count, int shard, int nshards) {
                     const int32_t e = entry_id(list[q]);
                     ok = e == e0 || in_row(v, e, i);
                 }
-                cnt += ok;
                 __syncwarp();
+                cnt += __popc(group_ballot(c, ok));
+                if (!count && cnt >= aux.y) len0 = 0;  // decided
+                if (!__any_sync(0xffffffffu, k - c.sub + kG < len0)) break;
             }
-            cnt = group_sum(cnt);
             if (j >= 0) {
                 if (count) {
                     if (c.sub == 0) v_cnt[j] = cnt;
@@ -1279,6 +1280,9 @@ __device__ __noinline__ void md_test(bool count, int shard, int nshards) {
                 ok = !__any_sync(0xffffffffu, !in);
             }
             if (ok && c.lane == 0) atomicAdd(&sh->pos, 1);
+            __syncwarp();
+            const bool decided = !count && vload(&sh->pos) >= aux.y;
+            if (__any_sync(0xffffffffu, decided)) break;
         }
         __syncthreads();
         const int32_t cnt = sh->pos;

@@ -288,3 +288,34 @@ def test_one_hyperedge_of_a_large_demand_leaves_the_lists(mhs):
         assert h.work_stats()[1] > 0
         got = h.result()
     _same(got, mhs.kernelize(inst, contraction="popcount"))
+
+
+def _shared(kind, c, h, m, f, seed):
+    """h long hyperedges over c common vertices beside m small ones."""
+    rng = np.random.Generator(np.random.PCG64(seed))
+    if kind == "twins":  # (and one vertex of its own each)
+        rows = [np.append(np.arange(c), c + q) for q in range(h)]
+    elif kind == "complement":  # every vertex misses one hyperedge
+        h = c
+        rows = [np.delete(np.arange(c), q) for q in range(h)]
+    else:
+        rows = [np.nonzero(rng.random(c) < 0.95)[0] for _ in range(h)]
+    lo = c + h
+    rows += [lo + np.sort(rng.choice(900, 6, replace=False)) for _ in range(m)]
+    return I.from_edges(lo + 900, rows, [f] * h + [2] * m, k=3)
+
+
+@pytest.mark.parametrize("kind,c,h,m,f", [
+    ("twins", 400, 20, 900, 1), ("twins", 400, 20, 900, 7), ("twins", 300, 300, 900, 2),
+    ("subsets", 300, 40, 900, 2), ("complement", 230, 230, 900, 1), ("complement", 60, 60, 0, 1),
+    ("complement", 300, 300, 3000, 1), ("twins", 400, 20, 900, 100)])
+def test_vertices_of_nearly_equal_hyperedges(mhs, kind, c, h, m, f):
+    """MD tests that go far: many members, most of them in most hyperedges."""
+    inst = _shared(kind, c, h, m, f, c + h)
+    for fe in (False, True):
+        ref = mhs.kernelize(inst, contraction="popcount", full_edges=fe)
+        _same(mhs.kernelize(inst, full_edges=fe), ref)
+        with mhs.Instance.load_batch([inst] * 180, full_edges=fe) as hd:
+            hd.kernelize()
+            _same(hd.result(0), ref)
+            _same(hd.result(179), ref)
