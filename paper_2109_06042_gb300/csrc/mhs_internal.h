@@ -75,6 +75,7 @@ struct SpRound {
     int32_t dp, md;             // deletions
     int32_t ntask;              // tasks reserved
     int32_t npair[2];           // pairs listed: by the walks, by the tasks
+    int32_t nbig;               // vertices left to whole CTAs by their groups
     int32_t scan_all;           // an instance-wide bound rose
 };
 // Sparse path: control words of one instance.

@@ -267,6 +267,7 @@ __device__ __noinline__ bool team_sync(const SpRound *p = nullptr) {
             sh->got.ntask = vload(&p->ntask);
             sh->got.npair[0] = vload(&p->npair[0]);
             sh->got.npair[1] = vload(&p->npair[1]);
+            sh->got.nbig = vload(&p->nbig);
         }
     }
     __syncthreads();
@@ -1203,6 +1204,62 @@ __device__ __forceinline__ void delete_vertex(Shared *sh, int32_t j, int4 rj, in
     for (int32_t q = sub; q < rj.z; q += step) v.estamp[entry_id(v.vedge[rj.w + q])] = next;
 }
 
+// The test of vertex j (below), by the whole CTA: of high degree, or left by a group.
+__device__ __noinline__ void md_whole(int32_t j, bool count) {
+    const Ctx c;
+    Shared *sh = c.sh;
+    const View &v = sh->view;
+    const int4 rj = v.vrec[j], aux = v.vaux[j];
+    const int32_t e0 = aux.x, len0 = rj.z > 0 ? aux.w : 0;
+    if (rj.z > 0 && !count && len0 - 1 < aux.y) return;
+    const uint32_t *row = v.row + aux.z;
+    const u64 *list = v.vedge + rj.w;
+    if (threadIdx.x == 0) sh->pos = 0;
+    __syncthreads();
+    // one member per warp, 32 hyperedges at a time
+#pragma unroll 1
+    for (int32_t k = c.warp; k < len0; k += blockDim.x >> 5) {
+        const uint32_t i = row[k];
+        bool ok = may_dominate(key_id(i), v.vrec[key_id(i)], j, rj);  // (all lanes alike)
+#pragma unroll 1
+        for (int32_t q0 = 0; q0 < rj.z && ok; q0 += 32) {
+            const int32_t q = q0 + c.lane;
+            const int32_t e = q < rj.z ? entry_id(list[q]) : e0;
+            const bool in = e == e0 || in_row(v, e, i);
+            __syncwarp();
+            ok = !__any_sync(0xffffffffu, !in);
+        }
+        if (ok && c.lane == 0) atomicAdd(&sh->pos, 1);
+        __syncwarp();
+        const bool decided = !count && vload(&sh->pos) >= aux.y;
+        if (__any_sync(0xffffffffu, decided)) break;
+    }
+    __syncthreads();
+    const int32_t cnt = sh->pos;
+    __syncthreads();  // (reset for the next)
+    if (count) {
+        if (threadIdx.x == 0) sh->s->v_cnt[j] = cnt;
+    } else if (rj.z == 0 || cnt >= aux.y) {
+        delete_vertex(sh, j, rj, threadIdx.x, blockDim.x);
+    }
+}
+
+// A group gives up a vertex after so many hyperedges looked at by a lane, if the
+// list of such vertices has room: whole CTAs take them, 32 hyperedges of a member
+// at a time.  (Every vertex in all hyperedges but one, 250 of each, beside 4,000
+// small ones, load and kernelization: 5.3 ms by groups alone, which look through
+// half of them for every member; 0.92 so, 1.17 by the contraction.)
+constexpr int32_t kMdBudget = 96;
+__device__ __noinline__ bool leave_to_cta(bool want, int32_t j) {
+    const Ctx c;
+    int32_t at = c.sh->task_cap;
+    if (want && c.sub == 0) {
+        at = atomicAdd(&c.sh->view.ctl->c[c.par].nbig, 1);
+        if (at < c.sh->task_cap) c.sh->task[at] = make_int4(j, 0, 0, 0);
+    }
+    return __shfl_sync(0xffffffffu, at, c.lead) < c.sh->task_cap;
+}
+
 // The dominators of the candidates (count: into v_cnt; else a vertex with
 // at least as many as its largest demand is deleted, and its hyperedges
 // become the next round's candidates).
@@ -1226,7 +1283,8 @@ __device__ __noinline__ void md_test(bool count, int shard, int nshards) {
             if (!count && len0 - 1 < aux.y) len0 = 0;  // too few members to dominate
             const uint32_t *row = v.row + aux.z;
             const u64 *list = v.vedge + rj.w;
-            int32_t cnt = 0;
+            int32_t cnt = 0, spent = 0;
+            bool mine = j >= 0;
             const int32_t maxlen = __reduce_max_sync(0xffffffffu, len0);
 #pragma unroll 1
             for (int32_t k = c.sub; k - c.sub < maxlen; k += kG) {
@@ -1236,13 +1294,26 @@ __device__ __noinline__ void md_test(bool count, int shard, int nshards) {
                 for (int32_t q = 0; q < rj.z && ok; ++q) {
                     const int32_t e = entry_id(list[q]);
                     ok = e == e0 || in_row(v, e, i);
+                    ++spent;
                 }
                 __syncwarp();
                 cnt += __popc(group_ballot(c, ok));
                 if (!count && cnt >= aux.y) len0 = 0;  // decided
-                if (!__any_sync(0xffffffffu, k - c.sub + kG < len0)) break;
+                const bool more = k - c.sub + kG < len0;
+                if (!__any_sync(0xffffffffu, more)) break;
+                const unsigned far = group_ballot(c, spent > kMdBudget);
+                const bool big = more && !count && far;
+                if (__any_sync(0xffffffffu, big)) {
+                    const bool left = leave_to_cta(big, j);
+                    if (big && left) {
+                        mine = false;
+                        len0 = 0;
+                    } else if (big) {
+                        spent = INT32_MIN / 2;  // (no room: go on)
+                    }
+                }
             }
-            if (j >= 0) {
+            if (mine) {
                 if (count) {
                     if (c.sub == 0) v_cnt[j] = cnt;
                 } else if (rj.z == 0 || cnt >= aux.y) {
@@ -1259,40 +1330,16 @@ __device__ __noinline__ void md_test(bool count, int shard, int nshards) {
                           (!count || nshards == 1 || (j >> 7) % nshards == shard);
         __syncthreads();  // (v_o2c[j] is written below)
         if (!mine) continue;
-        const int4 rj = vrec[j], aux = v.vaux[j];
-        const int32_t e0 = aux.x, len0 = rj.z > 0 ? aux.w : 0;
-        if (rj.z > 0 && !count && len0 - 1 < aux.y) continue;
-        const uint32_t *row = v.row + aux.z;
-        const u64 *list = v.vedge + rj.w;
-        if (threadIdx.x == 0) sh->pos = 0;
-        __syncthreads();
-        // one member per warp, 32 hyperedges at a time
-#pragma unroll 1
-        for (int32_t k = c.warp; k < len0; k += blockDim.x >> 5) {
-            const uint32_t i = row[k];
-            bool ok = may_dominate(key_id(i), vrec[key_id(i)], j, rj);  // (all lanes alike)
-#pragma unroll 1
-            for (int32_t q0 = 0; q0 < rj.z && ok; q0 += 32) {
-                const int32_t q = q0 + c.lane;
-                const int32_t e = q < rj.z ? entry_id(list[q]) : e0;
-                const bool in = e == e0 || in_row(v, e, i);
-                __syncwarp();
-                ok = !__any_sync(0xffffffffu, !in);
-            }
-            if (ok && c.lane == 0) atomicAdd(&sh->pos, 1);
-            __syncwarp();
-            const bool decided = !count && vload(&sh->pos) >= aux.y;
-            if (__any_sync(0xffffffffu, decided)) break;
-        }
-        __syncthreads();
-        const int32_t cnt = sh->pos;
-        __syncthreads();  // (reset for the next)
-        if (count) {
-            if (threadIdx.x == 0) v_cnt[j] = cnt;
-        } else if (rj.z == 0 || cnt >= aux.y) {
-            delete_vertex(sh, j, rj, threadIdx.x, blockDim.x);
-        }
+        md_whole(j, count);
     }
+}
+
+// The vertices whose groups gave up.
+__device__ __noinline__ void md_big() {
+    const Shared *sh = shared();
+    const int32_t nb = min(sh->got.nbig, sh->task_cap);
+#pragma unroll 1
+    for (int32_t t = sh->rank; t < nb; t += sh->size) md_whole(sh->task[t].x, false);
 }
 
 // Sharded passes: the decision from the (merged) counts.
@@ -2120,6 +2167,11 @@ __device__ __noinline__ bool run_instance(int32_t limit, BatchCounters *ctr, SpT
                 md_test(false, 0, 1);
                 flush(&sh->del2, &rc->md);
                 if (!team_sync(rc)) return false;
+                if (sh->got.nbig > 0) {
+                    md_big();
+                    flush(&sh->del2, &rc->md);
+                    if (!team_sync(rc)) return false;
+                }
                 if (lead) sh->g.t_md += globaltimer();
                 md = sh->got.md;
             }
