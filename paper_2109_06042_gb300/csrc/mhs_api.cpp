@@ -474,16 +474,24 @@ constexpr double kSparseMeanSize = 256;
 bool sparse_pays(double cost, double open, double pairs) {
     return cost <= kSparseBase + kSparsePerPair * pairs && open <= kSparseBase + kOpenPerPair * pairs;
 }
+// Hyperedges of most of the vertices have next to no rare ones, and most pairs
+// pass the signatures (us; demands 1..4 / 1, and the contraction's):
+//   n 60, m 4,000, 80 % of the incidences     1,785 / 287    469
+//   n 250, m 1,000, 90 %                      1,650 / 943    587
+//   n 250, m 1,000, 60 %                        466 / 306    506
+constexpr double kDenseShare = 0.7, kDenseSize = 32;
 // A lower estimate of the cost before anything is loaded: every hyperedge
 // walks one list of mean length.
 bool sparse_may_pay(int32_t count, const int32_t *n, const int32_t *m, const int64_t *nnz) {
-    double cost = 0, pairs = 0, edges = 0, inc = 0;
+    double cost = 0, pairs = 0, edges = 0, inc = 0, cells = 0;
     for (int32_t b = 0; b < count; ++b) {
         if (n[b] > 0) cost += (double)m[b] * (double)nnz[b] / n[b];
         pairs += (double)m[b] * m[b] + (double)n[b] * n[b];
         edges += m[b];
         inc += (double)nnz[b];
+        cells += (double)m[b] * n[b];
     }
+    if (inc > kDenseShare * cells && inc >= kDenseSize * edges) return false;
     return inc <= kSparseMeanSize * edges && sparse_pays(cost / 4, 0, pairs);
 }
 

@@ -319,3 +319,18 @@ def test_vertices_of_nearly_equal_hyperedges(mhs, kind, c, h, m, f):
             hd.kernelize()
             _same(hd.result(0), ref)
             _same(hd.result(179), ref)
+
+
+@pytest.mark.parametrize("n,m,share,leaves", [(60, 2000, .85, True), (250, 500, .9, True),
+                                              (250, 500, .6, False), (30, 2000, .9, False)])
+def test_dense_hypergraphs_go_to_the_contraction(mhs, n, m, share, leaves):
+    rng = np.random.Generator(np.random.PCG64(n))
+    inst = I.from_edges(n, [np.nonzero(rng.random(n) < share)[0] for _ in range(m)],
+                        rng.integers(1, 3, m), k=4)
+    ref = mhs.kernelize(inst, contraction="popcount")
+    with mhs.Instance.load(inst) as h:
+        h.kernelize()
+        assert (h.work_stats()[1] > 0) == leaves
+        _same(h.result(), ref)
+    if inst.nnz <= 65536:
+        _noalloc(mhs, inst, ref)
