@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <functional>
 #include <vector>
 
 #include "mhs.h"
@@ -60,10 +61,13 @@ struct GroupItem {
     mhs_status status;               // of this request
 };
 // Reduces the group on the sparse path, all requests in the same launches, on
-// `stream` (synchronises it).  *again: the path does not pay for this group;
-// nothing has been written.  opt: contraction auto.
+// `stream` (synchronises it).  reserve is asked before anything is allocated:
+// may the group hold so many bytes on the device?  *again: it may not, or the
+// path does not pay for this group; nothing has been written.  opt: contraction
+// auto.
 mhs_status solve_sparse_group(const mhs_options &opt, cudaStream_t stream,
-                              std::vector<GroupItem> &group, bool *again);
+                              std::vector<GroupItem> &group,
+                              const std::function<bool(int64_t)> &reserve, bool *again);
 // Would MHS_CONTRACT_AUTO try the sparse path with these options?
 bool auto_takes_sparse(const mhs_options &opt);
 

@@ -498,7 +498,7 @@ bool sparse_may_pay(int32_t count, const int32_t *n, const int32_t *m, const int
 mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64_t *nnz,
                   const int64_t *k, const mhs_options *opt_in, void *cuda_stream,
                   mhs_instance **out, std::vector<Layout> &lay, int64_t &glob_off,
-                  bool sparse = false) {
+                  bool sparse = false, const std::function<bool(int64_t)> &reserve = nullptr) {
     mhs_options opt;
     mhs_status st = check_options(opt_in, &opt);
     if (st) return st;
@@ -650,6 +650,10 @@ mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64
     }
     const int64_t ctl_end = ar.bytes;
     glob_off = off_tmaps;
+    if (reserve && !reserve(ar.bytes + h->dense_bytes)) {
+        destroy(h);
+        return MHS_EBUSY;
+    }
 
     cudaMemPool_t pool;
     cudaError_t ce = pool_for(h->device, &pool);
@@ -1220,7 +1224,8 @@ mhs_status run_rounds(mhs_instance *h, int32_t limit, mhs_round_stats *stats) {
 bool mhs::auto_takes_sparse(const mhs_options &opt) { return auto_sparse(&opt); }
 
 mhs_status mhs::solve_sparse_group(const mhs_options &opt, cudaStream_t stream,
-                                   std::vector<GroupItem> &group, bool *again) {
+                                   std::vector<GroupItem> &group,
+                                   const std::function<bool(int64_t)> &reserve, bool *again) {
     const int count = (int)group.size();
     *again = false;
     if (count == 0) return MHS_OK;
@@ -1244,8 +1249,12 @@ mhs_status mhs::solve_sparse_group(const mhs_options &opt, cudaStream_t stream,
     std::vector<Layout> lay;
     int64_t tmoff = 0;
     mhs_instance *h = nullptr;
-    mhs_status st =
-        create(count, n.data(), m.data(), nnz.data(), k.data(), &opt, stream, &h, lay, tmoff, true);
+    mhs_status st = create(count, n.data(), m.data(), nnz.data(), k.data(), &opt, stream, &h, lay,
+                           tmoff, true, [&](int64_t b) { return reserve(b + sum_n + sum_m); });
+    if (st == MHS_EBUSY) {
+        *again = true;
+        return MHS_OK;
+    }
     if (st) return st;
     // page-locked staging: the inputs, array by array as in the arena, then
     // room for the masks

@@ -305,8 +305,10 @@ mhs_status admit(Lane &Ln, int si, std::shared_ptr<Request> req) {
 
 // Contraction auto: reduce the admitted requests together on the sparse path,
 // on the load stream and beside the lane's loop.  Returns the ones it does
-// not pay for, which take slots of the loop.  (The footprint reserved for a
-// request is that of the loop's dense form, which it may need.)
+// not pay for, which take slots of the loop.  The footprint reserved for a
+// request is that of the loop's dense form; what the group's lists need beyond
+// those is reserved for as long as it runs, and a group without room for it
+// takes slots.
 std::vector<std::shared_ptr<Request>> solve_group(Lane &Ln,
                                                   std::vector<std::shared_ptr<Request>> reqs) {
     mhs_server *S = Ln.S;
@@ -322,12 +324,30 @@ std::vector<std::shared_ptr<Request>> solve_group(Lane &Ln,
         std::lock_guard<std::mutex> lk(S->mu);
         Ln.active_count += (int32_t)reqs.size();
     }
+    int64_t extra = 0;
+    auto reserve = [&](int64_t bytes) {
+        for (auto &r : reqs) bytes -= r->footprint;
+        std::lock_guard<std::mutex> lk(S->mu);
+        extra = std::max<int64_t>(bytes, 0);
+        if (S->in_use + extra > S->opt.hbm_budget_bytes) {
+            extra = 0;
+            return false;
+        }
+        S->in_use += extra;
+        S->peak = std::max(S->peak, S->in_use);
+        return true;
+    };
     bool again = false;
-    const mhs_status st = solve_sparse_group(opt, Ln.load, group, &again);
+    const mhs_status st = solve_sparse_group(opt, Ln.load, group, reserve, &again);
     const int64_t t = now_ns();
     std::lock_guard<std::mutex> lk(S->mu);
     Ln.active_count -= (int32_t)reqs.size();
-    if (again) return reqs;
+    S->in_use -= extra;
+    if (again) {
+        if (extra)
+            for (auto &ln : S->lanes) ln.cv_work.notify_one();
+        return reqs;
+    }
     int32_t rounds = 0;
     for (size_t i = 0; i < reqs.size(); ++i) {
         Request &r = *reqs[i];

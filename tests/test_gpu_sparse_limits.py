@@ -334,3 +334,29 @@ def test_dense_hypergraphs_go_to_the_contraction(mhs, n, m, share, leaves):
         _same(h.result(), ref)
     if inst.nnz <= 65536:
         _noalloc(mhs, inst, ref)
+
+
+def test_server_budget_covers_the_lists(mhs):
+    """What a group of requests holds by candidate lists is reserved too, and
+    where the budget has no room for that, the device loop takes them."""
+    inst = I.uniform_random(100, 200, 2, 8, 3, 5, seed=1)
+    ref = O.reduce(inst)
+    lists = 16 * 16384 + 8 * 65536  # tasks and pairs of a request alone, at least
+    for budget in (0, 600 << 10):
+        with mhs.Server(hbm_budget_bytes=budget) as srv:
+            for _ in range(3):
+                _same(srv.poll(srv.submit(inst)), ref, budget)
+            st = srv.stats()
+        assert st["completed"] == 3 and st["bytes_in_use"] == 0
+        if budget:
+            assert st["peak_bytes"] <= budget
+        else:
+            assert st["peak_bytes"] >= lists
+    wide = I.uniform_random(256, 4000, 180, 200, 2, 5, seed=2)
+    for budget in (8 << 20, 64 << 20):
+        with mhs.Server(hbm_budget_bytes=budget) as srv:
+            tickets = [srv.submit(i) for i in (wide, inst, inst, wide, inst)]
+            for t, i in zip(tickets, (wide, inst, inst, wide, inst)):
+                _same(srv.poll(t), ref if i is inst else mhs.kernelize(wide), budget)
+            st = srv.stats()
+        assert st["peak_bytes"] <= budget and st["bytes_in_use"] == 0
