@@ -502,10 +502,11 @@ void mhs_free(mhs_instance *inst);
 mhs_status mhs_selftest_bounded_wait(int64_t limit_ns, int32_t *status_out,
                                      int64_t *waited_ns_out);
 /*
- * Diagnostic: from now on, in calls made by this thread that reduce a single
- * instance by candidate lists, the kernels' barriers (of two or more CTAs)
- * wait limit_ns (<= 2 s) for a CTA that never comes, so that such calls return
- * MHS_EDEVICE.  0: off, as at the start.
+ * Diagnostic: from now on, in calls made by this thread that reduce instances
+ * by candidate lists with two or more CTAs for each, the kernels' barriers wait
+ * limit_ns (<= 2 s) for a CTA that never comes, so that such calls return
+ * MHS_EDEVICE.  A server created by this thread meanwhile does the same, and
+ * its requests are reduced by the device loop.  0: off, as at the start.
  */
 mhs_status mhs_selftest_team_wait(int64_t limit_ns);
 

@@ -62,9 +62,9 @@ struct GroupItem {
 };
 // Reduces the group on the sparse path, all requests in the same launches, on
 // `stream` (synchronises it).  reserve is asked before anything is allocated:
-// may the group hold so many bytes on the device?  *again: it may not, or the
-// path does not pay for this group; nothing has been written.  opt: contraction
-// auto.
+// may the group hold so many bytes on the device?  *again: it may not, the path
+// does not pay for this group, or it failed in a way that need not be every
+// request's; nothing has been written.  opt: contraction auto.
 mhs_status solve_sparse_group(const mhs_options &opt, cudaStream_t stream,
                               std::vector<GroupItem> &group,
                               const std::function<bool(int64_t)> &reserve, bool *again);

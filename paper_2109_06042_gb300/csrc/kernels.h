@@ -168,6 +168,7 @@ cudaError_t launch_sparse_pass(InstState *st, int team, int op, int shard, int n
 // Self-test: barriers of the teams that this thread launches wait ns for a CTA
 // that never comes (0: off).
 void set_team_absent(uint64_t ns);
+uint64_t team_absent();
 
 // tcgen05 contraction (contract_tc.cu)
 cudaError_t launch_tc_contract(InstState *st, Plan *plan, BatchCounters *ctr, int phase, int sms,

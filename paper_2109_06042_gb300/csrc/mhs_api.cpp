@@ -1251,7 +1251,8 @@ mhs_status mhs::solve_sparse_group(const mhs_options &opt, cudaStream_t stream,
     mhs_instance *h = nullptr;
     mhs_status st = create(count, n.data(), m.data(), nnz.data(), k.data(), &opt, stream, &h, lay,
                            tmoff, true, [&](int64_t b) { return reserve(b + sum_n + sum_m); });
-    if (st == MHS_EBUSY) {
+    // (no memory for all of them together, or not from the budget: one by one)
+    if (st == MHS_EBUSY || st == MHS_ENOMEM) {
         *again = true;
         return MHS_OK;
     }
@@ -1350,6 +1351,12 @@ mhs_status mhs::solve_sparse_group(const mhs_options &opt, cudaStream_t stream,
     st = body();
     if (masks) cudaFreeAsync(masks, h->stream);
     destroy(h);
+    // one request's failed wait, or no memory for all of them together, fails none
+    // of the others (nothing has been written before the end)
+    if (st == MHS_ENOMEM || st == MHS_EDEVICE) {
+        *again = true;
+        return MHS_OK;
+    }
     return st;
 }
 

@@ -184,6 +184,7 @@ struct mhs_server {
     mhs_server_options opt{};
     int contraction = kFp8;
     bool sparse = false;      // contraction auto: requests are tried on the sparse path first
+    uint64_t absent_ns = 0;   // self-test (mhs_selftest_team_wait) of the creating thread
     int device = 0, sms = 0;
     cudaMemPool_t pool = nullptr;
     int64_t small_items = 0;  // n + m at most for the small-request lane
@@ -484,6 +485,7 @@ void worker_loop(Lane *L) {
     Lane &Ln = *L;
     mhs_server *S = Ln.S;
     cudaSetDevice(S->device);
+    set_team_absent(S->absent_ns);
     for (;;) {
         bool progress = false;
         // ---- admission: load into free slots, then mark them ready ----
@@ -829,6 +831,7 @@ mhs_status mhs_server_create(const mhs_server_options *opt_in, void *cuda_stream
         o.contraction = opt.contraction;
         o.sparsity = opt.sparsity;
         S->sparse = auto_takes_sparse(o);
+        S->absent_ns = team_absent();
     }
     // < 0: one lane for every request; 0: default split
     S->small_items = opt.small_items < 0 ? INT64_MAX : (opt.small_items == 0 ? 8192 : opt.small_items);

@@ -2432,5 +2432,6 @@ cudaError_t launch_sparse_pass(InstState *st, int team, int op, int shard, int n
 }
 
 void set_team_absent(uint64_t ns) { t_absent_ns = ns; }
+uint64_t team_absent() { return t_absent_ns; }
 
 }  // namespace mhs

@@ -360,3 +360,23 @@ def test_server_budget_covers_the_lists(mhs):
                 _same(srv.poll(t), ref if i is inst else mhs.kernelize(wide), budget)
             st = srv.stats()
         assert st["peak_bytes"] <= budget and st["bytes_in_use"] == 0
+
+
+def test_server_group_that_fails_goes_to_the_device_loop(mhs):
+    """An error of a group's launch is not every request's result."""
+    insts = [I.uniform_random(n, 2 * n, 2, 8, 3, 5, seed=n) for n in (300, 900, 2000)]
+    for fe in (False, True):
+        refs = [O.reduce_variant(i, "dp", fe) for i in insts]
+        mhs.selftest_team_wait(1_000_000)
+        srv = mhs.Server(full_edges=fe)
+        mhs.selftest_team_wait(0)
+        try:
+            for _ in range(2):
+                tickets = [srv.submit(i) for i in insts]
+                for t, ref in zip(tickets, refs):
+                    got = srv.poll(t)
+                    _same(got, ref)
+                    if fe:
+                        assert got["forced"].tolist() == ref["forced"].tolist()
+        finally:
+            srv.close()
