@@ -72,3 +72,17 @@ def test_repeated_ids_from_the_device(mhs):
         got = h.result()
     assert got["vertices"].tolist() == ref["vertices"].tolist()
     assert got["edges"].tolist() == ref["edges"].tolist() and got["rounds"] == ref["rounds"]
+
+
+@pytest.mark.parametrize("n", [1, 31, 126, 127, 128, 254, 255, 256, 1023, 1024, 2047, 2048, 4095, 4096, 4098])
+def test_vertices_in_all_hyperedges(mhs, n):
+    """MD passes that walk whole lists: bitmaps of 1, 2, 4 .. 32 quads of words
+    (a hyperedge per 1 .. 32 lanes) and more, lists of more than 512."""
+    rng = np.random.Generator(np.random.PCG64(n))
+    rows = [np.append(np.sort(rng.choice(n, min(n, 6), replace=False)), [n, n + 1]) for _ in range(1500)]
+    inst = I.from_edges(n + 2, rows, np.full(1500, 3), k=5)
+    ref = O.reduce(inst)
+    got = mhs.kernelize(inst, contraction="popcount")
+    for key in ("vertices", "edges", "demands"):
+        assert got[key].tolist() == ref[key].tolist(), key
+    assert got["rounds"] == ref["rounds"]

@@ -146,3 +146,20 @@ def test_loop_restarts_and_admits_while_running(mhs):
     for wave, results in done:
         for idx, (inst, res) in enumerate(zip(wave, results)):
             _same(res, O.reduce(inst), f"oracle {idx}")
+
+
+def test_device_loop_asked_for_by_name(mhs):
+    """contraction="fp8": every request takes a slot of the loop, which goes
+    idle, starts again and admits at its round boundaries."""
+    insts = [I.config_batch_one(9300 + i) for i in range(12)] + [I.config_powerlaw(7, n=2500, m=5000)]
+    refs = [O.reduce(i) for i in insts]
+    with mhs.Server(max_slots=8, contraction="fp8") as srv:
+        for _ in range(2):
+            tickets = []
+            for inst in insts:
+                tickets.append(srv.submit(inst))
+                time.sleep(0.002)
+            for idx, (res, ref) in enumerate(zip(_poll_all(srv, tickets), refs)):
+                _same(res, ref, f"oracle {idx}")
+            time.sleep(0.05)
+        assert srv.stats()["completed"] == 2 * len(insts)
