@@ -86,7 +86,6 @@ struct SpCtl {
     int32_t full;               // the next round takes every hyperedge and vertex
     int32_t loose;              // largest f_i - |e_i| over nonempty hyperedges (> 0), else 0
     int32_t pairs_full;         // the pair table ran out of places: its bounds are incomplete
-    int32_t leave;              // (build) a row that is not for this path
     SpRound fe;                 // deletions of an FE pass
     unsigned long long empty;   // empty hyperedges: largest f << 32 | ~index
     SpRound c[2];

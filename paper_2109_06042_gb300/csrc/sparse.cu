@@ -420,7 +420,7 @@ __device__ __forceinline__ bool pair_hit(const Shared *sh, uint32_t x, uint32_t 
 //   one hyperedge of 600, demand 600, among 20,000 of 10 over 700 vertices
 //                                                          124,935 /  811 / 549
 //   20,000 of 30 over 1,000 vertices, of demand |e|          3,650 /  881 / 652
-constexpr int32_t kPairRow = 6, kPairTest = 256;
+constexpr int32_t kPairRow = 6, kPairTest = 64;
 __device__ __forceinline__ bool many_heavy(const uint32_t *row, int32_t len, int32_t most) {
     return len > most && row[len - 1 - most] >= kHeavyKey;  // (they end the row)
 }
@@ -590,7 +590,6 @@ __device__ __noinline__ void dp_bounds_all(int shard, int nshards) {
     const View &v = c.sh->view;
     const int32_t loose = vload(&v.ctl->loose);
     const u64 empty = *reinterpret_cast<volatile u64 *>(&v.ctl->empty);
-    const bool pairs = c.full && !vload(&v.ctl->pairs_full);  // (else the walks find theirs)
     const int32_t *const e_o2c = v.e_o2c, *const eptr = v.eptr;
     const int4 *const erec = v.erec;
     const uint32_t *const rows = v.row;
@@ -626,9 +625,9 @@ __device__ __noinline__ void dp_bounds_all(int shard, int nshards) {
             hit = hit && fj != kGone;
             // every two heavy ones, unless decided
             int32_t end = 0;
-            if (pairs && __any_sync(0xffffffffu, heavy != 0)) {
+            if (__any_sync(0xffffffffu, heavy != 0)) {
                 heavy = group_sum(heavy);
-                end = group_ballot(c, hit) == 0 && heavy > 1 ? len : 0;
+                end = group_ballot(c, hit) == 0 && heavy > 1 && heavy <= kPairTest ? len : 0;
                 end = __shfl_sync(0xffffffffu, end, c.lead);
             }
             const int32_t maxend = __reduce_max_sync(0xffffffffu, end);
@@ -1469,7 +1468,7 @@ __device__ __forceinline__ void first_places(int32_t *at, int lane) {
 // 10,000 ids among 300 rows over 10,000 vertices: 1,196 / 1,225 by the contraction.
 constexpr int32_t kRankRow = 64;
 constexpr int32_t kSortRow = 65536;
-constexpr int32_t kLeave = 1 << 30;  // (beside the kErr* bits)
+constexpr int32_t kLeave = 1 << 30;  // (of the status, beside the kErr* bits)
 constexpr int32_t kLongRow = 1 << 29;
 constexpr int32_t kInOrder = -1;
 
@@ -1918,15 +1917,13 @@ __device__ __noinline__ bool build_instance(int32_t max_rounds, SpTotals *out) {
         [&](int32_t e) { bad |= count_row(c, v, evtx, f, place, local, n0, nnz0, e); });
     if (kLong && __any_sync(0xffffffffu, bad & kLongRow))
         bad = (bad & ~kLongRow) | count_long_rows();
-    if (bad & ~kLeave) atomicOr(&s.status, bad & ~kLeave);
-    if (kLong && (bad & kLeave)) v.ctl->leave = 1;
+    if (bad) atomicOr(&s.status, bad);
     if (!team_sync()) return false;
     if (const int32_t st = vload(&s.status)) {
-        if (t0 == 0 && !(st & kLongRow)) atomicOr(&out->status, st);
-        return true;
-    }
-    if (kLong && vload(&v.ctl->leave)) {
-        if (t0 == 0) out->leave = 1;
+        if (t0 == 0 && !(st & kLongRow)) {
+            if (st == kLeave) out->leave = 1;
+            else atomicOr(&out->status, st & ~kLeave);
+        }
         return true;
     }
     // a place for every vertex's list (in any order): one atomic per warp
@@ -2330,10 +2327,10 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
                     uint64_t absent_ns) {
     Shared *sh = shared();
     bool ok = true;
-    if (masks.built &&
-        (masks.built->status || masks.built->leave ||
-         masks.built->cost + masks.built->open > masks.max_cost))
-        return;
+    if (masks.built) {  // (all words on their way together)
+        const SpTotals b = *masks.built;
+        if ((b.status | b.leave) | (int)(b.cost + b.open > masks.max_cost)) return;
+    }
     if (team > 0) {
         start(st + blockIdx.x / team, blockIdx.x % team, team, absent_ns);
         ok = run_instance(limit, ctr, times);
