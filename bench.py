@@ -551,10 +551,12 @@ def run_ours(args, rank, world, dist):
     # the DP contraction, k_compact_edges, k_plan, the fused A clear / A^T set
     # scatter, [k_tile_list], the MD contraction, the A^T clear scatter,
     # k_compact_vertices and the loop-condition kernel ([] tcgen05 only), plus
-    # the three FE kernels with --full-edges.  FP8 from 8,000 hyperedges on: the
-    # three kernels of the vertex bounds, once.
+    # the three FE kernels with --full-edges.  FP8 from 8,000 hyperedges on, up
+    # to a mean size of 24: the three kernels of the vertex bounds, once.
     load_kernels = 11 + (2 if batch else 0)
-    if args.contraction == "fp8" and (sum if batch else max)(i.m for i in insts) >= 8000:
+    edges = (sum if batch else max)(i.m for i in insts)
+    size = sum(i.nnz for i in insts) / max(sum(i.m for i in insts), 1)
+    if args.contraction == "fp8" and edges >= 8000 and size <= 24:
         load_kernels += 3
     per_round = (12 if args.contraction == "fp8" else 10) + (3 if args.full_edges else 0)
     line = {

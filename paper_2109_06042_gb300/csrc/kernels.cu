@@ -951,12 +951,12 @@ __device__ int32_t chain_exclusive(unsigned long long *status, uint32_t epoch, i
 
 // ---------------------------------------------------------- vertex bounds --
 //
-// tcgen05 path, first round (every hyperedge is a candidate): e_i supersedes every e_j that shares one vertex with it and
-// has f_j <= f_i - |e_i| + 1, so the largest such bound of each vertex (in
-// v_maxf, free until MD) deletes most of what the pass deletes, in two walks
-// over the incidences, before the operand is built.  "Supersedes or wins the
-// tie" is transitive, so the rest of the pass gives the same result without
-// them.  (|e_j| = 1: f_j < the bound, its own included; equal ones are left to
+// tcgen05 path, first round (every hyperedge is a candidate): e_i supersedes
+// every e_j that shares one vertex with it and has f_j <= f_i - |e_i| + 1, so
+// the largest such bound of each vertex (in v_maxf, free until MD) deletes most
+// of what the pass deletes, in two walks over the incidences, before the operand
+// is built.  "Supersedes or wins the tie" is transitive, so the rest of the pass
+// gives the same result without them.  (|e_j| = 1: f_j < the bound, its own included; equal ones are left to
 // the contraction.  Rule SE: only hyperedges of one vertex bound.)  A vertex
 // listed twice makes a size too large, which only weakens a bound; one vertex
 // alone is told by its smallest and largest position.
@@ -1548,8 +1548,8 @@ __global__ void __launch_bounds__(32 * kPopWarps, kPopDpBlocks)
 // bitmap takes as many lanes as it has quads of words (a power of two), and the
 // warp 4 x 32 / lanes hyperedges at a time: few vertices of high degree have
 // only their own warps.  (n 66, m 100,000, two vertices in all hyperedges: the
-// pass 6.4 ms with the whole warp on 4 hyperedges, 1.2 now; as 128 x 128 tiles of
-// bit counts 0.7, with a DP pass of 39 instead of 4.6.)
+// pass 6.4 ms with the whole warp on 4 hyperedges, 1.2 now; as tiles of bit
+// counts 0.7, with a DP pass of 39 instead of 4.6.)
 __global__ void __launch_bounds__(32 * kPopWarps, kPopMdBlocks)
     k_pop_md(InstState *st, const Plan *plan, int shard, int nshards) {
     __shared__ int32_t ids_all[kPopWarps][kPopIds];

@@ -380,3 +380,24 @@ def test_server_group_that_fails_goes_to_the_device_loop(mhs):
                         assert got["forced"].tolist() == ref["forced"].tolist()
         finally:
             srv.close()
+
+
+@pytest.mark.parametrize("fe", [False, True])
+def test_server_group_that_does_not_pay(mhs, fe):
+    """Requests whose build says that the lists do not pay, alone and among
+    others: all of the group take slots of the device loop."""
+    rng = np.random.Generator(np.random.PCG64(55))
+    wide = I.from_edges(300, [np.sort(rng.choice(300, rng.integers(20, 61), replace=False))
+                              for _ in range(3000)], rng.integers(1, 21, 3000), k=4)
+    with mhs.Instance.load(wide) as h:
+        h.kernelize()
+        assert h.work_stats()[1] > 0  # contracted
+    insts = [wide, I.uniform_random(400, 900, 2, 8, 3, 5, seed=3), I.uniform_random(90, 200, 2, 5, 3, 5, seed=4)]
+    refs = [mhs.kernelize(i, contraction="popcount", full_edges=fe) for i in insts]
+    with mhs.Server(full_edges=fe) as srv:
+        _same(srv.poll(srv.submit(wide)), refs[0])
+        srv.pause(True)
+        tickets = [srv.submit(i) for i in insts]
+        srv.pause(False)
+        for t, ref in zip(tickets, refs):
+            _same(srv.poll(t), ref)
