@@ -16,6 +16,7 @@
 // Per instance that reached its DP/MD fixpoint in this round (fe_stage = 1):
 //   k_fe_mark     full hyperedges -> e_del; their alive vertices -> v_del (S)
 //   k_fe_apply    other hyperedges: f -= |e & S|; f <= 0 -> e_del
+//                 (a vertex listed twice in a hyperedge counts once)
 //   k_fe_compact  order-preserving compaction of both, forced[] += S, k -= |S|;
 //                 if anything went the instance runs more rounds, otherwise
 //                 it is finished.
@@ -35,9 +36,8 @@ __global__ void k_fe_mark(InstState *st, int count) {
     if (!s.fe_stage || s.status) return;
     for (int32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < s.m; r += gridDim.x * blockDim.x) {
         const int32_t e = s.e_c2o[r];
-        int32_t size = 0;
-        for (int32_t p = s.eptr[e]; p < s.eptr[e + 1]; ++p) size += s.v_o2c[s.evtx[p]] >= 0;
-        if (size != s.f[e]) continue;
+        // (the last DP pass's size: no vertex went since; repeated ids count once)
+        if (s.e_s[r] != s.f[e]) continue;
         s.e_del[r] = 1;
         for (int32_t p = s.eptr[e]; p < s.eptr[e + 1]; ++p) {
             const int32_t cv = s.v_o2c[s.evtx[p]];
@@ -54,11 +54,21 @@ __global__ void k_fe_apply(InstState *st, int count) {
     for (int32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < s.m; r += gridDim.x * blockDim.x) {
         if (s.e_del[r]) continue;  // full: goes whole
         const int32_t e = s.e_c2o[r];
-        int32_t lost = 0;
-        for (int32_t p = s.eptr[e]; p < s.eptr[e + 1]; ++p) {
+        const int32_t p0 = s.eptr[e], p1 = s.eptr[e + 1];
+        int32_t lost = 0, alive = 0;
+        for (int32_t p = p0; p < p1; ++p) {
             const int32_t cv = s.v_o2c[s.evtx[p]];
+            alive += cv >= 0;
             lost += cv >= 0 && s.v_del[cv];
         }
+        if (lost && alive != s.e_s[r])  // some vertex is listed twice
+            for (int32_t p = p0; p < p1; ++p) {
+                const int32_t v = s.evtx[p], cv = s.v_o2c[v];
+                if (cv < 0 || !s.v_del[cv]) continue;
+                int32_t q = p0;
+                while (s.evtx[q] != v) ++q;
+                lost -= q < p;
+            }
         if (lost) {
             s.f[e] -= lost;
             if (s.f[e] <= 0) s.e_del[r] = 1;

@@ -65,3 +65,27 @@ def test_vertex_bounds_leave_long_rows_to_the_contraction(mhs, rule, long):
     for key in ("vertices", "edges", "demands"):
         assert got[key].tolist() == ref[key].tolist(), key
     assert got["rounds"] == ref["rounds"]
+
+
+@pytest.mark.parametrize("contraction", ["fp8", "popcount", "auto"])
+@pytest.mark.parametrize("rule", ["dp", "se"])
+def test_full_edges_with_vertices_listed_twice(mhs, contraction, rule):
+    """Device rows with repeats: a vertex counts once for a hyperedge's size and
+    for the demand that it loses."""
+    import torch
+    rng = np.random.Generator(np.random.PCG64(16))
+    for n, m, top in ((30, 40, 6), (60, 12, 50), (400, 900, 8), (252, 1, 214), (90, 300, 70)):
+        rows = [rng.choice(n, rng.integers(1, top + 1), replace=False) for _ in range(m)]
+        dem = [max(1, len(r) - int(rng.integers(0, 3))) for r in rows]
+        inst = I.from_edges(n, [sorted(r.tolist()) for r in rows], dem, k=9)
+        ref = O.reduce_variant(inst, rule, True)
+        rep = [rng.permutation(np.concatenate([r, r[:rng.integers(0, len(r) + 1)], r[:1]])) for r in rows]
+        d = [torch.from_numpy(np.ascontiguousarray(x, np.int32)).cuda()
+             for x in (np.concatenate([[0], np.cumsum([len(r) for r in rep])]), np.concatenate(rep), inst.demand)]
+        with mhs.Instance.load_device(n, m, *d, 9, contraction=contraction, rule=rule, full_edges=True) as h:
+            h.kernelize()
+            got = h.result()
+            assert h.forced()[0].tolist() == ref["forced"].tolist()
+        for key in ("vertices", "edges", "demands"):
+            assert got[key].tolist() == ref[key].tolist(), (key, n, m)
+        assert got["k"] == ref["k"] and got["rounds"] == ref["rounds"]
