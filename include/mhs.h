@@ -73,8 +73,10 @@ typedef enum {
     MHS_CONTRACT_AUTO = 0,     /* library choice: sparse hypergraphs by candidate lists (the pairs
                                   that can fire, found from the incidence lists; no contraction),
                                   others, and those whose tile shape or sparsity the options
-                                  name, as MHS_CONTRACT_FP8 */
-    MHS_CONTRACT_FP8 = 1,      /* tcgen05 tensor cores, E4M3 0/1, FP32 accumulate */
+                                  name, as MHS_CONTRACT_FP8; without such options, and with a
+                                  demand of 2^23 or more, as MHS_CONTRACT_POPCOUNT */
+    MHS_CONTRACT_FP8 = 1,      /* tcgen05 tensor cores, E4M3 0/1, FP32 accumulate; demands of
+                                  2^23 and more may be rounded */
     MHS_CONTRACT_POPCOUNT = 2  /* bit-packed, on the integer units */
 } mhs_contraction;
 

@@ -84,6 +84,7 @@ __global__ void k_validate(InstState *st, int count) {
     for (int64_t e = tid; e < s.m0; e += stride) {
         if (s.eptr[e + 1] < s.eptr[e]) atomicOr(&s.status, kErrBadPtr);
         if (s.f[e] < 1) atomicOr(&s.status, kErrBadDemand);
+        if (s.f[e] >= kBigDemand) s.big_demand = 1;
     }
     for (int64_t p = tid; p < s.nnz0; p += stride) {
         int32_t v = s.evtx[p];
@@ -91,12 +92,12 @@ __global__ void k_validate(InstState *st, int count) {
     }
 }
 
-// OR of the instances' status words, so that a batch load reads back one
-// word instead of every instance's state.
+// OR of the instances' status words (and kSawBigDemand), so that a batch load
+// reads back one word instead of every instance's state.
 __global__ void k_status_or(const InstState *st, int count, int32_t *out) {
     int32_t x = 0;
     for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < count; b += gridDim.x * blockDim.x)
-        x |= st[b].status;
+        x |= st[b].status | (st[b].big_demand ? kSawBigDemand : 0);
     x = __reduce_or_sync(0xffffffffu, x);
     if ((threadIdx.x & 31) == 0 && x) atomicOr(out, x);
 }

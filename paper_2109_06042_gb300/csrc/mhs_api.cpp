@@ -495,6 +495,21 @@ bool sparse_may_pay(int32_t count, const int32_t *n, const int32_t *m, const int
     return inc <= kSparseMeanSize * edges && sparse_pays(cost / 4, 0, pairs);
 }
 
+// What MHS_CONTRACT_AUTO takes where the lists do not pay: the tensor cores, or,
+// with demands that FP32 tests may round, the bit-packed form (32-bit integers).
+mhs_options exact_form(const mhs_options *opt) {
+    mhs_options o;
+    mhs_default_options(&o);
+    if (opt) o = *opt;
+    o.contraction = MHS_CONTRACT_POPCOUNT;
+    return o;
+}
+bool any_big(const int32_t *demand, int64_t m) {
+    int32_t top = 0;
+    for (int64_t e = 0; e < m; ++e) top = std::max(top, demand[e]);
+    return top >= kBigDemand;
+}
+
 mhs_status create(int32_t count, const int32_t *n, const int32_t *m, const int64_t *nnz,
                   const int64_t *k, const mhs_options *opt_in, void *cuda_stream,
                   mhs_instance **out, std::vector<Layout> &lay, int64_t &glob_off,
@@ -1403,7 +1418,10 @@ mhs_status mhs_load(int32_t n, int32_t m, const int32_t *edge_ptr, const int32_t
     size_t stage_cls = 0;
     bool checked = false;
     bool sparse = auto_sparse(opt) && sparse_may_pay(1, &n, &m, &nnz);
+    const mhs_options exact = exact_form(opt);
+    const bool choose = auto_sparse(opt);
     for (;;) {
+        if (choose && !sparse && any_big(demand, m)) opt = &exact;
         std::vector<Layout> lay;
         int64_t tmoff = 0;
         mhs_instance *h = nullptr;
@@ -1483,7 +1501,9 @@ mhs_status mhs_load_device(int32_t n, int32_t m, const int32_t *edge_ptr, const 
     if (nnz32 < 0) return fail(MHS_EINVAL, "edge_ptr[m] < 0");
     if (nnz32 > 0 && !edge_vtx) return fail(MHS_EINVAL, "edge_vtx is NULL");
     int64_t nnz = nnz32;
-    for (bool sparse = auto_sparse(opt) && sparse_may_pay(1, &n, &m, &nnz);; sparse = false) {
+    const mhs_options exact = exact_form(opt);
+    const bool choose = auto_sparse(opt);
+    for (bool sparse = choose && sparse_may_pay(1, &n, &m, &nnz);; sparse = false) {
         std::vector<Layout> lay;
         int64_t tmoff = 0;
         mhs_instance *h = nullptr;
@@ -1514,10 +1534,12 @@ mhs_status mhs_load_device(int32_t n, int32_t m, const int32_t *edge_ptr, const 
             e = cudaMemcpyAsync(h->dstate, h->hstate.data(), sizeof(InstState),
                                 cudaMemcpyHostToDevice, h->stream);
         if (e == cudaSuccess) e = launch_validate(h->dstate, 1, h->stream);
-        int32_t status = 0;
+        int32_t words[2] = {0, 0};  // status, big_demand
+        static_assert(offsetof(InstState, big_demand) == offsetof(InstState, status) + 4, "one copy");
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(&status, &h->dstate->status, 4, cudaMemcpyDeviceToHost, h->stream);
+            e = cudaMemcpyAsync(words, &h->dstate->status, 8, cudaMemcpyDeviceToHost, h->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        const int32_t status = words[0];
         if (e != cudaSuccess) {
             destroy(h);
             return fail(MHS_ECUDA, "device load failed: %s", cudaGetErrorString(e));
@@ -1526,6 +1548,11 @@ mhs_status mhs_load_device(int32_t n, int32_t m, const int32_t *edge_ptr, const 
             destroy(h);
             return fail(MHS_EINVAL, "malformed device instance (status 0x%x: %s)", status,
                         status_text(status));
+        }
+        if (choose && words[1] && opt != &exact) {
+            destroy(h);
+            opt = &exact;
+            continue;
         }
         st = finish_load(h, tmoff);  // device inputs: nothing to wait for before returning
         if (st) {
@@ -1637,8 +1664,11 @@ mhs_status mhs_load_batch(int32_t count, const int32_t *n, const int32_t *m,
         return st ? st : fail(MHS_EINVAL, "%s: malformed", what);
     };
     std::vector<int32_t> local_ptr;  // (without staging) local int32 offsets
-    bool sparse = auto_sparse(opt) && sparse_may_pay(count, n, m, nnz.data());
+    const bool choose = auto_sparse(opt);
+    bool sparse = choose && sparse_may_pay(count, n, m, nnz.data());
+    const mhs_options exact = exact_form(opt);
     for (bool first = true;; first = false, sparse = false) {
+        if (choose && !sparse && any_big(demand, sum_m)) opt = &exact;
         std::vector<Layout> lay;
         int64_t tmoff = 0;
         mhs_instance *h = nullptr;
@@ -1772,7 +1802,9 @@ mhs_status mhs_load_batch_device(int32_t count, const int32_t *n, const int32_t 
         cudaFreeAsync(tmp, cs);
         return fail(MHS_EINVAL, "edge_vtx is NULL");
     }
-    for (bool sparse = auto_sparse(opt) && sparse_may_pay(count, n, m, nnz.data());; sparse = false) {
+    const mhs_options exact = exact_form(opt);
+    const bool choose = auto_sparse(opt);
+    for (bool sparse = choose && sparse_may_pay(count, n, m, nnz.data());; sparse = false) {
         std::vector<Layout> lay;
         int64_t tmoff = 0;
         mhs_instance *h = nullptr;
@@ -1813,12 +1845,17 @@ mhs_status mhs_load_batch_device(int32_t count, const int32_t *n, const int32_t 
             e = cudaMemcpyAsync(&hany, any_status, sizeof(int32_t), cudaMemcpyDeviceToHost,
                                 h->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        if (e == cudaSuccess && choose && hany == kSawBigDemand && opt != &exact) {
+            destroy(h);
+            opt = &exact;
+            continue;
+        }
         cudaFreeAsync(tmp, h->stream);
         if (e != cudaSuccess) {
             destroy(h);
             return fail(MHS_ECUDA, "batch device load: %s", cudaGetErrorString(e));
         }
-        if (hany) {  // some instance is malformed: read the states to name the first
+        if (hany & ~kSawBigDemand) {  // some instance is malformed: read the states to name the first
             std::vector<InstState> chk(count);
             e = cudaMemcpyAsync(chk.data(), h->dstate, sizeof(InstState) * count,
                                 cudaMemcpyDeviceToHost, h->stream);

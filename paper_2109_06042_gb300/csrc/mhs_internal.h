@@ -33,6 +33,11 @@ constexpr int kTraceRounds = 32; // rounds whose sizes an instance records
 // (kSparse: no contraction; what MHS_CONTRACT_AUTO takes for sparse hypergraphs)
 enum Contraction : int32_t { kAuto = 0, kFp8 = 1, kPopcount = 2, kSparse = 3 };
 
+// Demands from here on may be rounded by the contraction's FP32 tests (sums of a
+// demand, a size and a count must stay below 2^24).
+constexpr int32_t kBigDemand = 1 << 23;
+constexpr int32_t kSawBigDemand = 1 << 28;  // beside the bits below, from launch_status_or
+
 // Status bits written by kernels (OR-ed into InstState::status).
 enum : int32_t {
     kErrBadVertex = 1,     // vertex id out of range in the input
@@ -119,6 +124,7 @@ struct InstState {
     int32_t dp_deleted, md_deleted;
     int32_t bounds_deleted; // of the running DP pass: deleted before its operand was built
     int32_t status;        // kErr* bits
+    int32_t big_demand;    // (validation of device inputs) some demand is kBigDemand or more
     int32_t layout_sorted; // 0: input order; 1: hyperedges by smallest vertex id;
                            // 2: vertices by degree class, hyperedges by smallest vertex position
 

@@ -73,6 +73,7 @@ struct Request {
     int64_t footprint = 0;
     int64_t tiles = 0;  // most tile-list entries one of its phases can need
     int64_t t_submit = 0, t_admit = 0, t_done = 0;
+    bool big = false;       // a demand that the contraction's FP32 tests may round
     bool done = false;
     mhs_status status = MHS_OK;
     std::vector<int32_t> vout, eout, dout, forced;
@@ -304,6 +305,21 @@ mhs_status admit(Lane &Ln, int si, std::shared_ptr<Request> req) {
     return MHS_OK;
 }
 
+// A request that leaves the device: its books.  Under S->mu.
+void complete_locked(Lane &Ln, Request &r, mhs_status st) {
+    mhs_server *S = Ln.S;
+    if (r.done) return;  // (failed by a shutdown)
+    r.status = st;
+    r.t_done = now_ns();
+    r.done = true;
+    r.ptr.clear();
+    r.vtx.clear();
+    r.dem.clear();
+    ++S->completed;
+    S->in_use -= r.footprint;
+    Ln.tiles_in_use -= r.tiles;
+}
+
 // Contraction auto: reduce the admitted requests together on the sparse path,
 // on the load stream and beside the lane's loop.  Returns the ones it does
 // not pay for, which take slots of the loop.  The footprint reserved for a
@@ -340,7 +356,6 @@ std::vector<std::shared_ptr<Request>> solve_group(Lane &Ln,
     };
     bool again = false;
     const mhs_status st = solve_sparse_group(opt, Ln.load, group, reserve, &again);
-    const int64_t t = now_ns();
     std::lock_guard<std::mutex> lk(S->mu);
     Ln.active_count -= (int32_t)reqs.size();
     S->in_use -= extra;
@@ -353,23 +368,63 @@ std::vector<std::shared_ptr<Request>> solve_group(Lane &Ln,
     for (size_t i = 0; i < reqs.size(); ++i) {
         Request &r = *reqs[i];
         if (r.done) continue;  // (failed by a shutdown)
-        r.status = st ? st : group[i].status;
         r.rounds = group[i].rounds;
         r.k = group[i].k;
         rounds = std::max(rounds, r.rounds);
-        r.t_done = t;
-        r.done = true;
-        r.ptr.clear();
-        r.vtx.clear();
-        r.dem.clear();
-        ++S->completed;
-        S->in_use -= r.footprint;
-        Ln.tiles_in_use -= r.tiles;
+        complete_locked(Ln, r, st ? st : group[i].status);
     }
     S->group_rounds += rounds;
     S->cv_done.notify_all();
     for (auto &ln : S->lanes) ln.cv_work.notify_one();
     return {};
+}
+
+// Contraction auto, a demand that the loop's FP32 tests may round, and lists that
+// do not pay: the request alone, bit-packed (an eighth of the footprint reserved).
+void solve_alone(Lane &Ln, Request &r) {
+    mhs_server *S = Ln.S;
+    mhs_options opt;
+    mhs_default_options(&opt);
+    opt.contraction = MHS_CONTRACT_POPCOUNT;
+    opt.edge_rule = S->opt.edge_rule;
+    opt.full_edges = S->opt.full_edges;
+    {
+        std::lock_guard<std::mutex> lk(S->mu);
+        ++Ln.active_count;
+    }
+    mhs_instance *h = nullptr;
+    std::vector<int32_t> v, e, d, forced;
+    int32_t n = 0, m = 0, rounds = 0, taken = 0;
+    int64_t k = r.k;
+    mhs_status st = mhs_load(r.n, r.m, r.ptr.data(), r.vtx.data(), r.dem.data(), r.k, &opt, Ln.load, &h);
+    if (st == MHS_OK) st = mhs_kernelize(h, nullptr);
+    if (st == MHS_OK) st = mhs_result(h, nullptr, 0, &n, nullptr, nullptr, 0, &m, &k, &rounds);
+    if (st == MHS_OK) {
+        v.resize(n);
+        e.resize(m);
+        d.resize(m);
+        if (n || m) st = mhs_result(h, v.data(), n, &n, e.data(), d.data(), m, &m, &k, &rounds);
+    }
+    if (st == MHS_OK && opt.full_edges) st = mhs_forced_at(h, 0, nullptr, 0, &taken, nullptr);
+    if (st == MHS_OK && taken) {
+        forced.resize(taken);
+        st = mhs_forced_at(h, 0, forced.data(), taken, &taken, nullptr);
+    }
+    mhs_free(h);
+    std::lock_guard<std::mutex> lk(S->mu);
+    --Ln.active_count;
+    if (!r.done) {
+        r.vout = std::move(v);
+        r.eout = std::move(e);
+        r.dout = std::move(d);
+        r.forced = std::move(forced);
+        r.rounds = rounds;
+        r.k = k;
+        S->group_rounds += rounds;
+        complete_locked(Ln, r, st);
+    }
+    S->cv_done.notify_all();
+    for (auto &ln : S->lanes) ln.cv_work.notify_one();
 }
 
 // Fail every request that has not finished (device error or shutdown).
@@ -523,10 +578,17 @@ void worker_loop(Lane *L) {
         }
         std::vector<int> loaded;
         if (S->sparse && !to_admit.empty()) {
-            std::vector<std::shared_ptr<Request>> reqs;
-            for (auto &p : to_admit) reqs.push_back(p.second);
+            std::vector<std::shared_ptr<Request>> reqs, big;
+            for (auto &p : to_admit) (p.second->big ? big : reqs).push_back(p.second);
             progress = true;
-            if (solve_group(Ln, std::move(reqs)).empty()) to_admit.clear();
+            if (!reqs.empty() && solve_group(Ln, std::move(reqs)).empty())
+                to_admit.clear();
+            else
+                to_admit.erase(std::remove_if(to_admit.begin(), to_admit.end(),
+                                              [](auto &p) { return p.second->big; }),
+                               to_admit.end());
+            if (!big.empty())
+                for (auto &r : solve_group(Ln, std::move(big))) solve_alone(Ln, *r);
         }
         for (auto &p : to_admit) {
             mhs_status st = admit(Ln, p.first, p.second);
@@ -877,10 +939,12 @@ mhs_status mhs_submit(mhs_server *S, int32_t n, int32_t m, const int32_t *edge_p
     if (nnz > 0 && !edge_vtx) return set_error(MHS_EINVAL, "edge_vtx is NULL");
     // structural checks on the host, before anything is queued
     std::vector<int32_t> mark;
+    bool big = false;
     for (int32_t e = 0; e < m; ++e) {
         if (edge_ptr[e + 1] < edge_ptr[e])
             return set_error(MHS_EINVAL, "edge_ptr decreases at hyperedge %d", e);
         if (demand[e] < 1) return set_error(MHS_EINVAL, "demand of hyperedge %d is < 1", e);
+        big |= demand[e] >= kBigDemand;
         const int32_t a = edge_ptr[e], b = edge_ptr[e + 1];
         if (a == b || ascending_row(edge_vtx + a, b - a, n)) continue;
         if (mark.empty()) mark.assign((size_t)n, -1);
@@ -896,6 +960,7 @@ mhs_status mhs_submit(mhs_server *S, int32_t n, int32_t m, const int32_t *edge_p
     r->n = n;
     r->m = m;
     r->k = k;
+    r->big = big;
     r->ptr.assign(edge_ptr, edge_ptr + m + 1);
     r->vtx.assign(edge_vtx, edge_vtx + nnz);
     r->dem.assign(demand, demand + m);

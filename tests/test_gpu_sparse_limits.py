@@ -401,3 +401,52 @@ def test_server_group_that_does_not_pay(mhs, fe):
         srv.pause(False)
         for t, ref in zip(tickets, refs):
             _same(srv.poll(t), ref)
+
+
+@pytest.mark.parametrize("rule,fe", VARIANTS)
+def test_large_demands_where_the_lists_do_not_pay(mhs, rule, fe):
+    """Demands that FP32 tests would round are decided in 32-bit integers by
+    every entry point that chooses its form itself."""
+    import torch
+    rng = np.random.Generator(np.random.PCG64(23))
+    insts = []
+    for n, m, lo, hi in ((60, 300, 40, 60), (300, 3000, 20, 60), (700, 60, 300, 500), (200, 300, 2, 9)):
+        rows = [np.sort(rng.choice(n, rng.integers(lo, hi + 1), replace=False)) for _ in range(m)]
+        top = int(rng.choice([2**23, 2**25, 2**30, TOP - 40]))
+        insts.append(I.from_edges(n, rows, top + rng.integers(0, 40, m), k=4))
+        insts.append(I.from_edges(n, rows, rng.choice([1, 2, top, top + 3], m), k=4))
+    opts = {"rule": rule, "full_edges": fe}
+    refs = [O.reduce_variant(i, rule, fe) for i in insts]
+    for b, (inst, ref) in enumerate(zip(insts, refs)):
+        _same(mhs.kernelize(inst, **opts), ref, f"host {b}")
+        d = _dev(inst.edge_ptr, inst.edge_vtx, inst.demand)
+        with mhs.Instance.load_device(inst.n, inst.m, *d, inst.k, **opts) as h:
+            h.kernelize()
+            assert h.work_stats() == (0, 0)
+            _same(h.result(), ref, f"device {b}")
+        for part in ([inst], [inst, insts[-1]]):
+            with mhs.Instance.load_batch(part, **opts) as h:
+                h.kernelize()
+                _same(h.result(0), ref, f"batch {b}")
+            n, m = (np.array([getattr(i, x) for i in part], np.int32) for x in "nm")
+            ptr = torch.from_numpy(np.concatenate(
+                [[0], np.cumsum(np.concatenate([np.diff(i.edge_ptr) for i in part]))])).cuda()
+            vtx, dem = _dev(np.concatenate([i.edge_vtx for i in part]),
+                            np.concatenate([i.demand for i in part]))
+            k = np.array([i.k for i in part], np.int64)
+            with mhs.Instance.load_batch_device(n, m, k, ptr, vtx, dem, **opts) as h:
+                h.kernelize()
+                _same(h.result(0), ref, f"device batch {b}")
+    small = I.uniform_random(400, 900, 2, 8, 3, 5, seed=3)
+    sref = O.reduce_variant(small, rule, fe)
+    with mhs.Server(**opts) as srv:
+        srv.pause(True)
+        tickets = [srv.submit(i) for i in insts + [small]]
+        srv.pause(False)
+        for b, (t, ref) in enumerate(zip(tickets, refs + [sref])):
+            got = srv.poll(t)
+            _same(got, ref, f"server {b}")
+            if fe:
+                assert got["forced"].tolist() == ref["forced"].tolist()
+        st = srv.stats()
+    assert st["completed"] == len(tickets) and st["active"] == 0 and st["bytes_in_use"] == 0
