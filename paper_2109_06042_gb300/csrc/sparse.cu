@@ -418,8 +418,8 @@ __device__ __forceinline__ bool pair_hit(const Shared *sh, uint32_t x, uint32_t 
 // Every pair of every row, as far as the table had room, took (load and
 // kernelization, us; so / now / by the contraction):
 //   one hyperedge of 600, demand 600, among 20,000 of 10 over 700 vertices
-//                                                          124,935 /  811 / 549
-//   20,000 of 30 over 1,000 vertices, of demand |e|          3,650 /  881 / 652
+//                                                          124,935 /  721 / 549
+//   20,000 of 30 over 1,000 vertices, of demand |e|          3,650 /  858 / 652
 constexpr int32_t kPairRow = 6, kPairTest = 64;
 __device__ __forceinline__ bool many_heavy(const uint32_t *row, int32_t len, int32_t most) {
     return len > most && row[len - 1 - most] >= kHeavyKey;  // (they end the row)
