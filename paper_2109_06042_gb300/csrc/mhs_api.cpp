@@ -929,8 +929,7 @@ mhs_status finish_load(mhs_instance *h, int64_t tmap_off) {
 }
 
 // Sparse path, once the inputs are on their way: the states, the build
-// kernel, and what it found.  Synchronises.  *pays: the instance stays on
-// this path.
+// kernel, and what it found.  Synchronises.  *pays: by the rule above.
 mhs_status build_sparse(mhs_instance *h, SpTotals *found, bool *pays) {
     SpTotals *host = reinterpret_cast<SpTotals *>(h->pin + 128);
     CUDA_TRY(launch_sparse_build(h->dstate, h->count, h->sp_team, h->opt.max_rounds, &h->sp->queue,
@@ -940,7 +939,7 @@ mhs_status build_sparse(mhs_instance *h, SpTotals *found, bool *pays) {
     double pairs = 0;
     for (const HostInst &i : h->hinst)
         pairs += (double)i.m0 * i.m0 + (double)i.n0 * i.n0;
-    *pays = !host->leave && sparse_pays((double)host->cost, (double)host->open, pairs);
+    *pays = sparse_pays((double)host->cost, (double)host->open, pairs);
     return MHS_OK;
 }
 
@@ -956,8 +955,9 @@ const char *status_text(int32_t st) {
 // The end of a load on the sparse path (inputs and states are on their
 // way): build and checks.  *again: the
 // instance is better contracted (the caller loads it again on that path).
-// On an error or *again the caller destroys the handle.
-mhs_status finish_sparse(mhs_instance *h, bool *again) {
+// On an error or *again the caller destroys the handle.  *could: the lists take
+// it all the same, should the contraction find no memory; force: that it did.
+mhs_status finish_sparse(mhs_instance *h, bool force, bool *again, bool *could) {
     SpTotals found;
     bool pays = true;
     mhs_status st = build_sparse(h, &found, &pays);
@@ -980,7 +980,8 @@ mhs_status finish_sparse(mhs_instance *h, bool *again) {
                             chk[b].status, status_text(chk[b].status));
         return fail(MHS_ECUDA, "batch device load: status read back inconsistent");
     }
-    *again = !pays;
+    *could = !found.leave;
+    *again = found.leave || (!pays && !force);
     return MHS_OK;
 }
 
@@ -1302,7 +1303,8 @@ mhs_status mhs::solve_sparse_group(const mhs_options &opt, cudaStream_t stream,
             CUDA_TRY(cudaMemcpyAsync(h->arena + h->in_f, in + 4 * (sum_m1 + sum_z),
                                      4 * (size_t)sum_m, cudaMemcpyHostToDevice, h->stream));
         CUDA_TRY(upload_states(h));
-        mhs_status st2 = finish_sparse(h, again);
+        bool could = false;
+        mhs_status st2 = finish_sparse(h, false, again, &could);
         if (st2 || *again) return st2;
         st2 = run_sparse(h, 0, nullptr);
         if (st2) return st2;
@@ -1420,12 +1422,17 @@ mhs_status mhs_load(int32_t n, int32_t m, const int32_t *edge_ptr, const int32_t
     bool sparse = auto_sparse(opt) && sparse_may_pay(1, &n, &m, &nnz);
     const mhs_options exact = exact_form(opt);
     const bool choose = auto_sparse(opt);
+    bool could = false, force = false;  // finish_sparse
     for (;;) {
         if (choose && !sparse && any_big(demand, m)) opt = &exact;
         std::vector<Layout> lay;
         int64_t tmoff = 0;
         mhs_instance *h = nullptr;
         mhs_status st = create(1, &n, &m, &nnz, &k, opt, cuda_stream, &h, lay, tmoff, sparse);
+        if (st == MHS_ENOMEM && !sparse && could) {
+            force = sparse = true;
+            continue;
+        }
         if (st) {
             pinned_give(stage, stage_cls);
             return st;
@@ -1469,7 +1476,7 @@ mhs_status mhs_load(int32_t n, int32_t m, const int32_t *edge_ptr, const int32_t
         }
         bool again = false;
         if (sparse && upload_states(h) != cudaSuccess) st = fail(MHS_ECUDA, "state copy failed");
-        else st = sparse ? finish_sparse(h, &again) : finish_load(h, tmoff);
+        else st = sparse ? finish_sparse(h, force, &again, &could) : finish_load(h, tmoff);
         if (st == MHS_OK && !sparse && cudaStreamSynchronize(h->stream) != cudaSuccess)
             st = fail(MHS_ECUDA, "load failed: %s", cudaGetErrorString(cudaGetLastError()));
         if (st) {
@@ -1503,11 +1510,16 @@ mhs_status mhs_load_device(int32_t n, int32_t m, const int32_t *edge_ptr, const 
     int64_t nnz = nnz32;
     const mhs_options exact = exact_form(opt);
     const bool choose = auto_sparse(opt);
-    for (bool sparse = choose && sparse_may_pay(1, &n, &m, &nnz);; sparse = false) {
+    bool could = false, force = false;  // finish_sparse
+    for (bool sparse = choose && sparse_may_pay(1, &n, &m, &nnz);; sparse = force) {
         std::vector<Layout> lay;
         int64_t tmoff = 0;
         mhs_instance *h = nullptr;
         mhs_status st = create(1, &n, &m, &nnz, &k, opt, cuda_stream, &h, lay, tmoff, sparse);
+        if (st == MHS_ENOMEM && !sparse && could) {
+            force = true;
+            continue;
+        }
         if (st) return st;
         InstState &s = h->hstate[0];
         cudaError_t e = cudaMemcpyAsync(const_cast<int32_t *>(s.eptr), edge_ptr,
@@ -1521,7 +1533,7 @@ mhs_status mhs_load_device(int32_t n, int32_t m, const int32_t *edge_ptr, const 
         bool again = false;
         if (e == cudaSuccess && sparse) e = upload_states(h);
         if (e == cudaSuccess && sparse) {
-            st = finish_sparse(h, &again);
+            st = finish_sparse(h, force, &again, &could);
             if (st || again) {
                 destroy(h);
                 if (st) return st;
@@ -1667,13 +1679,18 @@ mhs_status mhs_load_batch(int32_t count, const int32_t *n, const int32_t *m,
     const bool choose = auto_sparse(opt);
     bool sparse = choose && sparse_may_pay(count, n, m, nnz.data());
     const mhs_options exact = exact_form(opt);
-    for (bool first = true;; first = false, sparse = false) {
+    bool could = false, force = false;  // finish_sparse
+    for (bool first = true;; first = false, sparse = force) {
         if (choose && !sparse && any_big(demand, sum_m)) opt = &exact;
         std::vector<Layout> lay;
         int64_t tmoff = 0;
         mhs_instance *h = nullptr;
         mhs_status st =
             create(count, n, m, nnz.data(), k, opt, cuda_stream, &h, lay, tmoff, sparse);
+        if (st == MHS_ENOMEM && !sparse && could) {
+            force = true;
+            continue;
+        }
         if (st) {  // a malformed input is reported first, as a check before the allocation would
             const std::string msg = g_err;
             const mhs_status vst = first ? finish_checks() : MHS_OK;
@@ -1729,7 +1746,7 @@ mhs_status mhs_load_batch(int32_t count, const int32_t *n, const int32_t *m,
         }
         bool again = false;
         if (sparse && upload_states(h) != cudaSuccess) st = fail(MHS_ECUDA, "state copy failed");
-        else st = sparse ? finish_sparse(h, &again) : finish_load(h, tmoff);
+        else st = sparse ? finish_sparse(h, force, &again, &could) : finish_load(h, tmoff);
         if (st == MHS_OK && !sparse && cudaStreamSynchronize(h->stream) != cudaSuccess)
             st = fail(MHS_ECUDA, "load failed");
         if (st) {
@@ -1804,12 +1821,17 @@ mhs_status mhs_load_batch_device(int32_t count, const int32_t *n, const int32_t 
     }
     const mhs_options exact = exact_form(opt);
     const bool choose = auto_sparse(opt);
-    for (bool sparse = choose && sparse_may_pay(count, n, m, nnz.data());; sparse = false) {
+    bool could = false, force = false;  // finish_sparse
+    for (bool sparse = choose && sparse_may_pay(count, n, m, nnz.data());; sparse = force) {
         std::vector<Layout> lay;
         int64_t tmoff = 0;
         mhs_instance *h = nullptr;
         mhs_status st =
             create(count, n, m, nnz.data(), k, opt, cuda_stream, &h, lay, tmoff, sparse);
+        if (st == MHS_ENOMEM && !sparse && could) {
+            force = true;
+            continue;
+        }
         if (st) {
             cudaFreeAsync(tmp, cs);
             return st;
@@ -1826,7 +1848,7 @@ mhs_status mhs_load_batch_device(int32_t count, const int32_t *n, const int32_t 
         if (e == cudaSuccess) e = launch_localize_ptr(h->dstate, count, edge_ptr, tmp, h->stream);
         if (e == cudaSuccess && sparse) {
             bool again = false;
-            st = finish_sparse(h, &again);
+            st = finish_sparse(h, force, &again, &could);
             if (st || !again) cudaFreeAsync(tmp, h->stream);
             if (st || again) {
                 destroy(h);

@@ -450,3 +450,40 @@ def test_large_demands_where_the_lists_do_not_pay(mhs, rule, fe):
                 assert got["forced"].tolist() == ref["forced"].tolist()
         st = srv.stats()
     assert st["completed"] == len(tickets) and st["active"] == 0 and st["bytes_in_use"] == 0
+
+
+def test_no_memory_for_the_contraction():
+    """A load whose lists do not pay stays on them where the operands of the
+    contraction (9.8 GB here) find no memory.  (A process of its own, most of the
+    card's memory taken; nothing cached by other tests.)"""
+    import subprocess
+    import sys
+    code = """
+import numpy as np, torch
+from oracle import oracle as O
+from paper_2109_06042_gb300 import instances as I, mhs
+rng = np.random.Generator(np.random.PCG64(70))
+n = m = 70000
+rows = [np.unique(r) for r in rng.integers(0, n, (m, 3))] + [np.sort(rng.choice(n, 6000, replace=False))]
+inst = I.from_edges(n, rows, np.append([min(2, len(r)) for r in rows[:-1]], 6000), k=3)
+ref = O.reduce(inst)
+d = [torch.from_numpy(np.ascontiguousarray(a, np.int32)).cuda() for a in (inst.edge_ptr, inst.edge_vtx, inst.demand)]
+fill = torch.empty(torch.cuda.mem_get_info()[0] - (6 << 30), dtype=torch.uint8, device='cuda')
+for load in (lambda: mhs.Instance.load(inst), lambda: mhs.Instance.load_device(n, inst.m, *d, inst.k),
+             lambda: mhs.Instance.load_batch([inst])):
+    with load() as h:
+        h.kernelize()
+        got = h.result()
+    for key in ('vertices', 'edges', 'demands'):
+        assert got[key].tolist() == ref[key].tolist(), key
+    assert got['rounds'] == ref['rounds']
+try:
+    mhs.kernelize(inst, contraction='fp8')
+    raise SystemExit('the contraction found memory')
+except mhs.MhsError as e:
+    assert e.status == mhs.MHS_ENOMEM
+"""
+    import os
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
